@@ -224,7 +224,7 @@ int run_ssd(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, const voi
         if (rc != SWIMBA_OK) return fail(h, rc, "SSD tile kernel launch failed");
         return SWIMBA_OK;
     }
-    int rc = launch_ssd_sequential(ctx, c.dtype, x, BC, false, dt, w->A, w->dt_bias, w->D, h0, B, L,
+    int rc = launch_ssd_sequential(ctx, c.dtype, x, BC, dt, w->A, w->dt_bias, w->D, h0, B, L,
                                    c.n_heads, c.head_dim, c.d_state, c.n_groups, y, h_final);
     if (rc != SWIMBA_OK) return fail(h, rc, "SSD launch failed");
     return SWIMBA_OK;
@@ -746,7 +746,7 @@ int swimba_forward_packed(swimba_handle *h, const swimba_weights *w, const void 
                     continue;
                 }
                 rc = launch_ssd_sequential(ctx, c.dtype, (const char *)x + t0 * HP * es, (const char *)BC + t0 * S * es,
-                                           false, dt ? dt + t0 * c.n_heads : nullptr, w->A, w->dt_bias, w->D, hin, 1,
+                                           dt ? dt + t0 * c.n_heads : nullptr, w->A, w->dt_bias, w->D, hin, 1,
                                            len, c.n_heads, c.head_dim, c.d_state, c.n_groups,
                                            (char *)y + t0 * HP * es, hf);
                 if (rc != SWIMBA_OK) rc = fail(h, rc, "SSD launch failed");

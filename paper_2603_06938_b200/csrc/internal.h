@@ -129,11 +129,11 @@ int launch_gated_rmsnorm(LaunchCtx &ctx, int dtype, const void *y, const void *z
                          int64_t T, int D, int ngroups, float eps, void *out);
 int launch_dt_columns(LaunchCtx &ctx, int dtype, const void *zxdt, int64_t ld, int off, int64_t T, int H, float *dt);
 
-// Per-timestep SIMT evaluation of the recurrence (fp32 state in registers).
-int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *BC, bool bc_fp32,
-                          const float *dt, const float *A, const float *dt_bias, const float *D,
-                          const float *h0, int B, int L, int H, int P, int N, int G, void *y,
-                          float *h_final);
+// Chunked CUDA-core evaluation of the recurrence (fp32 arithmetic): the fp32 path and the bf16 shapes
+// the tile kernel does not take.
+int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *BC, const float *dt, const float *A,
+                          const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int P, int N,
+                          int G, void *y, float *h_final);
 
 // The per-timestep evaluation over n listed sequences of a packed batch (bf16 streams): seq_tab[i] =
 // (first token, tokens, sequence index, 0), a device array; x, BC, dt, y are the packed arrays, h0 /

@@ -821,6 +821,8 @@ project_mix_simt_kernel(const T *__restrict__ u, const T *__restrict__ W_e,
 {
     // (kst, joff): the k experts of token t are entries t*kst + joff .. + k - 1 of idx / w and the
     // output row is t*(kst/k) + joff/k ... used with k = 1, joff = j to write unmixed slots
+    grid_dep_launch();
+    grid_dep_wait();
     const int lane = threadIdx.x & 31;
     const int nblk = ceil_div(S, RW);
     const int64_t wid = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -886,9 +888,8 @@ static int launch_pm(LaunchCtx &ctx, const void *u, const void *W_e, const int32
     const int64_t nw = T_ * ceil_div(S, RW);
     dim3 grid((unsigned)ceil_div64(nw, warps)), block(warps * 32);
     ctx.begin(STAGE_PROJECT_SIMT);
-    project_mix_simt_kernel<T, TO, RW><<<grid, block, 0, ctx.stream>>>(
-        (const T *)u, (const T *)W_e, idx, w, T_, F, S, k, (TO *)BC, E, ctx.check_indices ? 1 : 0, ctx.d_status,
-        kst, joff);
+    launch_kernel(project_mix_simt_kernel<T, TO, RW>, grid, block, 0, ctx.stream, true, (const T *)u, (const T *)W_e,
+                  idx, w, T_, F, S, k, (TO *)BC, E, ctx.check_indices ? 1 : 0, ctx.d_status, kst, joff);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }

@@ -6,6 +6,331 @@
 
 namespace swimba {
 
+// Chunked evaluation on the CUDA cores (fp32 arithmetic throughout): the fp32 path of the forward and
+// the bf16 shapes that the tensor-core kernel does not take.  A cluster of up to eight CTAs owns one
+// (sequence, head); every CTA takes a run of CK_Q consecutive tokens, all CTAs at once:
+//   S_c[n,p] = sum_s w_s Btilde_s[n] x_s[p],  w_s = Delta_s exp(l_last - l_s)     local end state
+//   G[i,s]   = (Ctilde_i . Btilde_s) Delta_s exp(l_i - l_s)  for s <= i, else 0
+// then the local end states and decays are exchanged through distributed shared memory,
+//   H <- decay_r H + S_r  over the runs in front of this one,
+// and  y_i = exp(l_i) Ctilde_i^T H + sum_s G[i,s] x_s + D x_i.  Longer sequences repeat this with the
+// carried state (every CTA keeps its own copy).  All exponents are <= 0 and are formed from cumulative
+// sums in fp64, so a product of decays is rounded once.
+// What bounds it: the latency of a handful of dependent phases (load, G and S, exchange, y); the
+// arithmetic of a run is about 0.1 us of the SM.  One step per token with the state in registers
+// needed 0.66 us per token: 8 heads of 256 tokens (P = 64, N = 16) 168 us, this kernel 11 us.
+constexpr int CK_Q = 32;          // tokens per CTA and round
+constexpr int CK_THREADS = 256;
+constexpr int CK_MAX_CLUSTER = 8;
+
+namespace {
+__device__ __forceinline__ float4 ck_load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 ck_load4(const __nv_bfloat16 *p)
+{
+    const uint2 raw = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
+                       __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
+}
+__device__ __forceinline__ void ck_store4(float *p, const float (&v)[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void ck_store4(__nv_bfloat16 *p, const float (&v)[4])
+{
+    *reinterpret_cast<uint2 *>(p) = make_uint2(tc::pack_bf16x2(v[0], v[1]), tc::pack_bf16x2(v[2], v[3]));
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float4 cluster_load4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float cluster_load(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void fma4(float4 &acc, float a, const float4 &v)
+{
+    acc.x = fmaf(a, v.x, acc.x);
+    acc.y = fmaf(a, v.y, acc.y);
+    acc.z = fmaf(a, v.z, acc.z);
+    acc.w = fmaf(a, v.w, acc.w);
+}
+
+struct ChunkSmem {                 // offsets in floats; rows padded to whole float4s
+    int B, C, x, G, S, H, total;
+};
+__host__ __device__ inline ChunkSmem chunk_smem(int P, int N)
+{
+    const int Pp = (P + 3) & ~3;
+    ChunkSmem m;
+    int off = 0;
+    m.B = off; off += CK_Q * (N + 4);
+    m.C = off; off += CK_Q * (N + 4);
+    m.x = off; off += CK_Q * Pp;
+    m.G = off; off += CK_Q * (CK_Q + 4);
+    m.S = off; off += N * Pp;
+    m.H = off; off += N * Pp;
+    m.total = off;
+    return m;
+}
+}  // namespace
+
+template <typename T>
+__global__ void __launch_bounds__(CK_THREADS)
+ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float *__restrict__ dt,
+                 const float *__restrict__ A, const float *__restrict__ dt_bias, const float *__restrict__ D,
+                 const float *__restrict__ h0, int L, int H, int P, int N, int G, int ncta, T *__restrict__ y,
+                 float *__restrict__ h_final)
+{
+    extern __shared__ __align__(16) float csm[];
+    __shared__ double s_l[CK_Q];
+    __shared__ float s_delta[CK_Q], s_w[CK_Q], s_e[CK_Q];
+    __shared__ float s_decay;
+    const ChunkSmem m = chunk_smem(P, N);
+    float *sB = csm + m.B, *sC = csm + m.C, *sx = csm + m.x, *sG = csm + m.G, *sS = csm + m.S, *sH = csm + m.H;
+    const int Pp = (P + 3) & ~3, pq = Pp >> 2, Nr = N + 4, Gr = CK_Q + 4;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (int)(blockIdx.x % ncta);
+    const int64_t bh = blockIdx.x / ncta;
+    const int b = (int)(bh / H), h = (int)(bh % H);
+    const int g = h / (H / G), S = 2 * G * N;
+    const bool vec = (P & 3) == 0;
+    grid_dep_launch();
+    grid_dep_wait();
+    const double Ah = (double)A[h];
+    const float bias = dt_bias[h], Dh = D ? D[h] : 0.f;
+    const float *h0p = h0 ? h0 + bh * P * N : nullptr;
+    const int nrounds = ceil_div(L, CK_Q * ncta);
+    for (int rd = 0; rd < nrounds; ++rd) {
+        const int t0 = (rd * ncta + rank) * CK_Q;
+        const int nt = max(0, min(CK_Q, L - t0));
+        const int64_t tok0 = (int64_t)b * L + t0;
+        // ---- this run's rows; rows past the end are zero
+        for (int i = tid; i < CK_Q * (N >> 2); i += CK_THREADS) {
+            const int tt = i / (N >> 2), c = (i - tt * (N >> 2)) * 4;
+            float4 vb = make_float4(0.f, 0.f, 0.f, 0.f), vc = vb;
+            if (tt < nt) {
+                const T *row = BC + (tok0 + tt) * S + g * N + c;
+                vb = ck_load4(row);
+                vc = ck_load4(row + G * N);
+            }
+            *reinterpret_cast<float4 *>(sB + tt * Nr + c) = vb;
+            *reinterpret_cast<float4 *>(sC + tt * Nr + c) = vc;
+        }
+#pragma unroll 2
+        for (int i = tid; i < CK_Q * pq; i += CK_THREADS) {
+            const int tt = i / pq, c = (i - tt * pq) * 4;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (tt < nt) {
+                const T *row = x + ((tok0 + tt) * H + h) * P + c;
+                if (vec) {
+                    v = ck_load4(row);
+                } else {
+                    v.x = to_f32<T>(row[0]);
+                    if (c + 1 < P) v.y = to_f32<T>(row[1]);
+                    if (c + 2 < P) v.z = to_f32<T>(row[2]);
+                    if (c + 3 < P) v.w = to_f32<T>(row[3]);
+                }
+            }
+            *reinterpret_cast<float4 *>(sx + tt * Pp + c) = v;
+        }
+        if (warp == 0) {
+            const float d = lane < nt ? softplus_f((dt ? dt[(tok0 + lane) * H + h] : 0.f) + bias) : 0.f;
+            double l = (double)d * Ah;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double nb = __shfl_up_sync(0xffffffffu, l, o);
+                if (lane >= o) l += nb;
+            }
+            const double l_last = __shfl_sync(0xffffffffu, l, 31);
+            s_l[lane] = l;
+            s_delta[lane] = d;
+            s_w[lane] = d * expf((float)(l_last - l));
+            s_e[lane] = expf((float)l);
+            if (lane == 31) s_decay = expf((float)l);
+        }
+        if (rd == 0) {                       // the carried state, [n][p]
+            for (int i = tid; i < N * Pp; i += CK_THREADS) {
+                const int p = i / N, n = i - p * N;
+                sH[n * Pp + p] = (h0p && p < P) ? h0p[(int64_t)p * N + n] : 0.f;
+            }
+        }
+        __syncthreads();
+        // ---- local end state, two state rows x four channels per thread and step
+        for (int i = tid; i < (N >> 1) * pq; i += CK_THREADS) {
+            const int nn = (i / pq) * 2, c = (i % pq) * 4;
+            float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+#pragma unroll 8
+            for (int s = 0; s < CK_Q; ++s) {
+                const float w = s_w[s];
+                const float2 bv = *reinterpret_cast<const float2 *>(sB + s * Nr + nn);
+                const float4 xv = *reinterpret_cast<const float4 *>(sx + s * Pp + c);
+                fma4(a0, w * bv.x, xv);
+                fma4(a1, w * bv.y, xv);
+            }
+            *reinterpret_cast<float4 *>(sS + nn * Pp + c) = a0;
+            *reinterpret_cast<float4 *>(sS + (nn + 1) * Pp + c) = a1;
+        }
+        // ---- G: warp = rows i, lane = column s
+        for (int i = warp; i < CK_Q; i += CK_THREADS / 32) {
+            float v = 0.f;
+            if (lane <= i) {
+                const float4 *cr = reinterpret_cast<const float4 *>(sC + i * Nr);
+                const float4 *br = reinterpret_cast<const float4 *>(sB + lane * Nr);
+                float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+                for (int c = 0; c < (N >> 2); ++c) {
+                    const float4 cv = cr[c], bv = br[c];
+                    d4.x = fmaf(cv.x, bv.x, d4.x);
+                    d4.y = fmaf(cv.y, bv.y, d4.y);
+                    d4.z = fmaf(cv.z, bv.z, d4.z);
+                    d4.w = fmaf(cv.w, bv.w, d4.w);
+                }
+                v = ((d4.x + d4.y) + (d4.z + d4.w)) * s_delta[lane] * expf((float)(s_l[i] - s_l[lane]));
+            }
+            sG[i * Gr + lane] = v;
+        }
+        if (ncta > 1) cluster_sync();
+        else __syncthreads();
+        // ---- state entering this run: the runs in front of it, in order
+        const uint32_t s_addr = tc::smem_u32(sS), d_addr = tc::smem_u32(&s_decay);
+        for (int r = 0; r < rank; ++r) {
+            const float dr = cluster_load(cluster_addr(d_addr, r));
+            const uint32_t ra = cluster_addr(s_addr, r);
+#pragma unroll 4
+            for (int i = tid; i < N * pq; i += CK_THREADS) {
+                float4 cur = reinterpret_cast<float4 *>(sH)[i];
+                const float4 v = cluster_load4(ra + i * 16);
+                cur.x = fmaf(dr, cur.x, v.x);
+                cur.y = fmaf(dr, cur.y, v.y);
+                cur.z = fmaf(dr, cur.z, v.z);
+                cur.w = fmaf(dr, cur.w, v.w);
+                reinterpret_cast<float4 *>(sH)[i] = cur;
+            }
+        }
+        __syncthreads();
+        // ---- y: two tokens x four channels per thread and step
+        for (int i = tid; i < (CK_Q / 2) * pq; i += CK_THREADS) {
+            const int i0 = (i / pq) * 2, c = (i % pq) * 4;
+            if (i0 >= nt) continue;
+            float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+#pragma unroll 2
+            for (int n = 0; n < N; n += 4) {
+                const float4 c0 = *reinterpret_cast<const float4 *>(sC + i0 * Nr + n);
+                const float4 c1 = *reinterpret_cast<const float4 *>(sC + (i0 + 1) * Nr + n);
+                const float cv0[4] = {c0.x, c0.y, c0.z, c0.w}, cv1[4] = {c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 hv = *reinterpret_cast<const float4 *>(sH + (n + q) * Pp + c);
+                    fma4(a0, cv0[q], hv);
+                    fma4(a1, cv1[q], hv);
+                }
+            }
+            const float e0 = s_e[i0], e1 = s_e[i0 + 1];
+            a0.x *= e0; a0.y *= e0; a0.z *= e0; a0.w *= e0;
+            a1.x *= e1; a1.y *= e1; a1.z *= e1; a1.w *= e1;
+            for (int s = 0; s <= i0 + 1; s += 4) {          // (G is zero past the diagonal)
+                const float4 g0 = *reinterpret_cast<const float4 *>(sG + i0 * Gr + s);
+                const float4 g1 = *reinterpret_cast<const float4 *>(sG + (i0 + 1) * Gr + s);
+                const float gv0[4] = {g0.x, g0.y, g0.z, g0.w}, gv1[4] = {g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 xv = *reinterpret_cast<const float4 *>(sx + (s + q) * Pp + c);
+                    fma4(a0, gv0[q], xv);
+                    fma4(a1, gv1[q], xv);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                if (i0 + r >= nt) break;
+                float4 v = r ? a1 : a0;
+                fma4(v, Dh, *reinterpret_cast<const float4 *>(sx + (i0 + r) * Pp + c));
+                T *dst = y + ((tok0 + i0 + r) * H + h) * P + c;
+                const float o[4] = {v.x, v.y, v.z, v.w};
+                if (vec) {
+                    ck_store4(dst, o);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (c + q < P) dst[q] = from_f32<T>(o[q]);
+                }
+            }
+        }
+        // ---- the state after this round (carried on, or the call's end state)
+        if (rd + 1 < nrounds || (h_final && rank == 0)) {
+            __syncthreads();                                 // (y has read the entry state)
+            for (int r = rank; r < ncta; ++r) {
+                const float dr = cluster_load(cluster_addr(d_addr, r));
+                const uint32_t ra = cluster_addr(s_addr, r);
+#pragma unroll 4
+                for (int i = tid; i < N * pq; i += CK_THREADS) {
+                    float4 cur = reinterpret_cast<float4 *>(sH)[i];
+                    const float4 v = cluster_load4(ra + i * 16);
+                    cur.x = fmaf(dr, cur.x, v.x);
+                    cur.y = fmaf(dr, cur.y, v.y);
+                    cur.z = fmaf(dr, cur.z, v.z);
+                    cur.w = fmaf(dr, cur.w, v.w);
+                    reinterpret_cast<float4 *>(sH)[i] = cur;
+                }
+            }
+        }
+        // the local end states have been read by everyone (and no CTA leaves while it is being read)
+        if (ncta > 1) cluster_sync();
+        else __syncthreads();
+    }
+    if (h_final && rank == 0) {
+        float *dst = h_final + bh * P * N;
+        for (int i = tid; i < P * N; i += CK_THREADS) {
+            const int p = i / N, n = i - p * N;
+            dst[i] = sH[n * Pp + p];
+        }
+    }
+}
+
+template <typename T>
+static int launch_chunk_t(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
+                          const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int P, int N,
+                          int G, void *y, float *h_final)
+{
+    // as many CTAs per (sequence, head) as it has runs of CK_Q tokens, a power of two up to eight (the
+    // portable cluster size)
+    int ncta = 1;
+    while (ncta < CK_MAX_CLUSTER && ncta * CK_Q < L) ncta <<= 1;
+    const size_t smem = (size_t)chunk_smem(P, N).total * sizeof(float);
+    auto kern = ssd_chunk_kernel<T>;
+    if (smem > 40 * 1024 && !ensure_dynamic_smem((const void *)kern, smem)) return SWIMBA_ERR_CUDA;
+    ctx.begin(STAGE_SSD_SEQUENTIAL);
+    launch_kernel_cluster(kern, dim3((unsigned)((int64_t)B * H * ncta)), dim3(CK_THREADS), smem, ctx.stream, true,
+                          (unsigned)ncta, (const T *)x, (const T *)BC, dt, A, dt_bias, D, h0, L, H, P, N, G, ncta,
+                          (T *)y, h_final);
+    ctx.end();
+    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+}
+
+int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *BC, const float *dt, const float *A,
+                          const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int P, int N,
+                          int G, void *y, float *h_final)
+{
+    if (B <= 0 || L <= 0) return SWIMBA_OK;
+    if (dtype == SWIMBA_DTYPE_FP32)
+        return launch_chunk_t<float>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, y, h_final);
+    return launch_chunk_t<__nv_bfloat16>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, y, h_final);
+}
+
 constexpr int SEQ_TS = 32;   // tokens staged in shared memory per round
 constexpr int SEQ_NT = 16;   // state entries per thread
 
@@ -123,19 +448,6 @@ static int launch_seq_t(LaunchCtx &ctx, const void *x, const void *BC, const flo
                                              L, H, P, N, G, NS, (T *)y, h_final, seq_tab);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
-}
-
-int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *BC, bool bc_fp32,
-                          const float *dt, const float *A, const float *dt_bias, const float *D,
-                          const float *h0, int B, int L, int H, int P, int N, int G, void *y,
-                          float *h_final)
-{
-    if (B <= 0 || L <= 0) return SWIMBA_OK;
-    if (dtype == SWIMBA_DTYPE_FP32)
-        return launch_seq_t<float, float>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, y, h_final);
-    if (bc_fp32)
-        return launch_seq_t<__nv_bfloat16, float>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, y, h_final);
-    return launch_seq_t<__nv_bfloat16, __nv_bfloat16>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, y, h_final);
 }
 
 // The same over a list of sequences of a packed batch (device table of n entries: first token,
