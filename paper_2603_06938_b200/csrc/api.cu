@@ -430,6 +430,14 @@ int swimba_ssd_slots(swimba_handle *h, const swimba_weights *w, const void *x_sl
     // ordinary evaluation each, with slot j's own injection stream and input and the readout stream
     // mixed over all slots; the initial state enters through slot 0 only.  No skip term: the
     // paper's output equation has none, and with expert-specific inputs there is no single x.
+    if (ssd_tiles_supported(c.dtype, c.head_dim, c.d_state)) {
+        rc = launch_ssd_slots_tiles(ctx, x_slots, BC_slots, dt, w->A, w->dt_bias, h0, B, L, c.n_heads, c.n_groups, k,
+                                    c.chunk, h->sm_count, y, h_final, bcj, ws + l.ssd);
+        if (rc != SWIMBA_OK) fail(h, rc, "SSD tile kernel launch failed");
+        h->last_stream = ctx.stream;
+        h->last_launches = ctx.launches;
+        return rc;
+    }
     swimba_weights wj = *w;
     wj.D = nullptr;
     for (int j = 0; j < k && rc == SWIMBA_OK; ++j) {

@@ -69,6 +69,21 @@ int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float 
                      int chunk, int sm_count, void *y, float *h_final, void *workspace,
                      bool scalars_done);
 
+// One bf16 stream of G*N entries per token, rows ld elements apart.
+struct SsdStream {
+    const void *p;
+    int64_t ld;
+};
+// The same with the injection and readout streams given apart; add: y and h_final are added to.
+int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs, const SsdStream &Cs, const float *dt,
+                             const float *A, const float *dt_bias, const float *D, const float *h0, int B, int L,
+                             int H, int G, int chunk, int sm_count, void *y, float *h_final, void *workspace,
+                             bool scalars_done, bool add);
+// The general form on the tile kernel: k evaluations (one per slot) added up; cmix: T*G*N bf16 scratch.
+int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_slots, const float *dt, const float *A,
+                           const float *dt_bias, const float *h0, int B, int L, int H, int G, int k, int chunk,
+                           int sm_count, void *y, float *h_final, void *cmix, void *workspace);
+
 // The same over a packed batch: nseq sequences back to back in [T, ...] arrays, sequence b holding
 // tokens cu[b] .. cu[b+1]-1 (cu is a HOST array of nseq + 1 entries, read before the call returns).
 // h0 / h_final are [nseq, H, P, N].  The step sizes are produced inside the call.

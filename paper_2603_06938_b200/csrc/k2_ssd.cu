@@ -91,6 +91,8 @@ struct SsdParams {
     const int2 *items;
     int ntile_total, seg_states;
     void *y;
+    // 1: y and h_out are added to, not overwritten (the slots behind the first of the general form)
+    int add;
 };
 
 struct __align__(8) HeadBars {
@@ -218,8 +220,9 @@ __device__ __forceinline__ void scale_own_row(const uint8_t *s_x, uint8_t *s_xp,
 
 template <bool SPLIT>
 __global__ void __launch_bounds__(SSD_THREADS, 1)
-ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_constant__ CUtensorMap tmap_x,
-                 const __grid_constant__ CUtensorMap tmap_y, const SsdParams prm)
+ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_c,
+                 const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_y,
+                 const SsdParams prm)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     SsdSmall *sm = (SsdSmall *)(smem + SM_SMALL);
@@ -297,7 +300,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_const
         tc::tmem_relinquish();
     }
     if (warp == WARP_TMA && lane == 0) {
-        tc::prefetch_tmap(&tmap_bc);
+        tc::prefetch_tmap(&tmap_b);
+        tc::prefetch_tmap(&tmap_c);
         tc::prefetch_tmap(&tmap_x);
         tc::prefetch_tmap(&tmap_y);
     }
@@ -337,11 +341,11 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_const
             if (leader) {
                 tc::mbar_arrive_expect_tx(&bars->cb_full, full ? 4 * SLAB : 2 * SLAB);
                 if (full) {
-                    tc::tma_load_3d(smem + SM_CB + 0 * SLAB, &tmap_bc, &bars->cb_full, (prm.G + g) * SN, t0, bco);
-                    tc::tma_load_3d(smem + SM_CB + 1 * SLAB, &tmap_bc, &bars->cb_full, (prm.G + g) * SN + 64, t0, bco);
+                    tc::tma_load_3d(smem + SM_CB + 0 * SLAB, &tmap_c, &bars->cb_full, g * SN, t0, bco);
+                    tc::tma_load_3d(smem + SM_CB + 1 * SLAB, &tmap_c, &bars->cb_full, g * SN + 64, t0, bco);
                 }
-                tc::tma_load_3d(smem + SM_CB + 2 * SLAB, &tmap_bc, &bars->cb_full, g * SN, t0, bco);
-                tc::tma_load_3d(smem + SM_CB + 3 * SLAB, &tmap_bc, &bars->cb_full, g * SN + 64, t0, bco);
+                tc::tma_load_3d(smem + SM_CB + 2 * SLAB, &tmap_b, &bars->cb_full, g * SN, t0, bco);
+                tc::tma_load_3d(smem + SM_CB + 3 * SLAB, &tmap_b, &bars->cb_full, g * SN + 64, t0, bco);
             }
             if (j + 1 < ntiles) {                            // X one tile ahead
                 const int jn = j + 1, sx = jn & 1;
@@ -482,7 +486,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_const
                     // by the compute warps, the rows behind it belong to the next sequence)
                     tc::mbar_wait(&hb->y_staged, jf & 1, abort_flag, d_status);
                     if (leader && !(packed && t_begin + (j + 1) * ST > L)) {
-                        tc::tma_store_4d(&tmap_y, s_y, 0, head0 + hd, tok0 + t_begin + j * ST, bco);
+                        if (prm.add) tc::tma_reduce_add_4d(&tmap_y, s_y, 0, head0 + hd, tok0 + t_begin + j * ST, bco);
+                        else tc::tma_store_4d(&tmap_y, s_y, 0, head0 + hd, tok0 + t_begin + j * ST, bco);
                         tc::bulk_commit_group();
                     }
                     __syncwarp();
@@ -750,6 +755,10 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_const
         if (kfull) {
             if (prm.h_out && seg == nseg - 1 && !head_part) {
                 float *dst = prm.h_out + (((int64_t)b * H + h) * SP) * SN;
+                if (prm.add) {
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) Hst[q] += dst[(int64_t)(p0 + q) * SN + i];
+                }
 #pragma unroll
                 for (int q = 0; q < 32; ++q) dst[(int64_t)(p0 + q) * SN + i] = Hst[q];
             }
@@ -889,7 +898,7 @@ __host__ __device__ inline int quads_per_group(int H, int G) { return (H / G + N
 }  // namespace
 
 __global__ void __launch_bounds__(ST_THREADS, 1)
-ssd_state_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_constant__ CUtensorMap tmap_x,
+ssd_state_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_x,
                  const SsdParams prm)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -941,7 +950,7 @@ ssd_state_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_const
         tc::tmem_relinquish();
     }
     if (warp == 4 * NQ && lane == 0) {
-        tc::prefetch_tmap(&tmap_bc);
+        tc::prefetch_tmap(&tmap_b);
         tc::prefetch_tmap(&tmap_x);
     }
     tc::tc_fence_before();
@@ -962,8 +971,8 @@ ssd_state_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_const
                 uint8_t *stg = smem + s * ST_STAGE_BYTES;
                 const int t0 = tok0 + t_begin + q * HT;
                 tc::mbar_arrive_expect_tx(&sm->full[s], (2 + nh) * HSLAB + nh * (uint32_t)sizeof(TileScalars));
-                tc::tma_load_3d(stg, &tmap_bc, &sm->full[s], g * SN, t0, bco);
-                tc::tma_load_3d(stg + HSLAB, &tmap_bc, &sm->full[s], g * SN + 64, t0, bco);
+                tc::tma_load_3d(stg, &tmap_b, &sm->full[s], g * SN, t0, bco);
+                tc::tma_load_3d(stg + HSLAB, &tmap_b, &sm->full[s], g * SN + 64, t0, bco);
                 for (int hd = 0; hd < nh; ++hd) {
                     tc::tma_load_4d(stg + (2 + hd) * HSLAB, &tmap_x, &sm->full[s], 0, head0 + hd, t0, bco);
                     tc::bulk_load(&sm->sc[s][hd],
@@ -1063,21 +1072,33 @@ ssd_state_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_const
 
 static size_t ssd_state_smem_bytes() { return ST_SMALL + sizeof(StateSmall); }
 
-// The state-only launch behind both the dense and the packed segment passes.
-static int launch_state_pass(LaunchCtx &ctx, const void *x, const void *BC, int64_t rows, int nb, const SsdParams &p,
-                             unsigned grid_x, int H, int G, unsigned grid_z)
+// Tensor map over one mixed stream: nb x rows rows of G*N entries, boxes of 64 entries x box_rows rows.
+static bool stream_map(LaunchCtx &ctx, CUtensorMap *m, const SsdStream &s, int64_t rows, int nb, int G, int box_rows)
 {
-    // tensor maps with boxes of half a tile (64 tokens) over x [nb, rows, H, P] and BC [nb, rows, S]
-    CUtensorMap tm_bc, tm_x;
+    const uint64_t dims[3] = {(uint64_t)G * SN, (uint64_t)rows, (uint64_t)nb};
+    const uint64_t str[2] = {(uint64_t)s.ld * 2, (uint64_t)rows * s.ld * 2};
+    const uint32_t box[3] = {64, (uint32_t)box_rows, 1};
+    return encode_tmap_bf16_cached(ctx.tmaps, m, s.p, 3, dims, str, box);
+}
+
+// The two streams inside rows of mixed streams BC [rows, 2 G N].
+static SsdStream b_stream(const void *BC, int G) { return SsdStream{BC, 2 * (int64_t)G * SN}; }
+static SsdStream c_stream(const void *BC, int G)
+{
+    return SsdStream{(const __nv_bfloat16 *)BC + (int64_t)G * SN, 2 * (int64_t)G * SN};
+}
+
+// The state-only launch behind both the dense and the packed segment passes.
+static int launch_state_pass(LaunchCtx &ctx, const void *x, const SsdStream &Bs, int64_t rows, int nb,
+                             const SsdParams &p, unsigned grid_x, int H, int G, unsigned grid_z)
+{
+    // tensor maps with boxes of half a tile (64 tokens) over x [nb, rows, H, P] and Btilde
+    CUtensorMap tm_b, tm_x;
     {
-        const int S = 2 * G * SN;
-        const uint64_t dims3[3] = {(uint64_t)S, (uint64_t)rows, (uint64_t)nb};
-        const uint64_t str3[2] = {(uint64_t)S * 2, (uint64_t)rows * S * 2};
-        const uint32_t box3[3] = {64, (uint32_t)HT, 1};
         const uint64_t dims4[4] = {(uint64_t)SP, (uint64_t)H, (uint64_t)rows, (uint64_t)nb};
         const uint64_t str4[3] = {(uint64_t)SP * 2, (uint64_t)H * SP * 2, (uint64_t)rows * H * SP * 2};
         const uint32_t box4[4] = {SP, 1, (uint32_t)HT, 1};
-        if (!encode_tmap_bf16_cached(ctx.tmaps, &tm_bc, BC, 3, dims3, str3, box3) ||
+        if (!stream_map(ctx, &tm_b, Bs, rows, nb, G, HT) ||
             !encode_tmap_bf16_cached(ctx.tmaps, &tm_x, x, 4, dims4, str4, box4))
             return SWIMBA_ERR_CUDA;
     }
@@ -1085,7 +1106,7 @@ static int launch_state_pass(LaunchCtx &ctx, const void *x, const void *BC, int6
     if (!ensure_dynamic_smem((const void *)ssd_state_kernel, smem)) return SWIMBA_ERR_CUDA;
     ctx.begin(STAGE_SSD_STATE);
     launch_kernel(ssd_state_kernel, dim3(grid_x, (unsigned)(G * quads_per_group(H, G)), grid_z), dim3(ST_THREADS), smem,
-                  ctx.stream, true, tm_bc, tm_x, p);
+                  ctx.stream, true, tm_b, tm_x, p);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
@@ -1182,15 +1203,18 @@ int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float 
                      int chunk, int sm_count, void *y, float *h_final, void *workspace,
                      bool scalars_done)
 {
+    return launch_ssd_tiles_streams(ctx, x, b_stream(BC, G), c_stream(BC, G), dt, A, dt_bias, D, h0, B, L, H, G, chunk,
+                                    sm_count, y, h_final, workspace, scalars_done, false);
+}
+
+int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs, const SsdStream &Cs, const float *dt,
+                             const float *A, const float *dt_bias, const float *D, const float *h0, int B, int L,
+                             int H, int G, int chunk, int sm_count, void *y, float *h_final, void *workspace,
+                               bool scalars_done, bool add)
+{
     if (B <= 0 || L <= 0) return SWIMBA_OK;
-    const int S = 2 * G * SN;
-    CUtensorMap tm_bc, tm_x, tm_y;
-    {
-        const uint64_t dims[3] = {(uint64_t)S, (uint64_t)L, (uint64_t)B};
-        const uint64_t str[2] = {(uint64_t)S * 2, (uint64_t)L * S * 2};
-        const uint32_t box[3] = {64, ST, 1};
-        if (!encode_tmap_bf16_cached(ctx.tmaps, &tm_bc, BC, 3, dims, str, box)) return SWIMBA_ERR_CUDA;
-    }
+    CUtensorMap tm_b, tm_c, tm_x, tm_y;
+    if (!stream_map(ctx, &tm_b, Bs, L, B, G, ST) || !stream_map(ctx, &tm_c, Cs, L, B, G, ST)) return SWIMBA_ERR_CUDA;
     {
         const uint64_t dims[4] = {(uint64_t)SP, (uint64_t)H, (uint64_t)L, (uint64_t)B};
         const uint64_t str[3] = {(uint64_t)SP * 2, (uint64_t)H * SP * 2, (uint64_t)L * H * SP * 2};
@@ -1221,6 +1245,7 @@ int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float 
     p.L = L; p.Lpad = Lpad; p.H = H; p.G = G; p.nseg = nseg; p.seg_len = seg_len;
     p.d_status = ctx.d_status;
     p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = nseg > 1; p.y = y;
+    p.add = add ? 1 : 0;
     dim3 grid((unsigned)nseg, (unsigned)(G * pairs_per_group(H, G)), (unsigned)B);
     p.split_tiles = 0;
     if (nseg == 1) {
@@ -1229,9 +1254,9 @@ int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float 
         if (p.split_tiles > 0) grid = dim3((unsigned)B, (unsigned)(G * pairs_per_group(H, G)), 2u);
         ctx.begin(STAGE_SSD_TILES);
         if (p.split_tiles > 0)
-            launch_kernel(ssd_tiles_kernel<true>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_bc, tm_x, tm_y, p);
+            launch_kernel(ssd_tiles_kernel<true>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         else
-            launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_bc, tm_x, tm_y, p);
+            launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         ctx.end();
     } else {
         float *states = (float *)seg_ws;
@@ -1239,7 +1264,7 @@ int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float 
         p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY;
         {
             // (the last segment's end state is nobody's entry state: the full pass produces it)
-            const int rc = launch_state_pass(ctx, x, BC, L, B, p, (unsigned)(nseg - 1), H, G, (unsigned)B);
+            const int rc = launch_state_pass(ctx, x, Bs, L, B, p, (unsigned)(nseg - 1), H, G, (unsigned)B);
             if (rc != SWIMBA_OK) return rc;
         }
         const int PN4 = SP * SN / 4;
@@ -1249,8 +1274,72 @@ int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float 
         ctx.end();
         p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
         ctx.begin(STAGE_SSD_TILES);
-        launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_bc, tm_x, tm_y, p);
+        launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         ctx.end();
+    }
+    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+}
+
+// General form (expert-specific inputs): the readout stream is the sum of the k slots' readout halves,
+//   Cmix[t, :] = sum_j slots[t*k + j, GN:2GN]      (the slots carry their router weights)
+// and the same for every slot's evaluation, whose injection stream is read straight from the slots.  The
+// leading blocks compute the step sizes, which are shared by the slots too.
+__global__ void __launch_bounds__(256)
+slot_readout_kernel(const __nv_bfloat16 *__restrict__ slots, int64_t T, int GN, int k,
+                    __nv_bfloat16 *__restrict__ Cmix, int scalar_blocks, const ScalarsArgs scalars)
+{
+    grid_dep_wait();
+    grid_dep_launch();
+    if ((int)blockIdx.x < scalar_blocks) {
+        ssd_scalars_block(scalars, blockIdx.x);
+        return;
+    }
+    const int vpr = GN >> 3;
+    const int64_t n = T * vpr, stride = (int64_t)(gridDim.x - scalar_blocks) * blockDim.x;
+    for (int64_t i = (int64_t)(blockIdx.x - scalar_blocks) * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const int64_t t = i / vpr;
+        const int c = (int)(i - t * vpr) * 8;
+        const __nv_bfloat16 *src = slots + t * k * 2 * GN + GN + c;
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+        for (int j = 0; j < k; ++j) {
+            float v[8];
+            load8(src + (int64_t)j * 2 * GN, v);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc[q] += v[q];
+        }
+        *reinterpret_cast<uint4 *>(Cmix + t * GN + c) =
+            make_uint4(tc::pack_bf16x2(acc[0], acc[1]), tc::pack_bf16x2(acc[2], acc[3]),
+                       tc::pack_bf16x2(acc[4], acc[5]), tc::pack_bf16x2(acc[6], acc[7]));
+    }
+}
+
+// The layer as the sum over the slots of one evaluation each (the injection is linear in
+// (B^(e), X^(e))): slots behind the first add their y tile with the reducing TMA store and their end
+// state in place, so that no per-slot y exists. 8 x 2048 tokens of 24 heads, k = 2:
+// 240 us a call with a summing pass per slot and an assembled stream per slot, 147 us this way (bit-identical).
+int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_slots, const float *dt, const float *A,
+                           const float *dt_bias, const float *h0, int B, int L, int H, int G, int k, int chunk,
+                           int sm_count, void *y, float *h_final, void *cmix, void *workspace)
+{
+    if (B <= 0 || L <= 0) return SWIMBA_OK;
+    const int64_t T = (int64_t)B * L;
+    const int GN = G * SN;
+    const ScalarsArgs sa = ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace);
+    const int64_t extra = scalars_blocks(sa, 256);
+    int64_t blocks = ceil_div64(T * (GN / 8), 256);
+    if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
+    ctx.begin(STAGE_SLOT_STREAMS);
+    launch_kernel(slot_readout_kernel, dim3((unsigned)(extra + blocks)), dim3(256), 0, ctx.stream, true,
+                  (const __nv_bfloat16 *)BC_slots, T, GN, k, (__nv_bfloat16 *)cmix, (int)extra, sa);
+    ctx.end();
+    for (int j = 0; j < k; ++j) {
+        const SsdStream Bs{(const __nv_bfloat16 *)BC_slots + (int64_t)j * 2 * GN, (int64_t)k * 2 * GN};
+        const SsdStream Cs{cmix, GN};
+        const int rc = launch_ssd_tiles_streams(ctx, (const __nv_bfloat16 *)x_slots + (int64_t)j * T * H * SP, Bs, Cs, dt,
+                                                A, dt_bias, nullptr, j == 0 ? h0 : nullptr, B, L, H, G, chunk, sm_count,
+                                                y, h_final, workspace, true, j > 0);
+        if (rc != SWIMBA_OK) return rc;
     }
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
@@ -1377,14 +1466,9 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const void *x, const void *BC, const
     }
     if (pl.items.empty()) return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 
-    const int S = 2 * G * SN;
-    CUtensorMap tm_bc, tm_x, tm_y;
-    {
-        const uint64_t dims[3] = {(uint64_t)S, (uint64_t)T, 1};
-        const uint64_t str[2] = {(uint64_t)S * 2, (uint64_t)T * S * 2};
-        const uint32_t box[3] = {64, ST, 1};
-        if (!encode_tmap_bf16_cached(ctx.tmaps, &tm_bc, BC, 3, dims, str, box)) return SWIMBA_ERR_CUDA;
-    }
+    CUtensorMap tm_b, tm_c, tm_x, tm_y;
+    const SsdStream Bs = b_stream(BC, G), Cs = c_stream(BC, G);
+    if (!stream_map(ctx, &tm_b, Bs, T, 1, G, ST) || !stream_map(ctx, &tm_c, Cs, T, 1, G, ST)) return SWIMBA_ERR_CUDA;
     {
         const uint64_t dims[4] = {(uint64_t)SP, (uint64_t)H, (uint64_t)T, 1};
         const uint64_t str[3] = {(uint64_t)SP * 2, (uint64_t)H * SP * 2, (uint64_t)T * H * SP * 2};
@@ -1412,20 +1496,21 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const void *x, const void *BC, const
     p.seqs = (const SeqDesc *)(ws + lay.seqs);
     p.ntile_total = pl.total_tiles;
     p.y = y;
+    p.add = 0;
     const unsigned pairs = (unsigned)(G * pairs_per_group(H, G));
     if (!pl.segmented) {
         p.items = (const int2 *)(ws + lay.items);
         p.h_in = h0; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL; p.seg_states = 0;
         ctx.begin(STAGE_SSD_TILES);
         launch_kernel(ssd_tiles_kernel<false>, dim3((unsigned)pl.items.size(), pairs, 1), dim3(SSD_THREADS), smem,
-                      ctx.stream, true, tm_bc, tm_x, tm_y, p);
+                      ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         ctx.end();
     } else {
         float *states = (float *)(ws + lay.states);
         float *decay = (float *)(ws + lay.decay);
         p.items = (const int2 *)(ws + lay.pre);
         p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY; p.seg_states = 1;
-        rc = launch_state_pass(ctx, x, BC, T, 1, p, (unsigned)pl.pre.size(), H, G, 1u);
+        rc = launch_state_pass(ctx, x, Bs, T, 1, p, (unsigned)pl.pre.size(), H, G, 1u);
         if (rc != SWIMBA_OK) return rc;
         const int PN4 = SP * SN / 4;
         ctx.begin(STAGE_SEGMENT_SCAN);
@@ -1436,7 +1521,7 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const void *x, const void *BC, const
         p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
         ctx.begin(STAGE_SSD_TILES);
         launch_kernel(ssd_tiles_kernel<false>, dim3((unsigned)pl.items.size(), pairs, 1), dim3(SSD_THREADS), smem,
-                      ctx.stream, true, tm_bc, tm_x, tm_y, p);
+                      ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         ctx.end();
     }
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
@@ -1467,19 +1552,15 @@ ShardLayout shard_layout(int B, int L, int H, int G, int chunk, int sm_count)
 }
 
 bool shard_maps(LaunchCtx &ctx, const void *x, const void *BC, const void *y, int B, int L, int H, int G,
-                CUtensorMap *tm_bc, CUtensorMap *tm_x, CUtensorMap *tm_y)
+                CUtensorMap *tm_b, CUtensorMap *tm_c, CUtensorMap *tm_x, CUtensorMap *tm_y)
 {
-    const int S = 2 * G * SN;
-    const uint64_t dims3[3] = {(uint64_t)S, (uint64_t)L, (uint64_t)B};
-    const uint64_t str3[2] = {(uint64_t)S * 2, (uint64_t)L * S * 2};
-    const uint32_t box3[3] = {64, ST, 1};
-    if (!encode_tmap_bf16_cached(ctx.tmaps, tm_bc, BC, 3, dims3, str3, box3)) return false;
+    if (!stream_map(ctx, tm_b, b_stream(BC, G), L, B, G, ST) || !stream_map(ctx, tm_c, c_stream(BC, G), L, B, G, ST))
+        return false;
     const uint64_t dims[4] = {(uint64_t)SP, (uint64_t)H, (uint64_t)L, (uint64_t)B};
     const uint64_t str[3] = {(uint64_t)SP * 2, (uint64_t)H * SP * 2, (uint64_t)L * H * SP * 2};
     const uint32_t box[4] = {SP, 1, ST, 1};
     if (!encode_tmap_bf16_cached(ctx.tmaps, tm_x, x, 4, dims, str, box)) return false;
-    // (the state-only pass stores no y; its map is a copy of x's)
-    if (!encode_tmap_bf16_cached(ctx.tmaps, tm_y, y ? y : x, 4, dims, str, box)) return false;
+    if (!encode_tmap_bf16_cached(ctx.tmaps, tm_y, y, 4, dims, str, box)) return false;
     return ensure_dynamic_smem((const void *)ssd_tiles_kernel<false>, ssd_smem_bytes());
 }
 
@@ -1493,6 +1574,7 @@ SsdParams shard_params(LaunchCtx &ctx, const ShardLayout &lay, int B, int L, int
     p.split_tiles = 0;
     p.d_status = ctx.d_status;
     p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = 1; p.y = nullptr;
+    p.add = 0;
     return p;
 }
 }  // namespace
@@ -1515,8 +1597,6 @@ int launch_ssd_shard_summary(LaunchCtx &ctx, const void *x, const void *BC, cons
 {
     if (B <= 0 || L <= 0) return SWIMBA_OK;
     const ShardLayout lay = shard_layout(B, L, H, G, chunk, sm_count);
-    CUtensorMap tm_bc, tm_x, tm_y;
-    if (!shard_maps(ctx, x, BC, nullptr, B, L, H, G, &tm_bc, &tm_x, &tm_y)) return SWIMBA_ERR_CUDA;
     if (!scalars_done) {
         const int rc = launch_ssd_scalars(ctx, ssd_scalars_args(dt, A, dt_bias, B, L, H, (char *)workspace + lay.scal));
         if (rc != SWIMBA_OK) return rc;
@@ -1526,7 +1606,7 @@ int launch_ssd_shard_summary(LaunchCtx &ctx, const void *x, const void *BC, cons
     float *decay = (float *)((char *)workspace + lay.decay);
     p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY;
     {
-        const int rc = launch_state_pass(ctx, x, BC, L, B, p, (unsigned)lay.nseg, H, G, (unsigned)B);
+        const int rc = launch_state_pass(ctx, x, b_stream(BC, G), L, B, p, (unsigned)lay.nseg, H, G, (unsigned)B);
         if (rc != SWIMBA_OK) return rc;
     }
     const int PN4 = SP * SN / 4;
@@ -1543,8 +1623,8 @@ int launch_ssd_shard_finish(LaunchCtx &ctx, const void *x, const void *BC, const
 {
     if (B <= 0 || L <= 0) return SWIMBA_OK;
     const ShardLayout lay = shard_layout(B, L, H, G, chunk, sm_count);
-    CUtensorMap tm_bc, tm_x, tm_y;
-    if (!shard_maps(ctx, x, BC, y, B, L, H, G, &tm_bc, &tm_x, &tm_y)) return SWIMBA_ERR_CUDA;
+    CUtensorMap tm_b, tm_c, tm_x, tm_y;
+    if (!shard_maps(ctx, x, BC, y, B, L, H, G, &tm_b, &tm_c, &tm_x, &tm_y)) return SWIMBA_ERR_CUDA;
     SsdParams p = shard_params(ctx, lay, B, L, H, G, workspace);
     float *states = (float *)((char *)workspace + lay.states);
     float *decay = (float *)((char *)workspace + lay.decay);
@@ -1557,8 +1637,8 @@ int launch_ssd_shard_finish(LaunchCtx &ctx, const void *x, const void *BC, const
     p.h_in = states; p.h_out = h_end; p.seg_decay = nullptr; p.mode = MODE_FULL;
     const dim3 grid((unsigned)lay.nseg, (unsigned)(G * pairs_per_group(H, G)), (unsigned)B);
     ctx.begin(STAGE_SSD_TILES);
-    launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), ssd_smem_bytes(), ctx.stream, true, tm_bc, tm_x,
-                  tm_y, p);
+    launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), ssd_smem_bytes(), ctx.stream, true, tm_b, tm_c,
+                  tm_x, tm_y, p);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }

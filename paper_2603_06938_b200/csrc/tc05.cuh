@@ -121,6 +121,14 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *m, const void *s
         "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
 }
+// The same, adding into the destination (the element type of the tensor map, round to nearest).
+__device__ __forceinline__ void tma_reduce_add_4d(const CUtensorMap *m, const void *src, int c0, int c1,
+                                                  int c2, int c3) {
+    asm volatile(
+        "cp.reduce.async.bulk.tensor.4d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(m),
+        "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
 // Plain bulk copy global -> shared of `bytes` (a multiple of 16, both addresses 16-byte aligned);
 // completion is counted in bytes on the mbarrier.
 __device__ __forceinline__ void bulk_load(void *dst_smem, const void *src_global, uint32_t bytes,
