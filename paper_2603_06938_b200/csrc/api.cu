@@ -653,15 +653,19 @@ int swimba_forward(swimba_handle *h, const swimba_weights *w, const void *u, con
 namespace {
 // Workspace of the packed forward: the forward's regions for T tokens, with the SSD region sized for
 // the packed batch.
-FwdLayout packed_fwd_layout(const swimba_config &c, const int32_t *cu, int nseq, int sm_count)
+// (plan: the batch's plan, or NULL for shapes without a tile kernel)
+FwdLayout packed_fwd_layout(const swimba_config &c, int64_t T, const PackedPlan *plan, int sm_count)
 {
-    const int64_t T = cu[nseq];
     FwdLayout l = fwd_layout(c, 1, (int)(T > 0 ? T : 1), sm_count);
     size_t off = l.ssd;
-    if (ssd_tiles_supported(c.dtype, c.head_dim, c.d_state))
-        off += align_up(ssd_packed_workspace_bytes(cu, nseq, c.n_heads, c.n_groups, c.chunk, sm_count));
+    if (plan) off += align_up(ssd_packed_workspace_bytes(*plan, c.n_heads));
     l.total = off;
     return l;
+}
+std::shared_ptr<const PackedPlan> make_packed_plan(const swimba_config &c, const int32_t *cu, int nseq, int sm_count)
+{
+    if (!ssd_tiles_supported(c.dtype, c.head_dim, c.d_state)) return nullptr;
+    return ssd_packed_plan(cu, nseq, c.n_heads, c.n_groups, c.chunk, sm_count);
 }
 bool packed_offsets_ok(const int32_t *cu, int nseq)
 {
@@ -675,7 +679,8 @@ bool packed_offsets_ok(const int32_t *cu, int nseq)
 size_t swimba_packed_workspace_bytes(const swimba_handle *h, const int32_t *cu_seqlens, int32_t nseq)
 {
     if (!h || nseq <= 0 || !packed_offsets_ok(cu_seqlens, nseq) || cu_seqlens[nseq] <= 0) return 0;
-    return packed_fwd_layout(h->cfg, cu_seqlens, nseq, h->sm_count).total;
+    return packed_fwd_layout(h->cfg, cu_seqlens[nseq], make_packed_plan(h->cfg, cu_seqlens, nseq, h->sm_count).get(),
+                             h->sm_count).total;
 }
 
 int32_t swimba_packed_segments(const swimba_handle *h, const int32_t *cu_seqlens, int32_t nseq)
@@ -683,7 +688,7 @@ int32_t swimba_packed_segments(const swimba_handle *h, const int32_t *cu_seqlens
     if (!h || nseq <= 0 || !packed_offsets_ok(cu_seqlens, nseq)) return 0;
     const swimba_config &c = h->cfg;
     if (!ssd_tiles_supported(c.dtype, c.head_dim, c.d_state)) return nseq;
-    return ssd_packed_segments(cu_seqlens, nseq, c.n_heads, c.n_groups, c.chunk, h->sm_count);
+    return ssd_packed_segments(*make_packed_plan(c, cu_seqlens, nseq, h->sm_count));
 }
 
 int swimba_forward_packed(swimba_handle *h, const swimba_weights *w, const void *u, const void *x,
@@ -708,7 +713,8 @@ int swimba_forward_packed(swimba_handle *h, const swimba_weights *w, const void 
         !aligned16(h_final) || !aligned16(topk_idx) || !aligned16(topk_w) || !aligned16(workspace))
         return fail(h, SWIMBA_ERR_MISALIGNED, "tensors must be 16-byte aligned");
     const swimba_config &c = h->cfg;
-    const FwdLayout l = packed_fwd_layout(c, cu_seqlens, nseq, h->sm_count);
+    const std::shared_ptr<const PackedPlan> plan = make_packed_plan(c, cu_seqlens, nseq, h->sm_count);
+    const FwdLayout l = packed_fwd_layout(c, T, plan.get(), h->sm_count);
     if (T > 0 && workspace_bytes < l.total) return fail(h, SWIMBA_ERR_WORKSPACE_TOO_SMALL, "workspace too small");
     if ((rc = set_device(h)) != SWIMBA_OK) return rc;
     char *ws = (char *)workspace;
@@ -730,11 +736,17 @@ int swimba_forward_packed(swimba_handle *h, const swimba_weights *w, const void 
     float *wt = topk_w ? topk_w : (float *)(ws + l.w);
     void *BC = ws + l.bc;
     // routing, projection and mix are per token: the packed batch is one run of T tokens
-    rc = run_route_mix(h, ctx, w, u, T, BC, false, idx, wt, ws + l.gemm);
+    ScalarsArgs sa{};
+    if (plan) {
+        if (ssd_packed_upload(ctx, *plan, c.n_heads, ws + l.ssd) != SWIMBA_OK)
+            return fail(h, SWIMBA_ERR_CUDA, "copying the batch tables failed");
+        sa = ssd_packed_scalars_args(*plan, dt, w->A, w->dt_bias, T, c.n_heads, ws + l.ssd);
+    }
+    rc = run_route_mix(h, ctx, w, u, T, BC, false, idx, wt, ws + l.gemm, plan ? &sa : nullptr);
     if (rc == SWIMBA_OK) {
-        if (ssd_tiles_supported(c.dtype, c.head_dim, c.d_state)) {
-            rc = launch_ssd_tiles_packed(ctx, x, BC, dt, w->A, w->dt_bias, w->D, h0, cu_seqlens, nseq, c.n_heads,
-                                         c.n_groups, c.chunk, h->sm_count, y, h_final, ws + l.ssd);
+        if (plan) {
+            rc = launch_ssd_tiles_packed(ctx, *plan, x, BC, dt, w->A, w->dt_bias, w->D, h0, T, c.n_heads, c.n_groups, y,
+                                         h_final, ws + l.ssd);
             if (rc != SWIMBA_OK) rc = fail(h, rc, "SSD tile kernel launch failed");
         } else {
             // per-timestep evaluation, sequence by sequence

@@ -1,5 +1,7 @@
 // Launchers shared between the API translation unit and the kernel files.
 #pragma once
+#include <memory>
+
 #include "common.cuh"
 #include "ssd_scalars.cuh"
 
@@ -85,13 +87,19 @@ int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_s
                            int sm_count, void *y, float *h_final, void *cmix, void *workspace);
 
 // The same over a packed batch: nseq sequences back to back in [T, ...] arrays, sequence b holding
-// tokens cu[b] .. cu[b+1]-1 (cu is a HOST array of nseq + 1 entries, read before the call returns).
-// h0 / h_final are [nseq, H, P, N].  The step sizes are produced inside the call.
-size_t ssd_packed_workspace_bytes(const int32_t *cu, int nseq, int H, int G, int chunk, int sm_count);
-int ssd_packed_segments(const int32_t *cu, int nseq, int H, int G, int chunk, int sm_count);
-int launch_ssd_tiles_packed(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
-                            const float *dt_bias, const float *D, const float *h0, const int32_t *cu, int nseq,
-                            int H, int G, int chunk, int sm_count, void *y, float *h_final, void *workspace);
+// tokens cu[b] .. cu[b+1]-1 (cu is a HOST array of nseq + 1 entries).  h0 / h_final are [nseq, H, P, N].
+// A call makes its plan once (host work only), uploads the plan's tables in front of the router, has
+// the step sizes computed beside it (ssd_packed_scalars_args) and launches the rest behind the mix.
+struct PackedPlan;
+std::shared_ptr<const PackedPlan> ssd_packed_plan(const int32_t *cu, int nseq, int H, int G, int chunk, int sm_count);
+size_t ssd_packed_workspace_bytes(const PackedPlan &plan, int H);
+int ssd_packed_segments(const PackedPlan &plan);
+int ssd_packed_upload(LaunchCtx &ctx, const PackedPlan &plan, int H, void *workspace);
+ScalarsArgs ssd_packed_scalars_args(const PackedPlan &plan, const float *dt, const float *A, const float *dt_bias,
+                                    int64_t T, int H, void *workspace);
+int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &plan, const void *x, const void *BC, const float *dt,
+                            const float *A, const float *dt_bias, const float *D, const float *h0, int64_t T, int H,
+                            int G, void *y, float *h_final, void *workspace);
 
 // Sequence-sharded evaluation (every rank holds L consecutive tokens of each of B sequences), in two
 // halves around the exchange of the ranks' summaries.  summary: state-only pass + local scan from a
@@ -150,12 +158,12 @@ int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *
                           const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int P, int N,
                           int G, void *y, float *h_final);
 
-// The per-timestep evaluation over n listed sequences of a packed batch (bf16 streams): seq_tab[i] =
-// (first token, tokens, sequence index, 0), a device array; x, BC, dt, y are the packed arrays, h0 /
-// h_final are indexed by the sequence.
-int launch_ssd_sequential_listed(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
-                                 const float *dt_bias, const float *D, const float *h0, const int4 *seq_tab, int n,
-                                 int H, int P, int N, int G, void *y, float *h_final);
+// Sequences of a few tokens in a packed batch (bf16 streams, P = 64, N = 128), stepped token by token:
+// seq_tab[i] = (first token, tokens, sequence index, 0), a device array of n entries; x, BC, dt, y are
+// the packed arrays, h0 / h_final (may be NULL) are indexed by the sequence.
+int launch_step_sequences(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
+                          const float *dt_bias, const float *D, const float *h0, const int4 *seq_tab, int n, int H,
+                          int G, void *y, float *h_final);
 
 // K4: one-token state update, state[B,H,P,N] in place.
 // BC [B,S] is fp32 when bc_fp32, else bf16.

@@ -30,6 +30,8 @@
 // Long sequences with few (sequence, head) pairs are cut into segments: a first pass of this
 // kernel computes every segment's local end state (MMA 4 only), segment_scan_kernel (K3) chains
 // them, and a second pass evaluates each segment from its true incoming state.
+#include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "internal.h"
@@ -74,6 +76,7 @@ struct SsdParams {
     const TileScalars *rec; // [B,H,Lpad/128] per-tile weights and block ends
     const float *D;
     const float *h_in;      // initial states: [B,H,P,N] (nseg == 1) or [B,nseg,H,P,N]; may be null
+    const float *h_first;   // seg_states == 2: states entering the first segments, [B,H,P,N]; may be null
     float *h_out;           // MODE_FULL: h_final [B,H,P,N] (last segment writes) or null
                             // MODE_STATE_ONLY: local end states [B,nseg,H,P,N]
     float *seg_decay;       // MODE_STATE_ONLY: [B,nseg,H] product of a_t over the segment
@@ -85,7 +88,8 @@ struct SsdParams {
     // entry per sequence plus a closing one, items lists the (sequence, segment) pairs of this launch
     // (grid.x), the scalar arrays are laid out [H, tiles of the batch], and the per-segment state
     // arrays are indexed by seqs[b].seg0 + segment.  seg_states: h_in / state-only h_out are those
-    // per-segment arrays (else h_in is [sequences, H, P, N]).  y: base of the output (ragged last
+    // per-segment arrays (else h_in is [sequences, H, P, N]); 2: a sequence's first segment starts from
+    // h_first instead.  y: base of the output (ragged last
     // tiles are stored row by row).  Null seqs: dense [B, L].
     const SeqDesc *seqs;
     const int2 *items;
@@ -249,8 +253,13 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
     int seg_base = b * prm.nseg;                     // index of the sequence's first segment
     int64_t rec_base = (int64_t)b * H * (prm.Lpad / ST);   // tile record of head 0, tile 0: + h * rec_hstride
     int rec_hstride = prm.Lpad / ST;
+    const int HG = H / prm.G, ppg = pairs_per_group(H, prm.G);
+    int pair = blockIdx.y;
     if (packed) {
-        const int2 it = prm.items[blockIdx.x];
+        // (one grid dimension, the head pair fastest: CTAs start in the order of the items)
+        const int npairs = prm.G * ppg;
+        pair = blockIdx.x % npairs;
+        const int2 it = prm.items[blockIdx.x / npairs];
         b = it.x; seg = it.y;
         const SeqDesc sd = prm.seqs[b];
         L = sd.len; tok0 = sd.tok0; bco = 0;
@@ -259,8 +268,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         rec_base = sd.tile0;
         rec_hstride = prm.ntile_total;
     }
-    const int HG = H / prm.G, ppg = pairs_per_group(H, prm.G);
-    const int g = blockIdx.y / ppg, pr = blockIdx.y % ppg;
+    const int g = pair / ppg, pr = pair % ppg;
     const int head0 = g * HG + pr * NHD;
     const int nh = min(NHD, HG - pr * NHD);          // heads this CTA really has
     const int t_begin = seg * prm.seg_len;
@@ -512,9 +520,10 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         // fp32 master copy of the state: this thread holds H[n = i][p = p0 .. p0+31]
         float Hst[32];
         {
-            const float *h_in = prm.h_in;
+            const bool first = prm.seg_states == 2 && seg == 0;
+            const float *h_in = first ? prm.h_first : prm.h_in;
             if (h_in && kfull) {
-                const int64_t base = prm.seg_states
+                const int64_t base = (prm.seg_states && !first)
                     ? ((((int64_t)seg_base + seg) * H + h) * SP) * SN
                     : (((int64_t)b * H + h) * SP) * SN;
 #pragma unroll
@@ -777,18 +786,27 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
 // K3: chain the segments.  states[b,s,h,:,:] holds segment s's local end state (computed from a
 // zero initial state) on entry and the state ENTERING segment s on exit:
 //   H_in(0) = h0,   H_in(s+1) = decay(s) H_in(s) + S(s).
-// One thread per 4 consecutive state entries; segments are walked in order.
-// (packed batch: sequence b owns segments seqs[b].seg0 .. seqs[b+1].seg0 - 1 of the batch-wide list)
+// One thread per 4 consecutive state entries; segments are walked in order.  The first segment's
+// entry state is h0 itself and is written only when keep_first is set (a sequence shard, whose entry
+// state is not known yet): otherwise the full pass reads h0.
+// (packed batch: the z-th block plane works sequence multi[z], which owns segments seqs[b].seg0 ..
+// seqs[b+1].seg0 - 1 of the batch-wide list; sequences of one segment are not listed -- copying their
+// entry states was 57 of the 80 us this kernel took for 64 sequences, 57 of them a token long)
 __global__ void __launch_bounds__(256)
 segment_scan_kernel(float *__restrict__ states, const float *__restrict__ seg_decay,
                     const float *__restrict__ h0, int nseg, int H, int PN4, const SeqDesc *__restrict__ seqs,
-                    float *__restrict__ end_state, float *__restrict__ end_decay)
+                    const int *__restrict__ multi, int keep_first, float *__restrict__ end_state,
+                    float *__restrict__ end_decay)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // float4 index inside [P*N/4]
-    const int h = blockIdx.y, b = blockIdx.z;
+    const int h = blockIdx.y;
+    int b = blockIdx.z;
     if (v >= PN4) return;
     int64_t sb = (int64_t)b * nseg;
     if (seqs) {
+        b = multi[b];
         sb = seqs[b].seg0;
         nseg = seqs[b + 1].seg0 - seqs[b].seg0;
     }
@@ -815,7 +833,7 @@ segment_scan_kernel(float *__restrict__ states, const float *__restrict__ seg_de
         for (int q = 0; q < U; ++q) {
             const int s = s0 + q;
             if (s < nseg) {
-                reinterpret_cast<float4 *>(states)[((sb + s) * H + h) * PN4 + v] = run;
+                if (s > 0 || keep_first) reinterpret_cast<float4 *>(states)[((sb + s) * H + h) * PN4 + v] = run;
                 if (s >= nlocal) continue;
                 run.x = fmaf(d[q], run.x, loc[q].x);
                 run.y = fmaf(d[q], run.y, loc[q].y);
@@ -1244,7 +1262,8 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
     p.D = D;
     p.L = L; p.Lpad = Lpad; p.H = H; p.G = G; p.nseg = nseg; p.seg_len = seg_len;
     p.d_status = ctx.d_status;
-    p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = nseg > 1; p.y = y;
+    p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = nseg > 1 ? 2 : 0; p.y = y;
+    p.h_first = h0;
     p.add = add ? 1 : 0;
     dim3 grid((unsigned)nseg, (unsigned)(G * pairs_per_group(H, G)), (unsigned)B);
     p.split_tiles = 0;
@@ -1269,8 +1288,9 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
         }
         const int PN4 = SP * SN / 4;
         ctx.begin(STAGE_SEGMENT_SCAN);
-        segment_scan_kernel<<<dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)B), 256, 0, ctx.stream>>>(
-            states, decay, h0, nseg, H, PN4, nullptr, nullptr, nullptr);
+        launch_kernel(segment_scan_kernel, dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)B), dim3(256), 0,
+                      ctx.stream, true, states, (const float *)decay, h0, nseg, H, PN4, (const SeqDesc *)nullptr,
+                      (const int *)nullptr, 0, (float *)nullptr, (float *)nullptr);
         ctx.end();
         p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
         ctx.begin(STAGE_SSD_TILES);
@@ -1350,21 +1370,21 @@ int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_s
 // segment length is cut into segments (state-only pass, segment scan, full pass, as in the dense
 // case); the segment length is the per-SM share of the batch's tiles, so that one long sequence
 // among short ones does not serialise the launch.
-namespace {
 struct PackedPlan {
     std::vector<SeqDesc> seqs;        // nseq + 1
     std::vector<int2> tiles;          // (first token, valid tokens) per tile
     std::vector<int2> items, pre;     // (sequence, segment): all of them / those whose end state the scan needs
+    std::vector<int> multi;           // sequences of more than one segment
     std::vector<int4> shorts;         // (first token, tokens, sequence, 0) of the sequences stepped token by token
     int total_tiles = 0, total_segs = 0, seg_len = 0;
-    bool segmented = false;
 };
 
+namespace {
 PackedPlan packed_plan(const int32_t *cu, int nseq, int H, int G, int chunk, int sm_count)
 {
     PackedPlan pl;
     // Sequences of a few tokens (decode tokens riding in a prefill batch) do not take a 128-token
-    // tile and a CTA per head pair each: they are stepped token by token, one block per head.
+    // tile and a CTA per head pair each: they are stepped token by token, one warp per eight state rows.
     constexpr int SHORT_MAX = 4;
     auto is_short = [&](int b) { const int len = cu[b + 1] - cu[b]; return len >= 1 && len <= SHORT_MAX; };
     int64_t tiles = 0;
@@ -1396,72 +1416,104 @@ PackedPlan packed_plan(const int32_t *cu, int nseq, int H, int G, int chunk, int
             pl.items.push_back(make_int2(b, sgi));
             if (sgi + 1 < ns) pl.pre.push_back(make_int2(b, sgi));
         }
-        if (ns > 1) pl.segmented = true;
+        if (ns > 1) pl.multi.push_back(b);
         tile0 += nt;
         seg0 += ns;
     }
     pl.seqs[nseq] = SeqDesc{cu[nseq], 0, tile0, seg0};
     pl.total_tiles = tile0;
     pl.total_segs = seg0;
+    // CTAs start in the order of the list: the longest segments first, so that the short ones fill
+    // the SMs that come free at the end
+    auto tiles_of = [&](const int2 &it) {
+        const int left = pl.seqs[it.x].len - it.y * pl.seg_len;
+        return ceil_div(left < pl.seg_len ? left : pl.seg_len, ST);
+    };
+    std::stable_sort(pl.items.begin(), pl.items.end(),
+                     [&](const int2 &a, const int2 &b) { return tiles_of(a) > tiles_of(b); });
     return pl;
 }
 
 struct PackedLayout {
-    size_t seqs, tiles, items, pre, shorts, l2, rec, states, decay, total;
+    size_t seqs, tiles, items, pre, multi, shorts, tables, l2, rec, states, decay, total;
 };
-PackedLayout packed_layout(const PackedPlan &pl, int nseq, int H)
+PackedLayout packed_layout(const PackedPlan &pl, int H)
 {
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    auto up16 = [](size_t v) { return (v + 15) / 16 * 16; };
     PackedLayout l;
     size_t off = 0;
-    l.seqs = off;  off += up(((size_t)nseq + 1) * sizeof(SeqDesc));
-    l.tiles = off; off += up((size_t)pl.total_tiles * sizeof(int2));
-    l.items = off; off += up(pl.items.size() * sizeof(int2));
-    l.pre = off;   off += up(pl.pre.size() * sizeof(int2));
-    l.shorts = off; off += up(pl.shorts.size() * sizeof(int4));
+    // the tables, close together: they are copied in one piece
+    l.seqs = off;  off += up16(pl.seqs.size() * sizeof(SeqDesc));
+    l.tiles = off; off += up16(pl.tiles.size() * sizeof(int2));
+    l.items = off; off += up16(pl.items.size() * sizeof(int2));
+    l.pre = off;   off += up16(pl.pre.size() * sizeof(int2));
+    l.multi = off; off += up16(pl.multi.size() * sizeof(int));
+    l.shorts = off; off += up16(pl.shorts.size() * sizeof(int4));
+    l.tables = off;
+    off = up(off);
     l.l2 = off;    off += up((size_t)H * pl.total_tiles * ST * sizeof(float));
     l.rec = off;   off += up((size_t)H * pl.total_tiles * sizeof(TileScalars));
     l.states = off;
-    if (pl.segmented) off += up((size_t)pl.total_segs * H * SP * SN * sizeof(float));
+    if (!pl.multi.empty()) off += up((size_t)pl.total_segs * H * SP * SN * sizeof(float));
     l.decay = off;
-    if (pl.segmented) off += up((size_t)pl.total_segs * H * sizeof(float));
+    if (!pl.multi.empty()) off += up((size_t)pl.total_segs * H * sizeof(float));
     l.total = off;
     return l;
 }
 }  // namespace
 
-size_t ssd_packed_workspace_bytes(const int32_t *cu, int nseq, int H, int G, int chunk, int sm_count)
+std::shared_ptr<const PackedPlan> ssd_packed_plan(const int32_t *cu, int nseq, int H, int G, int chunk, int sm_count)
 {
-    const PackedPlan pl = packed_plan(cu, nseq, H, G, chunk, sm_count);
-    return packed_layout(pl, nseq, H).total;
+    return std::make_shared<const PackedPlan>(packed_plan(cu, nseq, H, G, chunk, sm_count));
 }
 
-int ssd_packed_segments(const int32_t *cu, int nseq, int H, int G, int chunk, int sm_count)
+size_t ssd_packed_workspace_bytes(const PackedPlan &pl, int H) { return packed_layout(pl, H).total; }
+
+int ssd_packed_segments(const PackedPlan &pl) { return pl.total_segs; }
+
+// The plan's tables go to the device in one copy, in stream order (the copy has read host memory when
+// it returns: pageable memory is staged by the runtime).
+int ssd_packed_upload(LaunchCtx &ctx, const PackedPlan &pl, int H, void *workspace)
 {
-    return packed_plan(cu, nseq, H, G, chunk, sm_count).total_segs;
+    const PackedLayout lay = packed_layout(pl, H);
+    std::vector<char> host(lay.tables);
+    auto put = [&](size_t off, const void *src, size_t bytes) { if (bytes) memcpy(host.data() + off, src, bytes); };
+    put(lay.seqs, pl.seqs.data(), pl.seqs.size() * sizeof(SeqDesc));
+    put(lay.tiles, pl.tiles.data(), pl.tiles.size() * sizeof(int2));
+    put(lay.items, pl.items.data(), pl.items.size() * sizeof(int2));
+    put(lay.pre, pl.pre.data(), pl.pre.size() * sizeof(int2));
+    put(lay.multi, pl.multi.data(), pl.multi.size() * sizeof(int));
+    put(lay.shorts, pl.shorts.data(), pl.shorts.size() * sizeof(int4));
+    return cudaMemcpyAsync(workspace, host.data(), lay.tables, cudaMemcpyHostToDevice, ctx.stream) == cudaSuccess
+               ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
-int launch_ssd_tiles_packed(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
-                            const float *dt_bias, const float *D, const float *h0, const int32_t *cu, int nseq,
-                            int H, int G, int chunk, int sm_count, void *y, float *h_final, void *workspace)
+ScalarsArgs ssd_packed_scalars_args(const PackedPlan &pl, const float *dt, const float *A, const float *dt_bias,
+                                    int64_t T, int H, void *workspace)
 {
-    const int64_t T = cu[nseq];
-    if (nseq <= 0 || T <= 0) return SWIMBA_OK;
-    const PackedPlan pl = packed_plan(cu, nseq, H, G, chunk, sm_count);
-    const PackedLayout lay = packed_layout(pl, nseq, H);
+    const PackedLayout lay = packed_layout(pl, H);
     char *ws = (char *)workspace;
-    // the tables go to the device in stream order (the copies read host memory before returning)
-    if (cudaMemcpyAsync(ws + lay.seqs, pl.seqs.data(), pl.seqs.size() * sizeof(SeqDesc), cudaMemcpyHostToDevice, ctx.stream) != cudaSuccess ||
-        cudaMemcpyAsync(ws + lay.tiles, pl.tiles.data(), pl.tiles.size() * sizeof(int2), cudaMemcpyHostToDevice, ctx.stream) != cudaSuccess ||
-        cudaMemcpyAsync(ws + lay.items, pl.items.data(), pl.items.size() * sizeof(int2), cudaMemcpyHostToDevice, ctx.stream) != cudaSuccess ||
-        (!pl.pre.empty() &&
-         cudaMemcpyAsync(ws + lay.pre, pl.pre.data(), pl.pre.size() * sizeof(int2), cudaMemcpyHostToDevice, ctx.stream) != cudaSuccess) ||
-        (!pl.shorts.empty() &&
-         cudaMemcpyAsync(ws + lay.shorts, pl.shorts.data(), pl.shorts.size() * sizeof(int4), cudaMemcpyHostToDevice, ctx.stream) != cudaSuccess))
-        return SWIMBA_ERR_CUDA;
+    ScalarsArgs sa{};
+    if (pl.total_tiles == 0) return sa;
+    sa.dt = dt; sa.A = A; sa.dt_bias = dt_bias;
+    sa.l2 = (float *)(ws + lay.l2);
+    sa.rec = (TileScalars *)(ws + lay.rec);
+    sa.L = (int)T; sa.Lpad = pl.total_tiles * ST; sa.H = H; sa.B = 1;
+    sa.tile_tab = (const int2 *)(ws + lay.tiles);
+    return sa;
+}
+
+// Everything behind the mixed streams (tables uploaded and step sizes computed before).
+int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &pl, const void *x, const void *BC, const float *dt,
+                            const float *A, const float *dt_bias, const float *D, const float *h0, int64_t T, int H,
+                            int G, void *y, float *h_final, void *workspace)
+{
+    const PackedLayout lay = packed_layout(pl, H);
+    char *ws = (char *)workspace;
     if (!pl.shorts.empty()) {
-        const int rc = launch_ssd_sequential_listed(ctx, x, BC, dt, A, dt_bias, D, h0, (const int4 *)(ws + lay.shorts),
-                                                    (int)pl.shorts.size(), H, SP, SN, G, y, h_final);
+        const int rc = launch_step_sequences(ctx, x, BC, dt, A, dt_bias, D, h0, (const int4 *)(ws + lay.shorts),
+                                             (int)pl.shorts.size(), H, G, y, h_final);
         if (rc != SWIMBA_OK) return rc;
     }
     if (pl.items.empty()) return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
@@ -1479,51 +1531,39 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const void *x, const void *BC, const
     const size_t smem = ssd_smem_bytes();
     if (!ensure_dynamic_smem((const void *)ssd_tiles_kernel<false>, smem)) return SWIMBA_ERR_CUDA;
 
-    ScalarsArgs sa;
-    sa.dt = dt; sa.A = A; sa.dt_bias = dt_bias;
-    sa.l2 = (float *)(ws + lay.l2);
-    sa.rec = (TileScalars *)(ws + lay.rec);
-    sa.L = (int)T; sa.Lpad = pl.total_tiles * ST; sa.H = H; sa.B = 1;
-    sa.tile_tab = (const int2 *)(ws + lay.tiles);
-    int rc = launch_ssd_scalars(ctx, sa);
-    if (rc != SWIMBA_OK) return rc;
-
     SsdParams p;
-    p.l2 = sa.l2; p.rec = sa.rec; p.D = D;
-    p.L = 0; p.Lpad = sa.Lpad; p.H = H; p.G = G; p.nseg = 1; p.seg_len = pl.seg_len;
+    p.l2 = (const float *)(ws + lay.l2); p.rec = (const TileScalars *)(ws + lay.rec); p.D = D;
+    p.L = 0; p.Lpad = pl.total_tiles * ST; p.H = H; p.G = G; p.nseg = 1; p.seg_len = pl.seg_len;
     p.split_tiles = 0;
     p.d_status = ctx.d_status;
     p.seqs = (const SeqDesc *)(ws + lay.seqs);
     p.ntile_total = pl.total_tiles;
     p.y = y;
     p.add = 0;
+    p.h_first = h0;
     const unsigned pairs = (unsigned)(G * pairs_per_group(H, G));
-    if (!pl.segmented) {
-        p.items = (const int2 *)(ws + lay.items);
-        p.h_in = h0; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL; p.seg_states = 0;
-        ctx.begin(STAGE_SSD_TILES);
-        launch_kernel(ssd_tiles_kernel<false>, dim3((unsigned)pl.items.size(), pairs, 1), dim3(SSD_THREADS), smem,
-                      ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
-        ctx.end();
-    } else {
+    p.h_in = h0; p.seg_states = 0;
+    if (!pl.multi.empty()) {
         float *states = (float *)(ws + lay.states);
         float *decay = (float *)(ws + lay.decay);
         p.items = (const int2 *)(ws + lay.pre);
-        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY; p.seg_states = 1;
-        rc = launch_state_pass(ctx, x, Bs, T, 1, p, (unsigned)pl.pre.size(), H, G, 1u);
+        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY; p.seg_states = 2;
+        const int rc = launch_state_pass(ctx, x, Bs, T, 1, p, (unsigned)pl.pre.size(), H, G, 1u);
         if (rc != SWIMBA_OK) return rc;
         const int PN4 = SP * SN / 4;
         ctx.begin(STAGE_SEGMENT_SCAN);
-        segment_scan_kernel<<<dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)nseq), 256, 0, ctx.stream>>>(
-            states, decay, h0, 0, H, PN4, p.seqs, nullptr, nullptr);
+        launch_kernel(segment_scan_kernel, dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)pl.multi.size()),
+                      dim3(256), 0, ctx.stream, true, states, (const float *)decay, h0, 0, H, PN4, p.seqs,
+                      (const int *)(ws + lay.multi), 0, (float *)nullptr, (float *)nullptr);
         ctx.end();
-        p.items = (const int2 *)(ws + lay.items);
-        p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
-        ctx.begin(STAGE_SSD_TILES);
-        launch_kernel(ssd_tiles_kernel<false>, dim3((unsigned)pl.items.size(), pairs, 1), dim3(SSD_THREADS), smem,
-                      ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
-        ctx.end();
+        p.h_in = states;
     }
+    p.items = (const int2 *)(ws + lay.items);
+    p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
+    ctx.begin(STAGE_SSD_TILES);
+    launch_kernel(ssd_tiles_kernel<false>, dim3((unsigned)pl.items.size() * pairs), dim3(SSD_THREADS), smem,
+                  ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
+    ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
@@ -1574,6 +1614,7 @@ SsdParams shard_params(LaunchCtx &ctx, const ShardLayout &lay, int B, int L, int
     p.split_tiles = 0;
     p.d_status = ctx.d_status;
     p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = 1; p.y = nullptr;
+    p.h_first = nullptr;
     p.add = 0;
     return p;
 }
@@ -1611,8 +1652,9 @@ int launch_ssd_shard_summary(LaunchCtx &ctx, const void *x, const void *BC, cons
     }
     const int PN4 = SP * SN / 4;
     ctx.begin(STAGE_SEGMENT_SCAN);
-    segment_scan_kernel<<<dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)B), 256, 0, ctx.stream>>>(
-        states, decay, nullptr, lay.nseg, H, PN4, nullptr, sum_state, sum_decay);
+    launch_kernel(segment_scan_kernel, dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)B), dim3(256), 0,
+                  ctx.stream, true, states, (const float *)decay, (const float *)nullptr, lay.nseg, H, PN4,
+                  (const SeqDesc *)nullptr, (const int *)nullptr, 1, sum_state, sum_decay);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
