@@ -470,6 +470,10 @@ int dense_linear(swimba_handle *h, LaunchCtx &ctx, const void *in, const void *W
                  void *out, char *scratch)
 {
     const int dtype = h->cfg.dtype;
+    if (dtype == SWIMBA_DTYPE_BF16 && pair_gemm_usable(T, Fi, So, h->sm_count)) {
+        const int rc = launch_pair_gemm(ctx, in, W, nullptr, nullptr, nullptr, T, Fi, So, 1, 1, false, h->sm_count, out, So);
+        return rc == SWIMBA_OK ? rc : fail(h, rc, "linear map launch failed");
+    }
     int32_t *idx = (int32_t *)scratch;
     float *wt = (float *)(scratch + align_up((size_t)T * sizeof(int32_t)));
     char *gws = (char *)wt + align_up((size_t)T * sizeof(float));

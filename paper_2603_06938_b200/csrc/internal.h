@@ -32,6 +32,13 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
                        int F, int S, int E, int k, int sm_count, void *BC, void *workspace,
                        void *slots_out = nullptr);
 
+// The same products on CTA pairs, 256 x 256 tiles, persistent: calls with enough tiles (pair_gemm_usable).
+// perm == NULL: the T rows of A as they lie (E = k = 1, no weights); out rows are ld_out elements apart.
+bool pair_gemm_usable(int64_t rows, int F, int S, int sm_count);
+int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *perm, const int *counts,
+                     const float *w_slot, int64_t T, int F, int S, int E, int k, bool add_rows, int sm_count,
+                     void *out, int64_t ld_out);
+
 // K1b (SIMT): project the k selected experts and mix.  BC is written in `dtype`, or as float
 // per slot-sum when bc_fp32 is set.
 int launch_project_mix_simt(LaunchCtx &ctx, int dtype, const void *u, const void *W_e,

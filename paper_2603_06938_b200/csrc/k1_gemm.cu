@@ -324,6 +324,20 @@ bool expert_gemm_supported(int F, int S)
     return S % 32 == 0 && F >= 64;
 }
 
+// The slot sum behind a projection that stored its slots (wanted: the call mixes them).
+static int mix_slots(LaunchCtx &ctx, const __nv_bfloat16 *slots, int64_t T, int S, int k, bool wanted, int sm_count,
+                     void *BC)
+{
+    if (k > 1 && wanted) {
+        int64_t blocks = ceil_div64(T * (S / 8), 256);
+        if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
+        ctx.begin(STAGE_MIX_SLOTS);
+        mix_slots_kernel<<<(unsigned)blocks, 256, 0, ctx.stream>>>(slots, T, S, k, (__nv_bfloat16 *)BC);
+        ctx.end();
+    }
+    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+}
+
 int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const float *w, int64_t T,
                        int F, int S, int E, int k, int sm_count, void *BC, void *workspace,
                        void *slots_out)
@@ -339,6 +353,11 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
         ? (__nv_bfloat16 *)((char *)perm + gemm_ws_up((size_t)E * T * sizeof(int)))
         : (__nv_bfloat16 *)BC;
 
+    if (pair_gemm_usable(T * k, F, S, sm_count)) {
+        const int rc = launch_pair_gemm(ctx, u, W_e, perm, counts, w, T, F, S, E, k, add_rows != 0, sm_count, slots, S);
+        if (rc != SWIMBA_OK) return rc;
+        return mix_slots(ctx, slots, T, S, k, !add_rows && !slots_out, sm_count, BC);
+    }
     // Widest column tile that divides S; narrower when there are too few row tiles to fill the
     // GPU (decode-sized calls), so that the weight rows are spread over more SMs.
     int BN = 32;
@@ -369,16 +388,7 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
     else SWIMBA_GEMM_CASE(32);
 #undef SWIMBA_GEMM_CASE
     ctx.end();
-    if (k > 1 && !add_rows && !slots_out) {
-        const int64_t nvec = T * (S / 8);
-        int64_t blocks = ceil_div64(nvec, 256);
-        if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
-        ctx.begin(STAGE_MIX_SLOTS);
-        mix_slots_kernel<<<(unsigned)blocks, 256, 0, ctx.stream>>>(slots, T, S, k,
-                                                                  (__nv_bfloat16 *)BC);
-        ctx.end();
-    }
-    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+    return mix_slots(ctx, slots, T, S, k, !add_rows && !slots_out, sm_count, BC);
 }
 
 }  // namespace swimba
