@@ -43,6 +43,8 @@ struct PairArgs {
     const __nv_bfloat16 *rows;     // the rows the lists index
     __nv_bfloat16 *out;
     int64_t ld_out;
+    float *tail;                   // columns from tail_col on go here as fp32, [rows, S - tail_col] (a
+    int tail_col;                  // multiple of 32; S: none)
     int E, F, S, k, add_rows, check;
     int *d_status;
 };
@@ -330,13 +332,23 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             tc::tc_fence_after();
             tc::bulk_wait_read_all();            // the previous tile's row has left its staging buffer
             __syncwarp();
-            const int ncols = min(PG_BN, p.S - ti.n0);
+            const int ncols = min(PG_BN, p.S - ti.n0);                   // all columns of the tile,
+            const int nmain = max(0, min(ncols, p.tail_col - ti.n0));     // those in front of the tail
             const uint32_t acc = tmem + buf * PG_BN + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
             for (int c = 0; c < ncols; c += 32) {
                 uint32_t v[32];
                 tc::tmem_ld32(acc + c, v);
                 tc::tmem_ld_wait();
+                if (DENSE && c >= nmain) {
+                    if (ok) {
+                        const int c0 = ti.n0 + c - p.tail_col, nt = p.S - p.tail_col;
+                        float *d = p.tail + dst * nt + c0;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) if (c0 + i < nt) d[i] = __uint_as_float(v[i]);
+                    }
+                    continue;
+                }
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
@@ -349,10 +361,10 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             tc::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) remote_arrive(leader_addr(&sm->acc_empty[buf]));
-            if (ok) {
+            if (ok && nmain > 0) {
                 __nv_bfloat16 *row = p.out + dst * p.ld_out + ti.n0;
-                if (p.add_rows) tc::bulk_reduce_add_bf16(row, srow, (uint32_t)ncols * 2);
-                else tc::bulk_store(row, srow, (uint32_t)ncols * 2);
+                if (p.add_rows) tc::bulk_reduce_add_bf16(row, srow, (uint32_t)nmain * 2);
+                else tc::bulk_store(row, srow, (uint32_t)nmain * 2);
             }
             tc::bulk_commit_group();
         }
@@ -368,7 +380,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
 
 int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *perm, const int *counts,
                      const float *w_slot, int64_t T, int F, int S, int E, int k, bool add_rows, int sm_count,
-                     void *out, int64_t ld_out)
+                     void *out, int64_t ld_out, float *tail, int tail_col)
 {
     const bool dense = perm == nullptr;
     CUtensorMap tm_a, tm_w;
@@ -388,6 +400,7 @@ int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *pe
     p.perm = perm; p.counts = counts; p.cap = T; p.w_slot = w_slot;
     p.rows = (const __nv_bfloat16 *)A;
     p.out = (__nv_bfloat16 *)out; p.ld_out = ld_out;
+    p.tail = tail; p.tail_col = tail ? tail_col : S;
     p.E = E; p.F = F; p.S = S; p.k = k; p.add_rows = add_rows ? 1 : 0;
     p.check = ctx.check_indices ? 1 : 0;
     p.d_status = ctx.d_status;

@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("dtype,L,H,G,d_conv", [("bf16", 15, 3, 1, 4), ("bf16", 16, 2, 2, 3), ("bf16", 17, 4, 2, 2),
                                                 ("bf16", 2, 2, 1, 4), ("bf16", 1, 3, 1, 1), ("bf16", 33, 65, 1, 4),
+                                                ("bf16", 600, 3, 1, 4), ("bf16", 530, 8, 2, 3),   # step sizes from the product's tail
                                                 ("fp32", 8, 3, 3, 4), ("fp32", 9, 2, 1, 2)])
 def test_block_edges_match_the_oracle_composition(dtype, L, H, G, d_conv):
     cfg = synth.LayerConfig("edges", dtype, 2, L, 64, H, 64, 128, G, 4, 2, 128)
