@@ -902,7 +902,7 @@ BwdLayout bwd_layout(const swimba_config &c, int B, int L, int sm_count)
     l.dg = off;    off += align_up(T * c.n_experts * sizeof(float));
     l.adj = off;
     if (ssd_tiles_supported(c.dtype, c.head_dim, c.d_state))
-        off += align_up(ssd_adjoint_tiles_workspace_bytes(B, L, c.n_heads, c.chunk, sm_count));
+        off += align_up(ssd_adjoint_tiles_workspace_bytes(B, L, c.n_heads, c.n_groups, sm_count));
     l.total = off;
     return l;
 }
@@ -960,7 +960,10 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
     void *slots = ws + l.slots;
     float *dBC = (float *)(ws + l.dbc);
     // forward quantities again: routing, mixed streams, and the unscaled projection of every kept slot
-    rc = run_route_mix(h, ctx, w, u, T, BC, false, idx, wt, ws + l.f.gemm);
+    const bool tiles = ssd_tiles_supported(c.dtype, c.head_dim, c.d_state);
+    const ScalarsArgs sa = tiles ? ssd_adjoint_scalars_args(dt, w->A, w->dt_bias, B, L, c.n_heads, ws + l.adj)
+                                 : ScalarsArgs{};
+    rc = run_route_mix(h, ctx, w, u, T, BC, false, idx, wt, ws + l.f.gemm, tiles ? &sa : nullptr);
     if (rc == SWIMBA_OK) rc = launch_fill(ctx, ones, T * c.top_k, 1.f);
     if (rc == SWIMBA_OK) {
         if (use_tensor_k1(c))
@@ -974,11 +977,9 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
     if (rc == SWIMBA_OK && cudaMemsetAsync(dBC, 0, (size_t)T * S * sizeof(float), ctx.stream) != cudaSuccess)
         rc = fail(h, SWIMBA_ERR_CUDA, "clearing dBC failed");
     if (rc == SWIMBA_OK) {
-        // shapes of the forward's tile kernel: the adjoint is two more evaluations of that kernel on
-        // re-arranged operands; everything else: per-timestep passes
-        if (ssd_tiles_supported(c.dtype, c.head_dim, c.d_state))
-            rc = launch_ssd_adjoint_tiles(ctx, x, dy, BC, dt, w->A, w->dt_bias, h0, B, L, c.n_heads, c.n_groups,
-                                          c.chunk, h->sm_count, dBC, ws + l.adj);
+        // shapes of the forward's tile kernel: tensor cores; everything else: per-timestep passes
+        if (tiles)
+            rc = launch_ssd_adjoint_tiles(ctx, x, dy, BC, h0, B, L, c.n_heads, c.n_groups, h->sm_count, dBC, ws + l.adj);
         else
             rc = launch_ssd_adjoint(ctx, c.dtype, x, dy, BC, dt, w->A, w->dt_bias, h0, B, L, c.n_heads, c.head_dim,
                                     c.d_state, c.n_groups, dBC);

@@ -8,7 +8,8 @@
 //   softmax (router equation)      dg_{t,i} = pi_{t,i} ([i in K_t] dpi_{t,i} - sum_{j in K_t} pi_{t,j} dpi_{t,j})
 //   logits                         dW_r += dg_t u_t^T
 // The active sets are constants; the kept weights are softmax values over all E (no
-// renormalisation) and are differentiated as such.  Plain CUDA-core kernels, fp32 accumulation.
+// renormalisation) and are differentiated as such.  The recurrence's adjoint for the tensor-core shapes is
+// in k2_adjoint.cu; here: the per-timestep adjoint of the other shapes, and what follows from dBC.
 #include "internal.h"
 #include "tc05.cuh"
 
@@ -290,193 +291,6 @@ dw_expert_kernel(const T *__restrict__ u, const float *__restrict__ dBC, const i
 }
 
 }  // namespace
-
-// ---------------------------------------------------------------------------------------------
-// The adjoint through the tile kernel of the forward.  For head h the contribution to dCtilde is
-//   dC_t[n] = sum_{s<=t} (prod_{r=s+1..t} a_r) (dy_t[h] . x_s[h]) Delta_s Btilde_s[n]  (+ the h0 term),
-// which is the forward's own form  y_t = sum_{s<=t} decay (C_t . B_s) Delta_s x_s  with the roles
-//   C := [dy_t[h] | 0],  B := [x_s[h] | 0]  (64 entries padded to the 128 of a state row),
-//   x := one 64-wide half c of Btilde_s,
-// i.e. a layer of 2H heads (h, c) in H groups.  dBtilde is the same in reversed time,
-//   dB_s[n] = Delta_s sum_{t>=s} (prod_{r=s+1..t} a_r) (x_s[h] . dy_t[h]) Ctilde_t[n],
-// with position rho = L-1-t carrying the step size of token t+1 (so that the decay between two
-// reversed positions is the product the adjoint needs) and x := Ctilde_t half / that step size (the
-// kernel multiplies its input by the step size).  The per-head results (bf16) are summed over the
-// heads of a group into dBC.  Shapes of the tile kernel only (bf16, P = 64, N = 128).
-namespace {
-constexpr int VP = 64, VN = 128;
-
-// Operand streams of the virtual layer.  One block per token, thread = (head, 8-element chunk).
-template <bool REVERSE>
-__global__ void __launch_bounds__(256)
-adjoint_pack_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ dy,
-                    const __nv_bfloat16 *__restrict__ BC, const float *__restrict__ dt,
-                    const float *__restrict__ dt_bias, int L, int H, int G,
-                    __nv_bfloat16 *__restrict__ BCv, __nv_bfloat16 *__restrict__ xv, float *__restrict__ dtv)
-{
-    const int64_t bt = blockIdx.x;                    // token of the ORIGINAL order
-    const int b = (int)(bt / L), t = (int)(bt % L);
-    const int64_t ot = REVERSE ? (int64_t)b * L + (L - 1 - t) : bt;      // its position in the virtual layer
-    const int S = 2 * G * VN, HG = H / G;
-    const int Sv = 2 * H * VN;                        // virtual streams: H groups
-    // C / B rows: [x | 0] and [dy | 0] (forward), [dy | 0] and [x | 0] (reverse)
-    for (int i = threadIdx.x; i < H * 16; i += blockDim.x) {
-        const int h = i >> 4, ch = i & 15;            // 16 chunks of 8 elements per 128-entry row
-        uint4 vb = make_uint4(0, 0, 0, 0), vc = make_uint4(0, 0, 0, 0);
-        if (ch < 8) {
-            const uint4 xr = *reinterpret_cast<const uint4 *>(x + (bt * H + h) * VP + ch * 8);
-            const uint4 dr = *reinterpret_cast<const uint4 *>(dy + (bt * H + h) * VP + ch * 8);
-            vb = REVERSE ? dr : xr;
-            vc = REVERSE ? xr : dr;
-        }
-        *reinterpret_cast<uint4 *>(BCv + ot * Sv + (int64_t)h * VN + ch * 8) = vb;
-        *reinterpret_cast<uint4 *>(BCv + ot * Sv + (int64_t)(H + h) * VN + ch * 8) = vc;
-    }
-    // step sizes of the virtual heads and their inputs
-    for (int i = threadIdx.x; i < 2 * H * 8; i += blockDim.x) {
-        const int vh = i >> 3, ch = i & 7;
-        const int h = vh >> 1, c = vh & 1, g = h / HG;
-        float raw;
-        if (REVERSE) raw = (t + 1 < L && dt) ? dt[(bt + 1) * H + h] : 0.f;
-        else raw = dt ? dt[bt * H + h] : 0.f;
-        if (ch == 0) dtv[ot * 2 * H + vh] = raw;
-        const __nv_bfloat16 *src = BC + bt * S + (int64_t)(REVERSE ? G + g : g) * VN + c * 64 + ch * 8;
-        uint4 v = *reinterpret_cast<const uint4 *>(src);
-        if (REVERSE) {
-            const float inv = 1.f / softplus_f(raw + dt_bias[h]);
-            uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float lo = __uint_as_float(wv[q] << 16) * inv, hi = __uint_as_float(wv[q] & 0xffff0000u) * inv;
-                const __nv_bfloat162 pr = __floats2bfloat162_rn(lo, hi);
-                wv[q] = *reinterpret_cast<const uint32_t *>(&pr);
-            }
-            v = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-        }
-        *reinterpret_cast<uint4 *>(xv + (ot * 2 * H + vh) * VP + ch * 8) = v;
-    }
-}
-
-// A, dt_bias of the virtual heads and the transposed initial state (forward pass only):
-// h0v[b, (h,c), p', n'] = h0[b, h, p = n', n = 64 c + p'] for n' < 64, else 0.
-__global__ void __launch_bounds__(256)
-adjoint_params_kernel(const float *__restrict__ A, const float *__restrict__ dt_bias, const float *__restrict__ h0,
-                      int B, int H, float *__restrict__ Av, float *__restrict__ biasv, float *__restrict__ h0v)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < 2 * H) {
-        Av[i] = A[i >> 1];
-        biasv[i] = dt_bias[i >> 1];
-    }
-    const int64_t total = (int64_t)B * 2 * H * VP * VN;
-    if (h0v && i < total) {
-        const int np = (int)(i % VN), pp = (int)((i / VN) % VP);
-        const int vh = (int)((i / ((int64_t)VN * VP)) % (2 * H));
-        const int64_t b = i / ((int64_t)VN * VP * 2 * H);
-        const int h = vh >> 1, c = vh & 1;
-        h0v[i] = (np < VP && h0) ? h0[((b * H + h) * VP + np) * VN + 64 * c + pp] : 0.f;
-    }
-}
-
-// dBC[t, column block] = sum over the heads of the group of the virtual layer's outputs (times the
-// head's own step size in the reverse pass).  One block per token, thread = column n.
-template <bool REVERSE>
-__global__ void __launch_bounds__(128)
-adjoint_reduce_kernel(const __nv_bfloat16 *__restrict__ yv, const float *__restrict__ dt,
-                      const float *__restrict__ dt_bias, int L, int H, int G, float *__restrict__ dBC)
-{
-    const int64_t bt = blockIdx.x;
-    const int b = (int)(bt / L), t = (int)(bt % L);
-    const int64_t ot = REVERSE ? (int64_t)b * L + (L - 1 - t) : bt;
-    const int S = 2 * G * VN, HG = H / G;
-    const int n = threadIdx.x, c = n >> 6, pp = n & 63;
-    __shared__ float s_delta[1024];                       // the token's step sizes, one per head
-    if (REVERSE) {
-        for (int h = threadIdx.x; h < H; h += blockDim.x)
-            s_delta[h] = softplus_f((dt ? dt[bt * H + h] : 0.f) + dt_bias[h]);
-        __syncthreads();
-    }
-    for (int g = 0; g < G; ++g) {
-        float acc = 0.f;
-        for (int hh = 0; hh < HG; ++hh) {
-            const int h = g * HG + hh;
-            float v = __bfloat162float(yv[(ot * 2 * H + 2 * h + c) * VP + pp]);
-            if (REVERSE) v *= s_delta[h];
-            acc += v;
-        }
-        dBC[bt * S + (int64_t)(REVERSE ? g : G + g) * VN + n] = acc;
-    }
-}
-
-struct AdjLayout {
-    size_t bcv, xv, yv, dtv, av, biasv, h0v, ssd, total;
-};
-AdjLayout adj_layout(int B, int L, int H, int chunk, int sm_count)
-{
-    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-    const size_t T = (size_t)B * L;
-    AdjLayout l;
-    size_t off = 0;
-    l.bcv = off;   off += up(T * 2 * H * VN * 2);
-    l.xv = off;    off += up(T * 2 * H * VP * 2);
-    l.yv = off;    off += up(T * 2 * H * VP * 2);
-    l.dtv = off;   off += up(T * 2 * H * sizeof(float));
-    l.av = off;    off += up(2 * (size_t)H * sizeof(float));
-    l.biasv = off; off += up(2 * (size_t)H * sizeof(float));
-    l.h0v = off;   off += up((size_t)B * 2 * H * VP * VN * sizeof(float));
-    l.ssd = off;   off += up(ssd_workspace_bytes(B, L, 2 * H, H, chunk, sm_count));
-    l.total = off;
-    return l;
-}
-}  // namespace
-
-size_t ssd_adjoint_tiles_workspace_bytes(int B, int L, int H, int chunk, int sm_count)
-{
-    return adj_layout(B, L, H, chunk, sm_count).total;
-}
-
-int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, const void *BC, const float *dt,
-                             const float *A, const float *dt_bias, const float *h0, int B, int L, int H, int G,
-                             int chunk, int sm_count, float *dBC, void *workspace)
-{
-    if (B <= 0 || L <= 0) return SWIMBA_OK;
-    const AdjLayout lay = adj_layout(B, L, H, chunk, sm_count);
-    char *ws = (char *)workspace;
-    __nv_bfloat16 *BCv = (__nv_bfloat16 *)(ws + lay.bcv), *xv = (__nv_bfloat16 *)(ws + lay.xv);
-    __nv_bfloat16 *yv = (__nv_bfloat16 *)(ws + lay.yv);
-    float *dtv = (float *)(ws + lay.dtv), *Av = (float *)(ws + lay.av), *biasv = (float *)(ws + lay.biasv);
-    float *h0v = (float *)(ws + lay.h0v);
-    const int64_t T = (int64_t)B * L;
-    const int64_t nparam = (int64_t)B * 2 * H * VP * VN;
-    ctx.begin(STAGE_ADJOINT_PACK);
-    adjoint_params_kernel<<<(unsigned)ceil_div64(h0 ? nparam : 2 * H, 256), 256, 0, ctx.stream>>>(
-        A, dt_bias, h0, B, H, Av, biasv, h0 ? h0v : nullptr);
-    ctx.end();
-    for (int pass = 0; pass < 2; ++pass) {
-        const bool rev = pass == 1;
-        ctx.begin(STAGE_ADJOINT_PACK);
-        if (rev)
-            adjoint_pack_kernel<true><<<(unsigned)T, 256, 0, ctx.stream>>>(
-                (const __nv_bfloat16 *)x, (const __nv_bfloat16 *)dy, (const __nv_bfloat16 *)BC, dt, dt_bias, L, H, G,
-                BCv, xv, dtv);
-        else
-            adjoint_pack_kernel<false><<<(unsigned)T, 256, 0, ctx.stream>>>(
-                (const __nv_bfloat16 *)x, (const __nv_bfloat16 *)dy, (const __nv_bfloat16 *)BC, dt, dt_bias, L, H, G,
-                BCv, xv, dtv);
-        ctx.end();
-        if (cudaGetLastError() != cudaSuccess) return SWIMBA_ERR_CUDA;
-        const int rc = launch_ssd_tiles(ctx, xv, BCv, dtv, Av, biasv, nullptr, (!rev && h0) ? h0v : nullptr, B, L, 2 * H,
-                                        H, chunk, sm_count, yv, nullptr, ws + lay.ssd, false);
-        if (rc != SWIMBA_OK) return rc;
-        ctx.begin(STAGE_ADJOINT_PACK);
-        if (rev)
-            adjoint_reduce_kernel<true><<<(unsigned)T, 128, 0, ctx.stream>>>(yv, dt, dt_bias, L, H, G, dBC);
-        else
-            adjoint_reduce_kernel<false><<<(unsigned)T, 128, 0, ctx.stream>>>(yv, dt, dt_bias, L, H, G, dBC);
-        ctx.end();
-    }
-    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
-}
 
 namespace {
 // The same sum on tensor cores (bf16 features): a 128 x 128 tile of one expert's matrix per block,

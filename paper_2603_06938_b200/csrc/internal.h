@@ -74,6 +74,10 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count);
 ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
                              void *workspace);
 int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &args);
+size_t ssd_scalars_bytes(int B, int L, int H);       // of the arrays ssd_scalars_args lays out
+// Chains nseg segment states per (sequence, head): states [B,nseg,H,P,N] holds local end states on entry
+// and, for all but the first segment, entry states on exit (P = 64, N = 128).
+int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const float *h0, int B, int nseg, int H);
 int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
                      const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int G,
                      int chunk, int sm_count, void *y, float *h_final, void *workspace,
@@ -137,12 +141,13 @@ int launch_fill(LaunchCtx &ctx, float *p, int64_t n, float v);
 int launch_ssd_adjoint(LaunchCtx &ctx, int dtype, const void *x, const void *dy, const void *BC, const float *dt,
                        const float *A, const float *dt_bias, const float *h0, int B, int L, int H, int P, int N,
                        int G, float *dBC);
-// The same adjoint through the forward's tile kernel (bf16, P = 64, N = 128): both passes are
-// evaluations of a virtual layer of 2H heads in H groups; dBC is overwritten, not accumulated.
-size_t ssd_adjoint_tiles_workspace_bytes(int B, int L, int H, int chunk, int sm_count);
-int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, const void *BC, const float *dt,
-                             const float *A, const float *dt_bias, const float *h0, int B, int L, int H, int G,
-                             int chunk, int sm_count, float *dBC, void *workspace);
+// The same adjoint on tensor cores (bf16, P = 64, N = 128).  The step sizes and tile log-decays of the
+// workspace (ssd_adjoint_scalars_args) are produced earlier in the stream; dBC (zeroed) is added to.
+size_t ssd_adjoint_tiles_workspace_bytes(int B, int L, int H, int G, int sm_count);
+ScalarsArgs ssd_adjoint_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
+                                     void *workspace);
+int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, const void *BC, const float *h0, int B,
+                             int L, int H, int G, int sm_count, float *dBC, void *workspace);
 int launch_weight_grads(LaunchCtx &ctx, int dtype, const void *u, const void *W_r, const void *slots,
                         const int32_t *idx, const float *w, const float *dBC, int64_t Tn, int F, int S, int E,
                         int k, float *pi, float *dg, float *dW_r, float *dW_e);

@@ -1156,7 +1156,7 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
 
 // Workspace: [log-decays B*H*Lpad float] [per-tile records B*H*(Lpad/128)] [segment states]
 // [segment decays].
-static size_t ssd_scalars_bytes(int B, int L, int H)
+size_t ssd_scalars_bytes(int B, int L, int H)
 {
     const size_t Lpad = (size_t)ceil_div(L, ST) * ST;
     const size_t l2_bytes = ((size_t)B * H * Lpad * sizeof(float) + 255) / 256 * 256;
@@ -1212,6 +1212,17 @@ int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &sa)
     ctx.begin(STAGE_SSD_SCALARS);
     launch_kernel(ssd_scalars_kernel, dim3((unsigned)scalars_blocks(sa, 256)), dim3(256), 0, ctx.stream,
                   true, sa);
+    ctx.end();
+    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+}
+
+int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const float *h0, int B, int nseg, int H)
+{
+    const int PN4 = SP * SN / 4;
+    ctx.begin(STAGE_SEGMENT_SCAN);
+    launch_kernel(segment_scan_kernel, dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)B), dim3(256), 0,
+                  ctx.stream, true, states, decay, h0, nseg, H, PN4, (const SeqDesc *)nullptr,
+                  (const int *)nullptr, 0, (float *)nullptr, (float *)nullptr);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
@@ -1286,12 +1297,10 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
             const int rc = launch_state_pass(ctx, x, Bs, L, B, p, (unsigned)(nseg - 1), H, G, (unsigned)B);
             if (rc != SWIMBA_OK) return rc;
         }
-        const int PN4 = SP * SN / 4;
-        ctx.begin(STAGE_SEGMENT_SCAN);
-        launch_kernel(segment_scan_kernel, dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)B), dim3(256), 0,
-                      ctx.stream, true, states, (const float *)decay, h0, nseg, H, PN4, (const SeqDesc *)nullptr,
-                      (const int *)nullptr, 0, (float *)nullptr, (float *)nullptr);
-        ctx.end();
+        {
+            const int rc = launch_segment_scan(ctx, states, decay, h0, B, nseg, H);
+            if (rc != SWIMBA_OK) return rc;
+        }
         p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
         ctx.begin(STAGE_SSD_TILES);
         launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
