@@ -884,10 +884,10 @@ int swimba_shard_finish(swimba_handle *h, const swimba_weights *w, const void *x
 }
 
 namespace {
-// Workspace of the backward: the forward's token regions, then [ones | slot projections | dBC | pi | dg].
+// Workspace of the backward: the forward's token regions, then [slot projections | dBC | pi | dg].
 struct BwdLayout {
     FwdLayout f;
-    size_t ones, slots, dbc, pi, dg, adj, total;
+    size_t slots, dbc, pi, dg, adj, total;
 };
 BwdLayout bwd_layout(const swimba_config &c, int B, int L, int sm_count)
 {
@@ -895,7 +895,6 @@ BwdLayout bwd_layout(const swimba_config &c, int B, int L, int sm_count)
     l.f = fwd_layout(c, B, L, sm_count);
     const size_t T = (size_t)B * L, S = 2u * c.n_groups * c.d_state;
     size_t off = l.f.ssd;
-    l.ones = off;  off += align_up(T * c.top_k * sizeof(float));
     l.slots = off; off += align_up(T * c.top_k * S * elt_size(c.dtype));
     l.dbc = off;   off += align_up(T * S * sizeof(float));
     l.pi = off;    off += align_up(T * c.n_experts * sizeof(float));
@@ -956,26 +955,38 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
     int32_t *idx = topk_idx ? topk_idx : (int32_t *)(ws + l.f.idx);
     float *wt = (float *)(ws + l.f.w);
     void *BC = ws + l.f.bc;
-    float *ones = (float *)(ws + l.ones);
     void *slots = ws + l.slots;
-    float *dBC = (float *)(ws + l.dbc);
-    // forward quantities again: routing, mixed streams, and the unscaled projection of every kept slot
-    const bool tiles = ssd_tiles_supported(c.dtype, c.head_dim, c.d_state);
+    float *dBC = (float *)(ws + l.dbc), *pi = (float *)(ws + l.pi);
+    if (cudaMemsetAsync(dBC, 0, (size_t)T * S * sizeof(float), ctx.stream) != cudaSuccess)
+        return fail(h, SWIMBA_ERR_CUDA, "clearing dBC failed");
+    // forward quantities again: routing (with the softmax over all experts), the unscaled projection of every
+    // kept slot, and the mixed streams as its weighted sum
+    const bool tiles = ssd_tiles_supported(c.dtype, c.head_dim, c.d_state), tensor = use_tensor_k1(c);
     const ScalarsArgs sa = tiles ? ssd_adjoint_scalars_args(dt, w->A, w->dt_bias, B, L, c.n_heads, ws + l.adj)
                                  : ScalarsArgs{};
-    rc = run_route_mix(h, ctx, w, u, T, BC, false, idx, wt, ws + l.f.gemm, tiles ? &sa : nullptr);
-    if (rc == SWIMBA_OK) rc = launch_fill(ctx, ones, T * c.top_k, 1.f);
-    if (rc == SWIMBA_OK) {
-        if (use_tensor_k1(c))
-            rc = launch_expert_gemm(ctx, u, w->W_expert, ones, T, c.d_model, (int)S, c.n_experts, c.top_k, h->sm_count,
-                                    BC, ws + l.f.gemm, slots);
-        else
-            rc = launch_project_slots_simt(ctx, c.dtype, u, w->W_expert, idx, ones, T, c.d_model, (int)S, c.n_experts,
-                                           c.top_k, slots);
-        if (rc != SWIMBA_OK) rc = fail(h, rc, "slot projection launch failed");
+    const void *Wr = w->W_router ? w->W_router : w->W_expert;
+    int *counts = nullptr, *perm = nullptr;
+    if (tensor) {
+        counts = expert_gemm_counts(ws + l.f.gemm);
+        perm = expert_gemm_perm(ws + l.f.gemm);
+        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
+            return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
-    if (rc == SWIMBA_OK && cudaMemsetAsync(dBC, 0, (size_t)T * S * sizeof(float), ctx.stream) != cudaSuccess)
-        rc = fail(h, SWIMBA_ERR_CUDA, "clearing dBC failed");
+    rc = launch_router(ctx, c.dtype, u, Wr, T, c.d_model, c.n_experts, c.top_k, idx, wt, counts, perm, T, h->sm_count,
+                       nullptr, 0, sa, pi);
+    if (rc != SWIMBA_OK) return fail(h, rc, "router launch failed");
+    if (tensor) {
+        rc = launch_expert_gemm(ctx, u, w->W_expert, nullptr, T, c.d_model, (int)S, c.n_experts, c.top_k, h->sm_count, BC,
+                                ws + l.f.gemm, slots);
+        if (rc == SWIMBA_OK) rc = launch_mix_slots(ctx, slots, wt, T, (int)S, c.top_k, h->sm_count, BC);
+    } else {
+        rc = launch_project_slots_simt(ctx, c.dtype, u, w->W_expert, idx, nullptr, T, c.d_model, (int)S, c.n_experts,
+                                       c.top_k, slots);
+        if (rc == SWIMBA_OK)
+            rc = launch_project_mix_simt(ctx, c.dtype, u, w->W_expert, idx, wt, T, c.d_model, (int)S, c.n_experts, c.top_k,
+                                         BC, false);
+    }
+    if (rc != SWIMBA_OK) rc = fail(h, rc, "projection launch failed");
     if (rc == SWIMBA_OK) {
         // shapes of the forward's tile kernel: tensor cores; everything else: per-timestep passes
         if (tiles)
@@ -986,10 +997,8 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
         if (rc != SWIMBA_OK) rc = fail(h, rc, "adjoint recurrence launch failed");
     }
     if (rc == SWIMBA_OK) {
-        const void *Wr = w->W_router ? w->W_router : w->W_expert;
-        rc = launch_weight_grads(ctx, c.dtype, u, Wr, slots, idx, wt, dBC, T, c.d_model, (int)S, c.n_experts, c.top_k,
-                                 (float *)(ws + l.pi), (float *)(ws + l.dg),
-                                 dW_router, dW_expert);
+        rc = launch_weight_grads(ctx, c.dtype, u, slots, idx, wt, dBC, T, c.d_model, (int)S, c.n_experts, c.top_k, pi,
+                                 (float *)(ws + l.dg), perm, counts, h->sm_count, dW_router, dW_expert);
         if (rc != SWIMBA_OK) rc = fail(h, rc, "weight gradient launch failed");
     }
     h->last_launches = ctx.launches;

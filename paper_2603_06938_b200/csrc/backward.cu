@@ -116,105 +116,112 @@ ssd_adjoint_kernel(const T *__restrict__ x, const T *__restrict__ dy, const T *_
     }
 }
 
-// Softmax over all E of the router logits, one warp per token: pi[T,E].  A lane takes 8 consecutive
-// features at a time (one 16- or 32-byte load of u, reused for every expert's row).
-template <typename T>
+// dpi and dg, one warp per token.  slots[t*k + j, :] = W_e[idx[t,j]] u_t (unscaled).  SCALED: the slots are
+// overwritten on the way by w[t,j] dBC[t, :], rounded to bf16, the rows the expert-matrix gradient sums.
+template <typename T, bool SCALED>
 __global__ void __launch_bounds__(256)
-router_softmax_kernel(const T *__restrict__ u, const T *__restrict__ W_r, int64_t Tn, int F, int E,
-                      float *__restrict__ pi)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t >= Tn) return;
-    float g[SWIMBA_MAX_EXPERTS];
-    for (int e = 0; e < E; ++e) g[e] = 0.f;
-    for (int f0 = lane * 8; f0 < F; f0 += 256) {            // (F is a multiple of 8)
-        float uv[8];
-        load8(u + t * F + f0, uv);
-        for (int e = 0; e < E; ++e) {
-            float wv[8];
-            load8(W_r + (int64_t)e * F + f0, wv);
-            float acc = g[e];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) acc = fmaf(wv[q], uv[q], acc);
-            g[e] = acc;
-        }
-    }
-    float m = -INFINITY;
-    for (int e = 0; e < E; ++e) {
-        g[e] = warp_sum(g[e]);
-        m = fmaxf(m, g[e]);
-    }
-    float z = 0.f;
-    for (int e = 0; e < E; ++e) { g[e] = expf(g[e] - m); z += g[e]; }
-    const float inv = 1.f / z;
-    for (int e = lane; e < E; e += 32) pi[t * E + e] = g[e] * inv;
-}
-
-// dpi and dg, one warp per token.  slots[t*k + j, :] = W_e[idx[t,j]] u_t (unscaled).
-template <typename T>
-__global__ void __launch_bounds__(256)
-dpi_dg_kernel(const float *__restrict__ dBC, const T *__restrict__ slots, const int32_t *__restrict__ idx,
+dpi_dg_kernel(const float *__restrict__ dBC, T *__restrict__ slots, const int32_t *__restrict__ idx,
               const float *__restrict__ w, const float *__restrict__ pi, int64_t Tn, int S, int E, int k,
               float *__restrict__ dg)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     const int lane = threadIdx.x & 31;
     const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (t >= Tn) return;
-    float inner = 0.f;
     float dpi[SWIMBA_MAX_TOPK];
-    for (int j = 0; j < k; ++j) {
-        float acc = 0.f;
-        const T *row = slots + (t * k + j) * (int64_t)S;
-        for (int s = lane; s < S; s += 32) acc = fmaf(dBC[t * S + s], to_f32<T>(row[s]), acc);
-        acc = warp_sum(acc);
-        dpi[j] = acc;
-        inner = fmaf(w[t * k + j], acc, inner);
+#pragma unroll
+    for (int j = 0; j < SWIMBA_MAX_TOPK; ++j) dpi[j] = 0.f;
+    for (int s = lane * 8; s < S; s += 256) {                 // (S is a multiple of 8)
+        float d[8];
+        load8(dBC + t * S + s, d);
+#pragma unroll
+        for (int j = 0; j < SWIMBA_MAX_TOPK; ++j) {
+            if (j < k) {
+                T *row = slots + (t * k + j) * (int64_t)S + s;
+                float v[8];
+                load8(row, v);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) dpi[j] = fmaf(d[q], v[q], dpi[j]);
+                if constexpr (SCALED) {
+                    const float wj = w[t * k + j];
+                    *reinterpret_cast<uint4 *>(row) =
+                        make_uint4(tc::pack_bf16x2(wj * d[0], wj * d[1]), tc::pack_bf16x2(wj * d[2], wj * d[3]),
+                                   tc::pack_bf16x2(wj * d[4], wj * d[5]), tc::pack_bf16x2(wj * d[6], wj * d[7]));
+                }
+            }
+        }
+    }
+    float inner = 0.f;
+#pragma unroll
+    for (int j = 0; j < SWIMBA_MAX_TOPK; ++j) {
+        if (j < k) {
+            dpi[j] = warp_sum(dpi[j]);
+            inner = fmaf(w[t * k + j], dpi[j], inner);
+        }
     }
     for (int e = lane; e < E; e += 32) {
         float v = -pi[t * E + e] * inner;
-        for (int j = 0; j < k; ++j)
-            if (idx[t * k + j] == e) v = fmaf(w[t * k + j], dpi[j], v);
+#pragma unroll
+        for (int j = 0; j < SWIMBA_MAX_TOPK; ++j)
+            if (j < k && idx[t * k + j] == e) v = fmaf(w[t * k + j], dpi[j], v);
         dg[t * E + e] = v;
     }
 }
 
-// dW_r[e,f] += sum_t dg[t,e] u[t,f] over the block's run of tokens; thread = one feature f,
-// eight experts at a time.
-constexpr int DWR_TOK = 512;
+// dW_r[e,f] += sum_t dg[t,e] u[t,f] over the block's run of tokens.  A thread takes 8 features (one 16-byte
+// load for bf16) and 8 experts; the block's threads cover the features, and where those are few, several
+// tokens at a time.  Bound by the read of u: 32768 x 2048, 8 experts 105 us with one feature per thread,
+// @DWR@ this way.
+constexpr int DWR_TOK = 128;
+__device__ __forceinline__ void add4(float *dst, float a, float b, float c, float d)
+{
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
 template <typename T>
 __global__ void __launch_bounds__(256)
-dw_router_kernel(const T *__restrict__ u, const float *__restrict__ dg, int64_t Tn, int F, int E,
+dw_router_kernel(const T *__restrict__ u, const float *__restrict__ dg, int64_t Tn, int F, int E, int lanes,
                  float *__restrict__ dW_r)
 {
-    __shared__ float sdg[64][8];
-    const int f = blockIdx.y * blockDim.x + threadIdx.x;
+    __shared__ __align__(16) float sdg[DWR_TOK][8];
+    grid_dep_wait();
+    grid_dep_launch();
+    const int width = blockDim.x / lanes;                       // threads along the features
+    const int lane = threadIdx.x / width;
+    const int f = (blockIdx.y * width + threadIdx.x % width) * 8;
     const int64_t t0 = (int64_t)blockIdx.x * DWR_TOK;
     const int nt = (int)min((int64_t)DWR_TOK, Tn - t0);
     for (int e0 = 0; e0 < E; e0 += 8) {
-        float acc[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-        for (int c0 = 0; c0 < nt; c0 += 64) {
-            const int nc = min(64, nt - c0);
-            __syncthreads();
-            for (int i = threadIdx.x; i < nc * 8; i += blockDim.x) {
-                const int tt = i >> 3, q = i & 7;
-                sdg[tt][q] = e0 + q < E ? dg[(t0 + c0 + tt) * E + e0 + q] : 0.f;
-            }
-            __syncthreads();
-            if (f < F) {
-                for (int tt = 0; tt < nc; ++tt) {
-                    const float uv = to_f32<T>(u[(t0 + c0 + tt) * F + f]);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) acc[q] = fmaf(sdg[tt][q], uv, acc[q]);
-                }
-            }
+        __syncthreads();
+        for (int i = threadIdx.x; i < nt * 8; i += blockDim.x) {
+            const int tt = i >> 3, q = i & 7;
+            sdg[tt][q] = e0 + q < E ? dg[(t0 + tt) * E + e0 + q] : 0.f;
         }
-        if (f < F) {
+        __syncthreads();
+        if (f < F) {                                            // (F is a multiple of 8)
+            float acc[8][8];
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (e0 + q < E) atomicAdd(dW_r + (int64_t)(e0 + q) * F + f, acc[q]);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[q][i] = 0.f;
+#pragma unroll 4
+            for (int tt = lane; tt < nt; tt += lanes) {
+                float uv[8], gv[8];
+                load8(u + (t0 + tt) * F + f, uv);
+                load8(&sdg[tt][0], gv);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) acc[q][i] = fmaf(gv[q], uv[i], acc[q][i]);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (e0 + q < E) {
+                    float *dst = dW_r + (int64_t)(e0 + q) * F + f;
+                    add4(dst, acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+                    add4(dst + 4, acc[q][4], acc[q][5], acc[q][6], acc[q][7]);
+                }
         }
     }
 }
@@ -293,122 +300,6 @@ dw_expert_kernel(const T *__restrict__ u, const float *__restrict__ dBC, const i
 }  // namespace
 
 namespace {
-// The same sum on tensor cores (bf16 features): a 128 x 128 tile of one expert's matrix per block,
-// eight warps of 32 (s) x 64 (f), the entries taken 32 at a time.  Both operands sit in shared memory
-// with the contraction index (the entry) as the row, so every fragment is a transposing ldmatrix:
-//   A[m = s][k = entry]  from sA[entry][s],   B[k = entry][n = f]  from sB[entry][f].
-// w dBC is rounded to bf16 once; accumulation in fp32; split over runs of tokens with atomics.
-constexpr int DWM_TOK = 4096, DWM_K = 32, DWM_LD = 136;      // row pitch 272 B: conflict-free ldmatrix
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-__global__ void __launch_bounds__(256)
-dw_expert_mma_kernel(const __nv_bfloat16 *__restrict__ u, const float *__restrict__ dBC,
-                     const int32_t *__restrict__ idx, const float *__restrict__ w, int64_t Tn, int F, int S,
-                     int E, int k, int nruns, float *__restrict__ dW_e)
-{
-    __shared__ int list[DWM_TOK];
-    __shared__ int list_n;
-    __shared__ __align__(16) __nv_bfloat16 sA[DWM_K][DWM_LD];
-    __shared__ __align__(16) __nv_bfloat16 sB[DWM_K][DWM_LD];
-    const int e = blockIdx.z / nruns, run = blockIdx.z % nruns;
-    const int s0 = blockIdx.x * 128, f0 = blockIdx.y * 128;
-    const int64_t t0 = (int64_t)run * DWM_TOK;
-    const int nt = (int)min((int64_t)DWM_TOK, Tn - t0);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid == 0) list_n = 0;
-    __syncthreads();
-    for (int i = tid; i < nt * k; i += blockDim.x)
-        if (idx[t0 * k + i] == e) list[atomicAdd(&list_n, 1)] = i;
-    __syncthreads();
-    const int cnt = list_n;
-    if (cnt == 0) return;
-    const int wm = (warp & 3) * 32, wn = (warp >> 2) * 64;       // the warp's corner inside the tile
-    float acc[2][8][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[a][c][q] = 0.f;
-    const int lj = lane >> 3, lr = lane & 7;
-    for (int c0 = 0; c0 < cnt; c0 += DWM_K) {
-        const int nc = min(DWM_K, cnt - c0);
-        __syncthreads();
-        // 32 entries x 128 columns of each operand, eight columns per thread and step
-        for (int i = tid; i < DWM_K * 16; i += blockDim.x) {
-            const int kk = i >> 4, col = (i & 15) * 8;
-            uint4 av = make_uint4(0, 0, 0, 0), bv = make_uint4(0, 0, 0, 0);
-            if (kk < nc) {
-                const int64_t r = t0 * k + list[c0 + kk];
-                const int64_t t = r / k;
-                const float wr = w[r];
-                if (s0 + col < S) {          // (S and F are multiples of 8)
-                    const float4 d0 = *reinterpret_cast<const float4 *>(dBC + t * S + s0 + col);
-                    const float4 d1 = *reinterpret_cast<const float4 *>(dBC + t * S + s0 + col + 4);
-                    const __nv_bfloat162 p0 = __floats2bfloat162_rn(wr * d0.x, wr * d0.y), p1 = __floats2bfloat162_rn(wr * d0.z, wr * d0.w);
-                    const __nv_bfloat162 p2 = __floats2bfloat162_rn(wr * d1.x, wr * d1.y), p3 = __floats2bfloat162_rn(wr * d1.z, wr * d1.w);
-                    av = make_uint4(*reinterpret_cast<const uint32_t *>(&p0), *reinterpret_cast<const uint32_t *>(&p1),
-                                    *reinterpret_cast<const uint32_t *>(&p2), *reinterpret_cast<const uint32_t *>(&p3));
-                }
-                if (f0 + col < F) bv = *reinterpret_cast<const uint4 *>(u + t * F + f0 + col);
-            }
-            *reinterpret_cast<uint4 *>(&sA[kk][col]) = av;
-            *reinterpret_cast<uint4 *>(&sB[kk][col]) = bv;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k0 = 0; k0 < DWM_K; k0 += 16) {
-            uint32_t af[2][4];
-#pragma unroll
-            for (int a = 0; a < 2; ++a)
-                ldmatrix_x4_trans(af[a], (uint32_t)__cvta_generic_to_shared(
-                                             &sA[k0 + (lj >> 1) * 8 + lr][wm + 16 * a + (lj & 1) * 8]));
-#pragma unroll
-            for (int c2 = 0; c2 < 4; ++c2) {
-                uint32_t bf[4];
-                ldmatrix_x4_trans(bf, (uint32_t)__cvta_generic_to_shared(
-                                          &sB[k0 + (lj & 1) * 8 + lr][wn + 16 * c2 + (lj >> 1) * 8]));
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    mma_16816(acc[a][2 * c2], af[a], bf[0], bf[1]);
-                    mma_16816(acc[a][2 * c2 + 1], af[a], bf[2], bf[3]);
-                }
-            }
-        }
-    }
-    const int g = lane >> 2, q2 = (lane & 3) * 2;
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-#pragma unroll
-            for (int hrow = 0; hrow < 2; ++hrow) {
-                const int srow = s0 + wm + 16 * a + g + 8 * hrow;
-                const int f = f0 + wn + 8 * c + q2;
-                if (srow < S && f < F) {            // (F is even)
-                    float *dst = dW_e + ((int64_t)e * S + srow) * F + f;
-                    atomicAdd(dst, acc[a][c][2 * hrow]);
-                    atomicAdd(dst + 1, acc[a][c][2 * hrow + 1]);
-                }
-            }
-}
-
-__global__ void fill_kernel(float *p, int64_t n, float v)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
-}
-
 int adjoint_ps(int P)
 {
     int ps = 1;
@@ -440,33 +331,30 @@ int launch_adjoint_t(LaunchCtx &ctx, const void *x, const void *dy, const void *
 }
 
 template <typename T>
-int launch_weight_grads_t(LaunchCtx &ctx, const void *u, const void *W_r, const void *slots, const int32_t *idx,
-                          const float *w, const float *dBC, int64_t Tn, int F, int S, int E, int k, float *pi,
-                          float *dg, float *dW_r, float *dW_e)
+int launch_weight_grads_t(LaunchCtx &ctx, const void *u, void *slots, const int32_t *idx, const float *w,
+                          const float *dBC, int64_t Tn, int F, int S, int E, int k, const float *pi, float *dg,
+                          const int *perm, const int *counts, int sm_count, float *dW_r, float *dW_e)
 {
     const unsigned tok_blocks = (unsigned)ceil_div64(Tn, 8);
-    ctx.begin(STAGE_ROUTER_SOFTMAX);
-    router_softmax_kernel<T><<<tok_blocks, 256, 0, ctx.stream>>>((const T *)u, (const T *)W_r, Tn, F, E, pi);
-    ctx.end();
     ctx.begin(STAGE_DPI_DG);
-    dpi_dg_kernel<T><<<tok_blocks, 256, 0, ctx.stream>>>(dBC, (const T *)slots, idx, w, pi, Tn, S, E, k, dg);
+    auto dpi = perm ? dpi_dg_kernel<T, sizeof(T) == 2> : dpi_dg_kernel<T, false>;
+    launch_kernel(dpi, dim3(tok_blocks), dim3(256), 0, ctx.stream, true, dBC, (T *)slots, idx, w, pi, Tn, S, E, k, dg);
     ctx.end();
     if (dW_r) {
+        // a block of up to 256 threads along the features; fewer features: several tokens at a time
+        const int need = ceil_div(F, 8);
+        int width = 256;
+        while (width > 32 && width / 2 >= need) width /= 2;
         ctx.begin(STAGE_DW_ROUTER);
-        dw_router_kernel<T><<<dim3((unsigned)ceil_div64(Tn, DWR_TOK), (unsigned)ceil_div(F, 256)), 256, 0, ctx.stream>>>(
-            (const T *)u, dg, Tn, F, E, dW_r);
+        launch_kernel(dw_router_kernel<T>, dim3((unsigned)ceil_div64(Tn, DWR_TOK), (unsigned)ceil_div(need, width)), dim3(256),
+                      0, ctx.stream, true, (const T *)u, (const float *)dg, Tn, F, E, 256 / width, dW_r);
         ctx.end();
     }
+    if (perm) return launch_pair_outer(ctx, slots, u, perm, counts, Tn, F, S, E, k, sm_count, dW_e);
+    const int nruns = (int)ceil_div64(Tn, DWE_TOK);
     ctx.begin(STAGE_DW_EXPERT);
-    if (sizeof(T) == 2 && F % 8 == 0 && S % 8 == 0) {
-        const int nruns = (int)ceil_div64(Tn, DWM_TOK);
-        dw_expert_mma_kernel<<<dim3((unsigned)ceil_div(S, 128), (unsigned)ceil_div(F, 128), (unsigned)(E * nruns)), 256, 0,
-                               ctx.stream>>>((const __nv_bfloat16 *)u, dBC, idx, w, Tn, F, S, E, k, nruns, dW_e);
-    } else {
-        const int nruns = (int)ceil_div64(Tn, DWE_TOK);
-        dw_expert_kernel<T><<<dim3((unsigned)ceil_div(S, 64), (unsigned)ceil_div(F, 64), (unsigned)(E * nruns)), 256, 0,
-                              ctx.stream>>>((const T *)u, dBC, idx, w, Tn, F, S, E, k, nruns, dW_e);
-    }
+    dw_expert_kernel<T><<<dim3((unsigned)ceil_div(S, 64), (unsigned)ceil_div(F, 64), (unsigned)(E * nruns)), 256, 0,
+                          ctx.stream>>>((const T *)u, dBC, idx, w, Tn, F, S, E, k, nruns, dW_e);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
@@ -475,14 +363,6 @@ int launch_weight_grads_t(LaunchCtx &ctx, const void *u, const void *W_r, const 
 bool ssd_adjoint_supported(int P, int N)
 {
     return N * adjoint_ps(P) <= 1024 && N >= 1;
-}
-
-int launch_fill(LaunchCtx &ctx, float *p, int64_t n, float v)
-{
-    if (n <= 0) return SWIMBA_OK;
-    fill_kernel<<<(unsigned)ceil_div64(n, 256), 256, 0, ctx.stream>>>(p, n, v);
-    ctx.launches++;
-    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
 int launch_ssd_adjoint(LaunchCtx &ctx, int dtype, const void *x, const void *dy, const void *BC, const float *dt,
@@ -495,14 +375,16 @@ int launch_ssd_adjoint(LaunchCtx &ctx, int dtype, const void *x, const void *dy,
     return launch_adjoint_t<__nv_bfloat16>(ctx, x, dy, BC, dt, A, dt_bias, h0, B, L, H, P, N, G, dBC);
 }
 
-int launch_weight_grads(LaunchCtx &ctx, int dtype, const void *u, const void *W_r, const void *slots,
-                        const int32_t *idx, const float *w, const float *dBC, int64_t Tn, int F, int S, int E,
-                        int k, float *pi, float *dg, float *dW_r, float *dW_e)
+int launch_weight_grads(LaunchCtx &ctx, int dtype, const void *u, void *slots, const int32_t *idx, const float *w,
+                        const float *dBC, int64_t Tn, int F, int S, int E, int k, const float *pi, float *dg,
+                        const int *perm, const int *counts, int sm_count, float *dW_r, float *dW_e)
 {
     if (Tn <= 0) return SWIMBA_OK;
     if (dtype == SWIMBA_DTYPE_FP32)
-        return launch_weight_grads_t<float>(ctx, u, W_r, slots, idx, w, dBC, Tn, F, S, E, k, pi, dg, dW_r, dW_e);
-    return launch_weight_grads_t<__nv_bfloat16>(ctx, u, W_r, slots, idx, w, dBC, Tn, F, S, E, k, pi, dg, dW_r, dW_e);
+        return launch_weight_grads_t<float>(ctx, u, slots, idx, w, dBC, Tn, F, S, E, k, pi, dg, nullptr, nullptr, sm_count,
+                                            dW_r, dW_e);
+    return launch_weight_grads_t<__nv_bfloat16>(ctx, u, slots, idx, w, dBC, Tn, F, S, E, k, pi, dg, perm, counts, sm_count,
+                                                dW_r, dW_e);
 }
 
 }  // namespace swimba

@@ -13,10 +13,12 @@ namespace swimba {
 // zero_out (may be NULL): a [T, zero_bytes_per_token] buffer the kernel clears on the way (the
 // mixed streams, when the projection adds its slots in place).  scalars.l2 != NULL: the call also
 // produces the SSD step sizes and tile log-decays of the same forward (they depend on dt only and
-// run beside the router, inside its launch or as a kernel in front of it).
+// run beside the router, inside its launch or as a kernel in front of it).  pi_out (may be NULL):
+// the softmax over all E, [T,E].
 int launch_router(LaunchCtx &ctx, int dtype, const void *u, const void *W_r, int64_t T, int F,
                   int E, int k, int32_t *idx, float *w, int *counts, int *perm, int64_t cap,
-                  int sm_count, void *zero_out, int zero_bytes_per_token, const ScalarsArgs &scalars);
+                  int sm_count, void *zero_out, int zero_bytes_per_token, const ScalarsArgs &scalars,
+                  float *pi_out = nullptr);
 
 // K1b (tensor cores): grouped GEMM over the per-expert lists + slot sum.  `workspace` is sized
 // by expert_gemm_workspace_bytes and holds the histogram (zeroed by the caller before the
@@ -27,10 +29,13 @@ bool expert_gemm_adds_rows(int k);   // true: BC must be zero before launch_expe
 int *expert_gemm_counts(void *workspace);
 int *expert_gemm_perm(void *workspace);
 // slots_out (may be NULL): [T*k, S] bf16; when given, the projection of (token t, slot j), scaled by
-// its router weight, is stored in row t*k + j and nothing is mixed (BC is not touched).
+// its router weight (w NULL: 1), is stored in row t*k + j and nothing is mixed (BC is not touched).
 int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const float *w, int64_t T,
                        int F, int S, int E, int k, int sm_count, void *BC, void *workspace,
                        void *slots_out = nullptr);
+
+// BC[t, :] = sum_j w[t,j] slots[t*k + j, :], bf16 (w NULL: 1).
+int launch_mix_slots(LaunchCtx &ctx, const void *slots, const float *w, int64_t T, int S, int k, int sm_count, void *BC);
 
 // The same products on CTA pairs, 256 x 256 tiles, persistent: calls with enough tiles (pair_gemm_usable).
 // perm == NULL: the T rows of A as they lie (E = k = 1, no weights); out rows are ld_out elements apart.
@@ -45,7 +50,7 @@ int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *pe
 int launch_project_mix_simt(LaunchCtx &ctx, int dtype, const void *u, const void *W_e,
                             const int32_t *idx, const float *w, int64_t T, int F, int S, int E,
                             int k, void *BC, bool bc_fp32);
-// The same without the mix: row t*k + j of slots_out (dtype) = w[t,j] * W_e[idx[t,j]] u_t.
+// The same without the mix: row t*k + j of slots_out (dtype) = w[t,j] * W_e[idx[t,j]] u_t (w NULL: 1).
 int launch_project_slots_simt(LaunchCtx &ctx, int dtype, const void *u, const void *W_e,
                               const int32_t *idx, const float *w, int64_t T, int F, int S, int E,
                               int k, void *slots_out);
@@ -131,13 +136,14 @@ int launch_ssd_shard_finish(LaunchCtx &ctx, const void *x, const void *BC, const
                             const float *all_state, const float *all_decay, int rank, int B, int L, int H, int G,
                             int chunk, int sm_count, void *y, float *h_end, void *workspace);
 
-// Backward for the trained weights (router and expert matrices), plain CUDA-core kernels.
+// Backward for the trained weights (router and expert matrices).
 // adjoint: both passes of the recurrence's adjoint; dBC [T,S] fp32 (zeroed by the caller) receives
-// dBtilde | dCtilde.  weight_grads: softmax over all E (pi [T,E] scratch), dpi / dg (dg [T,E]
-// scratch) from the unscaled slot projections slots [T*k,S] (dtype), then dW_r [E,F] and dW_e
-// [E,S,F] (fp32, zeroed by the caller, accumulated with atomics).
+// dBtilde | dCtilde.  weight_grads: dpi / dg (dg [T,E] scratch) from the softmax over all E (pi [T,E], left by
+// launch_router) and the unscaled slot projections slots [T*k,S] (dtype; overwritten when perm is given),
+// then dW_r [E,F] and dW_e [E,S,F] (fp32, zeroed by the caller, accumulated with atomics).  perm / counts:
+// the per-expert lists of launch_router (bf16; the gradient of the expert matrices then runs on the tensor
+// cores), or NULL.
 bool ssd_adjoint_supported(int P, int N);
-int launch_fill(LaunchCtx &ctx, float *p, int64_t n, float v);
 int launch_ssd_adjoint(LaunchCtx &ctx, int dtype, const void *x, const void *dy, const void *BC, const float *dt,
                        const float *A, const float *dt_bias, const float *h0, int B, int L, int H, int P, int N,
                        int G, float *dBC);
@@ -148,9 +154,11 @@ ScalarsArgs ssd_adjoint_scalars_args(const float *dt, const float *A, const floa
                                      void *workspace);
 int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, const void *BC, const float *h0, int B,
                              int L, int H, int G, int sm_count, float *dBC, void *workspace);
-int launch_weight_grads(LaunchCtx &ctx, int dtype, const void *u, const void *W_r, const void *slots,
-                        const int32_t *idx, const float *w, const float *dBC, int64_t Tn, int F, int S, int E,
-                        int k, float *pi, float *dg, float *dW_r, float *dW_e);
+int launch_weight_grads(LaunchCtx &ctx, int dtype, const void *u, void *slots, const int32_t *idx, const float *w,
+                        const float *dBC, int64_t Tn, int F, int S, int E, int k, const float *pi, float *dg,
+                        const int *perm, const int *counts, int sm_count, float *dW_r, float *dW_e);
+int launch_pair_outer(LaunchCtx &ctx, const void *g, const void *u, const int *perm, const int *counts, int64_t T,
+                      int F, int S, int E, int k, int sm_count, float *dW);
 
 // One warp waiting on a barrier nobody signals, with the given limit (see swimba_selftest_wait).
 // out_dev: three 64-bit words on the device.

@@ -169,7 +169,7 @@ expert_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __nv_bfloat
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
             const int row = hf * 128 + warp * 32 + lane;
-            wr2[hf] = (row < nrows && row_src[row] >= 0) ? w_slot[perm[row0 + row]] : 0.f;
+            wr2[hf] = (row < nrows && row_src[row] >= 0) ? (w_slot ? w_slot[perm[row0 + row]] : 1.f) : 0.f;
         }
 
         // ---- epilogue: thread = output row of each half.  All MMAs have completed, so the
@@ -268,11 +268,13 @@ expert_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __nv_bfloat
     if (uwarp == 5) tc::tmem_dealloc(tmem_base, TMEM_COLS);
 }
 
-// BC[t, :] = sum_j P[t*k + j, :]   (slots already carry their router weight).
+// BC[t, :] = sum_j w[t,j] P[t*k + j, :]   (w null: the slots already carry their router weight).
 __global__ void __launch_bounds__(256)
-mix_slots_kernel(const __nv_bfloat16 *__restrict__ P, int64_t T, int S, int k,
+mix_slots_kernel(const __nv_bfloat16 *__restrict__ P, const float *__restrict__ w, int64_t T, int S, int k,
                  __nv_bfloat16 *__restrict__ BC)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     const int vec_per_row = S >> 3;
     const int64_t nvec = T * vec_per_row;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec;
@@ -283,8 +285,9 @@ mix_slots_kernel(const __nv_bfloat16 *__restrict__ P, int64_t T, int S, int k,
         for (int j = 0; j < k; ++j) {
             float pv[8];
             load8(P + ((t * k + j) * S) + v * 8, pv);
+            const float wj = w ? w[t * k + j] : 1.f;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) acc[q] += pv[q];
+            for (int q = 0; q < 8; ++q) acc[q] = fmaf(wj, pv[q], acc[q]);
         }
         uint4 o = make_uint4(tc::pack_bf16x2(acc[0], acc[1]), tc::pack_bf16x2(acc[2], acc[3]),
                              tc::pack_bf16x2(acc[4], acc[5]), tc::pack_bf16x2(acc[6], acc[7]));
@@ -324,17 +327,14 @@ bool expert_gemm_supported(int F, int S)
     return S % 32 == 0 && F >= 64;
 }
 
-// The slot sum behind a projection that stored its slots (wanted: the call mixes them).
-static int mix_slots(LaunchCtx &ctx, const __nv_bfloat16 *slots, int64_t T, int S, int k, bool wanted, int sm_count,
-                     void *BC)
+int launch_mix_slots(LaunchCtx &ctx, const void *slots, const float *w, int64_t T, int S, int k, int sm_count, void *BC)
 {
-    if (k > 1 && wanted) {
-        int64_t blocks = ceil_div64(T * (S / 8), 256);
-        if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
-        ctx.begin(STAGE_MIX_SLOTS);
-        mix_slots_kernel<<<(unsigned)blocks, 256, 0, ctx.stream>>>(slots, T, S, k, (__nv_bfloat16 *)BC);
-        ctx.end();
-    }
+    int64_t blocks = ceil_div64(T * (S / 8), 256);
+    if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
+    ctx.begin(STAGE_MIX_SLOTS);
+    launch_kernel(mix_slots_kernel, dim3((unsigned)blocks), dim3(256), 0, ctx.stream, true, (const __nv_bfloat16 *)slots, w,
+                  T, S, k, (__nv_bfloat16 *)BC);
+    ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
@@ -353,10 +353,11 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
         ? (__nv_bfloat16 *)((char *)perm + gemm_ws_up((size_t)E * T * sizeof(int)))
         : (__nv_bfloat16 *)BC;
 
+    const bool mix = k > 1 && !add_rows && !slots_out;      // the slots were stored and are summed afterwards
     if (pair_gemm_usable(T * k, F, S, sm_count)) {
         const int rc = launch_pair_gemm(ctx, u, W_e, perm, counts, w, T, F, S, E, k, add_rows != 0, sm_count, slots, S);
-        if (rc != SWIMBA_OK) return rc;
-        return mix_slots(ctx, slots, T, S, k, !add_rows && !slots_out, sm_count, BC);
+        if (rc != SWIMBA_OK || !mix) return rc;
+        return launch_mix_slots(ctx, slots, nullptr, T, S, k, sm_count, BC);
     }
     // Widest column tile that divides S; narrower when there are too few row tiles to fill the
     // GPU (decode-sized calls), so that the weight rows are spread over more SMs.
@@ -388,7 +389,8 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
     else SWIMBA_GEMM_CASE(32);
 #undef SWIMBA_GEMM_CASE
     ctx.end();
-    return mix_slots(ctx, slots, T, S, k, !add_rows && !slots_out, sm_count, BC);
+    if (mix) return launch_mix_slots(ctx, slots, nullptr, T, S, k, sm_count, BC);
+    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
 }  // namespace swimba

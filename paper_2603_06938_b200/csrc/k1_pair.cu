@@ -13,7 +13,7 @@
 // (1.19 PFLOP/s), 32768 x 2048 x 8192 dense 1190 -> 661 us (1.66 PFLOP/s).  Gathered rows come by
 // cp.async: tile::gather4 loads (512 bytes each with the 128-byte swizzle) took 150 us for the first shape.
 #include "internal.h"
-#include "tc05.cuh"
+#include "pair.cuh"
 
 namespace swimba {
 
@@ -39,7 +39,7 @@ struct PairSmall {
 struct PairArgs {
     const int *perm, *counts;      // per-expert lists (entries t*k + j) and their lengths; null: dense rows
     int64_t cap;                   // list capacity = tokens
-    const float *w_slot;           // [T*k] row weights
+    const float *w_slot;           // [T*k] row weights; null: 1
     const __nv_bfloat16 *rows;     // the rows the lists index
     __nv_bfloat16 *out;
     int64_t ld_out;
@@ -49,32 +49,6 @@ struct PairArgs {
     int *d_status;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// Address of the same variable in the pair's first CTA, which issues the products and owns the barriers
-// that the loads report to.
-__device__ __forceinline__ uint32_t leader_addr(const void *p)
-{
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(tc::smem_u32(p)));
-    return r;
-}
-__device__ __forceinline__ void pair_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Arrival at a barrier of the first CTA.  What it announces -- rows in this SM's own shared memory that
-// this SM's tensor core will read, tensor memory of this SM that its tensor core may overwrite -- is
-// ordered by the proxy fence / tcgen05 fence in front; no other SM reads it, so that no cluster-wide
-// release is needed (with one, every step of the product took 2000 cycles).
-__device__ __forceinline__ void remote_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void pair_load_2d(void *dst, const CUtensorMap *m, uint32_t bar, int c0, int c1)
 {
     asm volatile(
@@ -91,23 +65,6 @@ __device__ __forceinline__ void pair_load_3d(void *dst, const CUtensorMap *m, ui
         "l"(m), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
-__device__ __forceinline__ void pair_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrives on the barrier at this offset in BOTH CTAs once all products issued so far have completed.
-__device__ __forceinline__ void pair_commit(uint64_t *bar)
-{
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            tc::smem_u32(bar)),
-        "h"((uint16_t)3)
-        : "memory");
-}
 }  // namespace
 
 // DENSE: rows are taken as they lie (one expert, no lists, no weights).
@@ -121,7 +78,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     int *abort_flag = &sm->abort_flag;
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const uint32_t rank = cluster_rank();
+    const uint32_t rank = tc::cluster_rank();
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     if ((tc::smem_u32(smem) & 1023u) != 0) {      // the swizzled tiles need a 1024-byte aligned base (the
         if (tid == 0) atomicCAS(p.d_status, 0, SWIMBA_ERR_DEVICE_BOUNDS);   // same in both CTAs)
@@ -144,10 +101,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         tc::prefetch_tmap(&tmap_w);
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         tc::smem_u32(&sm->tmem_slot)), "r"(512)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        tc::pair_tmem_alloc(&sm->tmem_slot);
     }
     grid_dep_launch();
     grid_dep_wait();        // lists, weights and rows come from the kernels in front
@@ -179,7 +133,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
     tc::tc_fence_before();
     __syncthreads();
-    pair_sync();            // barriers and tensor memory of both CTAs are ready
+    tc::pair_sync();            // barriers and tensor memory of both CTAs are ready
     tc::tc_fence_after();
     const uint32_t tmem = sm->tmem_slot;
     const int ncol = ceil_div(p.S, PG_BN);
@@ -226,7 +180,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                 tc::mbar_wait(&sm->empty[s], ((n / PG_STAGES) & 1) ^ 1, abort_flag, p.d_status);
                 uint8_t *sA = smem + s * PG_STAGE_BYTES, *sB = sA + PG_A_BYTES;
                 if (elected) {
-                    const uint32_t bar = leader_addr(&sm->full[s]);
+                    const uint32_t bar = tc::leader_addr(&sm->full[s]);
                     if (rank == 0) tc::mbar_arrive_expect_tx(&sm->full[s], DENSE ? 2 * PG_STAGE_BYTES : 2 * PG_A_BYTES);
                     pair_load_3d(sB, &tmap_w, bar, kb * PG_BK, ti.n0 + (int)rank * (ti.nt >> 1), ti.e);
                     if (DENSE) pair_load_2d(sA, &tmap_a, bar, kb * PG_BK, ti.row0 + (int)rank * 128);
@@ -255,10 +209,10 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                     const uint64_t dB = tc::smem_desc_advance(dA, PG_A_BYTES);
 #pragma unroll
                     for (int kk = 0; kk < PG_BK / 16; ++kk)
-                        pair_mma(acc, tc::smem_desc_advance(dA, kk * 32), tc::smem_desc_advance(dB, kk * 32), idesc,
+                        tc::pair_mma(acc, tc::smem_desc_advance(dA, kk * 32), tc::smem_desc_advance(dB, kk * 32), idesc,
                                  (kb | kk) != 0);
-                    pair_commit(&sm->empty[s]);
-                    if (kb == KB - 1) pair_commit(&sm->acc_full[buf]);
+                    tc::pair_commit(&sm->empty[s]);
+                    if (kb == KB - 1) tc::pair_commit(&sm->acc_full[buf]);
                 }
                 __syncwarp();
             }
@@ -278,7 +232,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                 tc::fence_proxy_async_smem();
                 if (elected) {
                     if (rank == 0) tc::mbar_arrive(&sm->full[s]);
-                    else remote_arrive(leader_addr(&sm->full[s]));
+                    else tc::remote_arrive(tc::leader_addr(&sm->full[s]));
                 }
                 __syncwarp();
             }
@@ -303,9 +257,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                 for (int i = 0; i < 8; ++i)
                     tc::cp_async16(a_base + tc::sw128_offset(q * 32 + i * 4 + (lane >> 3), chunk),
                                    in ? src[i] + kb * PG_BK : p.rows, in ? 16u : 0u);
-                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(
-                                 tc::smem_u32(&sm->gathered[s]))
-                             : "memory");
+                tc::cp_async_arrive(&sm->gathered[s]);
             }
         }
         tc::cp_async_commit();
@@ -325,7 +277,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             if (!DENSE) {
                 const int entry = entry_of(ti, r);
                 ok = ok && entry >= 0;
-                wr = ok ? p.w_slot[entry] : 0.f;
+                wr = (ok && p.w_slot) ? p.w_slot[entry] : 1.f;
                 dst = p.add_rows ? entry / p.k : entry;
             }
             tc::mbar_wait(&sm->acc_full[buf], (it >> 1) & 1, abort_flag, p.d_status);
@@ -360,7 +312,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             tc::tc_fence_before();
             tc::fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) remote_arrive(leader_addr(&sm->acc_empty[buf]));
+            if (lane == 0) tc::remote_arrive(tc::leader_addr(&sm->acc_empty[buf]));
             if (ok && nmain > 0) {
                 __nv_bfloat16 *row = p.out + dst * p.ld_out + ti.n0;
                 if (p.add_rows) tc::bulk_reduce_add_bf16(row, srow, (uint32_t)nmain * 2);
@@ -372,10 +324,9 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
     tc::tc_fence_before();
     __syncthreads();
-    pair_sync();            // nobody reads or signals the other CTA's memory any more
+    tc::pair_sync();            // nobody reads or signals the other CTA's memory any more
     tc::tc_fence_after();
-    if (warp == 1)
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    if (warp == 1) tc::pair_tmem_dealloc(tmem);
 }
 
 int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *perm, const int *counts,

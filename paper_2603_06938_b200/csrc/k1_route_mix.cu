@@ -30,7 +30,8 @@ __global__ void __launch_bounds__(256)
 router_topk_kernel(const T *__restrict__ u, const T *__restrict__ W_r, int64_t Ttok, int F, int E,
                    int k, int32_t *__restrict__ idx, float *__restrict__ w, int *__restrict__ counts,
                    int *__restrict__ perm, int64_t cap, int stage_w, int chunk,
-                   uint4 *__restrict__ zero_out, int zero_vec_per_token, int router_blocks)
+                   uint4 *__restrict__ zero_out, int zero_vec_per_token, int router_blocks,
+                   float *__restrict__ pi_out)
 {
     grid_dep_launch();      // the projection kernel may set itself up under this kernel's tail
     const int rblock = (int)blockIdx.x;
@@ -142,9 +143,13 @@ router_topk_kernel(const T *__restrict__ u, const T *__restrict__ W_r, int64_t T
             }
 #pragma unroll
             for (int o = GW / 2; o >= DUP; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+            const int64_t t = t0 + q_own;
+            if (pi_out && t < tend && (lane % GW) % DUP == 0) {
+#pragma unroll
+                for (int i = 0; i < R; ++i) if (e0 + i < E) pi_out[t * E + e0 + i] = pv[i] / z;
+            }
             // k rounds of "largest remaining logit, lowest index on ties"; weights are NOT
             // renormalised
-            const int64_t t = t0 + q_own;
             for (int j = 0; j < k; ++j) {
                 float bg = gv[0], bp = pv[0];
                 int be = e0;
@@ -218,7 +223,7 @@ router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__re
                   int64_t Ttok, int F, int E, int k, int32_t *__restrict__ idx, float *__restrict__ w,
                   int *__restrict__ counts, int *__restrict__ perm, int64_t cap, int stage_w,
                   int chunk, uint4 *__restrict__ zero_out, int zero_vec_per_token, int router_blocks,
-                  int scalar_blocks, const ScalarsArgs scalars)
+                  int scalar_blocks, const ScalarsArgs scalars, float *__restrict__ pi_out)
 {
     grid_dep_launch();      // the projection kernel may set itself up under this kernel's tail
     if ((int)blockIdx.x < scalar_blocks) {
@@ -329,9 +334,13 @@ router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__re
             }
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+            const int64_t t = t0 + tl;
+            if (pi_out && t < tend) {
+#pragma unroll
+                for (int i = 0; i < NT; ++i) if (sub + 8 * i < E) pi_out[t * E + sub + 8 * i] = pv[i] / z;
+            }
             // k rounds of "largest remaining logit, lowest index on ties"; weights are NOT
             // renormalised
-            const int64_t t = t0 + tl;
             for (int j = 0; j < k; ++j) {
                 float bg = gv[0], bp = pv[0];
                 int be = sub;
@@ -419,7 +428,7 @@ router_stream_kernel(const __grid_constant__ CUtensorMap tmap_u, const __nv_bflo
                      int64_t Ttok, int F, int E, int k, int32_t *__restrict__ idx, float *__restrict__ w,
                      int *__restrict__ counts, int *__restrict__ perm, int64_t cap,
                      uint4 *__restrict__ zero_out, int zero_vec_per_token, int router_ctas,
-                     int nstages, int *d_status)
+                     int nstages, int *d_status, float *__restrict__ pi_out)
 {
     grid_dep_launch();      // the projection kernel may set itself up under this kernel's tail
     const int cta = (int)blockIdx.x;
@@ -564,6 +573,13 @@ router_stream_kernel(const __grid_constant__ CUtensorMap tmap_u, const __nv_bflo
             }
             z += __shfl_xor_sync(0xffffffffu, z, 1);
             z += __shfl_xor_sync(0xffffffffu, z, 2);
+            if (pi_out && t < tend) {
+#pragma unroll
+                for (int i = 0; i < 2 * NT; ++i) {
+                    const int e = (i >> 1) * 8 + 2 * c + (i & 1);
+                    if (e < E) pi_out[t * E + e] = pv[i] / z;
+                }
+            }
             // k rounds of "largest remaining logit, lowest index on ties"; weights are NOT
             // renormalised
             for (int j = 0; j < k; ++j) {
@@ -615,13 +631,14 @@ router_stream_kernel(const __grid_constant__ CUtensorMap tmap_u, const __nv_bflo
 // One expert: the softmax is identically 1 and every token is routed to expert 0.
 __global__ void __launch_bounds__(256)
 router_single_expert_kernel(int64_t Ttok, int32_t *__restrict__ idx, float *__restrict__ w,
-                            int *__restrict__ counts, int *__restrict__ perm)
+                            int *__restrict__ counts, int *__restrict__ perm, float *__restrict__ pi_out)
 {
     grid_dep_launch();
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < Ttok;
          t += (int64_t)gridDim.x * blockDim.x) {
         idx[t] = 0;
         w[t] = 1.f;
+        if (pi_out) pi_out[t] = 1.f;
         if (counts) perm[t] = (int)t;
     }
     if (counts && blockIdx.x == 0 && threadIdx.x == 0) counts[0] = (int)Ttok;
@@ -658,7 +675,7 @@ static bool router_stream_usable(const void *u, int64_t Ttok, int F, int E, int 
 static int launch_router_stream(LaunchCtx &ctx, const __nv_bfloat16 *u, const __nv_bfloat16 *W_r,
                                 int64_t Ttok, int F, int E, int k, int32_t *idx, float *w, int *counts,
                                 int *perm, int64_t cap, int sm_count, void *zero_out,
-                                int zero_bytes_per_token, bool behind_scalars)
+                                int zero_bytes_per_token, bool behind_scalars, float *pi_out)
 {
     const int NT = E <= 8 ? 1 : E <= 16 ? 2 : E <= 32 ? 4 : 8;
     // ring depth: the deepest (up to RS_MAX_STAGES) that still lets two CTAs share an SM, else
@@ -684,7 +701,7 @@ static int launch_router_stream(LaunchCtx &ctx, const __nv_bfloat16 *u, const __
             return SWIMBA_ERR_CUDA;                                                             \
         launch_kernel(kern, dim3((unsigned)ctas), dim3(RS_THREADS), smem, ctx.stream, behind_scalars, tmap, \
                       W_r, Ttok, F, E, k, idx, w, counts, perm, cap, (uint4 *)zero_out,         \
-                      zero_bytes_per_token / 16, (int)ctas, nstages, ctx.d_status);             \
+                      zero_bytes_per_token / 16, (int)ctas, nstages, ctx.d_status, pi_out);             \
     } while (0)
     if (NT == 1) SWIMBA_ROUTER_STREAM_CASE(1);
     else if (NT == 2) SWIMBA_ROUTER_STREAM_CASE(2);
@@ -698,7 +715,7 @@ static int launch_router_stream(LaunchCtx &ctx, const __nv_bfloat16 *u, const __
 static int launch_router_mma(LaunchCtx &ctx, const __nv_bfloat16 *u, const __nv_bfloat16 *W_r,
                              int64_t Ttok, int F, int E, int k, int32_t *idx, float *w, int *counts,
                              int *perm, int64_t cap, int sm_count, void *zero_out,
-                             int zero_bytes_per_token, const ScalarsArgs &scalars)
+                             int zero_bytes_per_token, const ScalarsArgs &scalars, float *pi_out)
 {
     const int NT = E <= 8 ? 1 : E <= 16 ? 2 : E <= 32 ? 4 : 8;
     const int chunk = router_chunk(Ttok, sm_count);
@@ -721,7 +738,7 @@ static int launch_router_mma(LaunchCtx &ctx, const __nv_bfloat16 *u, const __nv_
         launch_kernel(kern, dim3((unsigned)(extra + blocks)), dim3(256), smem, ctx.stream, false, \
                       u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, stage_w, chunk,         \
                       (uint4 *)zero_out, zero_bytes_per_token / 16, (int)blocks, (int)extra,    \
-                      scalars);                                                                 \
+                      scalars, pi_out);                                                                 \
     } while (0)
     if (NT == 1) SWIMBA_ROUTER_MMA_CASE(1);
     else if (NT == 2) SWIMBA_ROUTER_MMA_CASE(2);
@@ -736,7 +753,7 @@ template <typename T>
 static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Ttok, int F, int E,
                            int k, int32_t *idx, float *w, int *counts, int *perm, int64_t cap,
                            int sm_count, void *zero_out, int zero_bytes_per_token,
-                           const ScalarsArgs &scalars)
+                           const ScalarsArgs &scalars, float *pi_out)
 {
     const int warps = 8;
     // The SSD step sizes of the same call (scalars.l2 != NULL) depend on dt only and run beside the
@@ -746,7 +763,7 @@ static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Tto
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (E > 1 && !router_stream_usable(u, Ttok, F, E, sm_count) && F % (32 * RM_KSPLIT) == 0 && E <= 64)
             return launch_router_mma(ctx, u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, sm_count,
-                                     zero_out, zero_bytes_per_token, scalars);
+                                     zero_out, zero_bytes_per_token, scalars, pi_out);
         behind_scalars = E > 1 && scalars.l2 && router_stream_usable(u, Ttok, F, E, sm_count);
     }
     if (scalars.l2) {
@@ -758,14 +775,14 @@ static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Tto
         if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
         ctx.begin(STAGE_ROUTER);
         launch_kernel(router_single_expert_kernel, dim3((unsigned)blocks), dim3(256), 0, ctx.stream,
-                      false, Ttok, idx, w, counts, perm);
+                      false, Ttok, idx, w, counts, perm, pi_out);
         ctx.end();
         return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
     }
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (router_stream_usable(u, Ttok, F, E, sm_count))
             return launch_router_stream(ctx, u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, sm_count,
-                                        zero_out, zero_bytes_per_token, behind_scalars);
+                                        zero_out, zero_bytes_per_token, behind_scalars, pi_out);
     }
     const size_t w_bytes = (size_t)E * F * sizeof(T);
     const int stage_w = (w_bytes <= 64 * 1024 && (w_bytes & 15) == 0) ? 1 : 0;
@@ -784,7 +801,7 @@ static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Tto
         if (blocks > cap_blocks) blocks = cap_blocks;                                          \
         launch_kernel(kern, dim3((unsigned)blocks), dim3(warps * 32), smem, ctx.stream, false,   \
                       u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, stage_w, chunk,        \
-                      (uint4 *)zero_out, zero_bytes_per_token / 16, (int)blocks);              \
+                      (uint4 *)zero_out, zero_bytes_per_token / 16, (int)blocks, pi_out);      \
     } while (0)
     if (E <= 2) SWIMBA_ROUTER_CASE(2, 8);
     else if (E <= 4) SWIMBA_ROUTER_CASE(4, 8);
@@ -799,15 +816,15 @@ static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Tto
 
 int launch_router(LaunchCtx &ctx, int dtype, const void *u, const void *W_r, int64_t T, int F,
                   int E, int k, int32_t *idx, float *w, int *counts, int *perm, int64_t cap,
-                  int sm_count, void *zero_out, int zero_bytes_per_token, const ScalarsArgs &scalars)
+                  int sm_count, void *zero_out, int zero_bytes_per_token, const ScalarsArgs &scalars, float *pi_out)
 {
     if (T <= 0) return SWIMBA_OK;
     if (dtype == SWIMBA_DTYPE_FP32)
         return launch_router_t<float>(ctx, (const float *)u, (const float *)W_r, T, F, E, k, idx, w,
-                                      counts, perm, cap, sm_count, zero_out, zero_bytes_per_token, scalars);
+                                      counts, perm, cap, sm_count, zero_out, zero_bytes_per_token, scalars, pi_out);
     return launch_router_t<__nv_bfloat16>(ctx, (const __nv_bfloat16 *)u,
                                           (const __nv_bfloat16 *)W_r, T, F, E, k, idx, w, counts,
-                                          perm, cap, sm_count, zero_out, zero_bytes_per_token, scalars);
+                                          perm, cap, sm_count, zero_out, zero_bytes_per_token, scalars, pi_out);
 }
 
 // One warp per (token, block of RW stream rows): BC[t, r] = sum_j w_j <W_e[e_j, r, :], u_t>.
@@ -834,7 +851,7 @@ project_mix_simt_kernel(const T *__restrict__ u, const T *__restrict__ W_e,
 #pragma unroll
     for (int j = 0; j < SWIMBA_MAX_TOPK; ++j) {
         ej[j] = (j < k) ? idx[t * kst + joff + j] : 0;
-        wj[j] = (j < k) ? w[t * kst + joff + j] : 0.f;
+        wj[j] = (j < k) ? (w ? w[t * kst + joff + j] : 1.f) : 0.f;
         if (check && (ej[j] < 0 || ej[j] >= E)) {      // a bad expert index is skipped, not followed
             if (lane == 0) atomicCAS(d_status, 0, SWIMBA_ERR_DEVICE_BOUNDS);
             ej[j] = 0;
