@@ -10,7 +10,7 @@
 // tile per pair, where runs of fixed length would add the whole matrix once per 1000 entries.
 // What bounds it: the rows gathered from L2, 64 KB per step and pair against 512 cycles of tensor time.
 // 65536 entries of 8 experts, S = 256, F = 2048: mma.sync tiles of 128 x 128 over runs of 4096 tokens
-// 711 us, this kernel @OUTER@.
+// 711 us, this kernel 75 us (0.92 PFLOP/s).
 #include "internal.h"
 #include "pair.cuh"
 
@@ -24,11 +24,15 @@ constexpr int PO_COLS = 64;                                  // columns of a sta
 constexpr uint32_t PO_ROW = PO_COLS * 4 + 16;
 constexpr uint32_t PO_OUT = PO_STAGES * PO_STAGE_BYTES;
 constexpr uint32_t PO_SMALL = PO_OUT + 128 * PO_ROW;
+constexpr int PO_LIST = 16;                                  // steps whose list entries are held
 constexpr int PO_EPI_WARP = 4, PO_GATHER_WARP = 8, PO_GATHER = 256;
 constexpr int PO_THREADS = 32 * PO_GATHER_WARP + PO_GATHER;
 
-struct OuterSmall {
+struct __align__(16) OuterSmall {
+    int list[PO_LIST][PO_BK + 4];                            // list entries of the steps ahead (from the 16-byte
+                                                             // boundary at or below the first one on)
     uint64_t full[PO_STAGES], empty[PO_STAGES], gathered[PO_STAGES], acc_full[2], acc_empty[2];
+    uint64_t list_full[PO_LIST], list_free[PO_LIST];
     uint32_t tmem_slot;
     int abort_flag;
     int64_t step_end[SWIMBA_MAX_EXPERTS];                    // steps of experts 0 .. e, summed
@@ -37,7 +41,7 @@ struct OuterSmall {
 
 struct OuterArgs {
     const __nv_bfloat16 *g, *u;       // [T*k, S], [T, F]
-    const int *perm, *counts;
+    const int *perm, *counts;         // (up to 256 bytes behind the last list are read, not used)
     int64_t cap;
     float *dW;                        // [E, S, F]
     int E, F, S, k, check;
@@ -71,6 +75,10 @@ pair_outer_kernel(const OuterArgs p)
             tc::mbar_init(&sm->full[s], 2);                 // the gathered rows of either CTA
             tc::mbar_init(&sm->gathered[s], PO_GATHER);
             tc::mbar_init(&sm->empty[s], 1);
+        }
+        for (int s = 0; s < PO_LIST; ++s) {
+            tc::mbar_init(&sm->list_full[s], 1);
+            tc::mbar_init(&sm->list_free[s], PO_GATHER / 32);
         }
         for (int s = 0; s < 2; ++s) {
             tc::mbar_init(&sm->acc_full[s], 1);
@@ -176,6 +184,27 @@ pair_outer_kernel(const OuterArgs p)
             }
             __syncwarp();
         }
+    } else if (warp == 3) {
+        // ------------------------------------------------------------------ lists, PO_LIST steps ahead
+        // (by bulk copies: ordinary loads return behind the gather warps' copies in flight, however far
+        // ahead they are issued, and hold the pipeline at a fraction of its depth: 150 us)
+        const bool elected = tc::elect_one();
+        uint32_t n = 0;
+        for (int64_t pos = run_a; pos < run_b;) {
+            const Part pt = part_at(pos);
+            for (int j = 0; j < pt.n; ++j, ++n) {
+                const uint32_t q = n % PO_LIST;
+                tc::mbar_wait(&sm->list_free[q], ((n / PO_LIST) & 1) ^ 1, abort_flag, p.d_status);
+                if (elected) {
+                    const int64_t first = (int64_t)pt.e * p.cap + (int64_t)(pt.k0 + j) * PO_BK;
+                    const uint32_t bytes = PO_BK * 4 + ((first & 3) ? 16 : 0);
+                    tc::mbar_arrive_expect_tx(&sm->list_full[q], bytes);
+                    tc::bulk_load(sm->list[q], p.perm + (first & ~(int64_t)3), bytes, &sm->list_full[q]);
+                }
+                __syncwarp();
+            }
+            pos += pt.n;
+        }
     } else if (warp >= PO_GATHER_WARP) {
         // ------------------------------------------------------------------ row gather (both CTAs)
         // thread -> 16-byte chunk `ch` of the 256 bytes of rows r0, r0 + 16, r0 + 32, r0 + 48, both operands
@@ -183,37 +212,34 @@ pair_outer_kernel(const OuterArgs p)
         uint32_t n = 0;
         for (int64_t pos = run_a; pos < run_b;) {
             const Part pt = part_at(pos);
-            const int *list = p.perm + (int64_t)pt.e * p.cap;
             const int sc = pt.s0 + (int)rank * 128 + ch * 8, fc = pt.f0 + (int)rank * 128 + ch * 8;
             const bool s_in = sc < p.S, f_in = fc < p.F;
-            int ent[4];
-            auto fetch = [&](int step) {
+            const __nv_bfloat16 *g0 = p.g + sc, *u0 = p.u + fc;
+            const int shift = (int)(((int64_t)pt.e * p.cap) & 3);
+            for (int j = 0; j < pt.n; ++j, ++n) {
+                const uint32_t s = n % PO_STAGES, q = n % PO_LIST;
+                tc::mbar_wait(&sm->list_full[q], (n / PO_LIST) & 1, abort_flag, p.d_status);
+                int ent[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int r = step * PO_BK + r0 + 16 * i;
-                    int v = r < pt.cnt ? list[r] : -1;
-                    if (p.check && r < pt.cnt && (v < 0 || v >= p.cap * p.k)) {
+                    const int r = r0 + 16 * i;
+                    ent[i] = (pt.k0 + j) * PO_BK + r < pt.cnt ? sm->list[q][shift + r] : -1;
+                    if (p.check && (ent[i] < -1 || ent[i] >= p.cap * p.k)) {
                         atomicCAS(p.d_status, 0, SWIMBA_ERR_DEVICE_BOUNDS);
-                        v = -1;
+                        ent[i] = -1;
                     }
-                    ent[i] = v;
                 }
-            };
-            fetch(pt.k0);
-            for (int j = 0; j < pt.n; ++j, ++n) {
-                const uint32_t s = n % PO_STAGES;
-                int cur[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) cur[i] = ent[i];
-                if (j + 1 < pt.n) fetch(pt.k0 + j + 1);
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&sm->list_free[q]);
                 tc::mbar_wait(&sm->empty[s], ((n / PO_STAGES) & 1) ^ 1, abort_flag, p.d_status);
                 const uint32_t base = tc::smem_u32(smem + s * PO_STAGE_BYTES) + (ch >> 3) * PO_SLAB;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const uint32_t off = tc::sw128_offset(r0 + 16 * i, ch & 7);
-                    const bool gi = cur[i] >= 0 && s_in, ui = cur[i] >= 0 && f_in;
-                    tc::cp_async16(base + off, gi ? p.g + (int64_t)cur[i] * p.S + sc : p.g, gi ? 16u : 0u);
-                    tc::cp_async16(base + 2 * PO_SLAB + off, ui ? p.u + (int64_t)(cur[i] / p.k) * p.F + fc : p.u, ui ? 16u : 0u);
+                    const bool gi = ent[i] >= 0 && s_in, ui = ent[i] >= 0 && f_in;
+                    const int tok = p.k == 2 ? ent[i] >> 1 : ent[i] / p.k;
+                    tc::cp_async16(base + off, gi ? g0 + (int64_t)ent[i] * p.S : p.g, gi ? 16u : 0u);
+                    tc::cp_async16(base + 2 * PO_SLAB + off, ui ? u0 + (int64_t)tok * p.F : p.u, ui ? 16u : 0u);
                 }
                 tc::cp_async_arrive(&sm->gathered[s]);
             }

@@ -240,14 +240,21 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         // ------------------------------------------------------------------ row gather (both CTAs)
         // thread -> 16-byte chunk lane % 8 of rows 4 i + lane / 8 of its warp's 32
         const int q = warp - PG_GATHER_WARP, chunk = lane & 7;
+        // the list entries are fetched a tile ahead: behind the copies in flight they would return late
         uint32_t n = 0;
-        for (int t = pair; t < ntiles; t += npairs) {
+        int ent[8];
+        auto fetch = [&](int t) {
+            if (t >= ntiles) return;
             const Tile ti = tile_of(t);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ent[i] = entry_of(ti, ti.row0 + (int)rank * 128 + q * 32 + i * 4 + (lane >> 3));
+        };
+        fetch(pair);
+        for (int t = pair; t < ntiles; t += npairs) {
             const __nv_bfloat16 *src[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                src[i] = p.rows + chunk * 8 +
-                         (int64_t)(max(entry_of(ti, ti.row0 + (int)rank * 128 + q * 32 + i * 4 + (lane >> 3)), 0) / p.k) * p.F;
+            for (int i = 0; i < 8; ++i) src[i] = p.rows + chunk * 8 + (int64_t)(max(ent[i], 0) / p.k) * p.F;
+            fetch(t + npairs);
             for (int kb = 0; kb < KB; ++kb, ++n) {
                 const uint32_t s = n % PG_STAGES;
                 tc::mbar_wait(&sm->empty[s], ((n / PG_STAGES) & 1) ^ 1, abort_flag, p.d_status);
