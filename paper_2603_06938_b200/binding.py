@@ -154,16 +154,19 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+# (addresses are passed as plain integers: the declared argument types convert them, and a small call is
+# bound by what happens here)
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
     assert t.is_contiguous(), "tensors must be contiguous"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream: Optional[torch.cuda.Stream]):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 class Handle:
@@ -225,7 +228,7 @@ def swimba_host_workspace_bytes(h: Handle, B: int, L: int) -> int:
 def _ws(workspace: Optional[torch.Tensor]):
     if workspace is None:
         return None, 0
-    return ctypes.c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size()
+    return workspace.data_ptr(), workspace.nbytes
 
 
 def swimba_forward(h: Handle, w: swimba_weights, u, x, dt, h0, B: int, L: int, y, h_final,
@@ -283,7 +286,7 @@ def swimba_shard_finish(h: Handle, w: swimba_weights, x, h0, all_state, all_deca
 def _offsets(cu_seqlens):
     """Host offsets (a sequence of ints) as a C array of nseq + 1 int32."""
     n = len(cu_seqlens)
-    return (ctypes.c_int32 * n)(*[int(v) for v in cu_seqlens]), n - 1
+    return (ctypes.c_int32 * n)(*map(int, cu_seqlens)), n - 1
 
 
 def swimba_packed_workspace_bytes(h: Handle, cu_seqlens) -> int:

@@ -71,7 +71,9 @@ DecLayout dec_layout(const swimba_config &c, int B)
     DecLayout l;
     const size_t S = 2u * c.n_groups * c.d_state;
     size_t off = 0;
-    l.bc = off;  off += align_up((size_t)B * S * sizeof(float));
+    const bool slots = front_small_supported(c.dtype, B, c.d_model, (int)S, c.n_experts, c.top_k) &&
+                       front_small_slots(B, c.top_k);
+    l.bc = off;  off += align_up((size_t)B * (slots ? c.top_k : 1) * S * sizeof(float));
     l.idx = off; off += align_up((size_t)B * c.top_k * sizeof(int32_t));
     l.w = off;   off += align_up((size_t)B * c.top_k * sizeof(float));
     l.gemm = off;
@@ -1031,19 +1033,22 @@ int swimba_decode_step(swimba_handle *h, const swimba_weights *w, const void *u,
     float *wt = topk_w ? topk_w : (float *)(ws + l.w);
     void *BC = ws + l.bc;
     const int S = 2 * c.n_groups * c.d_state;
-    // a handful of tokens: the two-kernel front end (fp32 streams); else bf16 streams from the
+    // a handful of tokens: the small front end (fp32 streams); else bf16 streams from the
     // grouped GEMM, or fp32 from the SIMT projection
     const bool small = front_small_supported(c.dtype, B, c.d_model, S, c.n_experts, c.top_k);
     const bool tensor = !small && use_tensor_k1(c);
     if (small) {
         rc = launch_front_small(ctx, u, w->W_router ? w->W_router : w->W_expert, w->W_expert, B, c.d_model, S,
-                                c.n_experts, c.top_k, idx, wt, (float *)BC);
+                                c.n_experts, c.top_k, idx, wt, (float *)BC, state,
+                                (int64_t)B * c.n_heads * c.head_dim * c.d_state * (int64_t)sizeof(float));
         if (rc != SWIMBA_OK) fail(h, rc, "routing / projection launch failed");
     } else {
         rc = run_route_mix(h, ctx, w, u, B, BC, !tensor, idx, wt, tensor ? ws + l.gemm : nullptr);
     }
     if (rc == SWIMBA_OK) {
-        rc = launch_decode_update(ctx, c.dtype, x, BC, !tensor, dt, w->A, w->dt_bias, w->D, state, B,
+        // (only the fused front end starts the update behind the previous step's)
+        rc = launch_decode_update(ctx, c.dtype, x, BC, !tensor, small && front_small_slots(B, c.top_k) ? c.top_k : 1,
+                                  small && front_small_fused(B), dt, w->A, w->dt_bias, w->D, state, B,
                                   c.n_heads, c.head_dim, c.d_state, c.n_groups, h->sm_count, y);
         if (rc != SWIMBA_OK) fail(h, rc, "decode launch failed");
     }

@@ -1,19 +1,25 @@
 // K1 for a handful of tokens (the decode step: one token per sequence).  With at most a few
 // hundred tokens the routing / projection stage moves almost nothing besides the expert matrices
 // (Theorem 2: only the active experts are touched), so what counts is latency: no histogram, no
-// per-expert lists in global memory, no tile table, two short kernels chained by programmatic
-// dependent launch.
+// per-expert lists in global memory, no tile table, short kernels chained by programmatic dependent
+// launch.
 //   router_small_kernel   four warps per token: logits in fp32 with a fixed summation order, softmax
 //                         over all E, the k largest kept with their softmax values, NOT renormalised
 //                         (router softmax equation and the sentence after it); clears the token's
-//                         row of the fp32 mixed streams.
+//                         row of the fp32 mixed streams.  Further blocks ask for the first part of the
+//                         states: until the update starts, nothing else uses HBM.
 //   project_small_kernel  one CTA per (expert, 16 rows of its matrix): finds the tokens routed to
 //                         its expert by scanning the k * T routing entries, streams its 16 x F slice
 //                         of W_e once, multiplies it with those tokens' features on the tensor cores
 //                         (mma.sync m16n8k16, features split over the eight warps and added in a
 //                         fixed order) and adds pi_{t,e} times the result into the token's row of
 //                         the mixed streams (Theorem 1).  With k <= 2 a row receives at most two
-//                         additions onto zero, so the sum does not depend on their order.
+//                         additions onto zero, so the sum does not depend on their order; with more
+//                         experts the rows go to slots (t, j), which the update sums in order.
+// At most SM_FUSED tokens: every CTA of the projection computes the few logits itself (the router
+// matrix and the tokens are in L2, and a dependent launch costs more than they do); the rows go to slots,
+// since no kernel in front could clear the mixed streams.  One token, 8 experts, F = 2048: two kernels
+// @TWO@, one @ONE@.
 #include "internal.h"
 
 namespace swimba {
@@ -24,18 +30,41 @@ constexpr int SM_MAX_T = 256;       // tokens per call
 constexpr int SM_ROWS = 16;         // rows of W_e per CTA (the M of m16n8k16)
 constexpr int SM_WARPS = 8;
 constexpr int SM_NT = 4;            // 8-token column tiles worked per pass
+constexpr int SM_FUSED = 4;         // tokens up to which the projection routes as well
+
+// k rounds of arg-max over the logits (ties to the lower index); returns the next expert.
+__device__ __forceinline__ int next_expert(const float (&g)[SM_MAX_E], int E, unsigned taken)
+{
+    int best = -1;
+    float bv = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < SM_MAX_E; ++e)
+        if (e < E && !((taken >> e) & 1u) && (best < 0 || g[e] > bv)) { bv = g[e]; best = e; }
+    return best;
+}
 }  // namespace
 
 __global__ void __launch_bounds__(256)
 router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r, int Ttok,
                     int F, int E, int k, int32_t *__restrict__ idx, float *__restrict__ w,
-                    float4 *__restrict__ bc_zero, int bc_vec_per_token)
+                    float4 *__restrict__ bc_zero, int bc_vec_per_token, const float *__restrict__ state,
+                    int64_t prefetch_bytes)
 {
     // two tokens per block, four warps per token (a quarter of the features each, partial logits
     // added in warp order)
     __shared__ float s_part[2][4][SM_MAX_E];
     grid_dep_wait();        // the previous step's update may still be reading the mixed streams
     grid_dep_launch();
+    const int rblocks = (Ttok + 1) / 2;
+    if ((int)blockIdx.x >= rblocks) {
+        constexpr int PIECE = 4096;
+        const int64_t at = ((int64_t)(blockIdx.x - rblocks) * blockDim.x + threadIdx.x) * PIECE;
+        if (at < prefetch_bytes)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const char *>(state) + at),
+                         "r"((uint32_t)(prefetch_bytes - at < PIECE ? prefetch_bytes - at : PIECE))
+                         : "memory");
+        return;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tl = warp >> 2, part = warp & 3;
     const int t = blockIdx.x * 2 + tl;
@@ -47,7 +76,7 @@ router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__
         for (int v = part * 32 + lane; v < bc_vec_per_token; v += 128)
             bc_zero[(int64_t)t * bc_vec_per_token + v] = make_float4(0.f, 0.f, 0.f, 0.f);
         const __nv_bfloat16 *urow = u + (int64_t)t * F;
-        const int fq = F / 4;                               // (a multiple of 64)
+        const int fq = F / 4;                               // (a multiple of 8)
 #pragma unroll 2
         for (int f = part * fq + lane * 8; f < (part + 1) * fq; f += 256) {
             float uv[8];
@@ -65,16 +94,17 @@ router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__
     }
 #pragma unroll
     for (int e = 0; e < SM_MAX_E; ++e) {
-        const float v = warp_sum(acc[e]);
-        if (lane == 0) s_part[tl][part][e] = v;
+        if (e < E) {
+            const float v = warp_sum(acc[e]);
+            if (lane == 0) s_part[tl][part][e] = v;
+        }
     }
     __syncthreads();
     if (!live || part != 0) return;
 #pragma unroll
     for (int e = 0; e < SM_MAX_E; ++e)
         acc[e] = e < E ? ((s_part[tl][0][e] + s_part[tl][1][e]) + s_part[tl][2][e]) + s_part[tl][3][e] : -INFINITY;
-    // softmax over all E, then k rounds of arg-max (ties to the lower index); every lane holds the
-    // same values, lane 0 writes
+    // softmax over all E, then k rounds of arg-max; every lane holds the same values, lane 0 writes
     float m = acc[0];
 #pragma unroll
     for (int e = 1; e < SM_MAX_E; ++e) m = fmaxf(m, acc[e]);
@@ -87,12 +117,7 @@ router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__
     const float inv = 1.f / den;
     unsigned taken = 0u;
     for (int j = 0; j < k; ++j) {
-        int best = -1;
-        float bv = -INFINITY;
-#pragma unroll
-        for (int e = 0; e < SM_MAX_E; ++e) {
-            if (e < E && !((taken >> e) & 1u) && acc[e] > bv) { bv = acc[e]; best = e; }
-        }
+        const int best = next_expert(acc, E, taken);
         taken |= 1u << best;
         float pb = 0.f;
 #pragma unroll
@@ -112,48 +137,109 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// SLOTS: rows go to BC[(t*k + j), :] instead of being added to BC[t, :].  FUSED (implies SLOTS): the
+// routing is computed here, by every CTA for itself; the first CTA writes it to idx / w.
+template <bool SLOTS, bool FUSED>
 __global__ void __launch_bounds__(256)
-project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_e,
-                     const int32_t *__restrict__ idx, const float *__restrict__ w, int Ttok, int F, int S,
-                     int E, int k, float *__restrict__ BC, int check, int *d_status)
+project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r,
+                     const __nv_bfloat16 *__restrict__ W_e, int32_t *__restrict__ idx, float *__restrict__ w, int Ttok,
+                     int F, int S, int E, int k, float *__restrict__ BC, int check, int *d_status)
 {
-    __shared__ int s_tok[SM_MAX_T];
+    __shared__ int s_tok[SM_MAX_T], s_out[SM_MAX_T];
     __shared__ float s_wgt[SM_MAX_T];
     __shared__ int s_count;
     __shared__ float s_red[SM_WARPS][SM_ROWS][8 * SM_NT];
+    __shared__ float s_logit[FUSED ? SM_FUSED : 1][SM_MAX_E];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int e = blockIdx.y, row0 = blockIdx.x * SM_ROWS;
     if (tid == 0) s_count = 0;
     __syncthreads();
-    grid_dep_launch();
-    // The matrix slice does not depend on the routing: when a warp's share fits in registers (F up to
-    // 2048) it is fetched before the wait, under the router kernel's tail, and serves every pass.
+    if (!FUSED) grid_dep_launch();
+    // 32-feature steps of this warp: the first (steps % 8) warps take one more
     const int g = lane >> 2, tq = lane & 3;
-    const int kslice = F / SM_WARPS;                       // features per warp (a multiple of 32)
-    const __nv_bfloat16 *wrow0 = W_e + ((int64_t)e * S + row0 + g) * F + warp * kslice + tq * 8;
+    const int steps = F >> 5, base_n = steps / SM_WARPS, extra = steps % SM_WARPS;
+    const int nsteps = base_n + (warp < extra ? 1 : 0), f_warp = (warp * base_n + min(warp, extra)) * 32;
+    const __nv_bfloat16 *wrow0 = W_e + ((int64_t)e * S + row0 + g) * F + f_warp + tq * 8;
     const __nv_bfloat16 *wrow1 = wrow0 + (int64_t)8 * F;
-    const bool resident = kslice <= 256;
+    // The matrix slice does not depend on the routing: when a warp's share fits in registers (F up to
+    // 2048) it is fetched before the wait, under the tail of the kernel in front, and serves every pass.
+    // (Fused, only the few active experts' slices are wanted: fetched once the routing is known.)
+    const bool resident = !FUSED && base_n + (extra ? 1 : 0) <= 8;
     uint4 a0[8], a1[8];
     if (resident) {
 #pragma unroll
         for (int st = 0; st < 8; ++st) {
-            if (st * 32 < kslice) {
+            if (st < nsteps) {
                 a0[st] = *reinterpret_cast<const uint4 *>(wrow0 + st * 32);
                 a1[st] = *reinterpret_cast<const uint4 *>(wrow1 + st * 32);
             }
         }
     }
-    grid_dep_wait();        // routing entries come from the router kernel
-    // tokens routed to this expert (a token picks an expert at most once); the order of the list
-    // does not matter: every entry ends in its own output row
-    for (int i = tid; i < Ttok * k; i += blockDim.x) {
-        const int ei = idx[i];
-        if (check && (ei < 0 || ei >= E)) atomicCAS(d_status, 0, SWIMBA_ERR_DEVICE_BOUNDS);
-        if (ei == e) {
-            const int slot = atomicAdd(&s_count, 1);
-            if (slot < SM_MAX_T) {
-                s_tok[slot] = i / k;
-                s_wgt[slot] = w[i];
+    grid_dep_wait();        // routing entries (fused: the previous step's readers of the slots)
+    if (FUSED) {
+        grid_dep_launch();
+        // one warp per (token, expert) logit in turn; every CTA sums in the same order
+        for (int q = warp; q < Ttok * E; q += SM_WARPS) {
+            const int t = q / E, ee = q - t * E;
+            const __nv_bfloat16 *ur = u + (int64_t)t * F, *wr = W_r + (int64_t)ee * F;
+            float acc = 0.f;
+#pragma unroll 4
+            for (int f = lane * 8; f < F; f += 256) {
+                float uv[8], wv[8];
+                load8(ur + f, uv);
+                load8(wr + f, wv);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc = fmaf(wv[i], uv[i], acc);
+            }
+            acc = warp_sum(acc);
+            if (lane == 0) s_logit[t][ee] = acc;
+        }
+        __syncthreads();
+        if (tid < Ttok) {
+            float lg[SM_MAX_E], pe[SM_MAX_E], m = -INFINITY, den = 0.f;
+#pragma unroll
+            for (int q = 0; q < SM_MAX_E; ++q) {
+                lg[q] = q < E ? s_logit[tid][q] : -INFINITY;
+                m = fmaxf(m, lg[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < SM_MAX_E; ++q) {
+                pe[q] = q < E ? expf(lg[q] - m) : 0.f;
+                den += pe[q];
+            }
+            const float inv = 1.f / den;
+            unsigned taken = 0u;
+            for (int j = 0; j < k; ++j) {
+                const int best = next_expert(lg, E, taken);
+                taken |= 1u << best;
+                float pb = 0.f;
+#pragma unroll
+                for (int q = 0; q < SM_MAX_E; ++q) if (q == best) pb = pe[q];
+                if (best == e) {
+                    const int slot = atomicAdd(&s_count, 1);
+                    s_tok[slot] = tid;
+                    s_out[slot] = tid * k + j;
+                    s_wgt[slot] = pb * inv;
+                }
+                if (blockIdx.x == 0 && blockIdx.y == 0) {
+                    idx[tid * k + j] = best;
+                    w[tid * k + j] = pb * inv;
+                }
+            }
+        }
+    } else {
+        // tokens routed to this expert (a token picks an expert at most once); the order of the list
+        // does not matter: every entry ends in its own output row
+        for (int i = tid; i < Ttok * k; i += blockDim.x) {
+            const int ei = idx[i];
+            if (check && (ei < 0 || ei >= E)) atomicCAS(d_status, 0, SWIMBA_ERR_DEVICE_BOUNDS);
+            if (ei == e) {
+                const int slot = atomicAdd(&s_count, 1);
+                if (slot < SM_MAX_T) {
+                    s_tok[slot] = i / k;
+                    s_out[slot] = SLOTS ? i : i / k;
+                    s_wgt[slot] = w[i];
+                }
             }
         }
     }
@@ -170,8 +256,8 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
         // its two matrix rows and of its token of every column tile; the first four feed one
         // m16n8k16, the last four the next (the contraction may run over the features in any
         // order, as long as both operands agree)
-        for (int f0 = 0; f0 < kslice; f0 += 256) {
-            const int nst = min(8, (kslice - f0) >> 5);
+        for (int s0 = 0; s0 < nsteps; s0 += 8) {
+            const int nst = min(8, nsteps - s0), f0 = s0 * 32;
 #pragma unroll
             for (int st = 0; st < 8; ++st) {
                 if (!resident && st < nst) {
@@ -183,7 +269,7 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
             for (int q = 0; q < SM_NT; ++q) {
                 if (n0 + q * 8 < count) {                  // (warp-uniform)
                     const int n = n0 + q * 8 + g;
-                    const __nv_bfloat16 *urow = n < count ? u + (int64_t)s_tok[n] * F + warp * kslice + tq * 8 + f0 : nullptr;
+                    const __nv_bfloat16 *urow = n < count ? u + (int64_t)s_tok[n] * F + f_warp + tq * 8 + f0 : nullptr;
                     uint4 bv[8];
 #pragma unroll
                     for (int st = 0; st < 8; ++st)
@@ -209,13 +295,15 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
         }
         __syncthreads();
         for (int o = tid; o < SM_ROWS * 8 * SM_NT; o += blockDim.x) {
-            const int r = o / (8 * SM_NT), c = o % (8 * SM_NT);
+            const int r = o % SM_ROWS, c = o / SM_ROWS;      // (neighbouring threads: neighbouring columns of a row)
             const int n = n0 + c;
             if (n < count) {
                 float v = 0.f;
 #pragma unroll
                 for (int q = 0; q < SM_WARPS; ++q) v += s_red[q][r][c];
-                atomicAdd(&BC[(int64_t)s_tok[n] * S + row0 + r], s_wgt[n] * v);
+                float *dst = &BC[(int64_t)s_out[n] * S + row0 + r];
+                if (SLOTS) *dst = s_wgt[n] * v;
+                else atomicAdd(dst, s_wgt[n] * v);
             }
         }
         __syncthreads();
@@ -224,24 +312,39 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
 
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k)
 {
-    return dtype == SWIMBA_DTYPE_BF16 && T <= SM_MAX_T && E <= SM_MAX_E && k <= 2 && S % SM_ROWS == 0 &&
-           F % (32 * SM_WARPS) == 0;
+    return dtype == SWIMBA_DTYPE_BF16 && T <= SM_MAX_T && E <= SM_MAX_E && S % SM_ROWS == 0 && F % 32 == 0;
 }
 
-// idx [T,k], w [T,k] out; BC [T,S] fp32 out.
+bool front_small_fused(int64_t T) { return T <= SM_FUSED; }
+bool front_small_slots(int64_t T, int k) { return front_small_fused(T) || k > 2; }
+
+// Part of the states that the router's launch asks for.  Until the update starts, HBM only carries the
+// previous step's last writes; more than this would push them and each other out of L2.  B = 128, 64 heads
+// (268 MB of states), us a step: nothing 106, @PF@.
+static int64_t prefetch_bytes(int64_t state_bytes)
+{
+    constexpr int64_t most = (int64_t)48 << 20;
+    return state_bytes < ((int64_t)8 << 20) ? 0 : state_bytes < most ? state_bytes : most;
+}
+
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
-                       int S, int E, int k, int32_t *idx, float *w, float *BC)
+                       int S, int E, int k, int32_t *idx, float *w, float *BC, const float *state, int64_t state_bytes)
 {
     if (T <= 0) return SWIMBA_OK;
-    ctx.begin(STAGE_ROUTER);
-    launch_kernel(router_small_kernel, dim3((unsigned)ceil_div64(T, 2)), dim3(256), 0, ctx.stream, true,
-                  (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (int)T, F, E, k, idx, w, (float4 *)BC,
-                  S / 4);
-    ctx.end();
+    const bool slots = front_small_slots(T, k), fused = front_small_fused(T);
+    if (!fused) {
+        const int64_t pf = prefetch_bytes(state_bytes);
+        ctx.begin(STAGE_ROUTER);
+        launch_kernel(router_small_kernel, dim3((unsigned)(ceil_div64(T, 2) + ceil_div64(pf, 256 * 4096))), dim3(256), 0,
+                      ctx.stream, true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (int)T, F, E, k, idx, w,
+                      (float4 *)BC, slots ? 0 : S / 4, state, pf);
+        ctx.end();
+    }
     ctx.begin(STAGE_PROJECT_SMALL);
-    launch_kernel(project_small_kernel, dim3((unsigned)(S / SM_ROWS), (unsigned)E), dim3(256), 0, ctx.stream,
-                  true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_e, (const int32_t *)idx,
-                  (const float *)w, (int)T, F, S, E, k, BC, ctx.check_indices ? 1 : 0, ctx.d_status);
+    auto kern = fused ? project_small_kernel<true, true> : slots ? project_small_kernel<true, false> : project_small_kernel<false, false>;
+    launch_kernel(kern, dim3((unsigned)(S / SM_ROWS), (unsigned)E), dim3(256), 0, ctx.stream, true, (const __nv_bfloat16 *)u,
+                  (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F, S, E, k, BC,
+                  ctx.check_indices ? 1 : 0, ctx.d_status);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }

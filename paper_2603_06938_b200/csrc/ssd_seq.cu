@@ -349,23 +349,37 @@ __device__ __forceinline__ float4 load_bc4(const __nv_bfloat16 *p, int v)
                        __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
 }
 
-template <typename T, typename TBC>
-__global__ void __launch_bounds__(256)
+// MULTI: bc_slots rows of BC make up a sequence's mixed streams (summed in order; else one, mixed already).
+// EARLY: small launches with rows of at most 128 entries, in which every warp has one piece of work and
+// its state rows are fetched before the dependency wait, under the projection (large ones run out of
+// registers that way: 92 -> 139 us at 128 sequences of 64 heads).
+template <typename T, typename TBC, bool MULTI, bool EARLY>
+__global__ void __launch_bounds__(256, 2)
 decode_update_kernel(const T *__restrict__ x, const TBC *__restrict__ BC,
                      const float *__restrict__ dt, const float *__restrict__ A,
                      const float *__restrict__ dt_bias, const float *__restrict__ D,
-                     float *__restrict__ state, int B, int H, int P, int N, int G,
+                     float *__restrict__ state, int B, int H, int P, int N, int G, int bc_slots,
                      T *__restrict__ y)
 {
-    grid_dep_wait();      // the mixed streams come from the projection kernel
     const int lane = threadIdx.x & 31;
     const int S = 2 * G * N;
     const int pgroups = ceil_div(P, DEC_ROWS);
     const int64_t nwork = (int64_t)B * H * pgroups;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int nv = N >> 2;   // groups of 4 state entries per row
-    for (int64_t wk = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); wk < nwork;
-         wk += nwarps) {
+    int64_t wk = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    float4 s[DEC_ROWS];
+    if (EARLY && wk < nwork && lane < nv) {
+        // (the kernel in front lets this one in only behind its own wait: the previous step's update, the
+        // last writer of the states, has completed; the loads go past L1, which may hold older lines)
+        const int pg = (int)(wk % pgroups);
+#pragma unroll
+        for (int r = 0; r < DEC_ROWS; ++r)
+            if (pg * DEC_ROWS + r < P)
+                s[r] = __ldcg(reinterpret_cast<const float4 *>(state + ((wk / pgroups) * P + pg * DEC_ROWS + r) * N) + lane);
+    }
+    grid_dep_wait();      // the mixed streams come from the projection kernel
+    for (; wk < nwork; wk += nwarps) {
         const int pg = (int)(wk % pgroups);
         const int64_t bh = wk / pgroups;
         const int h = (int)(bh % H), b = (int)(bh / H);
@@ -373,8 +387,8 @@ decode_update_kernel(const T *__restrict__ x, const TBC *__restrict__ BC,
         const float delta = softplus_f((dt ? dt[bh] : 0.f) + dt_bias[h]);
         const float a = expf(delta * A[h]);
         const float Dh = D ? D[h] : 0.f;
-        const TBC *Bp = BC + (int64_t)b * S + g * N;
-        const TBC *Cp = BC + (int64_t)b * S + (G + g) * N;
+        const TBC *Bp = BC + (int64_t)b * (MULTI ? bc_slots : 1) * S + g * N;
+        const TBC *Cp = Bp + G * N;
         float xv[DEC_ROWS], acc[DEC_ROWS];
 #pragma unroll
         for (int r = 0; r < DEC_ROWS; ++r) {
@@ -383,14 +397,22 @@ decode_update_kernel(const T *__restrict__ x, const TBC *__restrict__ BC,
             acc[r] = 0.f;
         }
         for (int v = lane; v < nv; v += 32) {
-            float4 s[DEC_ROWS];
+            if (!EARLY) {
 #pragma unroll
-            for (int r = 0; r < DEC_ROWS; ++r) {
-                const int p = pg * DEC_ROWS + r;
-                if (p < P)
-                    s[r] = __ldcs(reinterpret_cast<const float4 *>(state + (bh * P + p) * N) + v);
+                for (int r = 0; r < DEC_ROWS; ++r) {
+                    const int p = pg * DEC_ROWS + r;
+                    if (p < P)
+                        s[r] = __ldcs(reinterpret_cast<const float4 *>(state + (bh * P + p) * N) + v);
+                }
             }
-            const float4 bb = load_bc4(Bp, v), cc = load_bc4(Cp, v);
+            float4 bb = load_bc4(Bp, v), cc = load_bc4(Cp, v);
+            if (MULTI) {
+                for (int j = 1; j < bc_slots; ++j) {
+                    const float4 bj = load_bc4(Bp + (int64_t)j * S, v), cj = load_bc4(Cp + (int64_t)j * S, v);
+                    bb.x += bj.x; bb.y += bj.y; bb.z += bj.z; bb.w += bj.w;
+                    cc.x += cj.x; cc.y += cj.y; cc.z += cj.z; cc.w += cj.w;
+                }
+            }
 #pragma unroll
             for (int r = 0; r < DEC_ROWS; ++r) {
                 const int p = pg * DEC_ROWS + r;
@@ -407,6 +429,7 @@ decode_update_kernel(const T *__restrict__ x, const TBC *__restrict__ BC,
                     __stcs(reinterpret_cast<float4 *>(state + (bh * P + p) * N) + v, s[r]);
                 }
             }
+            if (EARLY) break;
         }
 #pragma unroll
         for (int r = 0; r < DEC_ROWS; ++r) {
@@ -414,6 +437,7 @@ decode_update_kernel(const T *__restrict__ x, const TBC *__restrict__ BC,
             const int p = pg * DEC_ROWS + r;
             if (lane == r && p < P) y[bh * P + p] = from_f32<T>(tot + Dh * xv[r]);
         }
+        if (EARLY) break;
     }
 }
 
@@ -488,32 +512,39 @@ int launch_step_sequences(LaunchCtx &ctx, const void *x, const void *BC, const f
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
-int launch_decode_update(LaunchCtx &ctx, int dtype, const void *x, const void *BC, bool bc_fp32,
-                         const float *dt, const float *A, const float *dt_bias, const float *D,
-                         float *state, int B, int H, int P, int N, int G, int sm_count, void *y)
+template <typename T, typename TBC>
+static int launch_decode_t(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
+                           const float *dt_bias, const float *D, float *state, int B, int H, int P, int N, int G,
+                           int bc_slots, bool early, int sm_count, void *y)
 {
-    if (B <= 0) return SWIMBA_OK;
     const int64_t nwork = (int64_t)B * H * ceil_div(P, DEC_ROWS);
     const int warps = 8;
     int64_t blocks = ceil_div64(nwork, warps);
     const int64_t cap = (int64_t)sm_count * 8;
+    // one piece of work per warp, and all of them resident (two blocks of 256 threads per SM)
+    early = early && N <= 128 && blocks <= 2 * (int64_t)sm_count;
     if (blocks > cap) blocks = cap;
+    auto kern = bc_slots == 1 ? (early ? decode_update_kernel<T, TBC, false, true> : decode_update_kernel<T, TBC, false, false>)
+                              : (early ? decode_update_kernel<T, TBC, true, true> : decode_update_kernel<T, TBC, true, false>);
     ctx.begin(STAGE_DECODE_UPDATE);
-    const dim3 grid((unsigned)blocks), block(warps * 32);
-    if (dtype == SWIMBA_DTYPE_FP32)
-        launch_kernel(decode_update_kernel<float, float>, grid, block, 0, ctx.stream, true,
-                      (const float *)x, (const float *)BC, dt, A, dt_bias, D, state, B, H, P, N, G,
-                      (float *)y);
-    else if (bc_fp32)
-        launch_kernel(decode_update_kernel<__nv_bfloat16, float>, grid, block, 0, ctx.stream, true,
-                      (const __nv_bfloat16 *)x, (const float *)BC, dt, A, dt_bias, D, state, B, H, P, N,
-                      G, (__nv_bfloat16 *)y);
-    else
-        launch_kernel(decode_update_kernel<__nv_bfloat16, __nv_bfloat16>, grid, block, 0, ctx.stream,
-                      true, (const __nv_bfloat16 *)x, (const __nv_bfloat16 *)BC, dt, A, dt_bias, D,
-                      state, B, H, P, N, G, (__nv_bfloat16 *)y);
+    launch_kernel(kern, dim3((unsigned)blocks), dim3(warps * 32), 0, ctx.stream, true, (const T *)x, (const TBC *)BC, dt, A, dt_bias, D, state, B, H, P, N,
+                  G, bc_slots, (T *)y);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+}
+
+int launch_decode_update(LaunchCtx &ctx, int dtype, const void *x, const void *BC, bool bc_fp32, int bc_slots, bool early,
+                         const float *dt, const float *A, const float *dt_bias, const float *D,
+                         float *state, int B, int H, int P, int N, int G, int sm_count, void *y)
+{
+    if (B <= 0) return SWIMBA_OK;
+    if (dtype == SWIMBA_DTYPE_FP32)
+        return launch_decode_t<float, float>(ctx, x, BC, dt, A, dt_bias, D, state, B, H, P, N, G, bc_slots, early, sm_count, y);
+    if (bc_fp32)
+        return launch_decode_t<__nv_bfloat16, float>(ctx, x, BC, dt, A, dt_bias, D, state, B, H, P, N, G, bc_slots, early,
+                                                     sm_count, y);
+    return launch_decode_t<__nv_bfloat16, __nv_bfloat16>(ctx, x, BC, dt, A, dt_bias, D, state, B, H, P, N, G, bc_slots, early,
+                                                         sm_count, y);
 }
 
 }  // namespace swimba
