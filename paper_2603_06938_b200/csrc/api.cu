@@ -1039,8 +1039,7 @@ int swimba_decode_step(swimba_handle *h, const swimba_weights *w, const void *u,
     const bool tensor = !small && use_tensor_k1(c);
     if (small) {
         rc = launch_front_small(ctx, u, w->W_router ? w->W_router : w->W_expert, w->W_expert, B, c.d_model, S,
-                                c.n_experts, c.top_k, idx, wt, (float *)BC, state,
-                                (int64_t)B * c.n_heads * c.head_dim * c.d_state * (int64_t)sizeof(float));
+                                c.n_experts, c.top_k, idx, wt, (float *)BC);
         if (rc != SWIMBA_OK) fail(h, rc, "routing / projection launch failed");
     } else {
         rc = run_route_mix(h, ctx, w, u, B, BC, !tensor, idx, wt, tensor ? ws + l.gemm : nullptr);

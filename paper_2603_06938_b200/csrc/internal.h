@@ -65,13 +65,12 @@ int launch_accumulate(LaunchCtx &ctx, int dtype, void *y, const void *y_add, int
 
 // K1 for at most a few hundred tokens (decode): one or two short kernels, no lists in global memory.
 // idx [T,k], w [T,k] and the fp32 streams BC are written: [T,S] mixed, or, where front_small_slots says so,
-// [T,k,S] per slot (weights applied), summed by the reader.  state: read by the caller's next kernel
-// (state_bytes of it; the launch may ask for a part of it ahead).
+// [T,k,S] per slot (weights applied), summed by the reader.
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
 bool front_small_slots(int64_t T, int k);
 bool front_small_fused(int64_t T);        // one kernel, which starts the next one behind its own wait
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
-                       int S, int E, int k, int32_t *idx, float *w, float *BC, const float *state, int64_t state_bytes);
+                       int S, int E, int k, int32_t *idx, float *w, float *BC);
 
 // K2/K3 (tensor cores): tiled SSD with the carried state kept on chip; bf16, P == 64, N == 128.
 bool ssd_tiles_supported(int dtype, int P, int N);

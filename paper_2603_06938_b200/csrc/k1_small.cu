@@ -6,8 +6,7 @@
 //   router_small_kernel   four warps per token: logits in fp32 with a fixed summation order, softmax
 //                         over all E, the k largest kept with their softmax values, NOT renormalised
 //                         (router softmax equation and the sentence after it); clears the token's
-//                         row of the fp32 mixed streams.  Further blocks ask for the first part of the
-//                         states: until the update starts, nothing else uses HBM.
+//                         row of the fp32 mixed streams
 //   project_small_kernel  one CTA per (expert, 16 rows of its matrix): finds the tokens routed to
 //                         its expert by scanning the k * T routing entries, streams its 16 x F slice
 //                         of W_e once, multiplies it with those tokens' features on the tensor cores
@@ -47,24 +46,13 @@ __device__ __forceinline__ int next_expert(const float (&g)[SM_MAX_E], int E, un
 __global__ void __launch_bounds__(256)
 router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r, int Ttok,
                     int F, int E, int k, int32_t *__restrict__ idx, float *__restrict__ w,
-                    float4 *__restrict__ bc_zero, int bc_vec_per_token, const float *__restrict__ state,
-                    int64_t prefetch_bytes)
+                    float4 *__restrict__ bc_zero, int bc_vec_per_token)
 {
     // two tokens per block, four warps per token (a quarter of the features each, partial logits
     // added in warp order)
     __shared__ float s_part[2][4][SM_MAX_E];
     grid_dep_wait();        // the previous step's update may still be reading the mixed streams
     grid_dep_launch();
-    const int rblocks = (Ttok + 1) / 2;
-    if ((int)blockIdx.x >= rblocks) {
-        constexpr int PIECE = 4096;
-        const int64_t at = ((int64_t)(blockIdx.x - rblocks) * blockDim.x + threadIdx.x) * PIECE;
-        if (at < prefetch_bytes)
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const char *>(state) + at),
-                         "r"((uint32_t)(prefetch_bytes - at < PIECE ? prefetch_bytes - at : PIECE))
-                         : "memory");
-        return;
-    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tl = warp >> 2, part = warp & 3;
     const int t = blockIdx.x * 2 + tl;
@@ -148,7 +136,7 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
     __shared__ int s_tok[SM_MAX_T], s_out[SM_MAX_T];
     __shared__ float s_wgt[SM_MAX_T];
     __shared__ int s_count;
-    __shared__ float s_red[SM_WARPS][SM_ROWS][8 * SM_NT];
+    __shared__ float s_red[SM_WARPS][SM_ROWS][8 * SM_NT + 1];
     __shared__ float s_logit[FUSED ? SM_FUSED : 1][SM_MAX_E];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int e = blockIdx.y, row0 = blockIdx.x * SM_ROWS;
@@ -318,26 +306,16 @@ bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k)
 bool front_small_fused(int64_t T) { return T <= SM_FUSED; }
 bool front_small_slots(int64_t T, int k) { return front_small_fused(T) || k > 2; }
 
-// Part of the states that the router's launch asks for.  Until the update starts, HBM only carries the
-// previous step's last writes; more than this would push them and each other out of L2.  B = 128, 64 heads
-// (268 MB of states), us a step: nothing 106, @PF@.
-static int64_t prefetch_bytes(int64_t state_bytes)
-{
-    constexpr int64_t most = (int64_t)48 << 20;
-    return state_bytes < ((int64_t)8 << 20) ? 0 : state_bytes < most ? state_bytes : most;
-}
-
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
-                       int S, int E, int k, int32_t *idx, float *w, float *BC, const float *state, int64_t state_bytes)
+                       int S, int E, int k, int32_t *idx, float *w, float *BC)
 {
     if (T <= 0) return SWIMBA_OK;
     const bool slots = front_small_slots(T, k), fused = front_small_fused(T);
     if (!fused) {
-        const int64_t pf = prefetch_bytes(state_bytes);
         ctx.begin(STAGE_ROUTER);
-        launch_kernel(router_small_kernel, dim3((unsigned)(ceil_div64(T, 2) + ceil_div64(pf, 256 * 4096))), dim3(256), 0,
-                      ctx.stream, true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (int)T, F, E, k, idx, w,
-                      (float4 *)BC, slots ? 0 : S / 4, state, pf);
+        launch_kernel(router_small_kernel, dim3((unsigned)ceil_div64(T, 2)), dim3(256), 0, ctx.stream, true,
+                      (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (int)T, F, E, k, idx, w,
+                      (float4 *)BC, slots ? 0 : S / 4);
         ctx.end();
     }
     ctx.begin(STAGE_PROJECT_SMALL);

@@ -407,6 +407,7 @@ decode_update_kernel(const T *__restrict__ x, const TBC *__restrict__ BC,
             }
             float4 bb = load_bc4(Bp, v), cc = load_bc4(Cp, v);
             if (MULTI) {
+#pragma unroll 1
                 for (int j = 1; j < bc_slots; ++j) {
                     const float4 bj = load_bc4(Bp + (int64_t)j * S, v), cj = load_bc4(Cp + (int64_t)j * S, v);
                     bb.x += bj.x; bb.y += bj.y; bb.z += bj.z; bb.w += bj.w;
