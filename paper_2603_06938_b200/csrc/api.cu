@@ -1045,9 +1045,9 @@ int swimba_decode_step(swimba_handle *h, const swimba_weights *w, const void *u,
         rc = run_route_mix(h, ctx, w, u, B, BC, !tensor, idx, wt, tensor ? ws + l.gemm : nullptr);
     }
     if (rc == SWIMBA_OK) {
-        // (only the fused front end starts the update behind the previous step's)
+        // (the small front end starts the update behind the previous step's)
         rc = launch_decode_update(ctx, c.dtype, x, BC, !tensor, small && front_small_slots(B, c.top_k) ? c.top_k : 1,
-                                  small && front_small_fused(B), dt, w->A, w->dt_bias, w->D, state, B,
+                                  small, dt, w->A, w->dt_bias, w->D, state, B,
                                   c.n_heads, c.head_dim, c.d_state, c.n_groups, h->sm_count, y);
         if (rc != SWIMBA_OK) fail(h, rc, "decode launch failed");
     }

@@ -65,10 +65,10 @@ int launch_accumulate(LaunchCtx &ctx, int dtype, void *y, const void *y_add, int
 
 // K1 for at most a few hundred tokens (decode): one or two short kernels, no lists in global memory.
 // idx [T,k], w [T,k] and the fp32 streams BC are written: [T,S] mixed, or, where front_small_slots says so,
-// [T,k,S] per slot (weights applied), summed by the reader.
+// [T,k,S] per slot (weights applied), summed by the reader.  The kernel behind starts only after everything
+// in front of this call has completed, so it may read what earlier calls wrote before its own wait.
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
 bool front_small_slots(int64_t T, int k);
-bool front_small_fused(int64_t T);        // one kernel, which starts the next one behind its own wait
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
                        int S, int E, int k, int32_t *idx, float *w, float *BC);
 
@@ -190,8 +190,9 @@ int launch_step_sequences(LaunchCtx &ctx, const void *x, const void *BC, const f
                           int G, void *y, float *h_final);
 
 // K4: one-token state update, state[B,H,P,N] in place.
-// BC [B,bc_slots,S] is fp32 when bc_fp32, else bf16; the slots are summed.  early: the kernel in front
-// lets the next one in only after its own dependency wait, so that the states may be read before it ends.
+// BC [B,bc_slots,S] is fp32 when bc_fp32, else bf16; the slots are summed.  early: what was
+// launched in front lets this kernel in only after the previous writer of the states has completed
+// (launch_front_small), so that they may be read before the dependency wait.
 int launch_decode_update(LaunchCtx &ctx, int dtype, const void *x, const void *BC, bool bc_fp32, int bc_slots, bool early,
                          const float *dt, const float *A, const float *dt_bias, const float *D,
                          float *state, int B, int H, int P, int N, int G, int sm_count, void *y);

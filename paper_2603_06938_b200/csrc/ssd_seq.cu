@@ -333,8 +333,11 @@ int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *
 
 // ------------------------------------------------------------------------------------------
 // K4: decode.  The state [B,H,P,N] fp32 is read and written exactly once: the kernel is a pure
-// HBM stream.  One warp owns ROWS consecutive channels p of one (b,h); a row is N floats read
-// as float4 per lane, all ROWS loads are issued before any use.
+// HBM stream (128 sequences of 64 heads, 537 MB in and out: 92 us, 5.8 TB/s).  One warp owns ROWS consecutive channels p of one (b,h); a row is N floats read
+// as float4 per lane, all ROWS loads are issued before any use.  (A ring of 4 KB pieces per warp in shared
+// memory, filled and emptied by bulk copies, took 95 us with neighbouring warps on neighbouring pieces and
+// 103 us with a contiguous run per warp; asking L2 for the first 16 to 80 MB of the states under the front
+// end cost 3 to 8 us: the previous step's last writes still occupy HBM then.)
 // ------------------------------------------------------------------------------------------
 constexpr int DEC_ROWS = 8;
 
