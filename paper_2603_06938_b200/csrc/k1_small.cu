@@ -34,11 +34,11 @@ constexpr int SM_FUSED = 4;         // tokens up to which the projection routes 
 // k rounds of arg-max over the logits (ties to the lower index); returns the next expert.
 __device__ __forceinline__ int next_expert(const float (&g)[SM_MAX_E], int E, unsigned taken)
 {
-    int best = -1;
+    int best = 0;
     float bv = -INFINITY;
 #pragma unroll
     for (int e = 0; e < SM_MAX_E; ++e)
-        if (e < E && !((taken >> e) & 1u) && (best < 0 || g[e] > bv)) { bv = g[e]; best = e; }
+        if (e < E && !((taken >> e) & 1u) && g[e] > bv) { bv = g[e]; best = e; }
     return best;
 }
 }  // namespace
@@ -80,13 +80,20 @@ router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__
             }
         }
     }
+    // sixteen sums over the lanes by halving exchanges: expert 8 b4 + 4 b3 + 2 b2 + b1 ends on the lanes
+    // whose bits 4 .. 1 are b4 .. b1 (unused experts are zero)
+    static_assert(SM_MAX_E == 16, "the reduction is for sixteen values");
 #pragma unroll
-    for (int e = 0; e < SM_MAX_E; ++e) {
-        if (e < E) {
-            const float v = warp_sum(acc[e]);
-            if (lane == 0) s_part[tl][part][e] = v;
+    for (int o = 16, m = 8; m >= 1; o >>= 1, m >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < m; ++q) {
+            const float send = up ? acc[q] : acc[q + m], keep = up ? acc[q + m] : acc[q];
+            acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+    if ((lane & 1) == 0) s_part[tl][part][lane >> 1] = acc[0];
     __syncthreads();
     if (!live || part != 0) return;
 #pragma unroll
