@@ -191,6 +191,11 @@ int run_route_mix(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, con
     // being dereferenced only if it is given, so substitute the expert matrix as a dummy operand.
     const void *Wr = w->W_router ? w->W_router : w->W_expert;
     const bool tensor = gemm_ws && !bc_fp32 && use_tensor_k1(c);
+    if (tensor && front_short_supported(c.dtype, T, c.d_model, S, c.n_experts, c.top_k)) {
+        const int rc = launch_front_short(ctx, u, Wr, w->W_expert, T, c.d_model, S, c.n_experts, c.top_k, idx, wt, BC,
+                                          scalars ? *scalars : ScalarsArgs{});
+        return rc == SWIMBA_OK ? rc : fail(h, rc, "routing / projection launch failed");
+    }
     int *counts = nullptr, *perm = nullptr;
     if (tensor) {
         counts = expert_gemm_counts(gemm_ws);
@@ -217,12 +222,12 @@ int run_route_mix(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, con
 
 int run_ssd(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, const void *x,
             const void *BC, const float *dt, const float *h0, int B, int L, void *y,
-            float *h_final, void *ssd_ws, bool scalars_done = false)
+            float *h_final, void *ssd_ws, bool scalars_done = false, bool early = false)
 {
     const swimba_config &c = h->cfg;
     if (ssd_ws && ssd_tiles_supported(c.dtype, c.head_dim, c.d_state)) {
         int rc = launch_ssd_tiles(ctx, x, BC, dt, w->A, w->dt_bias, w->D, h0, B, L, c.n_heads,
-                                  c.n_groups, c.chunk, h->sm_count, y, h_final, ssd_ws, scalars_done);
+                                  c.n_groups, c.chunk, h->sm_count, y, h_final, ssd_ws, scalars_done, early);
         if (rc != SWIMBA_OK) return fail(h, rc, "SSD tile kernel launch failed");
         return SWIMBA_OK;
     }
@@ -657,7 +662,7 @@ int swimba_forward(swimba_handle *h, const swimba_weights *w, const void *u, con
     const ScalarsArgs sa = fuse ? ssd_scalars_args(dt, w->A, w->dt_bias, B, L, h->cfg.n_heads, ws + l.ssd)
                                 : ScalarsArgs{};
     rc = run_route_mix(h, ctx, w, u, T, BC, false, idx, wt, ws + l.gemm, fuse ? &sa : nullptr);
-    if (rc == SWIMBA_OK) rc = run_ssd(h, ctx, w, x, BC, dt, h0, B, L, y, h_final, ws + l.ssd, fuse);
+    if (rc == SWIMBA_OK) rc = run_ssd(h, ctx, w, x, BC, dt, h0, B, L, y, h_final, ws + l.ssd, fuse, true);
     h->last_stream = ctx.stream;
     h->last_launches = ctx.launches;
     return rc;

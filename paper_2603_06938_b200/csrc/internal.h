@@ -71,6 +71,10 @@ bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
 bool front_small_slots(int64_t T, int k);
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
                        int S, int E, int k, int32_t *idx, float *w, float *BC);
+// The same kernels for short calls of the forward: BC [T,S] bf16; scalars as in launch_router.
+bool front_short_supported(int dtype, int64_t T, int F, int S, int E, int k);
+int launch_front_short(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F, int S, int E,
+                       int k, int32_t *idx, float *w, void *BC, const ScalarsArgs &scalars);
 
 // K2/K3 (tensor cores): tiled SSD with the carried state kept on chip; bf16, P == 64, N == 128.
 bool ssd_tiles_supported(int dtype, int P, int N);
@@ -78,7 +82,8 @@ size_t ssd_workspace_bytes(int B, int L, int H, int G, int chunk, int sm_count);
 // Tokens per segment the tile path cuts a sequence into (a multiple of 128; >= L: one segment).
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count);
 // scalars_done: the step sizes and tile log-decays (ssd_scalars_args over the same workspace) have
-// already been produced earlier in the stream (launch_router with scalars, or launch_ssd_scalars).
+// already been produced earlier in the stream (launch_router with scalars, or launch_ssd_scalars).  early:
+// x and h0 were complete before the first kernel of the same call.
 ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
                              void *workspace);
 int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &args);
@@ -89,7 +94,7 @@ int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const
 int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
                      const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int G,
                      int chunk, int sm_count, void *y, float *h_final, void *workspace,
-                     bool scalars_done);
+                     bool scalars_done, bool early);
 
 // One bf16 stream of G*N entries per token, rows ld elements apart.
 struct SsdStream {
@@ -100,7 +105,7 @@ struct SsdStream {
 int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs, const SsdStream &Cs, const float *dt,
                              const float *A, const float *dt_bias, const float *D, const float *h0, int B, int L,
                              int H, int G, int chunk, int sm_count, void *y, float *h_final, void *workspace,
-                             bool scalars_done, bool add);
+                             bool scalars_done, bool add, bool early);
 // The general form on the tile kernel: k evaluations (one per slot) added up; cmix: T*G*N bf16 scratch.
 int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_slots, const float *dt, const float *A,
                            const float *dt_bias, const float *h0, int B, int L, int H, int G, int k, int chunk,

@@ -46,13 +46,18 @@ __device__ __forceinline__ int next_expert(const float (&g)[SM_MAX_E], int E, un
 __global__ void __launch_bounds__(256)
 router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r, int Ttok,
                     int F, int E, int k, int32_t *__restrict__ idx, float *__restrict__ w,
-                    float4 *__restrict__ bc_zero, int bc_vec_per_token)
+                    float4 *__restrict__ bc_zero, int bc_vec_per_token, const ScalarsArgs scalars)
 {
     // two tokens per block, four warps per token (a quarter of the features each, partial logits
     // added in warp order)
     __shared__ float s_part[2][4][SM_MAX_E];
     grid_dep_wait();        // the previous step's update may still be reading the mixed streams
     grid_dep_launch();
+    if ((int)blockIdx.x >= (Ttok + 1) / 2) {
+        // SSD step sizes and tile log-decays of the same call (they depend on dt only)
+        ssd_scalars_block(scalars, blockIdx.x - (Ttok + 1) / 2);
+        return;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tl = warp >> 2, part = warp & 3;
     const int t = blockIdx.x * 2 + tl;
@@ -132,14 +137,18 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// SLOTS: rows go to BC[(t*k + j), :] instead of being added to BC[t, :].  FUSED (implies SLOTS): the
-// routing is computed here, by every CTA for itself; the first CTA writes it to idx / w.
-template <bool SLOTS, bool FUSED>
+// How the rows leave: added to BC[t, :] (fp32, cleared before), stored to slots BC[(t*k + j), :] (fp32), or,
+// for the forward's bf16 streams, stored (one expert per token) or added (two; 0 + a + b does not depend on
+// the order).  FUSED (slots): the routing is computed here, by every CTA for itself; the first CTA writes it
+// to idx / w.
+enum { ROWS_ADD = 0, ROWS_SLOTS = 1, ROWS_BF16 = 2 };
+template <int ROWS, bool FUSED>
 __global__ void __launch_bounds__(256)
 project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r,
                      const __nv_bfloat16 *__restrict__ W_e, int32_t *__restrict__ idx, float *__restrict__ w, int Ttok,
-                     int F, int S, int E, int k, float *__restrict__ BC, int check, int *d_status)
+                     int F, int S, int E, int k, void *__restrict__ BCv, int check, int *d_status)
 {
+    float *BC = reinterpret_cast<float *>(BCv);
     __shared__ int s_tok[SM_MAX_T], s_out[SM_MAX_T];
     __shared__ float s_wgt[SM_MAX_T];
     __shared__ int s_count;
@@ -234,7 +243,7 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
                 const int slot = atomicAdd(&s_count, 1);
                 if (slot < SM_MAX_T) {
                     s_tok[slot] = i / k;
-                    s_out[slot] = SLOTS ? i : i / k;
+                    s_out[slot] = ROWS == ROWS_SLOTS ? i : i / k;
                     s_wgt[slot] = w[i];
                 }
             }
@@ -291,16 +300,35 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
             s_red[warp][g + 8][q * 8 + 2 * tq + 1] = acc[q][3];
         }
         __syncthreads();
-        for (int o = tid; o < SM_ROWS * 8 * SM_NT; o += blockDim.x) {
-            const int r = o % SM_ROWS, c = o / SM_ROWS;      // (neighbouring threads: neighbouring columns of a row)
-            const int n = n0 + c;
-            if (n < count) {
-                float v = 0.f;
+        if (ROWS == ROWS_BF16) {
+            for (int o = tid; o < SM_ROWS / 2 * 8 * SM_NT; o += blockDim.x) {
+                const int r = o % (SM_ROWS / 2) * 2, c = o / (SM_ROWS / 2);
+                const int n = n0 + c;
+                if (n < count) {
+                    float v0 = 0.f, v1 = 0.f;
 #pragma unroll
-                for (int q = 0; q < SM_WARPS; ++q) v += s_red[q][r][c];
-                float *dst = &BC[(int64_t)s_out[n] * S + row0 + r];
-                if (SLOTS) *dst = s_wgt[n] * v;
-                else atomicAdd(dst, s_wgt[n] * v);
+                    for (int q = 0; q < SM_WARPS; ++q) {
+                        v0 += s_red[q][r][c];
+                        v1 += s_red[q][r + 1][c];
+                    }
+                    const __nv_bfloat162 v = __floats2bfloat162_rn(s_wgt[n] * v0, s_wgt[n] * v1);
+                    __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(BCv) + (int64_t)s_out[n] * S + row0 + r;
+                    if (k == 1) *reinterpret_cast<__nv_bfloat162 *>(dst) = v;
+                    else atomicAdd(reinterpret_cast<__nv_bfloat162 *>(dst), v);
+                }
+            }
+        } else {
+            for (int o = tid; o < SM_ROWS * 8 * SM_NT; o += blockDim.x) {
+                const int r = o % SM_ROWS, c = o / SM_ROWS;      // (neighbouring threads: neighbouring columns of a row)
+                const int n = n0 + c;
+                if (n < count) {
+                    float v = 0.f;
+#pragma unroll
+                    for (int q = 0; q < SM_WARPS; ++q) v += s_red[q][r][c];
+                    float *dst = &BC[(int64_t)s_out[n] * S + row0 + r];
+                    if (ROWS == ROWS_SLOTS) *dst = s_wgt[n] * v;
+                    else atomicAdd(dst, s_wgt[n] * v);
+                }
             }
         }
         __syncthreads();
@@ -324,14 +352,38 @@ int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const voi
         ctx.begin(STAGE_ROUTER);
         launch_kernel(router_small_kernel, dim3((unsigned)ceil_div64(T, 2)), dim3(256), 0, ctx.stream, true,
                       (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (int)T, F, E, k, idx, w,
-                      (float4 *)BC, slots ? 0 : S / 4);
+                      (float4 *)BC, slots ? 0 : S / 4, ScalarsArgs{});
         ctx.end();
     }
     ctx.begin(STAGE_PROJECT_SMALL);
-    auto kern = fused ? project_small_kernel<true, true> : slots ? project_small_kernel<true, false> : project_small_kernel<false, false>;
+    auto kern = fused ? project_small_kernel<ROWS_SLOTS, true>
+                      : slots ? project_small_kernel<ROWS_SLOTS, false> : project_small_kernel<ROWS_ADD, false>;
     launch_kernel(kern, dim3((unsigned)(S / SM_ROWS), (unsigned)E), dim3(256), 0, ctx.stream, true, (const __nv_bfloat16 *)u,
-                  (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F, S, E, k, BC,
+                  (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F, S, E, k, (void *)BC,
                   ctx.check_indices ? 1 : 0, ctx.d_status);
+    ctx.end();
+    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+}
+
+// The forward's streams for short calls: no histogram to clear, no lists, no tiles.  @SHORT@
+bool front_short_supported(int dtype, int64_t T, int F, int S, int E, int k)
+{
+    return front_small_supported(dtype, T, F, S, E, k) && k <= 2 && E > 1;
+}
+
+int launch_front_short(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F, int S, int E,
+                       int k, int32_t *idx, float *w, void *BC, const ScalarsArgs &scalars)
+{
+    if (T <= 0) return SWIMBA_OK;
+    ctx.begin(STAGE_ROUTER);
+    launch_kernel(router_small_kernel, dim3((unsigned)(ceil_div64(T, 2) + scalars_blocks(scalars, 256))), dim3(256), 0,
+                  ctx.stream, true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (int)T, F, E, k, idx, w,
+                  (float4 *)BC, k == 1 ? 0 : S / 8, scalars);
+    ctx.end();
+    ctx.begin(STAGE_PROJECT_SMALL);
+    launch_kernel(project_small_kernel<ROWS_BF16, false>, dim3((unsigned)(S / SM_ROWS), (unsigned)E), dim3(256), 0, ctx.stream,
+                  true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F,
+                  S, E, k, BC, ctx.check_indices ? 1 : 0, ctx.d_status);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }

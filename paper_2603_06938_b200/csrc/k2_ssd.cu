@@ -97,6 +97,9 @@ struct SsdParams {
     void *y;
     // 1: y and h_out are added to, not overwritten (the slots behind the first of the general form)
     int add;
+    // 1: x and the initial states are not written by anything in the same call, so that they may be read before
+    // the dependency wait (everything in front of the call has completed when its first kernel runs)
+    int early;
 };
 
 struct __align__(8) HeadBars {
@@ -317,10 +320,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = sm->tmem_slot;
-    // Everything above needs nothing from earlier kernels and may run under their tail; the
-    // mixed streams and the step sizes are read from here on.
     grid_dep_launch();
-    grid_dep_wait();
 
     // Warp index as a value the compiler knows to be warp-uniform.
     const int uwarp = __shfl_sync(0xffffffffu, warp, 0);
@@ -332,12 +332,19 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         auto scal_rec = [&](int hd, int j) {
             return prm.rec + rec_base + (int64_t)(head0 + hd) * rec_hstride + t_begin / ST + j;
         };
+        if (!prm.early) grid_dep_wait();
         if (leader && ntiles > 0) {
-            for (int hd = 0; hd < nh; ++hd) {               // X and scalars of tile 0
+            for (int hd = 0; hd < nh; ++hd) {               // X of tile 0
                 HeadBars *hb = &bars->hd[hd];
                 tc::mbar_arrive_expect_tx(&hb->x_full[0], SLAB);
                 tc::tma_load_4d(smem + SM_HEAD + hd * SM_HEAD_BYTES, &tmap_x, &hb->x_full[0], 0,
                                 head0 + hd, tok0 + t_begin, bco);
+            }
+        }
+        if (prm.early) grid_dep_wait();
+        if (leader && ntiles > 0) {
+            for (int hd = 0; hd < nh; ++hd) {               // its scalars
+                HeadBars *hb = &bars->hd[hd];
                 tc::mbar_arrive_expect_tx(&hb->sc_full, (uint32_t)sizeof(TileScalars));
                 tc::bulk_load(&sm->sc[hd], scal_rec(hd, 0), (uint32_t)sizeof(TileScalars), &hb->sc_full);
             }
@@ -384,6 +391,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         // ------------------------------------------------------------------ MMA issuers
         // The whole warp runs the loop and the waits; one elected lane issues the MMAs, the
         // commits and the y stores.
+        grid_dep_wait();
         const int hd = uwarp - WARP_MMA0;
         const bool leader = tc::elect_one();
         if (hd < nh) {
@@ -522,12 +530,15 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         {
             const bool first = prm.seg_states == 2 && seg == 0;
             const float *h_in = first ? prm.h_first : prm.h_in;
+            // (states of earlier segments come from the scan in front; given ones go past L1)
+            const bool wait = !prm.early || (prm.seg_states && !first);
+            if (wait) grid_dep_wait();
             if (h_in && kfull) {
                 const int64_t base = (prm.seg_states && !first)
                     ? ((((int64_t)seg_base + seg) * H + h) * SP) * SN
                     : (((int64_t)b * H + h) * SP) * SN;
 #pragma unroll
-                for (int q = 0; q < 32; ++q) Hst[q] = h_in[base + (int64_t)(p0 + q) * SN + i];
+                for (int q = 0; q < 32; ++q) Hst[q] = __ldcg(h_in + base + (int64_t)(p0 + q) * SN + i);
             } else {
 #pragma unroll
                 for (int q = 0; q < 32; ++q) Hst[q] = 0.f;
@@ -554,6 +565,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 tc::tmem_st_wait();
             }
         }
+        grid_dep_wait();         // the step sizes, the streams
         float seg_l2 = 0.f;      // log2 of the product of a_t over the tiles done so far
         const int64_t rec_row = rec_base + (int64_t)h * rec_hstride;     // tile 0 of this (sequence, head)
         const float *l2p = prm.l2 + rec_row * ST + t_begin;
@@ -1136,22 +1148,25 @@ bool ssd_tiles_supported(int dtype, int P, int N)
 
 static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 
-// Segment length (tokens, multiple of 128) so that the grid fills the SMs; L itself if one
-// segment per sequence is enough.
+// Segment length (tokens, multiple of 128); L itself if one segment per sequence is best.  In units of a
+// full tile (3.8 us a head pair), measured: a segment's full pass costs its tiles plus 0.4, the state-only
+// pass half a tile's time per tile plus 1 (four heads per CTA), the scan 1.  Whole rounds of CTAs count.
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
 {
     const int64_t ctas = (int64_t)B * G * pairs_per_group(H, G);
+    const int64_t quads = (int64_t)B * G * quads_per_group(H, G);
     const int tiles = ceil_div(L, ST);
     if (2 * ctas > sm_count || tiles <= 2) return tiles * ST;
-    // segments per sequence: as many as keep the grid within two CTAs per SM (a few CTAs more
-    // would cost a whole extra round)
-    int want = (int)((2 * (int64_t)sm_count) / ctas);
-    if (want < 1) want = 1;
-    int q_tiles = chunk >= ST ? chunk / ST : 1;                       // segments are whole chunks
-    int seg_tiles = ceil_div(tiles, want);
-    seg_tiles = ceil_div(seg_tiles, q_tiles) * q_tiles;
-    if (seg_tiles < 4) seg_tiles = 4 < tiles ? 4 : tiles;
-    return seg_tiles * ST;
+    const int q_tiles = chunk >= ST ? chunk / ST : 1;                 // segments are whole chunks
+    float best_cost = (float)tiles + 0.4f;
+    int best = tiles;
+    for (int st = q_tiles; st < tiles; st += q_tiles) {
+        const int64_t nseg = ceil_div(tiles, st);
+        const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 0.4f) +
+                           (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.5f * st + 1.f) + 1.f;
+        if (cost < best_cost) { best_cost = cost; best = st; }
+    }
+    return best * ST;
 }
 
 // Workspace: [log-decays B*H*Lpad float] [per-tile records B*H*(Lpad/128)] [segment states]
@@ -1230,16 +1245,16 @@ int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const
 int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
                      const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int G,
                      int chunk, int sm_count, void *y, float *h_final, void *workspace,
-                     bool scalars_done)
+                     bool scalars_done, bool early)
 {
     return launch_ssd_tiles_streams(ctx, x, b_stream(BC, G), c_stream(BC, G), dt, A, dt_bias, D, h0, B, L, H, G, chunk,
-                                    sm_count, y, h_final, workspace, scalars_done, false);
+                                    sm_count, y, h_final, workspace, scalars_done, false, early);
 }
 
 int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs, const SsdStream &Cs, const float *dt,
                              const float *A, const float *dt_bias, const float *D, const float *h0, int B, int L,
                              int H, int G, int chunk, int sm_count, void *y, float *h_final, void *workspace,
-                               bool scalars_done, bool add)
+                               bool scalars_done, bool add, bool early)
 {
     if (B <= 0 || L <= 0) return SWIMBA_OK;
     CUtensorMap tm_b, tm_c, tm_x, tm_y;
@@ -1276,6 +1291,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
     p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = nseg > 1 ? 2 : 0; p.y = y;
     p.h_first = h0;
     p.add = add ? 1 : 0;
+    p.early = early ? 1 : 0;
     dim3 grid((unsigned)nseg, (unsigned)(G * pairs_per_group(H, G)), (unsigned)B);
     p.split_tiles = 0;
     if (nseg == 1) {
@@ -1367,7 +1383,7 @@ int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_s
         const SsdStream Cs{cmix, GN};
         const int rc = launch_ssd_tiles_streams(ctx, (const __nv_bfloat16 *)x_slots + (int64_t)j * T * H * SP, Bs, Cs, dt,
                                                 A, dt_bias, nullptr, j == 0 ? h0 : nullptr, B, L, H, G, chunk, sm_count,
-                                                y, h_final, workspace, true, j > 0);
+                                                y, h_final, workspace, true, j > 0, true);
         if (rc != SWIMBA_OK) return rc;
     }
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
@@ -1402,7 +1418,7 @@ PackedPlan packed_plan(const int32_t *cu, int nseq, int H, int G, int chunk, int
     const int64_t pairs = (int64_t)G * pairs_per_group(H, G);
     const int q_tiles = chunk >= ST ? chunk / ST : 1;
     int64_t seg_tiles = ceil_div64(tiles * pairs, sm_count);
-    if (seg_tiles < 4) seg_tiles = 4;
+    if (seg_tiles < 2) seg_tiles = 2;
     seg_tiles = ceil_div64(seg_tiles, q_tiles) * q_tiles;
     if (seg_tiles > (1 << 22)) seg_tiles = 1 << 22;
     pl.seg_len = (int)seg_tiles * ST;
@@ -1549,6 +1565,7 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &pl, const void *x,
     p.ntile_total = pl.total_tiles;
     p.y = y;
     p.add = 0;
+    p.early = 1;
     p.h_first = h0;
     const unsigned pairs = (unsigned)(G * pairs_per_group(H, G));
     p.h_in = h0; p.seg_states = 0;
@@ -1625,6 +1642,7 @@ SsdParams shard_params(LaunchCtx &ctx, const ShardLayout &lay, int B, int L, int
     p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = 1; p.y = nullptr;
     p.h_first = nullptr;
     p.add = 0;
+    p.early = 0;
     return p;
 }
 }  // namespace
