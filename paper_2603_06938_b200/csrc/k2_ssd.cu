@@ -1149,7 +1149,7 @@ bool ssd_tiles_supported(int dtype, int P, int N)
 static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 
 // Segment length (tokens, multiple of 128); L itself if one segment per sequence is best.  In units of a
-// full tile (3.8 us a head pair), measured: a segment's full pass costs its tiles plus 0.4, the state-only
+// full tile (3.8 us a head pair), measured: a segment's full pass costs its tiles plus 1.2, the state-only
 // pass half a tile's time per tile plus 1 (four heads per CTA), the scan 1.  Whole rounds of CTAs count.
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
 {
@@ -1158,11 +1158,11 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
     const int tiles = ceil_div(L, ST);
     if (2 * ctas > sm_count || tiles <= 2) return tiles * ST;
     const int q_tiles = chunk >= ST ? chunk / ST : 1;                 // segments are whole chunks
-    float best_cost = (float)tiles + 0.4f;
+    float best_cost = (float)tiles + 1.2f;
     int best = tiles;
     for (int st = q_tiles; st < tiles; st += q_tiles) {
         const int64_t nseg = ceil_div(tiles, st);
-        const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 0.4f) +
+        const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 1.2f) +
                            (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.5f * st + 1.f) + 1.f;
         if (cost < best_cost) { best_cost = cost; best = st; }
     }
@@ -1418,7 +1418,7 @@ PackedPlan packed_plan(const int32_t *cu, int nseq, int H, int G, int chunk, int
     const int64_t pairs = (int64_t)G * pairs_per_group(H, G);
     const int q_tiles = chunk >= ST ? chunk / ST : 1;
     int64_t seg_tiles = ceil_div64(tiles * pairs, sm_count);
-    if (seg_tiles < 2) seg_tiles = 2;
+    if (seg_tiles < 4) seg_tiles = 4;
     seg_tiles = ceil_div64(seg_tiles, q_tiles) * q_tiles;
     if (seg_tiles > (1 << 22)) seg_tiles = 1 << 22;
     pl.seg_len = (int)seg_tiles * ST;
