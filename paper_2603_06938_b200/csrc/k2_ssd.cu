@@ -828,30 +828,35 @@ segment_scan_kernel(float *__restrict__ states, const float *__restrict__ seg_de
     // Local end states exist for all segments but a sequence's last one, unless the caller wants the
     // state after the last segment (a sequence shard's summary): that one was computed too.
     const int nlocal = (end_state || end_decay) ? nseg : nseg - 1;
-    // the loads do not depend on the running state: four segments are fetched at a time
-    constexpr int U = 4;
-    for (int s0 = 0; s0 < nseg; s0 += U) {
-        float4 loc[U];
-        float d[U];
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const int s = s0 + q;
-            if (s < nlocal) {
-                loc[q] = reinterpret_cast<const float4 *>(states)[((sb + s) * H + h) * PN4 + v];
-                d[q] = seg_decay[(sb + s) * H + h];
-            }
+    // The loads do not depend on the running state: eight segments are fetched ahead, each slot refilled as soon
+    // as it is used (the kernel moves 128 KB a segment and four heads at 2.6 KB in flight per thread block and
+    // segment: a latency per group of four took 10.6 us for 17 segments of 32 heads, 22.8 us for 36).
+    constexpr int U = 8;
+    float4 loc[U];
+    float d[U];
+    auto fetch = [&](int q, int s) {
+        if (s < nlocal) {
+            loc[q] = reinterpret_cast<const float4 *>(states)[((sb + s) * H + h) * PN4 + v];
+            d[q] = seg_decay[(sb + s) * H + h];
         }
+    };
+#pragma unroll
+    for (int q = 0; q < U; ++q) fetch(q, q);
+    for (int s0 = 0; s0 < nseg; s0 += U) {
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const int s = s0 + q;
             if (s < nseg) {
-                if (s > 0 || keep_first) reinterpret_cast<float4 *>(states)[((sb + s) * H + h) * PN4 + v] = run;
-                if (s >= nlocal) continue;
-                run.x = fmaf(d[q], run.x, loc[q].x);
-                run.y = fmaf(d[q], run.y, loc[q].y);
-                run.z = fmaf(d[q], run.z, loc[q].z);
-                run.w = fmaf(d[q], run.w, loc[q].w);
-                dtot *= d[q];
+                const float4 in = run;
+                if (s < nlocal) {
+                    run.x = fmaf(d[q], run.x, loc[q].x);
+                    run.y = fmaf(d[q], run.y, loc[q].y);
+                    run.z = fmaf(d[q], run.z, loc[q].z);
+                    run.w = fmaf(d[q], run.w, loc[q].w);
+                    dtot *= d[q];
+                    fetch(q, s + U);
+                }
+                if (s > 0 || keep_first) reinterpret_cast<float4 *>(states)[((sb + s) * H + h) * PN4 + v] = in;
             }
         }
     }
@@ -1149,8 +1154,9 @@ bool ssd_tiles_supported(int dtype, int P, int N)
 static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 
 // Segment length (tokens, multiple of 128); L itself if one segment per sequence is best.  In units of a
-// full tile (3.8 us a head pair), measured: a segment's full pass costs its tiles plus 1.2, the state-only
-// pass half a tile's time per tile plus 1 (four heads per CTA), the scan 1.  Whole rounds of CTAs count.
+// full tile (3.7 us a head pair), measured: a segment's full pass costs its tiles plus 1.2, the state-only
+// pass half a tile's time per tile plus 2 (four heads per CTA), the scan 1 and its 64 KB per head and segment
+// at 5 TB/s.  Whole rounds of CTAs count.
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
 {
     const int64_t ctas = (int64_t)B * G * pairs_per_group(H, G);
@@ -1163,7 +1169,8 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
     for (int st = q_tiles; st < tiles; st += q_tiles) {
         const int64_t nseg = ceil_div(tiles, st);
         const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 1.2f) +
-                           (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.5f * st + 1.f) + 1.f;
+                           (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.5f * st + 2.f) + 1.f +
+                           (float)(nseg - 1) * B * H * 0.0035f;
         if (cost < best_cost) { best_cost = cost; best = st; }
     }
     return best * ST;
