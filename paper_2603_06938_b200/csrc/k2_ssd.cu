@@ -829,8 +829,8 @@ segment_scan_kernel(float *__restrict__ states, const float *__restrict__ seg_de
     // state after the last segment (a sequence shard's summary): that one was computed too.
     const int nlocal = (end_state || end_decay) ? nseg : nseg - 1;
     // The loads do not depend on the running state: eight segments are fetched ahead, each slot refilled as soon
-    // as it is used (the kernel moves 128 KB a segment and four heads at 2.6 KB in flight per thread block and
-    // segment: a latency per group of four took 10.6 us for 17 segments of 32 heads, 22.8 us for 36).
+    // as it is used (groups of four waited a latency per group: 22.8 us for 36 local states of 32 heads, now
+    // 17 us for 42, of which 13 us are the 86 MB moved).
     constexpr int U = 8;
     float4 loc[U];
     float d[U];
@@ -1153,10 +1153,12 @@ bool ssd_tiles_supported(int dtype, int P, int N)
 
 static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 
-// Segment length (tokens, multiple of 128); L itself if one segment per sequence is best.  In units of a
-// full tile (3.7 us a head pair), measured: a segment's full pass costs its tiles plus 1.2, the state-only
-// pass half a tile's time per tile plus 2 (four heads per CTA), the scan 1 and its 64 KB per head and segment
-// at 5 TB/s.  Whole rounds of CTAs count.
+// Segment length (tokens, multiple of 128); L itself if one segment per sequence is best.  Costs in units of
+// a full tile of a head pair (3.3 us), from a sweep of lengths 400..32768 at 12..128 (sequence, head) pairs:
+// a segment's full pass takes its tiles plus 1.2, the state-only pass 0.35 a tile plus 1.2 (four heads per
+// CTA), the scan 1 and 0.005 per head and segment (128 KB moved).  Whole rounds of CTAs count.  Of the
+// lengths tried the one picked was the best or within 2 % of it; filling two CTAs per SM whatever it costs
+// took 72 us instead of 66 at 24 heads and 8192 tokens.
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
 {
     const int64_t ctas = (int64_t)B * G * pairs_per_group(H, G);
@@ -1169,8 +1171,8 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
     for (int st = q_tiles; st < tiles; st += q_tiles) {
         const int64_t nseg = ceil_div(tiles, st);
         const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 1.2f) +
-                           (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.5f * st + 2.f) + 1.f +
-                           (float)(nseg - 1) * B * H * 0.0035f;
+                           (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.35f * st + 1.2f) + 1.f +
+                           (float)((nseg - 1) * B * H) * 0.005f;
         if (cost < best_cost) { best_cost = cost; best = st; }
     }
     return best * ST;
