@@ -1213,21 +1213,23 @@ ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bi
 // already fills the GPU (or the segmented path applies), else the number of leading tiles a.  The
 // CTAs that walk the whole sequence (started first, one per SM) cost (n - a) full tiles plus a
 // state-only tiles at about 0.47 of a full one; the CTAs that produce y of the leading tiles run
-// on the SMs left over, in ceil(ctas / spare) rounds of a tiles.  a minimises the later of the two.
+// on the SMs left over, in ceil(ctas / spare) rounds of a tiles and 1.2 for starting and draining one.
+// a minimises the later of the two.  4 sequences of 64 heads and 64 tiles: 219 us at a = 7, 228 us at the
+// a = 8 that a rule without the 1.2 picks, 234 us unsplit.
 static int ssd_split_tiles(int B, int L, int H, int G, int sm_count)
 {
     const int64_t ctas = (int64_t)B * G * pairs_per_group(H, G);
     const int n = ceil_div(L, ST);
     if (2 * ctas <= sm_count || ctas >= sm_count || n < 4) return 0;
     const int64_t spare = sm_count - ctas, rounds = ceil_div64(ctas, spare);
-    float best = (float)n;
+    float best = (float)n + 1.2f;
     int best_a = 0;
     for (int a = 1; a < n; ++a) {
-        const float whole = (float)n - 0.53f * a, lead = (float)(rounds * a);
+        const float whole = (float)n + 1.2f - 0.53f * a, lead = (float)rounds * ((float)a + 1.2f);
         const float m = whole > lead ? whole : lead;
         if (m < best) { best = m; best_a = a; }
     }
-    return best < 0.95f * n ? best_a : 0;
+    return best < 0.97f * ((float)n + 1.2f) ? best_a : 0;
 }
 
 int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &sa)
