@@ -434,6 +434,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 }
                 __syncwarp();
             };
+            if (hd == 0 && kfull && n_pre == 0 && ntiles > 0) issue_g(0);
             for (int j = 0; j < ntiles; ++j) {
                 const int sx = j & 1;
                 const bool full = SPLIT ? (kfull && j >= n_pre) : kfull;
@@ -458,9 +459,6 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                             for (int q = 0; q < nh; ++q) tc::mma_commit(&bars->hd[q].yoff_full);
                         }
                         __syncwarp();
-                        // MMA 1 of this tile goes behind MMA 3 in the tensor pipe: the product with
-                        // the carried state is needed first (it is scaled before the mask is built)
-                        issue_g(j);
                     }
                     // MMA 4: dH^T[n,p] = sum_s Btilde[s,n] (w_s x_s[p])   (K = token)
                     for (int q = 0; q < nh; ++q)
@@ -490,6 +488,9 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                         tc::mma_commit(&hb->yd_full);
                     }
                 }
+                // MMA 1 of the next tile needs no state: it runs under this tile's state update and
+                // epilogue, and the next tile's mask is built while MMA 3 is still waiting for them
+                if (hd == 0 && kfull && j + 1 < ntiles && j + 1 >= n_pre) issue_g(j + 1);
                 // (state-only pass: the second issuer has no product of its own; it follows the
                 // tile loop at the pace of its head's w.X scaling, whose end frees the X slot)
                 if (!full && hd > 0) tc::mbar_wait(&hb->xp_full, j & 1, abort_flag, d_status);
@@ -621,21 +622,6 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             tc::mbar_arrive(&hb->xp_full);
 
             if (full) {
-                // ---- Y = exp(l_i) * (Ctilde Hprev^T), in place
-                tc::mbar_wait(&hb->yoff_full, jf & 1, abort_flag, d_status);
-                tc::tc_fence_after();
-                {
-                    const float e_i = tc::ex2_approx(l2);
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t yo[16];
-                        tc::tmem_ld16(tm + TM_Y + p0 + 16 * hh, yo);
-                        tc::tmem_ld_wait();
-#pragma unroll
-                        for (int q = 0; q < 16; ++q) yo[q] = __float_as_uint(e_i * __uint_as_float(yo[q]));
-                        tc::tmem_st16(tm + TM_Y + p0 + 16 * hh, yo);
-                    }
-                }
                 // ---- decay mask: G (fp32, TMEM) -> M (bf16, TMEM); this thread owns row i and
                 // columns 16 hf .. 16 hf + 15 of every 32-column block
                 tc::mbar_wait(&bars->g_full, jf & 1, abort_flag, d_status);
@@ -690,9 +676,22 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                         tc::tmem_st8(tm + TM_M + c * 16 + 8 * hf, pk);
                     }
                 }
-                tc::tmem_st_wait();
                 tc::tc_fence_before();
                 tc::mbar_arrive(&bars->g_free);
+                // ---- Y = exp(l_i) * (Ctilde Hprev^T), in place
+                tc::mbar_wait(&hb->yoff_full, jf & 1, abort_flag, d_status);
+                tc::tc_fence_after();
+                {
+                    const float e_i = tc::ex2_approx(l2);
+                    uint32_t yo[32];
+                    tc::tmem_ld32(tm + TM_Y + p0, yo);
+                    tc::tmem_ld_wait();
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) yo[q] = __float_as_uint(e_i * __uint_as_float(yo[q]));
+                    tc::tmem_st32(tm + TM_Y + p0, yo);
+                }
+                tc::tmem_st_wait();
+                tc::tc_fence_before();
                 // (the scalars record read above is refilled by a bulk copy once m_full completes)
                 tc::fence_proxy_async_smem();
                 tc::mbar_arrive(&hb->m_full);
@@ -705,11 +704,13 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             tc::mbar_wait(&hb->dh_full, j & 1, abort_flag, d_status);
             tc::tc_fence_after();
             const float dec = tc::ex2_approx(full ? l2_last : run_total);
+            uint32_t dhv[2][16];
+            tc::tmem_ld16(tm + TM_DH + p0, dhv[0]);
+            tc::tmem_ld16(tm + TM_DH + p0 + 16, dhv[1]);
+            tc::tmem_ld_wait();
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-                uint32_t dh[16];
-                tc::tmem_ld16(tm + TM_DH + p0 + 16 * hh, dh);
-                tc::tmem_ld_wait();
+                const uint32_t (&dh)[16] = dhv[hh];
 #pragma unroll
                 for (int q = 0; q < 16; ++q)
                     Hst[16 * hh + q] = fmaf(dec, Hst[16 * hh + q], __uint_as_float(dh[q]));
@@ -735,11 +736,13 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 // ---- epilogue: y_i = Y_i + D x_i, staged in shared memory for the TMA store
                 tc::mbar_wait(&hb->yd_full, jf & 1, abort_flag, d_status);
                 tc::tc_fence_after();
+                uint32_t ydv[2][16];
+                tc::tmem_ld16(tm + TM_Y + p0, ydv[0]);
+                tc::tmem_ld16(tm + TM_Y + p0 + 16, ydv[1]);
+                tc::tmem_ld_wait();
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
-                    uint32_t yd[16];
-                    tc::tmem_ld16(tm + TM_Y + p0 + 16 * hh, yd);
-                    tc::tmem_ld_wait();
+                    const uint32_t (&yd)[16] = ydv[hh];
 #pragma unroll
                     for (int c2 = 0; c2 < 2; ++c2) {
                         const uint32_t off = tc::sw128_offset(i, 4 * hf + 2 * hh + c2);
