@@ -225,6 +225,11 @@ __device__ __forceinline__ void scale_own_row(const uint8_t *s_x, uint8_t *s_xp,
     }
 }
 
+__device__ __forceinline__ uint64_t f32x2_bits(uint32_t a, uint32_t b)
+{
+    return tc::f32x2(__uint_as_float(a), __uint_as_float(b));
+}
+
 template <bool SPLIT>
 __global__ void __launch_bounds__(SSD_THREADS, 1)
 ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_c,
@@ -526,8 +531,9 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
         const uint32_t tm = tmem + TM_HEAD + hd * TM_HEAD_COLS + lane_base;
         const float Dh = prm.D ? prm.D[h] : 0.f;
-        // fp32 master copy of the state: this thread holds H[n = i][p = p0 .. p0+31]
-        float Hst[32];
+        const uint64_t Dh2 = tc::f32x2(Dh, Dh);
+        // fp32 master copy of the state: this thread holds H[n = i][p = p0 .. p0+31], two to a register pair
+        uint64_t Hst[16];
         {
             const bool first = prm.seg_states == 2 && seg == 0;
             const float *h_in = first ? prm.h_first : prm.h_in;
@@ -539,19 +545,19 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     ? ((((int64_t)seg_base + seg) * H + h) * SP) * SN
                     : (((int64_t)b * H + h) * SP) * SN;
 #pragma unroll
-                for (int q = 0; q < 32; ++q) Hst[q] = __ldcg(h_in + base + (int64_t)(p0 + q) * SN + i);
+                for (int q = 0; q < 16; ++q)
+                    Hst[q] = tc::f32x2(__ldcg(h_in + base + (int64_t)(p0 + 2 * q) * SN + i),
+                                       __ldcg(h_in + base + (int64_t)(p0 + 2 * q + 1) * SN + i));
             } else {
 #pragma unroll
-                for (int q = 0; q < 32; ++q) Hst[q] = 0.f;
+                for (int q = 0; q < 16; ++q) Hst[q] = 0;
             }
             if (kfull && n_pre == 0) {
                 // bf16 copy of the state the first tile starts from
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
-                    uint4 v = make_uint4(tc::pack_bf16x2(Hst[8 * ch + 0], Hst[8 * ch + 1]),
-                                         tc::pack_bf16x2(Hst[8 * ch + 2], Hst[8 * ch + 3]),
-                                         tc::pack_bf16x2(Hst[8 * ch + 4], Hst[8 * ch + 5]),
-                                         tc::pack_bf16x2(Hst[8 * ch + 6], Hst[8 * ch + 7]));
+                    uint4 v = make_uint4(tc::f32x2_bf16(Hst[4 * ch]), tc::f32x2_bf16(Hst[4 * ch + 1]),
+                                         tc::f32x2_bf16(Hst[4 * ch + 2]), tc::f32x2_bf16(Hst[4 * ch + 3]));
                     *reinterpret_cast<uint4 *>(s_hb + tc::sw128_offset(i, 4 * hf + ch)) = v;
                 }
                 tc::fence_proxy_async_smem();
@@ -607,10 +613,9 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             // memory.
             tc::mbar_wait(&hb->x_full[sx], (j >> 1) & 1, abort_flag, d_status);
             if (full) {
-                if (wq == 0) scale_units<0, 6>(s_x, s_xp, s_wp, lane, hf);
-                else if (wq == 1) scale_units<6, 11>(s_x, s_xp, s_wp, lane, hf);
-                else if (wq == 2) scale_units<11, 14>(s_x, s_xp, s_wp, lane, hf);
-                else scale_units<14, 16>(s_x, s_xp, s_wp, lane, hf);
+                if (wq == 0) scale_units<0, 8>(s_x, s_xp, s_wp, lane, hf);
+                else if (wq == 1) scale_units<8, 14>(s_x, s_xp, s_wp, lane, hf);
+                else if (wq == 2) scale_units<14, 16>(s_x, s_xp, s_wp, lane, hf);
             } else {
                 // a tile of a run: the X' slab is free once the previous tile's product has read it
                 run_done += l2_last;
@@ -642,14 +647,15 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                             const float up = l2 - Lend;
                             if (Lw - Lend < 96.f) {
                                 const float rf = tc::ex2_approx(up);
+                                const uint64_t rf2 = tc::f32x2(rf, rf);
 #pragma unroll
                                 for (int q = 0; q < 8; ++q) {
-                                    const float2 cb = *reinterpret_cast<const float2 *>(&s_cb[c * 32 + 16 * hf + 2 * q]);
-                                    float m0 = __uint_as_float(cur[2 * q]) * cb.x * rf;
-                                    float m1 = __uint_as_float(cur[2 * q + 1]) * cb.y * rf;
-                                    if (16 * hf + 2 * q > lane) m0 = 0.f;
-                                    if (16 * hf + 2 * q + 1 > lane) m1 = 0.f;
-                                    pk[q] = tc::pack_bf16x2(m0, m1);
+                                    const uint64_t cb = *reinterpret_cast<const uint64_t *>(&s_cb[c * 32 + 16 * hf + 2 * q]);
+                                    float2 m = tc::f32x2_get(tc::f32x2_mul(
+                                        tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rf2));
+                                    if (16 * hf + 2 * q > lane) m.x = 0.f;
+                                    if (16 * hf + 2 * q + 1 > lane) m.y = 0.f;
+                                    pk[q] = tc::pack_bf16x2(m.x, m.y);
                                 }
                             } else {
 #pragma unroll
@@ -666,11 +672,12 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                             // l at the end of column block c, relative to the start of my block
                             const float Lc1 = c == 0 ? L1 : (c == 1 ? L2 : L3);
                             const float rowf = r_i * tc::ex2_approx(Lw - Lc1);
+                            const uint64_t rowf2 = tc::f32x2(rowf, rowf);
 #pragma unroll
                             for (int q = 0; q < 8; ++q) {
-                                const float2 cb = *reinterpret_cast<const float2 *>(&s_cb[c * 32 + 16 * hf + 2 * q]);
-                                pk[q] = tc::pack_bf16x2(__uint_as_float(cur[2 * q]) * cb.x * rowf,
-                                                        __uint_as_float(cur[2 * q + 1]) * cb.y * rowf);
+                                const uint64_t cb = *reinterpret_cast<const uint64_t *>(&s_cb[c * 32 + 16 * hf + 2 * q]);
+                                pk[q] = tc::f32x2_bf16(tc::f32x2_mul(
+                                    tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rowf2));
                             }
                         }
                         tc::tmem_st8(tm + TM_M + c * 16 + 8 * hf, pk);
@@ -686,8 +693,13 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     uint32_t yo[32];
                     tc::tmem_ld32(tm + TM_Y + p0, yo);
                     tc::tmem_ld_wait();
+                    const uint64_t e2 = tc::f32x2(e_i, e_i);
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) yo[q] = __float_as_uint(e_i * __uint_as_float(yo[q]));
+                    for (int q = 0; q < 32; q += 2) {
+                        const float2 v = tc::f32x2_get(tc::f32x2_mul(e2, f32x2_bits(yo[q], yo[q + 1])));
+                        yo[q] = __float_as_uint(v.x);
+                        yo[q + 1] = __float_as_uint(v.y);
+                    }
                     tc::tmem_st32(tm + TM_Y + p0, yo);
                 }
                 tc::tmem_st_wait();
@@ -704,6 +716,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             tc::mbar_wait(&hb->dh_full, j & 1, abort_flag, d_status);
             tc::tc_fence_after();
             const float dec = tc::ex2_approx(full ? l2_last : run_total);
+            const uint64_t dec2 = tc::f32x2(dec, dec);
             uint32_t dhv[2][16];
             tc::tmem_ld16(tm + TM_DH + p0, dhv[0]);
             tc::tmem_ld16(tm + TM_DH + p0 + 16, dhv[1]);
@@ -712,16 +725,14 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             for (int hh = 0; hh < 2; ++hh) {
                 const uint32_t (&dh)[16] = dhv[hh];
 #pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    Hst[16 * hh + q] = fmaf(dec, Hst[16 * hh + q], __uint_as_float(dh[q]));
+                for (int q = 0; q < 8; ++q)
+                    Hst[8 * hh + q] = tc::f32x2_fma(dec2, Hst[8 * hh + q], f32x2_bits(dh[2 * q], dh[2 * q + 1]));
                 if (hb_next) {
 #pragma unroll
                     for (int c2 = 0; c2 < 2; ++c2) {
                         const int ch = 2 * hh + c2;
-                        uint4 v = make_uint4(tc::pack_bf16x2(Hst[8 * ch + 0], Hst[8 * ch + 1]),
-                                             tc::pack_bf16x2(Hst[8 * ch + 2], Hst[8 * ch + 3]),
-                                             tc::pack_bf16x2(Hst[8 * ch + 4], Hst[8 * ch + 5]),
-                                             tc::pack_bf16x2(Hst[8 * ch + 6], Hst[8 * ch + 7]));
+                        uint4 v = make_uint4(tc::f32x2_bf16(Hst[4 * ch]), tc::f32x2_bf16(Hst[4 * ch + 1]),
+                                             tc::f32x2_bf16(Hst[4 * ch + 2]), tc::f32x2_bf16(Hst[4 * ch + 3]));
                         *reinterpret_cast<uint4 *>(s_hb + tc::sw128_offset(i, 4 * hf + ch)) = v;
                     }
                 }
@@ -752,10 +763,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int e0 = c2 * 8 + 2 * q;
-                            const float x0 = __uint_as_float(xw[q] << 16);
-                            const float x1 = __uint_as_float(xw[q] & 0xffff0000u);
-                            o[q] = tc::pack_bf16x2(fmaf(Dh, x0, __uint_as_float(yd[e0])),
-                                                   fmaf(Dh, x1, __uint_as_float(yd[e0 + 1])));
+                            o[q] = tc::f32x2_bf16(tc::f32x2_fma(Dh2, f32x2_bits(xw[q] << 16, xw[q] & 0xffff0000u),
+                                                                f32x2_bits(yd[e0], yd[e0 + 1])));
                         }
                         *reinterpret_cast<uint4 *>(s_y + off) = make_uint4(o[0], o[1], o[2], o[3]);
                         if (packed && t_begin + (j + 1) * ST > L && t_begin + j * ST + i < L) {
@@ -779,17 +788,25 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         if (kfull) {
             if (prm.h_out && seg == nseg - 1 && !head_part) {
                 float *dst = prm.h_out + (((int64_t)b * H + h) * SP) * SN;
-                if (prm.add) {
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) Hst[q] += dst[(int64_t)(p0 + q) * SN + i];
+                for (int q = 0; q < 16; ++q) {
+                    float2 v = tc::f32x2_get(Hst[q]);
+                    if (prm.add) {
+                        v.x += dst[(int64_t)(p0 + 2 * q) * SN + i];
+                        v.y += dst[(int64_t)(p0 + 2 * q + 1) * SN + i];
+                    }
+                    dst[(int64_t)(p0 + 2 * q) * SN + i] = v.x;
+                    dst[(int64_t)(p0 + 2 * q + 1) * SN + i] = v.y;
                 }
-#pragma unroll
-                for (int q = 0; q < 32; ++q) dst[(int64_t)(p0 + q) * SN + i] = Hst[q];
             }
         } else {
             float *dst = prm.h_out + ((((int64_t)seg_base + seg) * H + h) * SP) * SN;
 #pragma unroll
-            for (int q = 0; q < 32; ++q) dst[(int64_t)(p0 + q) * SN + i] = Hst[q];
+            for (int q = 0; q < 16; ++q) {
+                const float2 v = tc::f32x2_get(Hst[q]);
+                dst[(int64_t)(p0 + 2 * q) * SN + i] = v.x;
+                dst[(int64_t)(p0 + 2 * q + 1) * SN + i] = v.y;
+            }
             if (i == 0 && hf == 0) prm.seg_decay[((int64_t)seg_base + seg) * H + h] = tc::ex2_approx(seg_l2);
         }
     }
