@@ -20,6 +20,16 @@
 // the head dimension) and its own MMA-issuing warp, so that one head's tensor-core and memory
 // latencies are covered by the other warps' CUDA-core work.
 //
+// What bounds it: shared memory (about 4500 of a tile's 5500 cycles carry products, TMA and the CUDA cores'
+// reads and writes at 128 bytes a cycle) and the row-block-3 scheduler, not the tensor cores (30 %).  So G of
+// the next tile is issued under this tile's state update (it needs no state) and the mask is built before the
+// product with the carried state is waited for; fp32 work goes two to an instruction; the mask's column
+// weights are read 16 bytes at a time; w.X stays off the warps that have the longest mask rows.  4 x 8192
+// tokens of 64 heads: 228 us a call before these and with 8 leading tiles, 215 with 7, 205 with the mask
+// first, 200 with packed pairs and the new shares of w.X, 193 with the wide reads and one barrier for x and
+// the scalars.  Measured and not taken: the streams loaded as soon as they are free (217: G then displaces
+// the products that are waited for), tensor-memory loads one block ahead (232), 112 registers (no change).
+//
 // The decay mask needs exp(l_i - l_s) for every kept (i, s).  Only the four 32x32 blocks on the
 // diagonal evaluate it entry by entry.  A block strictly below the diagonal (rows in block w,
 // columns in block b < w) factors as
@@ -104,7 +114,7 @@ struct SsdParams {
 
 struct __align__(8) HeadBars {
     uint64_t x_full[2], x_free[2];
-    uint64_t yoff_full, m_full, yd_full, xp_full, dh_full, h_ready, y_free, y_staged, sc_full;
+    uint64_t yoff_full, m_full, yd_full, xp_full, dh_full, h_ready, y_free, y_staged;
 };
 struct __align__(8) SsdBars {
     uint64_t cb_full, cb_empty, g_full, g_free;
@@ -306,7 +316,6 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             tc::mbar_init(&hb->h_ready, HEAD_THREADS);
             tc::mbar_init(&hb->y_free, HEAD_THREADS);
             tc::mbar_init(&hb->y_staged, HEAD_THREADS);
-            tc::mbar_init(&hb->sc_full, 1);
         }
         *abort_flag = 0;
         tc::fence_mbar_init();
@@ -341,7 +350,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         if (leader && ntiles > 0) {
             for (int hd = 0; hd < nh; ++hd) {               // X of tile 0
                 HeadBars *hb = &bars->hd[hd];
-                tc::mbar_arrive_expect_tx(&hb->x_full[0], SLAB);
+                tc::mbar_arrive_expect_tx(&hb->x_full[0], SLAB + (uint32_t)sizeof(TileScalars));
                 tc::tma_load_4d(smem + SM_HEAD + hd * SM_HEAD_BYTES, &tmap_x, &hb->x_full[0], 0,
                                 head0 + hd, tok0 + t_begin, bco);
             }
@@ -350,8 +359,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         if (leader && ntiles > 0) {
             for (int hd = 0; hd < nh; ++hd) {               // its scalars
                 HeadBars *hb = &bars->hd[hd];
-                tc::mbar_arrive_expect_tx(&hb->sc_full, (uint32_t)sizeof(TileScalars));
-                tc::bulk_load(&sm->sc[hd], scal_rec(hd, 0), (uint32_t)sizeof(TileScalars), &hb->sc_full);
+                tc::bulk_load(&sm->sc[hd], scal_rec(hd, 0), (uint32_t)sizeof(TileScalars), &hb->x_full[0]);
             }
         }
         for (int j = 0; j < ntiles; ++j) {
@@ -373,7 +381,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     HeadBars *hb = &bars->hd[hd];
                     tc::mbar_wait(&hb->x_free[sx], ((jn >> 1) & 1) ^ 1, abort_flag, d_status);
                     if (leader) {
-                        tc::mbar_arrive_expect_tx(&hb->x_full[sx], SLAB);
+                        tc::mbar_arrive_expect_tx(&hb->x_full[sx], SLAB + (uint32_t)sizeof(TileScalars));
                         tc::tma_load_4d(smem + SM_HEAD + hd * SM_HEAD_BYTES + sx * SLAB, &tmap_x,
                                         &hb->x_full[sx], 0, head0 + hd, t0 + ST, bco);
                     }
@@ -384,10 +392,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     HeadBars *hb = &bars->hd[hd];
                     if (full) tc::mbar_wait(&hb->m_full, (SPLIT ? j - n_pre : j) & 1, abort_flag, d_status);
                     else tc::mbar_wait(&hb->xp_full, j & 1, abort_flag, d_status);
-                    if (leader) {
-                        tc::mbar_arrive_expect_tx(&hb->sc_full, (uint32_t)sizeof(TileScalars));
-                        tc::bulk_load(&sm->sc[hd], scal_rec(hd, jn), (uint32_t)sizeof(TileScalars), &hb->sc_full);
-                    }
+                    if (leader)
+                        tc::bulk_load(&sm->sc[hd], scal_rec(hd, jn), (uint32_t)sizeof(TileScalars), &hb->x_full[sx]);
                 }
             }
             __syncwarp();
@@ -600,18 +606,17 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             // the weights of all rows and the block ends arrive in shared memory
             const float l2 = l2_next;
             if (j + 1 < ntiles) l2_next = l2p[(j + 1) * ST + i];
-            tc::mbar_wait(&hb->sc_full, j & 1, abort_flag, d_status);
+            tc::mbar_wait(&hb->x_full[sx], (j >> 1) & 1, abort_flag, d_status);
             const float4 ends = *reinterpret_cast<const float4 *>(s_ends);
             const float L1 = ends.x, L2 = ends.y, L3 = ends.z, l2_last = ends.w;
             const float Lw = wq == 0 ? 0.f : (wq == 1 ? L1 : (wq == 2 ? L2 : L3));    // l before my block
             const float Lend = wq == 0 ? L1 : (wq == 1 ? L2 : (wq == 2 ? L3 : l2_last));  // l at its end
 
             // ---- w . X  (rows of the X slab -> rows of the X' slab, this thread's half of the
-            // head dim).  The decay mask below costs row block wq about wq + 1 units of work, so in
-            // the full pass the 16 (row block, 16-byte chunk) units of a lane are dealt 6 / 5 / 3 / 2
-            // to row blocks 0 .. 3 instead of 4 each; a foreign row's weight is read from shared
-            // memory.
-            tc::mbar_wait(&hb->x_full[sx], (j >> 1) & 1, abort_flag, d_status);
+            // head dim).  Row block wq has wq + 1 blocks of the decay mask to build, all of them on one
+            // scheduler (a warp reads only its quarter of the tensor memory), so in the full pass the 16
+            // (row block, 16-byte chunk) units of a lane are dealt 8 / 6 / 2 / 0 to row blocks 0 .. 3; a
+            // foreign row's weight is read from shared memory.
             if (full) {
                 if (wq == 0) scale_units<0, 8>(s_x, s_xp, s_wp, lane, hf);
                 else if (wq == 1) scale_units<8, 14>(s_x, s_xp, s_wp, lane, hf);
@@ -638,6 +643,10 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     if (c <= wq) {
                         uint32_t cur[16], pk[8];
                         tc::tmem_ld16(g_addr + c * 32, cur);
+                        ulonglong2 cb4[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            cb4[q] = *reinterpret_cast<const ulonglong2 *>(&s_cb[c * 32 + 16 * hf + 4 * q]);
                         tc::tmem_ld_wait();
                         if (c == wq) {
                             // diagonal block: Delta_j 2^(l_i - l_j) = cb_j 2^(l_i - l_blockend).  The
@@ -650,7 +659,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                                 const uint64_t rf2 = tc::f32x2(rf, rf);
 #pragma unroll
                                 for (int q = 0; q < 8; ++q) {
-                                    const uint64_t cb = *reinterpret_cast<const uint64_t *>(&s_cb[c * 32 + 16 * hf + 2 * q]);
+                                    const uint64_t cb = (q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x;
                                     float2 m = tc::f32x2_get(tc::f32x2_mul(
                                         tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rf2));
                                     if (16 * hf + 2 * q > lane) m.x = 0.f;
@@ -660,7 +669,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                             } else {
 #pragma unroll
                                 for (int q = 0; q < 8; ++q) {
-                                    const float2 cb = *reinterpret_cast<const float2 *>(&s_cb[c * 32 + 16 * hf + 2 * q]);
+                                    const float2 cb = tc::f32x2_get((q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x);
                                     float m0 = __uint_as_float(cur[2 * q]) * tc::ex2_approx(up + tc::lg2_approx(cb.x));
                                     float m1 = __uint_as_float(cur[2 * q + 1]) * tc::ex2_approx(up + tc::lg2_approx(cb.y));
                                     if (16 * hf + 2 * q > lane) m0 = 0.f;
@@ -675,7 +684,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                             const uint64_t rowf2 = tc::f32x2(rowf, rowf);
 #pragma unroll
                             for (int q = 0; q < 8; ++q) {
-                                const uint64_t cb = *reinterpret_cast<const uint64_t *>(&s_cb[c * 32 + 16 * hf + 2 * q]);
+                                const uint64_t cb = (q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x;
                                 pk[q] = tc::f32x2_bf16(tc::f32x2_mul(
                                     tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rowf2));
                             }
