@@ -86,8 +86,7 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count);
 // x and h0 were complete before the first kernel of the same call.
 ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
                              void *workspace);
-// beside: launched right behind the streaming router, to run together with it
-int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &args, bool beside = false);
+int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &args);
 size_t ssd_scalars_bytes(int B, int L, int H);       // of the arrays ssd_scalars_args lays out
 // Chains nseg segment states per (sequence, head): states [B,nseg,H,P,N] holds local end states on entry
 // and, for all but the first segment, entry states on exit (P = 64, N = 128).

@@ -675,7 +675,7 @@ static bool router_stream_usable(const void *u, int64_t Ttok, int F, int E, int 
 static int launch_router_stream(LaunchCtx &ctx, const __nv_bfloat16 *u, const __nv_bfloat16 *W_r,
                                 int64_t Ttok, int F, int E, int k, int32_t *idx, float *w, int *counts,
                                 int *perm, int64_t cap, int sm_count, void *zero_out,
-                                int zero_bytes_per_token, float *pi_out)
+                                int zero_bytes_per_token, bool behind_scalars, float *pi_out)
 {
     const int NT = E <= 8 ? 1 : E <= 16 ? 2 : E <= 32 ? 4 : 8;
     // ring depth: the deepest (up to RS_MAX_STAGES) that still lets two CTAs share an SM, else
@@ -699,7 +699,7 @@ static int launch_router_stream(LaunchCtx &ctx, const __nv_bfloat16 *u, const __
         if (!ensure_dynamic_smem((const void *)kern,             \
                                  smem))                                     \
             return SWIMBA_ERR_CUDA;                                                             \
-        launch_kernel(kern, dim3((unsigned)ctas), dim3(RS_THREADS), smem, ctx.stream, false, tmap, \
+        launch_kernel(kern, dim3((unsigned)ctas), dim3(RS_THREADS), smem, ctx.stream, behind_scalars, tmap, \
                       W_r, Ttok, F, E, k, idx, w, counts, perm, cap, (uint4 *)zero_out,         \
                       zero_bytes_per_token / 16, (int)ctas, nstages, ctx.d_status, pi_out);             \
     } while (0)
@@ -757,17 +757,14 @@ static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Tto
 {
     const int warps = 8;
     // The SSD step sizes of the same call (scalars.l2 != NULL) depend on dt only and run beside the
-    // router: as the leading blocks of the register-fed tensor-core kernel, as a kernel of their own that
-    // starts with the streaming router, else in front of the router.
+    // router: as the leading blocks of the register-fed tensor-core kernel, else as a kernel of
+    // their own in front of the router (the streaming router then starts while it runs).
+    bool behind_scalars = false;
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-        if (E > 1 && router_stream_usable(u, Ttok, F, E, sm_count)) {
-            const int rc = launch_router_stream(ctx, u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, sm_count,
-                                                zero_out, zero_bytes_per_token, pi_out);
-            return rc == SWIMBA_OK && scalars.l2 ? launch_ssd_scalars(ctx, scalars, true) : rc;
-        }
-        if (E > 1 && F % (32 * RM_KSPLIT) == 0 && E <= 64)
+        if (E > 1 && !router_stream_usable(u, Ttok, F, E, sm_count) && F % (32 * RM_KSPLIT) == 0 && E <= 64)
             return launch_router_mma(ctx, u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, sm_count,
                                      zero_out, zero_bytes_per_token, scalars, pi_out);
+        behind_scalars = E > 1 && scalars.l2 && router_stream_usable(u, Ttok, F, E, sm_count);
     }
     if (scalars.l2) {
         const int rc = launch_ssd_scalars(ctx, scalars);
@@ -781,6 +778,11 @@ static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Tto
                       false, Ttok, idx, w, counts, perm, pi_out);
         ctx.end();
         return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+    }
+    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+        if (router_stream_usable(u, Ttok, F, E, sm_count))
+            return launch_router_stream(ctx, u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, sm_count,
+                                        zero_out, zero_bytes_per_token, behind_scalars, pi_out);
     }
     const size_t w_bytes = (size_t)E * F * sizeof(T);
     const int stage_w = (w_bytes <= 64 * 1024 && (w_bytes & 15) == 0) ? 1 : 0;

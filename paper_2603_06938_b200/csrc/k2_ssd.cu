@@ -132,17 +132,15 @@ struct __align__(16) SsdSmall {
 __host__ __device__ inline int pairs_per_group(int H, int G) { return (H / G + NHD - 1) / NHD; }
 }  // namespace
 
-// Stand-alone launch of the step sizes and tile log-decays.  BESIDE: behind the streaming router, which lets it
-// in at once and which it does not depend on; both then run together.  The kernels behind wait for this grid
-// only, so one of its blocks stays until the router has completed.
-template <bool BESIDE>
+// Stand-alone launch of the step sizes and tile log-decays.
 __global__ void __launch_bounds__(256)
 ssd_scalars_kernel(const ScalarsArgs args)
 {
-    if (!BESIDE) grid_dep_wait();
+    // Everything earlier in the stream has completed once the wait returns; only then may the
+    // kernel behind this one (the streaming router, which writes without waiting) be let in.
+    grid_dep_wait();
     grid_dep_launch();
     ssd_scalars_block(args, blockIdx.x);
-    if (BESIDE && blockIdx.x == 0) grid_dep_wait();
 }
 
 // Self-test of the bounded wait every tensor-core kernel here relies on: one warp waits, with the
@@ -1263,12 +1261,12 @@ static int ssd_split_tiles(int B, int L, int H, int G, int sm_count)
     return best < 0.97f * ((float)n + 1.2f) ? best_a : 0;
 }
 
-int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &sa, bool beside)
+int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &sa)
 {
     if (scalars_units(sa) <= 0) return SWIMBA_OK;
     ctx.begin(STAGE_SSD_SCALARS);
-    launch_kernel(beside ? ssd_scalars_kernel<true> : ssd_scalars_kernel<false>, dim3((unsigned)scalars_blocks(sa, 256)),
-                  dim3(256), 0, ctx.stream, true, sa);
+    launch_kernel(ssd_scalars_kernel, dim3((unsigned)scalars_blocks(sa, 256)), dim3(256), 0, ctx.stream,
+                  true, sa);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }

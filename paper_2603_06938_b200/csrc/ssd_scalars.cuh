@@ -59,9 +59,8 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
     for (int q = 0; q < NU; ++q) {
         const int64_t unit = unit0 + q;
         const bool act = unit < nunits;
-        // (heads fastest: a token's step sizes lie side by side, so the units of a block share what they fetch)
-        const int h = act ? (int)(unit % a.H) : 0;
-        const int tile = act ? (int)((unit / a.H) % ntile) : 0;
+        const int tile = act ? (int)(unit % ntile) : 0;
+        const int h = act ? (int)((unit / ntile) % a.H) : 0;
         const int64_t b = act ? unit / ((int64_t)ntile * a.H) : 0;
         // first token of the lane's four in dt, and tokens of the tile that exist from there on
         int64_t tok = b * a.L + tile * SCALARS_TILE + lane * 4;
