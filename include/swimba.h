@@ -89,8 +89,8 @@ typedef struct {
  * Uses the current CUDA device.  *out is set only on success.
  * Which kernels serve a configuration: with SWIMBA_DTYPE_BF16, P == 64 and N == 128 the SSD runs
  * on the tensor cores in 128-token tiles; every other shape, and SWIMBA_DTYPE_FP32, evaluates the
- * recurrence token by token with one block per (sequence, head), which is exact in fp32 but
- * serial over L (orders of magnitude slower on long sequences).  The expert projection uses the
+ * same chunked form in fp32 on the CUDA cores, up to eight blocks of 32 tokens per (sequence, head)
+ * at a time (several times slower on long sequences).  The expert projection uses the
  * tensor cores for SWIMBA_DTYPE_BF16 with F >= 64 and S % 32 == 0. */
 int swimba_create(const swimba_config *cfg, swimba_handle **out);
 
@@ -228,7 +228,7 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
  *   dt, h0, y, h_final as in swimba_forward; there is no skip term (w->D is not read).
  * The injection is linear in (B^(e), X^(e)), so the call evaluates k ordinary chunked recurrences
  * (one per slot, each with its own injection stream and the readout stream mixed over all slots)
- * and adds them; cost is k times swimba_ssd plus two streaming passes per extra slot, and the state
+ * and adds them; cost is k times swimba_ssd (slots behind the first add to y and the state), and the state
  * stays [B,H,P,N] whatever E is (Theorem 1).  Workspace: swimba_ssd_slots_workspace_bytes. */
 int swimba_route_project_slots(swimba_handle *h, const swimba_weights *w, const void *u, int64_t T,
                                void *BC_slots, int32_t *topk_idx, float *topk_w, void *workspace,
@@ -326,8 +326,8 @@ int swimba_route_mix_static(swimba_handle *h, const swimba_weights *w, const voi
  * every kernel a call enqueues is bracketed by CUDA events on the call's stream.
  * swimba_profile_read synchronises that stream and returns how many kernels the most recent call
  * (for swimba_forward_host: its last batch slice) launched (at most max_entries), with kernel_ids[i] in 1..24 (1 router + grouping by
- * expert (for fewer than about 28000 tokens the launch also computes the SSD step sizes), 4 expert GEMM, 5 slot mix, 6 SIMT projection, 7 per-timestep SSM, 8 decode update, 9 SSD
- * tile kernel, 10 segment scan, 11 SSD step sizes and decays, 12 slot stream assembly, 13 slot sum, 14 small-batch projection, 15 convolution + SiLU, 16 gated norm, 17 step-size columns, 18 adjoint recurrence pass, 19 router softmax over all experts, 20 weight / logit adjoints, 21 router-matrix gradient, 22 expert-matrix gradient, 23 states at the tile boundaries for the adjoint, 24 state-only SSD pass; 2 and 3 are not in use) and ms[i] its duration in milliseconds.
+ * expert (for fewer than about 28000 tokens the launch also computes the SSD step sizes), 4 expert GEMM, 5 slot mix, 6 SIMT projection, 7 fp32 chunked SSM and packed decode tokens, 8 decode update, 9 SSD
+ * tile kernel, 10 segment scan, 11 SSD step sizes and decays, 12 slot stream assembly, 13 slot sum, 14 small-batch projection (short forwards too), 15 convolution + SiLU, 16 gated norm, 17 step-size columns, 18 adjoint recurrence pass, 20 weight / logit adjoints, 21 router-matrix gradient, 22 expert-matrix gradient, 23 states at the tile boundaries for the adjoint, 24 state-only SSD pass; 2, 3 and 19 are not in use) and ms[i] its duration in milliseconds.
  * Both arrays are HOST arrays. */
 int swimba_profile(swimba_handle *h, int enable);
 int swimba_profile_read(swimba_handle *h, int32_t *kernel_ids, float *ms, int32_t max_entries);

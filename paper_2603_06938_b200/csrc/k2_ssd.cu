@@ -258,7 +258,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // Split launch (grid = [B, head pairs, 2]; used when one CTA per (sequence, head pair) would
-    // leave a third of the SMs idle): the CTAs of the first z-plane, which start first, walk the whole
+    // leave SMs idle): the CTAs of the first z-plane, which start first, walk the whole
     // sequence but evaluate the first split_tiles tiles for their end state only (about half the
     // cost of a full tile) and produce y from there on; the CTAs of the second plane produce y of
     // those first tiles.  No CTA waits for another.
@@ -1402,7 +1402,7 @@ slot_readout_kernel(const __nv_bfloat16 *__restrict__ slots, int64_t T, int GN, 
 // The layer as the sum over the slots of one evaluation each (the injection is linear in
 // (B^(e), X^(e))): slots behind the first add their y tile with the reducing TMA store and their end
 // state in place, so that no per-slot y exists. 8 x 2048 tokens of 24 heads, k = 2:
-// 240 us a call with a summing pass per slot and an assembled stream per slot, 147 us this way (bit-identical).
+// 240 us a call with a summing pass per slot and an assembled stream per slot, 143 us this way (bit-identical).
 int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_slots, const float *dt, const float *A,
                            const float *dt_bias, const float *h0, int B, int L, int H, int G, int k, int chunk,
                            int sm_count, void *y, float *h_final, void *cmix, void *workspace)

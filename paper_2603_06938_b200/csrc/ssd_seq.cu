@@ -1,6 +1,6 @@
-// Per-timestep evaluation of the single selective-SSM recurrence (selective-SSM equation with
-// the channelwise convention; Theorem 1) with the state held in registers: the fp32 path of the
-// forward, and K4, the one-token decode update.
+// The recurrence on the CUDA cores (selective-SSM equation with the channelwise convention; Theorem 1):
+// the chunked fp32 path of the forward, packed sequences of a few tokens stepped token by token, and K4,
+// the one-token decode update.
 #include "internal.h"
 #include "tc05.cuh"
 
