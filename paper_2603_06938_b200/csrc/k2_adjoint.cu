@@ -459,9 +459,9 @@ adjoint_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_c
         const int srow = tid >> 2, sch = (tid & 3) * 2;
         const int wq = warp & 3, cq = warp >> 2, i = wq * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
-        float acc[32];
+        uint64_t acc[16];                                    // two fp32 sums each
 #pragma unroll
-        for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+        for (int e = 0; e < 16; ++e) acc[e] = 0;
         for (int n = 0; n < nheads; ++n) {
             const int s = n % AC_STAGES;
             tc::mbar_wait(&sm->full[s], (n / AC_STAGES) & 1, abort_flag, d_status);
@@ -498,21 +498,31 @@ adjoint_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_c
                 const float l_beg = cq == 0 ? 0.f : sc->ends[cq - 1];
                 const bool prod = cq < wq || l_beg - l_end < 96.f;
                 const float rf = tc::ex2_approx(prod ? up : 0.f);
+                const uint64_t rf2 = tc::f32x2(rf, rf);
+                uint32_t v[32];
+                tc::tmem_ld32(sa, v);
+                tc::tmem_ld_wait();
+                if (cq == wq) {
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t v[16];
-                    tc::tmem_ld16(sa + 16 * c, v);
-                    tc::tmem_ld_wait();
+                    for (int e = 0; e < 32; ++e) v[e] = e <= lane ? v[e] : 0u;
+                }
+                if (prod) {
 #pragma unroll
-                    for (int e = 0; e < 16; e += 4) {
-                        const float4 w4 = *reinterpret_cast<const float4 *>(cb + 16 * c + e);
-                        const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
+                    for (int e = 0; e < 32; e += 4) {
+                        const ulonglong2 w4 = *reinterpret_cast<const ulonglong2 *>(cb + e);
+                        acc[e / 2] = tc::f32x2_fma(tc::f32x2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
+                                                   tc::f32x2_mul(w4.x, rf2), acc[e / 2]);
+                        acc[e / 2 + 1] = tc::f32x2_fma(tc::f32x2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3])),
+                                                       tc::f32x2_mul(w4.y, rf2), acc[e / 2 + 1]);
+                    }
+                } else {
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const float f = prod ? wv[k] * rf : tc::ex2_approx(up + tc::lg2_approx(wv[k]));
-                            const bool keep = cq < wq || 16 * c + e + k <= lane;
-                            if (keep) acc[16 * c + e + k] = fmaf(__uint_as_float(v[e + k]), f, acc[16 * c + e + k]);
-                        }
+                    for (int e = 0; e < 32; e += 2) {
+                        // (behind the diagonal the exponent is positive: the entry there is zero, its factor must be finite)
+                        const float f0 = e <= lane ? tc::ex2_approx(up + tc::lg2_approx(cb[e])) : 0.f;
+                        const float f1 = e + 1 <= lane ? tc::ex2_approx(up + tc::lg2_approx(cb[e + 1])) : 0.f;
+                        acc[e / 2] = tc::f32x2_fma(tc::f32x2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
+                                                   tc::f32x2(f0, f1), acc[e / 2]);
                     }
                 }
             }
@@ -528,8 +538,8 @@ adjoint_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_c
 #pragma unroll
             for (int c = 0; c < 4; ++c)
                 *reinterpret_cast<uint4 *>(m + tc::sw128_offset(i, (cq & 1) * 4 + c)) =
-                    make_uint4(tc::pack_bf16x2(acc[8 * c], acc[8 * c + 1]), tc::pack_bf16x2(acc[8 * c + 2], acc[8 * c + 3]),
-                               tc::pack_bf16x2(acc[8 * c + 4], acc[8 * c + 5]), tc::pack_bf16x2(acc[8 * c + 6], acc[8 * c + 7]));
+                    make_uint4(tc::f32x2_bf16(acc[4 * c]), tc::f32x2_bf16(acc[4 * c + 1]), tc::f32x2_bf16(acc[4 * c + 2]),
+                               tc::f32x2_bf16(acc[4 * c + 3]));
         }
         tc::fence_proxy_async_smem();
         tc::mbar_arrive(&sm->m_ready);
