@@ -46,14 +46,13 @@ TIMED_SECONDS = 1.5   # the K-step timed region is repeated until it has covered
 # the current kernel reports null.  ncu flushes caches before a launch, and part of a kernel's
 # writes can still sit in L2 when it ends.
 NCU_TRAFFIC_BYTES = {
-    # profiles/forward_small_lm_kernels.md (the router launch includes the SSD step sizes)
-    "small_lm": {"router_topk": 26.790e6, "expert_gemm": 36.989e6, "ssd_tiles": 82.690e6},
-    # profiles/forward_mid_kernels.md
-    "mid": {"ssd_scalars": 8.413e6, "router_topk": 147.230e6, "expert_gemm": 256.823e6, "ssd_tiles": 584.555e6},
-    # profiles/ssd_segmented_long_seq.md (the state-only pass is a kernel of its own)
-    "long_seq": {"ssd_state": 306.343e6, "ssd_tiles": 619.930e6, "segment_scan": 17.834e6},
-    # profiles/decode_step_kernels.md
-    "decode": {"router_topk": 0.593e6, "project_small": 9.070e6, "decode_update": 479.990e6},
+    # profiles/case_launch_lists.md (at small_lm the router launch includes the SSD step sizes; the state-only
+    # pass of long_seq is a kernel of its own)
+    "small_lm": {"router_topk": 26.791e6, "expert_gemm": 37.000e6, "ssd_tiles": 77.479e6},
+    "mid": {"ssd_scalars": 8.413e6, "router_topk": 144.258e6, "expert_gemm": 242.470e6, "ssd_tiles": 571.672e6},
+    "long_seq": {"ssd_scalars": 8.413e6, "router_topk": 151.871e6, "expert_gemm": 288.257e6, "ssd_state": 302.795e6,
+                 "segment_scan": 17.864e6, "ssd_tiles": 611.674e6},
+    "decode": {"router_topk": 0.613e6, "project_small": 9.072e6, "decode_update": 476.994e6},
 }
 
 
