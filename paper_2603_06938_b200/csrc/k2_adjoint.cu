@@ -16,7 +16,8 @@
 //   adjoint_tiles_kernel   one CTA per (tile, group, share of its heads) sums over the heads in tensor
 //                          memory and registers and adds dBtilde | dCtilde to dBC.
 // What bounds them: HBM.  Both read x and dy once; the boundary states (32 KB per head and tile) are
-// written once and read once.  4 x 8192 tokens of 64 heads: 214 us (5.0 TB/s) and 251 us (4.3 TB/s); two
+// written once and read once.  4 x 8192 tokens of 64 heads: 214 us (5.0 TB/s) and 220 us (4.9 TB/s; 251 us
+// while the mask chose its factor entry by entry, exponentials included); two
 // evaluations of the forward's tile kernel on a virtual layer of 2H heads, with its operands re-arranged
 // and its per-head outputs summed by kernels of their own, took 1960 us.
 #include "internal.h"
