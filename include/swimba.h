@@ -19,6 +19,9 @@
  *     row-major with the last index contiguous and must be 16-byte aligned.
  *   - The caller owns every tensor and the workspace; the library owns only the handle (a few
  *     bytes of device memory for a status word).  Nothing is allocated or freed after create.
+ *   - Workspaces: swimba_workspace_bytes, _ssd_slots_, _block_, _backward_ and _shard_workspace_bytes
+ *     grow with B and with L, so a buffer sized for a handle's largest call serves its smaller ones.
+ *     The other queries are asked for every call's own sizes.
  *   - Calls enqueue work on the given CUDA stream and return without synchronising.
  *   - Return value: SWIMBA_OK or a negative SWIMBA_ERR_* code.  When an error is detected on
  *     the host nothing is enqueued and no output is touched.  Nothing throws or aborts.
@@ -136,7 +139,7 @@ int swimba_ssd(swimba_handle *h, const swimba_weights *w, const void *x, const v
  * "Mamba-2 and SSD": a linear recurrence between blocks of tokens).  1: each sequence is walked
  * once with the carried state kept on chip.  More than 1 (long sequences, few of them): a first
  * pass computes every segment's end state, a scan chains them, a second pass produces y; the
- * workspace then holds segments * B*H*P*N floats of segment states.  0 if B or L is not
+ * workspace then holds them (segments * B*H*P*N floats).  0 if B or L is not
  * positive.  The result does not depend on the segmentation beyond rounding. */
 int32_t swimba_ssd_segments(const swimba_handle *h, int32_t B, int32_t L);
 

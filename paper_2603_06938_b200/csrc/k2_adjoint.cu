@@ -20,6 +20,8 @@
 // while the mask chose its factor entry by entry, exponentials included); two
 // evaluations of the forward's tile kernel on a virtual layer of 2H heads, with its operands re-arranged
 // and its per-head outputs summed by kernels of their own, took 1960 us.
+#include <algorithm>
+
 #include "internal.h"
 #include "ssd_scalars.cuh"
 #include "tc05.cuh"
@@ -590,6 +592,14 @@ int adj_seg_tiles(int B, int nt, int H, int G, int sm_count)
     const int st = (int)ceil_div64(nt, nseg);
     return st < 2 ? 2 : st;
 }
+// States at segment starts (of all heads each) that a call reserves: at least what any call with no more
+// sequences of no more tokens takes (at most `cut` sequences are few enough to be cut).
+int64_t adj_segment_states(int B, int nt, int H, int G, int sm_count)
+{
+    const int64_t quads = (int64_t)G * adj_quads(H, G);
+    const int64_t cut = std::min<int64_t>(B, sm_count / (6 * quads));
+    return nt < 6 ? 0 : std::min<int64_t>(2 * cut * ceil_div(nt, 2), sm_count / quads);
+}
 struct AdjLayout {
     size_t scal, states, seg_states, seg_decay, total;
     int nt, seg_tiles, nseg;
@@ -601,13 +611,12 @@ AdjLayout adj_layout(int B, int L, int H, int G, int sm_count)
     l.nt = ceil_div(L, AT);
     l.seg_tiles = adj_seg_tiles(B, l.nt, H, G, sm_count);
     l.nseg = ceil_div(l.nt, l.seg_tiles);
+    const size_t nstates = (size_t)adj_segment_states(B, l.nt, H, G, sm_count);
     size_t off = 0;
     l.scal = off;   off += ssd_scalars_bytes(B, L, H);
     l.states = off; off += up((size_t)2 * B * l.nt * H * AN * AP * 2);
-    l.seg_states = off;
-    if (l.nseg > 1) off += up((size_t)2 * B * l.nseg * H * AN * AP * sizeof(float));
-    l.seg_decay = off;
-    if (l.nseg > 1) off += up((size_t)2 * B * l.nseg * H * sizeof(float));
+    l.seg_states = off; off += up(nstates * H * AN * AP * sizeof(float));
+    l.seg_decay = off;  off += up(nstates * H * sizeof(float));
     l.total = off;
     return l;
 }

@@ -1188,6 +1188,11 @@ static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 // CTA), the scan 1 and 0.005 per head and segment (128 KB moved).  Whole rounds of CTAs count.  Of the
 // lengths tried the one picked was the best or within 2 % of it; filling two CTAs per SM whatever it costs
 // took 72 us instead of 66 at 24 heads and 8192 tokens.
+// No more segments than SEG_ROUNDS rounds of CTAs, or than segments of SEG_TILES tiles make: the costs pick
+// more at none of 200 000 shapes (1 to 64 heads, 1 to 24 sequences of up to 150000 tokens), and
+// ssd_segment_states can reserve for every shorter call without knowing its pick.
+constexpr int SEG_ROUNDS = 4, SEG_TILES = 12;
+
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
 {
     const int64_t ctas = (int64_t)B * G * pairs_per_group(H, G);
@@ -1195,16 +1200,36 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
     const int tiles = ceil_div(L, ST);
     if (2 * ctas > sm_count || tiles <= 2) return tiles * ST;
     const int q_tiles = chunk >= ST ? chunk / ST : 1;                 // segments are whole chunks
+    const int64_t most = std::max<int64_t>(SEG_ROUNDS * (int64_t)sm_count / ctas, tiles / SEG_TILES);
     float best_cost = (float)tiles + 1.2f;
     int best = tiles;
     for (int st = q_tiles; st < tiles; st += q_tiles) {
         const int64_t nseg = ceil_div(tiles, st);
+        if (nseg > most) continue;
         const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 1.2f) +
                            (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.35f * st + 1.2f) + 1.f +
                            (float)((nseg - 1) * B * H) * 0.005f;
         if (cost < best_cost) { best_cost = cost; best = st; }
     }
     return best * ST;
+}
+
+// Segment states (of all H heads each) a B x L call reserves: at least what any call of the handle with no
+// more sequences of no more tokens takes, so that a buffer sized for the largest call serves the others.
+// (Sequences are cut only while two CTAs per SM are not reached: at most `cut` of them.)
+static int64_t ssd_segment_states(int B, int L, int H, int G, int chunk, int sm_count)
+{
+    const int64_t pairs = (int64_t)G * pairs_per_group(H, G), tiles = ceil_div(L, ST);
+    const int64_t cut = std::min<int64_t>(B, sm_count / (2 * pairs));
+    if (tiles <= 2) return 0;
+    const int q_tiles = chunk >= ST ? chunk / ST : 1;
+    return std::min(cut * ceil_div64(tiles, q_tiles),
+                    std::max(SEG_ROUNDS * (int64_t)sm_count / pairs, cut * (tiles / SEG_TILES)));
+}
+
+static size_t ssd_states_bytes(int64_t n, int H)
+{
+    return (size_t)n * H * SP * SN * sizeof(float) + ((size_t)n * H * sizeof(float) + 255) / 256 * 256;
 }
 
 // Workspace: [log-decays B*H*Lpad float] [per-tile records B*H*(Lpad/128)] [segment states]
@@ -1219,12 +1244,7 @@ size_t ssd_scalars_bytes(int B, int L, int H)
 
 size_t ssd_workspace_bytes(int B, int L, int H, int G, int chunk, int sm_count)
 {
-    const int seg_len = ssd_segment_len(B, L, H, G, chunk, sm_count);
-    const int nseg = ceil_div(L, seg_len);
-    size_t tot = ssd_scalars_bytes(B, L, H);
-    if (nseg > 1)
-        tot += (size_t)B * nseg * H * SP * SN * sizeof(float) + ((size_t)B * nseg * H * sizeof(float) + 255) / 256 * 256;
-    return tot;
+    return ssd_scalars_bytes(B, L, H) + ssd_states_bytes(ssd_segment_states(B, L, H, G, chunk, sm_count), H);
 }
 
 ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
@@ -1651,8 +1671,9 @@ ShardLayout shard_layout(int B, int L, int H, int G, int chunk, int sm_count)
     l.nseg = ceil_div(L, l.seg_len);
     size_t off = 0;
     l.scal = off;   off += ssd_scalars_bytes(B, L, H);
-    l.states = off; off += ((size_t)B * l.nseg * H * SP * SN * sizeof(float) + 255) / 256 * 256;
-    l.decay = off;  off += ((size_t)B * l.nseg * H * sizeof(float) + 255) / 256 * 256;
+    l.states = off;
+    l.decay = off + (size_t)B * l.nseg * H * SP * SN * sizeof(float);
+    off += ssd_states_bytes(std::max<int64_t>(B, ssd_segment_states(B, L, H, G, chunk, sm_count)), H);
     l.total = off;
     return l;
 }

@@ -1,0 +1,56 @@
+"""Workspace queries over ranges of sizes, without a device: they read nothing of a handle but its
+configuration and the SM count, which lead it."""
+import ctypes
+import random
+
+import pytest
+
+from paper_2603_06938_b200 import binding as sb
+from paper_2603_06938_b200 import build as sbuild
+
+SMS = 148
+
+
+def handle(F, H, G, E, k, chunk, P=64, N=128, dtype=sb.DTYPE_BF16):
+    sbuild.build()
+    block = (ctypes.c_int32 * 4096)(F, H, P, N, G, E, k, chunk, dtype, 0, 0, SMS)
+    return block, ctypes.cast(block, ctypes.c_void_p)
+
+
+LAYERS = [(768, 24, 1, 8, 2, 256), (2048, 64, 1, 8, 2, 128), (1152, 36, 2, 16, 4, 256), (64, 3, 1, 4, 1, 64),
+          (768, 96, 1, 64, 3, 128), (512, 2, 2, 1, 1, 256), (2048, 160, 1, 8, 2, 128)]
+
+
+@pytest.mark.parametrize("name", ["workspace", "ssd_slots_workspace", "block_workspace", "backward_workspace",
+                                  "shard_workspace"])
+@pytest.mark.parametrize("layer", LAYERS)
+def test_smaller_calls_need_no_more(name, layer):
+    """128-token tiles decide the segments: every tile count of a sequence, then batches."""
+    keep, h = handle(*layer)
+    need = getattr(sb.lib(), f"swimba_{name}_bytes")
+    lengths = [1, 100] + list(range(128, 128 * 200, 128)) + list(range(25600, 140000, 3712))
+    for B in (1, 2, 3, 7):
+        sizes = [need(h, B, L) for L in lengths]
+        assert sizes == sorted(sizes)
+    for L in (90, 300, 1500, 2432, 5376, 24704, 100000):
+        sizes = [need(h, B, L) for B in range(1, 80)]
+        assert sizes == sorted(sizes)
+
+
+def test_segment_states_fit_what_is_reserved():
+    """The forward's regions, by the sizes that include/swimba.h names, with the states of the segments that
+    the call really makes."""
+    up = lambda v: (v + 255) // 256 * 256
+    rnd = random.Random(5)
+    need, segments = sb.lib().swimba_workspace_bytes, sb.lib().swimba_ssd_segments
+    for F, H, G, E, k, chunk in LAYERS:
+        keep, h = handle(F, H, G, E, k, chunk)
+        S, PN = 2 * G * 128, 64 * 128
+        for _ in range(1500):
+            B, L = rnd.randint(1, 20), int(2 ** rnd.uniform(0, 17))
+            T, tiles, nseg = B * L, (L + 127) // 128, segments(h, B, L)
+            size = up(T * S * 2) + 2 * up(T * k * 4) + up(256 + up(E * T * 4) + (up(T * k * S * 2) if k > 2 else 0))
+            size += up(B * H * tiles * 512) + up(B * H * tiles * 1040)
+            if nseg > 1:
+                size += B * nseg * H * (PN + 1) * 4
+            assert size <= need(h, B, L), (B, L, nseg)
