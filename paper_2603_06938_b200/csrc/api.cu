@@ -124,9 +124,9 @@ HostLayout host_layout(const swimba_config &c, int B, int L, int sm_count)
     l.hf2 = off; off += align_up((size_t)B * HP * c.d_state * sizeof(float));   // (carried states alternate)
     l.idx = off; off += align_up(T * c.top_k * sizeof(int32_t));
     l.w = off;   off += align_up(T * c.top_k * sizeof(float));
-    // the forward runs slice by slice on the same scratch
-    const HostPlan hp = host_plan(c, B, L);
-    l.fwd = off; off += fwd_layout(c, hp.seqs, hp.piece, sm_count).total;
+    // the forward runs slice by slice on the same scratch: sized for the whole call, which serves every slice
+    // (they differ: the last one has fewer sequences or tokens) and lets a larger call's buffer serve this one
+    l.fwd = off; off += fwd_layout(c, B, L, sm_count).total;
     l.total = off;
     return l;
 }

@@ -22,7 +22,7 @@ LAYERS = [(768, 24, 1, 8, 2, 256), (2048, 64, 1, 8, 2, 128), (1152, 36, 2, 16, 4
 
 
 @pytest.mark.parametrize("name", ["workspace", "ssd_slots_workspace", "block_workspace", "backward_workspace",
-                                  "shard_workspace"])
+                                  "shard_workspace", "host_workspace"])
 @pytest.mark.parametrize("layer", LAYERS)
 def test_smaller_calls_need_no_more(name, layer):
     """128-token tiles decide the segments: every tile count of a sequence, then batches."""
@@ -54,3 +54,17 @@ def test_segment_states_fit_what_is_reserved():
             if nseg > 1:
                 size += B * nseg * H * (PN + 1) * 4
             assert size <= need(h, B, L), (B, L, nseg)
+
+
+@pytest.mark.parametrize("F,H,E,k,chunk,B,L", [(768, 64, 4, 1, 256, 4, 9956), (768, 32, 16, 2, 256, 5, 9924),
+                                               (768, 48, 8, 2, 128, 9, 600), (2048, 64, 8, 2, 128, 4, 9984)])
+def test_host_workspace_serves_every_slice(F, H, E, k, chunk, B, L):
+    """Behind the staged tensors (u, x, dt, y, two state buffers, routing) the forward's workspace for any slice:
+    up to an eighth of the sequences, or a run of tokens of one."""
+    up = lambda v: (v + 255) // 256 * 256
+    keep, h = handle(F, H, 1, E, k, chunk)
+    T, HP = B * L, H * 64
+    staged = up(T * F * 2) + 2 * up(T * HP * 2) + up(T * H * 4) + 2 * up(B * HP * 128 * 4) + 2 * up(T * k * 4)
+    left = sb.lib().swimba_host_workspace_bytes(h, B, L) - staged
+    assert max(sb.lib().swimba_workspace_bytes(h, n, L) for n in range(1, (B + 7) // 8 + 1)) <= left
+    assert max(sb.lib().swimba_workspace_bytes(h, 1, n) for n in range(1, L + 1)) <= left
