@@ -20,8 +20,8 @@
  *   - The caller owns every tensor and the workspace; the library owns only the handle (a few
  *     bytes of device memory for a status word).  Nothing is allocated or freed after create.
  *   - Workspaces: swimba_workspace_bytes, _ssd_slots_, _block_, _backward_, _shard_ and
- *     _host_workspace_bytes grow with B and with L, so a buffer sized for a handle's largest call serves
- *     its smaller ones.  The other queries are asked for every call's own sizes.
+ *     _host_workspace_bytes grow with B and with L, _decode_workspace_bytes with B, so a buffer sized for
+ *     a handle's largest call serves its smaller ones.  _packed_workspace_bytes is asked for every batch.
  *   - Calls enqueue work on the given CUDA stream and return without synchronising.
  *   - Return value: SWIMBA_OK or a negative SWIMBA_ERR_* code.  When an error is detected on
  *     the host nothing is enqueued and no output is touched.  Nothing throws or aborts.

@@ -71,9 +71,10 @@ DecLayout dec_layout(const swimba_config &c, int B)
     DecLayout l;
     const size_t S = 2u * c.n_groups * c.d_state;
     size_t off = 0;
-    const bool slots = front_small_supported(c.dtype, B, c.d_model, (int)S, c.n_experts, c.top_k) &&
-                       front_small_slots(B, c.top_k);
-    l.bc = off;  off += align_up((size_t)B * (slots ? c.top_k : 1) * S * sizeof(float));
+    // fp32 rows: as many as any batch of up to B sequences takes
+    const int64_t rows = front_small_supported(c.dtype, 1, c.d_model, (int)S, c.n_experts, c.top_k)
+                             ? front_small_max_rows(B, c.top_k) : B;
+    l.bc = off;  off += align_up((size_t)rows * S * sizeof(float));
     l.idx = off; off += align_up((size_t)B * c.top_k * sizeof(int32_t));
     l.w = off;   off += align_up((size_t)B * c.top_k * sizeof(float));
     l.gemm = off;

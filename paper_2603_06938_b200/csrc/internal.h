@@ -69,6 +69,7 @@ int launch_accumulate(LaunchCtx &ctx, int dtype, void *y, const void *y_add, int
 // in front of this call has completed, so it may read what earlier calls wrote before its own wait.
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
 bool front_small_slots(int64_t T, int k);
+int64_t front_small_max_rows(int64_t T, int k);     // rows of S streams that any call of up to T tokens takes
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
                        int S, int E, int k, int32_t *idx, float *w, float *BC);
 // The same kernels for short calls of the forward: BC [T,S] bf16; scalars as in launch_router.

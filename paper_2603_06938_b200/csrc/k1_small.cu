@@ -19,6 +19,8 @@
 // matrix and the tokens are in L2, and a dependent launch costs more than they do); the rows go to slots,
 // since no kernel in front could clear the mixed streams.  A decode step of one token, 64 heads, 8 experts,
 // F = 2048: router and projection apart 14.7 us, one kernel (and the states read under it) 8.5 us.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace swimba {
@@ -342,6 +344,12 @@ bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k)
 
 static bool front_small_fused(int64_t T) { return T <= SM_FUSED; }
 bool front_small_slots(int64_t T, int k) { return front_small_fused(T) || k > 2; }
+int64_t front_small_max_rows(int64_t T, int k)
+{
+    // (more tokens may take fewer rows: slots up to SM_FUSED tokens, or for k > 2 as far as this front end goes)
+    const int64_t slots = k * std::min<int64_t>(T, k > 2 ? SM_MAX_T : SM_FUSED);
+    return std::max(T, slots);
+}
 
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
                        int S, int E, int k, int32_t *idx, float *w, float *BC)

@@ -68,3 +68,13 @@ def test_host_workspace_serves_every_slice(F, H, E, k, chunk, B, L):
     left = sb.lib().swimba_host_workspace_bytes(h, B, L) - staged
     assert max(sb.lib().swimba_workspace_bytes(h, n, L) for n in range(1, (B + 7) // 8 + 1)) <= left
     assert max(sb.lib().swimba_workspace_bytes(h, 1, n) for n in range(1, L + 1)) <= left
+
+
+@pytest.mark.parametrize("F,G,E,k,dtype", [(2048, 1, 8, 2, "bf16"), (768, 1, 16, 4, "bf16"), (4096, 2, 16, 8, "bf16"),
+                                           (96, 1, 4, 1, "bf16"), (2048, 1, 64, 3, "bf16"), (256, 1, 8, 3, "fp32")])
+def test_smaller_decode_batches_need_no_more(F, G, E, k, dtype):
+    keep, h = handle(F, 8, G, E, k, 128, dtype=sb.DTYPE_FP32 if dtype == "fp32" else sb.DTYPE_BF16)
+    sizes = [sb.lib().swimba_decode_workspace_bytes(h, B) for B in range(1, 1200)]
+    assert sizes == sorted(sizes)
+    if E <= 16 and dtype == "bf16":      # the small front end: k fp32 rows per sequence up to B = 4
+        assert sizes[3] >= 4 * k * 256 * G * 4
