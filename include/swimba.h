@@ -22,6 +22,8 @@
  *   - Workspaces: swimba_workspace_bytes, _ssd_slots_, _block_, _backward_, _shard_ and
  *     _host_workspace_bytes grow with B and with L, _decode_workspace_bytes with B, so a buffer sized for
  *     a handle's largest call serves its smaller ones.  _packed_workspace_bytes is asked for every batch.
+ *   - States may be updated in place: h_final may be h0 itself (forward, packed, slots, block, ssd, and
+ *     shard_finish's h_end).  Inputs and outputs must not overlap otherwise.
  *   - Calls enqueue work on the given CUDA stream and return without synchronising.
  *   - Return value: SWIMBA_OK or a negative SWIMBA_ERR_* code.  When an error is detected on
  *     the host nothing is enqueued and no output is touched.  Nothing throws or aborts.

@@ -742,7 +742,7 @@ int swimba_forward_packed(swimba_handle *h, const swimba_weights *w, const void 
     const size_t PN = (size_t)c.n_heads * c.head_dim * c.d_state;
     if (T == 0) {
         // nothing but empty sequences: every state passes through
-        if (h_final) {
+        if (h_final && h_final != h0) {
             const cudaError_t e = h0 ? cudaMemcpyAsync(h_final, h0, (size_t)nseq * PN * sizeof(float), cudaMemcpyDeviceToDevice, ctx.stream)
                                      : cudaMemsetAsync(h_final, 0, (size_t)nseq * PN * sizeof(float), ctx.stream);
             if (e != cudaSuccess) return fail(h, SWIMBA_ERR_CUDA, "copying the states failed");
@@ -777,7 +777,7 @@ int swimba_forward_packed(swimba_handle *h, const swimba_weights *w, const void 
                 float *hf = h_final ? h_final + (size_t)b * PN : nullptr;
                 const float *hin = h0 ? h0 + (size_t)b * PN : nullptr;
                 if (len == 0) {
-                    if (hf) {
+                    if (hf && hf != hin) {
                         const cudaError_t e = hin ? cudaMemcpyAsync(hf, hin, PN * sizeof(float), cudaMemcpyDeviceToDevice, ctx.stream)
                                                   : cudaMemsetAsync(hf, 0, PN * sizeof(float), ctx.stream);
                         if (e != cudaSuccess) rc = fail(h, SWIMBA_ERR_CUDA, "copying a state failed");

@@ -90,8 +90,9 @@ ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bi
 int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &args);
 size_t ssd_scalars_bytes(int B, int L, int H);       // of the arrays ssd_scalars_args lays out
 // Chains nseg segment states per (sequence, head): states [B,nseg,H,P,N] holds local end states on entry
-// and, for all but the first segment, entry states on exit (P = 64, N = 128).
-int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const float *h0, int B, int nseg, int H);
+// and, for all but the first segment (keep_first: for all), entry states on exit (P = 64, N = 128).
+int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const float *h0, int B, int nseg, int H,
+                        bool keep_first);
 int launch_ssd_tiles(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
                      const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int G,
                      int chunk, int sm_count, void *y, float *h_final, void *workspace,

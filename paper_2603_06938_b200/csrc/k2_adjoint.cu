@@ -693,7 +693,7 @@ int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, cons
         for (int dir = 0; dir < 2; ++dir) {
             const int rc = launch_segment_scan(ctx, p.seg_states + (size_t)dir * B * lay.nseg * H * AN * AP,
                                                p.seg_decay + (size_t)dir * B * lay.nseg * H, dir == 0 ? h0 : nullptr, B,
-                                               lay.nseg, H);
+                                               lay.nseg, H, false);
             if (rc != SWIMBA_OK) return rc;
         }
     }

@@ -86,7 +86,7 @@ struct SsdParams {
     const TileScalars *rec; // [B,H,Lpad/128] per-tile weights and block ends
     const float *D;
     const float *h_in;      // initial states: [B,H,P,N] (nseg == 1) or [B,nseg,H,P,N]; may be null
-    const float *h_first;   // seg_states == 2: states entering the first segments, [B,H,P,N]; may be null
+    const float *h_first;   // seg_states >= 2: states entering the first segments, [B,H,P,N]; may be null
     float *h_out;           // MODE_FULL: h_final [B,H,P,N] (last segment writes) or null
                             // MODE_STATE_ONLY: local end states [B,nseg,H,P,N]
     float *seg_decay;       // MODE_STATE_ONLY: [B,nseg,H] product of a_t over the segment
@@ -99,7 +99,8 @@ struct SsdParams {
     // (grid.x), the scalar arrays are laid out [H, tiles of the batch], and the per-segment state
     // arrays are indexed by seqs[b].seg0 + segment.  seg_states: h_in / state-only h_out are those
     // per-segment arrays (else h_in is [sequences, H, P, N]); 2: a sequence's first segment starts from
-    // h_first instead.  y: base of the output (ragged last
+    // h_first instead; 3: so does a sequence of one segment (in-place states: the first of several reads
+    // the scan's copy, since the last one writes over h_first in the same launch).  y: base of the output (ragged last
     // tiles are stored row by row).  Null seqs: dense [B, L].
     const SeqDesc *seqs;
     const int2 *items;
@@ -541,7 +542,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         // fp32 master copy of the state: this thread holds H[n = i][p = p0 .. p0+31], two to a register pair
         uint64_t Hst[16];
         {
-            const bool first = prm.seg_states == 2 && seg == 0;
+            const bool first = seg == 0 && (prm.seg_states == 2 || (prm.seg_states == 3 && nseg == 1));
             const float *h_in = first ? prm.h_first : prm.h_in;
             // (states of earlier segments come from the scan in front; given ones go past L1)
             const bool wait = !prm.early || (prm.seg_states && !first);
@@ -829,7 +830,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
 //   H_in(0) = h0,   H_in(s+1) = decay(s) H_in(s) + S(s).
 // One thread per 4 consecutive state entries; segments are walked in order.  The first segment's
 // entry state is h0 itself and is written only when keep_first is set (a sequence shard, whose entry
-// state is not known yet): otherwise the full pass reads h0.
+// state is not known yet; states updated in place): otherwise the full pass reads h0.
 // (packed batch: the z-th block plane works sequence multi[z], which owns segments seqs[b].seg0 ..
 // seqs[b+1].seg0 - 1 of the batch-wide list; sequences of one segment are not listed -- copying their
 // entry states was 57 of the 80 us this kernel took for 64 sequences, 57 of them a token long)
@@ -1291,13 +1292,14 @@ int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &sa)
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
-int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const float *h0, int B, int nseg, int H)
+int launch_segment_scan(LaunchCtx &ctx, float *states, const float *decay, const float *h0, int B, int nseg, int H,
+                        bool keep_first)
 {
     const int PN4 = SP * SN / 4;
     ctx.begin(STAGE_SEGMENT_SCAN);
     launch_kernel(segment_scan_kernel, dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)B), dim3(256), 0,
                   ctx.stream, true, states, decay, h0, nseg, H, PN4, (const SeqDesc *)nullptr,
-                  (const int *)nullptr, 0, (float *)nullptr, (float *)nullptr);
+                  (const int *)nullptr, keep_first ? 1 : 0, (float *)nullptr, (float *)nullptr);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
@@ -1348,7 +1350,9 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
     p.D = D;
     p.L = L; p.Lpad = Lpad; p.H = H; p.G = G; p.nseg = nseg; p.seg_len = seg_len;
     p.d_status = ctx.d_status;
-    p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = nseg > 1 ? 2 : 0; p.y = y;
+    // h_final over h0: no CTA may read the given state while another one writes the final one
+    const bool in_place = h0 && h0 == h_final;
+    p.seqs = nullptr; p.items = nullptr; p.ntile_total = 0; p.seg_states = nseg > 1 ? (in_place ? 1 : 2) : 0; p.y = y;
     p.h_first = h0;
     p.add = add ? 1 : 0;
     p.early = early ? 1 : 0;
@@ -1356,7 +1360,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
     p.split_tiles = 0;
     if (nseg == 1) {
         p.h_in = h0; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
-        p.split_tiles = ssd_split_tiles(B, L, H, G, sm_count);
+        p.split_tiles = in_place ? 0 : ssd_split_tiles(B, L, H, G, sm_count);
         if (p.split_tiles > 0) grid = dim3((unsigned)B, (unsigned)(G * pairs_per_group(H, G)), 2u);
         ctx.begin(STAGE_SSD_TILES);
         if (p.split_tiles > 0)
@@ -1374,7 +1378,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
             if (rc != SWIMBA_OK) return rc;
         }
         {
-            const int rc = launch_segment_scan(ctx, states, decay, h0, B, nseg, H);
+            const int rc = launch_segment_scan(ctx, states, decay, h0, B, nseg, H, in_place);
             if (rc != SWIMBA_OK) return rc;
         }
         p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
@@ -1633,14 +1637,15 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &pl, const void *x,
         float *states = (float *)(ws + lay.states);
         float *decay = (float *)(ws + lay.decay);
         p.items = (const int2 *)(ws + lay.pre);
-        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY; p.seg_states = 2;
+        const bool in_place = h0 && h0 == h_final;
+        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY; p.seg_states = in_place ? 3 : 2;
         const int rc = launch_state_pass(ctx, x, Bs, T, 1, p, (unsigned)pl.pre.size(), H, G, 1u);
         if (rc != SWIMBA_OK) return rc;
         const int PN4 = SP * SN / 4;
         ctx.begin(STAGE_SEGMENT_SCAN);
         launch_kernel(segment_scan_kernel, dim3((unsigned)ceil_div(PN4, 256), (unsigned)H, (unsigned)pl.multi.size()),
                       dim3(256), 0, ctx.stream, true, states, (const float *)decay, h0, 0, H, PN4, p.seqs,
-                      (const int *)(ws + lay.multi), 0, (float *)nullptr, (float *)nullptr);
+                      (const int *)(ws + lay.multi), in_place ? 1 : 0, (float *)nullptr, (float *)nullptr);
         ctx.end();
         p.h_in = states;
     }
