@@ -243,7 +243,9 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
             const float e0 = s_e[i0], e1 = s_e[i0 + 1];
             a0.x *= e0; a0.y *= e0; a0.z *= e0; a0.w *= e0;
             a1.x *= e1; a1.y *= e1; a1.z *= e1; a1.w *= e1;
-            for (int s = 0; s <= i0 + 1; s += 4) {          // (G is zero past the diagonal)
+            // columns up to the diagonal and none behind it (G's zeros there would meet later tokens' infinities)
+            int s = 0;
+            for (; s + 4 <= i0; s += 4) {
                 const float4 g0 = *reinterpret_cast<const float4 *>(sG + i0 * Gr + s);
                 const float4 g1 = *reinterpret_cast<const float4 *>(sG + (i0 + 1) * Gr + s);
                 const float gv0[4] = {g0.x, g0.y, g0.z, g0.w}, gv1[4] = {g1.x, g1.y, g1.z, g1.w};
@@ -254,11 +256,27 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
                     fma4(a1, gv1[q], xv);
                 }
             }
+            if (s < i0) {
+                const float2 g0 = *reinterpret_cast<const float2 *>(sG + i0 * Gr + s);
+                const float2 g1 = *reinterpret_cast<const float2 *>(sG + (i0 + 1) * Gr + s);
+                const float4 x0 = *reinterpret_cast<const float4 *>(sx + s * Pp + c);
+                const float4 x1 = *reinterpret_cast<const float4 *>(sx + (s + 1) * Pp + c);
+                fma4(a0, g0.x, x0);
+                fma4(a1, g1.x, x0);
+                fma4(a0, g0.y, x1);
+                fma4(a1, g1.y, x1);
+            }
+            const float4 xi0 = *reinterpret_cast<const float4 *>(sx + i0 * Pp + c);
+            const float4 xi1 = *reinterpret_cast<const float4 *>(sx + (i0 + 1) * Pp + c);
+            const float2 gd = *reinterpret_cast<const float2 *>(sG + (i0 + 1) * Gr + i0);
+            fma4(a0, sG[i0 * Gr + i0], xi0);
+            fma4(a1, gd.x, xi0);
+            fma4(a1, gd.y, xi1);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 if (i0 + r >= nt) break;
                 float4 v = r ? a1 : a0;
-                fma4(v, Dh, *reinterpret_cast<const float4 *>(sx + (i0 + r) * Pp + c));
+                fma4(v, Dh, r ? xi1 : xi0);
                 T *dst = y + ((tok0 + i0 + r) * H + h) * P + c;
                 const float o[4] = {v.x, v.y, v.z, v.w};
                 if (vec) {
