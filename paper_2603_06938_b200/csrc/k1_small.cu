@@ -33,10 +33,12 @@ constexpr int SM_WARPS = 8;
 constexpr int SM_NT = 4;            // 8-token column tiles worked per pass
 constexpr int SM_FUSED = 4;         // tokens up to which the projection routes as well
 
-// k rounds of arg-max over the logits (ties to the lower index); returns the next expert.
+// k rounds of arg-max over the logits (ties to the lower index); returns the next expert.  Logits that compare
+// with nothing (NaN) leave the lowest expert not taken yet: a token never picks one twice, so that an
+// expert's list holds no more entries than there are tokens.
 __device__ __forceinline__ int next_expert(const float (&g)[SM_MAX_E], int E, unsigned taken)
 {
-    int best = 0;
+    int best = __ffs(~taken) - 1;
     float bv = -INFINITY;
 #pragma unroll
     for (int e = 0; e < SM_MAX_E; ++e)
