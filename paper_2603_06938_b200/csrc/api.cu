@@ -193,8 +193,8 @@ int run_route_mix(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, con
     const void *Wr = w->W_router ? w->W_router : w->W_expert;
     const bool tensor = gemm_ws && !bc_fp32 && use_tensor_k1(c);
     if (tensor && front_short_supported(c.dtype, T, c.d_model, S, c.n_experts, c.top_k)) {
-        const int rc = launch_front_short(ctx, u, Wr, w->W_expert, T, c.d_model, S, c.n_experts, c.top_k, idx, wt, BC,
-                                          scalars ? *scalars : ScalarsArgs{});
+        const int rc = launch_front_short(ctx, u, Wr, w->W_expert, T, c.d_model, S, c.n_experts, c.top_k, h->sm_count, idx,
+                                          wt, BC, scalars ? *scalars : ScalarsArgs{});
         return rc == SWIMBA_OK ? rc : fail(h, rc, "routing / projection launch failed");
     }
     int *counts = nullptr, *perm = nullptr;
@@ -1045,7 +1045,7 @@ int swimba_decode_step(swimba_handle *h, const swimba_weights *w, const void *u,
     const bool tensor = !small && use_tensor_k1(c);
     if (small) {
         rc = launch_front_small(ctx, u, w->W_router ? w->W_router : w->W_expert, w->W_expert, B, c.d_model, S,
-                                c.n_experts, c.top_k, idx, wt, (float *)BC);
+                                c.n_experts, c.top_k, h->sm_count, idx, wt, (float *)BC);
         if (rc != SWIMBA_OK) fail(h, rc, "routing / projection launch failed");
     } else {
         rc = run_route_mix(h, ctx, w, u, B, BC, !tensor, idx, wt, tensor ? ws + l.gemm : nullptr);

@@ -71,11 +71,11 @@ bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
 bool front_small_slots(int64_t T, int k);
 int64_t front_small_max_rows(int64_t T, int k);     // rows of S streams that any call of up to T tokens takes
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
-                       int S, int E, int k, int32_t *idx, float *w, float *BC);
+                       int S, int E, int k, int sm_count, int32_t *idx, float *w, float *BC);
 // The same kernels for short calls of the forward: BC [T,S] bf16; scalars as in launch_router.
 bool front_short_supported(int dtype, int64_t T, int F, int S, int E, int k);
 int launch_front_short(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F, int S, int E,
-                       int k, int32_t *idx, float *w, void *BC, const ScalarsArgs &scalars);
+                       int k, int sm_count, int32_t *idx, float *w, void *BC, const ScalarsArgs &scalars);
 
 // K2/K3 (tensor cores): tiled SSD with the carried state kept on chip; bf16, P == 64, N == 128.
 bool ssd_tiles_supported(int dtype, int P, int N);

@@ -7,7 +7,7 @@
 //                         over all E, the k largest kept with their softmax values, NOT renormalised
 //                         (router softmax equation and the sentence after it); clears the token's
 //                         row of the fp32 mixed streams
-//   project_small_kernel  one CTA per (expert, 16 rows of its matrix): finds the tokens routed to
+//   project_small_kernel  one CTA per (expert, 16 rows of its matrix, share of the tokens): finds the tokens routed to
 //                         its expert by scanning the k * T routing entries, streams its 16 x F slice
 //                         of W_e once, multiplies it with those tokens' features on the tensor cores
 //                         (mma.sync m16n8k16, features split over the eight warps and added in a
@@ -238,9 +238,10 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
             }
         }
     } else {
-        // tokens routed to this expert (a token picks an expert at most once); the order of the list
-        // does not matter: every entry ends in its own output row
-        for (int i = tid; i < Ttok * k; i += blockDim.x) {
+        // tokens of this CTA's share routed to its expert (a token picks an expert at most once); the order
+        // of the list does not matter: every entry ends in its own output row
+        const int t_end = (int)((int64_t)Ttok * (blockIdx.z + 1) / gridDim.z) * k;
+        for (int i = (int)((int64_t)Ttok * blockIdx.z / gridDim.z) * k + tid; i < t_end; i += blockDim.x) {
             const int ei = idx[i];
             if (check && (ei < 0 || ei >= E)) atomicCAS(d_status, 0, SWIMBA_ERR_DEVICE_BOUNDS);
             if (ei == e) {
@@ -353,8 +354,19 @@ int64_t front_small_max_rows(int64_t T, int k)
     return std::max(T, slots);
 }
 
+// Shares the tokens of a projection are cut into (grid z; a CTA lists and works its share): sixteen entries of
+// an expert or more each, two CTAs per SM at most.  Few experts make few CTAs (32 with two experts), which
+// walked their lists 32 entries at a time: two experts, k = 2, F = 768, 256 tokens 34.0 us (the grouped
+// product: 16.4), in shares 13; four experts, k = 1, F = 2048, 128 tokens 10.5, in shares 9.  32 entries a
+// share are 5 % slower over 1083 calls, four CTAs per SM 3 %.
+static unsigned project_shares(int64_t T, int S, int E, int k, int sm_count)
+{
+    const int64_t by_work = T * k / (16 * (int64_t)E), by_sms = 2 * (int64_t)sm_count / ((int64_t)(S / SM_ROWS) * E);
+    return (unsigned)std::max<int64_t>(1, std::min(by_work, by_sms));
+}
+
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
-                       int S, int E, int k, int32_t *idx, float *w, float *BC)
+                       int S, int E, int k, int sm_count, int32_t *idx, float *w, float *BC)
 {
     if (T <= 0) return SWIMBA_OK;
     const bool slots = front_small_slots(T, k), fused = front_small_fused(T);
@@ -368,7 +380,8 @@ int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const voi
     ctx.begin(STAGE_PROJECT_SMALL);
     auto kern = fused ? project_small_kernel<ROWS_SLOTS, true>
                       : slots ? project_small_kernel<ROWS_SLOTS, false> : project_small_kernel<ROWS_ADD, false>;
-    launch_kernel(kern, dim3((unsigned)(S / SM_ROWS), (unsigned)E), dim3(256), 0, ctx.stream, true, (const __nv_bfloat16 *)u,
+    launch_kernel(kern, dim3((unsigned)(S / SM_ROWS), (unsigned)E, fused ? 1u : project_shares(T, S, E, k, sm_count)),
+                  dim3(256), 0, ctx.stream, true, (const __nv_bfloat16 *)u,
                   (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F, S, E, k, (void *)BC,
                   ctx.check_indices ? 1 : 0, ctx.d_status);
     ctx.end();
@@ -377,14 +390,16 @@ int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const voi
 
 // The forward's streams for short calls: no histogram to clear, no lists, no tiles.  One prompt of
 // 93 tokens, 24 heads, F = 768, one of four experts: 22.5 us a call through router, lists and grouped product,
-// 16.8 us this way (the first tile and the states fetched ahead of the wait included).
+// 16.8 us this way (the first tile and the states fetched ahead of the wait included).  With few features the
+// grouped product has little to do and keeps its lead: sixteen experts, k = 2, F = 256, 192 tokens 14.4 us
+// this way, 12.3 there; F = 512, 256 tokens 15.1 and 14.4; F = 768 15.4 and 18.0.
 bool front_short_supported(int dtype, int64_t T, int F, int S, int E, int k)
 {
-    return front_small_supported(dtype, T, F, S, E, k) && k <= 2 && E > 1;
+    return front_small_supported(dtype, T, F, S, E, k) && k <= 2 && E > 1 && T * k < F;
 }
 
 int launch_front_short(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F, int S, int E,
-                       int k, int32_t *idx, float *w, void *BC, const ScalarsArgs &scalars)
+                       int k, int sm_count, int32_t *idx, float *w, void *BC, const ScalarsArgs &scalars)
 {
     if (T <= 0) return SWIMBA_OK;
     ctx.begin(STAGE_ROUTER);
@@ -393,7 +408,8 @@ int launch_front_short(LaunchCtx &ctx, const void *u, const void *W_r, const voi
                   (float4 *)BC, k == 1 ? 0 : S / 8, scalars);
     ctx.end();
     ctx.begin(STAGE_PROJECT_SMALL);
-    launch_kernel(project_small_kernel<ROWS_BF16, false>, dim3((unsigned)(S / SM_ROWS), (unsigned)E), dim3(256), 0, ctx.stream,
+    launch_kernel(project_small_kernel<ROWS_BF16, false>,
+                  dim3((unsigned)(S / SM_ROWS), (unsigned)E, project_shares(T, S, E, k, sm_count)), dim3(256), 0, ctx.stream,
                   true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F,
                   S, E, k, BC, ctx.check_indices ? 1 : 0, ctx.d_status);
     ctx.end();
