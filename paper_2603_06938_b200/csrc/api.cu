@@ -73,7 +73,7 @@ DecLayout dec_layout(const swimba_config &c, int B)
     size_t off = 0;
     // fp32 rows: as many as any batch of up to B sequences takes
     const int64_t rows = front_small_supported(c.dtype, 1, c.d_model, (int)S, c.n_experts, c.top_k)
-                             ? front_small_max_rows(B, c.top_k) : B;
+                             ? front_small_max_rows(B, c.d_model, c.top_k) : B;
     l.bc = off;  off += align_up((size_t)rows * S * sizeof(float));
     l.idx = off; off += align_up((size_t)B * c.top_k * sizeof(int32_t));
     l.w = off;   off += align_up((size_t)B * c.top_k * sizeof(float));

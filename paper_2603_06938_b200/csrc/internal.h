@@ -69,7 +69,7 @@ int launch_accumulate(LaunchCtx &ctx, int dtype, void *y, const void *y_add, int
 // in front of this call has completed, so it may read what earlier calls wrote before its own wait.
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
 bool front_small_slots(int64_t T, int k);
-int64_t front_small_max_rows(int64_t T, int k);     // rows of S streams that any call of up to T tokens takes
+int64_t front_small_max_rows(int64_t T, int F, int k);     // rows of S streams that any call of up to T tokens takes
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
                        int S, int E, int k, int sm_count, int32_t *idx, float *w, float *BC);
 // The same kernels for short calls of the forward: BC [T,S] bf16; scalars as in launch_router.
@@ -200,7 +200,7 @@ int launch_step_sequences(LaunchCtx &ctx, const void *x, const void *BC, const f
 // BC [B,bc_slots,S] is fp32 when bc_fp32, else bf16; the slots are summed.  early: what was
 // launched in front lets this kernel in only after the previous writer of the states has completed
 // (launch_front_small), so that they may be read before the dependency wait.
-int launch_decode_update(LaunchCtx &ctx, int dtype, const void *x, const void *BC, bool bc_fp32, int bc_slots, bool early,
+int launch_decode_update(LaunchCtx &ctx, int dtype, const void *x, void *BC, bool bc_fp32, int bc_slots, bool early,
                          const float *dt, const float *A, const float *dt_bias, const float *D,
                          float *state, int B, int H, int P, int N, int G, int sm_count, void *y);
 

@@ -1,6 +1,8 @@
 // The recurrence on the CUDA cores (selective-SSM equation with the channelwise convention; Theorem 1):
 // the chunked fp32 path of the forward, packed sequences of a few tokens stepped token by token, and K4,
 // the one-token decode update.
+#include <type_traits>
+
 #include "internal.h"
 #include "tc05.cuh"
 
@@ -370,7 +372,7 @@ __device__ __forceinline__ float4 load_bc4(const __nv_bfloat16 *p, int v)
                        __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
 }
 
-// MULTI: bc_slots rows of BC make up a sequence's mixed streams (summed in order; else one, mixed already).
+// A sequence's mixed streams are bc_slots rows of BC: MULTI, to be summed in order here; else the first one.
 // EARLY: small launches with rows of at most 128 entries, in which every warp has one piece of work and
 // its state rows are fetched before the dependency wait, under the projection (large ones run out of
 // registers that way: 92 -> 139 us at 128 sequences of 64 heads).
@@ -408,7 +410,7 @@ decode_update_kernel(const T *__restrict__ x, const TBC *__restrict__ BC,
         const float delta = softplus_f((dt ? dt[bh] : 0.f) + dt_bias[h]);
         const float a = expf(delta * A[h]);
         const float Dh = D ? D[h] : 0.f;
-        const TBC *Bp = BC + (int64_t)b * (MULTI ? bc_slots : 1) * S + g * N;
+        const TBC *Bp = BC + (int64_t)b * bc_slots * S + g * N;
         const TBC *Cp = Bp + G * N;
         float xv[DEC_ROWS], acc[DEC_ROWS];
 #pragma unroll
@@ -534,8 +536,26 @@ int launch_step_sequences(LaunchCtx &ctx, const void *x, const void *BC, const f
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
+// The first row of every sequence's k rows becomes their sum, in order.
+__global__ void __launch_bounds__(256)
+sum_slots_kernel(float *__restrict__ BC, int64_t T, int S, int k)
+{
+    grid_dep_launch();
+    grid_dep_wait();
+    const int vpr = S >> 2;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= T * vpr) return;
+    float4 *p = reinterpret_cast<float4 *>(BC) + (i / vpr) * k * vpr + i % vpr;
+    float4 sum = p[0];
+    for (int j = 1; j < k; ++j) {
+        const float4 v = p[(int64_t)j * vpr];
+        sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+    }
+    p[0] = sum;
+}
+
 template <typename T, typename TBC>
-static int launch_decode_t(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
+static int launch_decode_t(LaunchCtx &ctx, const void *x, void *BC, const float *dt, const float *A,
                            const float *dt_bias, const float *D, float *state, int B, int H, int P, int N, int G,
                            int bc_slots, bool early, int sm_count, void *y)
 {
@@ -546,7 +566,21 @@ static int launch_decode_t(LaunchCtx &ctx, const void *x, const void *BC, const 
     // one piece of work per warp, and all of them resident (two blocks of 256 threads per SM)
     early = early && N <= 128 && blocks <= 2 * (int64_t)sm_count;
     if (blocks > cap) blocks = cap;
-    auto kern = bc_slots == 1 ? (early ? decode_update_kernel<T, TBC, false, true> : decode_update_kernel<T, TBC, false, false>)
+    // Every warp of a sequence would sum its rows again, H ceil(P / 8) of them.  Where that reads more than a
+    // launch costs (20 MB out of L2; 5 or 80 MB in the rule are 1 and 2 % slower over 435 calls), a kernel of
+    // its own sums them once: 256 sequences of 64 heads, 16 experts, k = 8, F = 1024 283 us, now 205.
+    bool multi = bc_slots > 1;
+    if constexpr (std::is_same<TBC, float>::value) {
+        if (multi && nwork * (bc_slots - 1) * 2 * N * (int64_t)sizeof(float) > 20 << 20) {
+            const int S = 2 * G * N;
+            ctx.begin(STAGE_SLOT_SUM);
+            launch_kernel(sum_slots_kernel, dim3((unsigned)ceil_div64((int64_t)B * (S / 4), 256)), dim3(256), 0, ctx.stream,
+                          true, (float *)BC, (int64_t)B, S, bc_slots);
+            ctx.end();
+            multi = false;
+        }
+    }
+    auto kern = !multi ? (early ? decode_update_kernel<T, TBC, false, true> : decode_update_kernel<T, TBC, false, false>)
                               : (early ? decode_update_kernel<T, TBC, true, true> : decode_update_kernel<T, TBC, true, false>);
     ctx.begin(STAGE_DECODE_UPDATE);
     launch_kernel(kern, dim3((unsigned)blocks), dim3(warps * 32), 0, ctx.stream, true, (const T *)x, (const TBC *)BC, dt, A, dt_bias, D, state, B, H, P, N,
@@ -555,7 +589,7 @@ static int launch_decode_t(LaunchCtx &ctx, const void *x, const void *BC, const 
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
-int launch_decode_update(LaunchCtx &ctx, int dtype, const void *x, const void *BC, bool bc_fp32, int bc_slots, bool early,
+int launch_decode_update(LaunchCtx &ctx, int dtype, const void *x, void *BC, bool bc_fp32, int bc_slots, bool early,
                          const float *dt, const float *A, const float *dt_bias, const float *D,
                          float *state, int B, int H, int P, int N, int G, int sm_count, void *y)
 {

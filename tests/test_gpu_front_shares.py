@@ -10,8 +10,11 @@ import test_gpu_decode_front as front
 pytestmark = pytest.mark.gpu
 
 
+# shares; slots summed in the update and by their own kernel; sizes around the grouped product's (with 32 features
+# the projection that takes over has fp32 streams as well, which the tolerance is for)
 @pytest.mark.parametrize("B,F,H,P,N,E,k", [(256, 96, 1, 16, 16, 2, 2), (97, 64, 1, 16, 16, 2, 1), (50, 64, 1, 16, 16, 3, 2),
-                                           (255, 64, 1, 16, 16, 1, 1)])
+                                           (255, 64, 1, 16, 16, 1, 1), (130, 64, 3, 64, 128, 8, 8), (256, 64, 3, 64, 128, 16, 5),
+                                           (160, 32, 1, 16, 16, 8, 8), (161, 32, 1, 16, 16, 8, 8)])
 def test_decode_step(B, F, H, P, N, E, k):
     front.test_two_decode_steps_match_oracle(B, F, H, P, N, 1, E, k)
 
