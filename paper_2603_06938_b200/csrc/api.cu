@@ -478,7 +478,7 @@ int dense_linear(swimba_handle *h, LaunchCtx &ctx, const void *in, const void *W
                  void *out, char *scratch)
 {
     const int dtype = h->cfg.dtype;
-    if (dtype == SWIMBA_DTYPE_BF16 && pair_gemm_usable(T, Fi, So, h->sm_count)) {
+    if (dtype == SWIMBA_DTYPE_BF16 && pair_gemm_usable(T, Fi, So, 1, h->sm_count)) {
         const int rc = launch_pair_gemm(ctx, in, W, nullptr, nullptr, nullptr, T, Fi, So, 1, 1, false, h->sm_count, out, So);
         return rc == SWIMBA_OK ? rc : fail(h, rc, "linear map launch failed");
     }
@@ -572,7 +572,7 @@ int swimba_block_forward(swimba_handle *h, const swimba_weights *w, const swimba
     int32_t *idx = topk_idx ? topk_idx : (int32_t *)(fws + fl.idx);
     float *wt = topk_w ? topk_w : (float *)(fws + fl.w);
     // shared in-projection: [z | x'] (2 D columns) and the raw step sizes (H columns)
-    if (c.dtype == SWIMBA_DTYPE_BF16 && pair_gemm_usable(T, F, 2 * D, h->sm_count) && D % 16 == 0) {
+    if (c.dtype == SWIMBA_DTYPE_BF16 && pair_gemm_usable(T, F, 2 * D, 1, h->sm_count) && D % 16 == 0) {
         // one product over all 2D + H rows of W_in; the step sizes leave its epilogue as fp32 (a product of
         // their own read u again: 39 us at 32768 x 2048, and 13 us for the conversion)
         rc = launch_pair_gemm(ctx, u, bw->W_in, nullptr, nullptr, nullptr, T, F, 2 * D + H, 1, 1, false, h->sm_count,

@@ -40,7 +40,7 @@ int launch_mix_slots(LaunchCtx &ctx, const void *slots, const float *w, int64_t 
 // The same products on CTA pairs, 256 x 256 tiles, persistent: calls with enough tiles (pair_gemm_usable).
 // perm == NULL: the T rows of A as they lie (E = k = 1, no weights); out rows are ld_out elements apart.
 // tail (dense rows only): columns tail_col .. S-1 (tail_col % 32 == 0) go there as fp32, [T, S - tail_col].
-bool pair_gemm_usable(int64_t rows, int F, int S, int sm_count);
+bool pair_gemm_usable(int64_t rows, int F, int S, int E, int sm_count);
 int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *perm, const int *counts,
                      const float *w_slot, int64_t T, int F, int S, int E, int k, bool add_rows, int sm_count,
                      void *out, int64_t ld_out, float *tail = nullptr, int tail_col = 0);

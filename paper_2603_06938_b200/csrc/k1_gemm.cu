@@ -354,7 +354,7 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
         : (__nv_bfloat16 *)BC;
 
     const bool mix = k > 1 && !add_rows && !slots_out;      // the slots were stored and are summed afterwards
-    if (pair_gemm_usable(T * k, F, S, sm_count)) {
+    if (pair_gemm_usable(T * k, F, S, E, sm_count)) {
         const int rc = launch_pair_gemm(ctx, u, W_e, perm, counts, w, T, F, S, E, k, add_rows != 0, sm_count, slots, S);
         if (rc != SWIMBA_OK || !mix) return rc;
         return launch_mix_slots(ctx, slots, nullptr, T, S, k, sm_count, BC);

@@ -374,13 +374,28 @@ int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *pe
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
-// Calls that take the pair kernel: eight 256 x 256 tiles or more.  Below that the narrow column tiles of
-// expert_gemm_kernel spread the weight rows over more SMs.  Measured (F = 2048, S = 256, E = 8, k = 2, us
-// with about 5 us of event overhead): 300 tokens 18.9 narrow / 21.0 pairs, 1024 tokens 21.0 / 21.0, 4096
-// tokens 23.0 / 21.0, 16384 tokens 47.5 / 33.2; F = 768: 12.8 / 14.8, 14.8 / 14.8, 16.9 / 14.8, 27.1 / 18.9.
-bool pair_gemm_usable(int64_t rows, int F, int S, int sm_count)
+// Calls that take the pair kernel: eight full 256 x 256 tiles or more, except grouped rows that the narrow column
+// tiles of expert_gemm_kernel spread over more SMs (it can narrow them while all its tiles fit half of the SMs)
+// when there is little to gain: short products, or lists that fill one 128-row half of a tile.  Measured (router,
+// lists and product, S = 256, us, narrow / pairs):
+//             F = 512       F = 768       F = 1024      F = 2048
+//   E = 4      8 tiles  14.3 / 16.4   16.4 / 17.2   18.5 / 18.5   26.7 / 24.7
+//             17        14.6 / 16.4   17.4 / 18.2   19.6 / 18.6   26.6 / 26.6
+//   E = 8     13        16.4 / 16.4   18.4 / 18.4   20.5 / 20.5   28.8 / 26.6
+//   E = 16     8        15.4 / 17.8   17.9 / 19.5   20.5 / 22.2   32.8 / 30.8
+//             13        18.4 / 18.4   20.5 / 20.0   22.6 / 22.5   34.8 / 31.0
+//   E = 32     9        18.0 / 18.5   20.5 / 22.5   24.6 / 25.2   37.9 / 38.7
+//             13        18.4 / 19.3   20.5 / 22.5   24.7 / 26.6   37.0 / 38.9
+//             17        18.5 / 19.4   22.5 / 22.5   26.6 / 26.6   40.1 / 38.9
+//   E = 64     9        22.6 / 24.6   28.7 / 30.1   33.0 / 35.0   55.1 / 55.5
+//             11        26.6 / 24.6   32.8 / 30.0   39.0 / 34.9   65.8 / 55.9
+bool pair_gemm_usable(int64_t rows, int F, int S, int E, int sm_count)
 {
-    return sm_count >= 2 && F >= 64 && F % 8 == 0 && S % 8 == 0 && ceil_div64(rows, PG_BM) * ceil_div(S, PG_BN) >= 8;
+    const int cols = ceil_div(S, PG_BN);
+    const int64_t row_tiles = ceil_div64(rows, PG_BM);
+    if (sm_count < 2 || F < 64 || F % 8 != 0 || S % 8 != 0 || row_tiles * cols < 8) return false;
+    if (E == 1 || 2 * (row_tiles + E) * cols > sm_count) return true;
+    return F < 1024 ? row_tiles * cols >= 32 : E <= (F < 2048 ? 8 : 16) || rows > 120 * (int64_t)E;
 }
 
 }  // namespace swimba
