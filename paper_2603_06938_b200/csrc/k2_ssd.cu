@@ -1186,7 +1186,8 @@ static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 // Segment length (tokens, multiple of 128); L itself if one segment per sequence is best.  Costs in units of
 // a full tile of a head pair (3.3 us), from a sweep of lengths 400..32768 at 12..128 (sequence, head) pairs:
 // a segment's full pass takes its tiles plus 1.2, the state-only pass 0.35 a tile plus 1.2 (four heads per
-// CTA), the scan 1 and 0.005 per head and segment (128 KB moved).  Whole rounds of CTAs count.  Of the
+// CTA), the scan 1 and 0.005 per head and segment (128 KB moved), or 0.05 per segment where few heads leave it
+// bound by its chain (one head, 16000 tokens: 49 us in 125 segments, 43 in 63).  Whole rounds of CTAs count.  Of the
 // lengths tried the one picked was the best or within 2 % of it; filling two CTAs per SM whatever it costs
 // took 72 us instead of 66 at 24 heads and 8192 tokens.
 // No more segments than SEG_ROUNDS rounds of CTAs, or than segments of SEG_TILES tiles make: the costs pick
@@ -1209,7 +1210,7 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
         if (nseg > most) continue;
         const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 1.2f) +
                            (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.35f * st + 1.2f) + 1.f +
-                           (float)((nseg - 1) * B * H) * 0.005f;
+                           (float)(nseg - 1) * std::max(0.005f * B * H, 0.05f);
         if (cost < best_cost) { best_cost = cost; best = st; }
     }
     return best * ST;
