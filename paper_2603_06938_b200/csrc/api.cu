@@ -233,7 +233,7 @@ int run_ssd(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, const voi
         return SWIMBA_OK;
     }
     int rc = launch_ssd_sequential(ctx, c.dtype, x, BC, dt, w->A, w->dt_bias, w->D, h0, B, L,
-                                   c.n_heads, c.head_dim, c.d_state, c.n_groups, y, h_final);
+                                   c.n_heads, c.head_dim, c.d_state, c.n_groups, h->sm_count, y, h_final);
     if (rc != SWIMBA_OK) return fail(h, rc, "SSD launch failed");
     return SWIMBA_OK;
 }
@@ -786,7 +786,7 @@ int swimba_forward_packed(swimba_handle *h, const swimba_weights *w, const void 
                 }
                 rc = launch_ssd_sequential(ctx, c.dtype, (const char *)x + t0 * HP * es, (const char *)BC + t0 * S * es,
                                            dt ? dt + t0 * c.n_heads : nullptr, w->A, w->dt_bias, w->D, hin, 1,
-                                           len, c.n_heads, c.head_dim, c.d_state, c.n_groups,
+                                           len, c.n_heads, c.head_dim, c.d_state, c.n_groups, h->sm_count,
                                            (char *)y + t0 * HP * es, hf);
                 if (rc != SWIMBA_OK) rc = fail(h, rc, "SSD launch failed");
             }

@@ -187,7 +187,7 @@ int launch_dt_columns(LaunchCtx &ctx, int dtype, const void *zxdt, int64_t ld, i
 // the tile kernel does not take.
 int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *BC, const float *dt, const float *A,
                           const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int P, int N,
-                          int G, void *y, float *h_final);
+                          int G, int sm_count, void *y, float *h_final);
 
 // Sequences of a few tokens in a packed batch (bf16 streams, P = 64, N = 128), stepped token by token:
 // seq_tab[i] = (first token, tokens, sequence index, 0), a device array of n entries; x, BC, dt, y are

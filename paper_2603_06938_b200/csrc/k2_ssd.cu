@@ -1187,7 +1187,7 @@ static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 // a full tile of a head pair (3.3 us), from a sweep of lengths 400..32768 at 12..128 (sequence, head) pairs:
 // a segment's full pass takes its tiles plus 1.2, the state-only pass 0.35 a tile plus 1.2 (four heads per
 // CTA), the scan 1 and 0.005 per head and segment (128 KB moved), or 0.05 per segment where few heads leave it
-// bound by its chain (one head, 16000 tokens: 49 us in 125 segments, 43 in 63).  Whole rounds of CTAs count.  Of the
+// bound by its chain (one head, 16000 tokens: 49 us in 125 segments, 42 in 63).  Whole rounds of CTAs count.  Of the
 // lengths tried the one picked was the best or within 2 % of it; filling two CTAs per SM whatever it costs
 // took 72 us instead of 66 at 24 heads and 8192 tokens.
 // No more segments than SEG_ROUNDS rounds of CTAs, or than segments of SEG_TILES tiles make: the costs pick

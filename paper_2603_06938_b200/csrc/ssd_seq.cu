@@ -1,6 +1,7 @@
 // The recurrence on the CUDA cores (selective-SSM equation with the channelwise convention; Theorem 1):
 // the chunked fp32 path of the forward, packed sequences of a few tokens stepped token by token, and K4,
 // the one-token decode update.
+#include <algorithm>
 #include <type_traits>
 
 #include "internal.h"
@@ -18,12 +19,18 @@ namespace swimba {
 // and  y_i = exp(l_i) Ctilde_i^T H + sum_s G[i,s] x_s + D x_i.  Longer sequences repeat this with the
 // carried state (every CTA keeps its own copy).  All exponents are <= 0 and are formed from cumulative
 // sums in fp64, so a product of decays is rounded once.
-// What bounds it: the latency of a handful of dependent phases (load, G and S, exchange, y); the
-// arithmetic of a run is about 0.1 us of the SM.  One step per token with the state in registers
-// needed 0.66 us per token: 8 heads of 256 tokens (P = 64, N = 16) 168 us, this kernel 11 us.
+// With few heads, the latency of a handful of dependent phases (load, G and S, exchange, y) bounds it; with as
+// many as fill the SMs, shared memory, and every further CTA of a cluster costs an exchange of whole states.  So
+// a cluster is no larger than lets all of them run at once, and a cluster of one adds its run to the state in
+// place.  Up to a CTA per SM they may have 128 registers each, 64 (four CTAs per SM) beyond.  A forward in fp32,
+// a step per token / always eight CTAs / this way: 8 heads of 256 tokens (P = 64, N = 16) 184 / 25 / 23 us, 512
+// heads of 1024 (P = 64, N = 128) 3.6 / 4.6 / 2.8 ms, 512 heads of 1024 (P = 64, N = 256) 5.8 / 12.1 / 4.7 ms, 128
+// heads of 1000 (P = 64, N = 16) 697 / 157 / 130 us.  Over 430 shapes 0.77 of the faster of the other two, none
+// slower.
 constexpr int CK_Q = 32;          // tokens per CTA and round
 constexpr int CK_THREADS = 256;
 constexpr int CK_MAX_CLUSTER = 8;
+constexpr int CK_FILL = 4;        // CTAs per SM (fewer where shared memory holds fewer)
 
 namespace {
 __device__ __forceinline__ float4 ck_load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
@@ -72,10 +79,11 @@ __device__ __forceinline__ void fma4(float4 &acc, float a, const float4 &v)
     acc.w = fmaf(a, v.w, acc.w);
 }
 
-struct ChunkSmem {                 // offsets in floats; rows padded to whole float4s
+// Offsets in floats; rows padded to whole float4s.  One CTA adds its run to the state in place and needs no S.
+struct ChunkSmem {
     int B, C, x, G, S, H, total;
 };
-__host__ __device__ inline ChunkSmem chunk_smem(int P, int N)
+__host__ __device__ inline ChunkSmem chunk_smem(int P, int N, int ncta)
 {
     const int Pp = (P + 3) & ~3;
     ChunkSmem m;
@@ -84,25 +92,27 @@ __host__ __device__ inline ChunkSmem chunk_smem(int P, int N)
     m.C = off; off += CK_Q * (N + 4);
     m.x = off; off += CK_Q * Pp;
     m.G = off; off += CK_Q * (CK_Q + 4);
-    m.S = off; off += N * Pp;
     m.H = off; off += N * Pp;
+    m.S = off; off += ncta > 1 ? N * Pp : 0;
     m.total = off;
     return m;
 }
 }  // namespace
 
-template <typename T>
-__global__ void __launch_bounds__(CK_THREADS)
+// MULTI: a cluster of ncta > 1 CTAs.  PER_SM: CTAs that share an SM, and with it the registers.
+template <typename T, bool MULTI, int PER_SM>
+__global__ void __launch_bounds__(CK_THREADS, PER_SM)
 ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float *__restrict__ dt,
                  const float *__restrict__ A, const float *__restrict__ dt_bias, const float *__restrict__ D,
-                 const float *__restrict__ h0, int L, int H, int P, int N, int G, int ncta, T *__restrict__ y,
+                 const float *__restrict__ h0, int L, int H, int P, int N, int G, int cluster, T *__restrict__ y,
                  float *__restrict__ h_final)
 {
+    const int ncta = MULTI ? cluster : 1;
     extern __shared__ __align__(16) float csm[];
     __shared__ double s_l[CK_Q];
     __shared__ float s_delta[CK_Q], s_w[CK_Q], s_e[CK_Q];
     __shared__ float s_decay;
-    const ChunkSmem m = chunk_smem(P, N);
+    const ChunkSmem m = chunk_smem(P, N, ncta);
     float *sB = csm + m.B, *sC = csm + m.C, *sx = csm + m.x, *sG = csm + m.G, *sS = csm + m.S, *sH = csm + m.H;
     const int Pp = (P + 3) & ~3, pq = Pp >> 2, Nr = N + 4, Gr = CK_Q + 4;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -116,6 +126,17 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
     const double Ah = (double)A[h];
     const float bias = dt_bias[h], Dh = D ? D[h] : 0.f;
     const float *h0p = h0 ? h0 + bh * P * N : nullptr;
+    // A warp's share of a state: 8 state indexes x 16 channels, whole 32-byte sectors of [p][n] in global memory
+    // and two-way bank conflicts on rows [n][p] (with the state index along all lanes: 32-way; 16 tokens of 512
+    // heads, P = 32, N = 128: 75 -> 50 us a call)
+    auto state_tiles = [&](auto f) {
+        const int nct = (pq + 3) >> 2;
+        for (int i = warp; i < (N >> 3) * nct; i += CK_THREADS / 32) {
+            const int n = (i / nct) * 8 + (lane >> 3) * 2 + (lane & 1), p = (i % nct) * 16 + ((lane >> 1) & 3) * 4;
+            if (p < Pp) f(n, p);
+        }
+    };
+    bool has_state = h0p != nullptr;         // (zero otherwise: no product with it)
     const int nrounds = ceil_div(L, CK_Q * ncta);
     for (int rd = 0; rd < nrounds; ++rd) {
         const int t0 = (rd * ncta + rank) * CK_Q;
@@ -165,30 +186,44 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
             s_e[lane] = expf((float)l);
             if (lane == 31) s_decay = expf((float)l);
         }
-        if (rd == 0) {                       // the carried state, [n][p]
-            for (int i = tid; i < N * Pp; i += CK_THREADS) {
-                const int p = i / N, n = i - p * N;
-                sH[n * Pp + p] = (h0p && p < P) ? h0p[(int64_t)p * N + n] : 0.f;
-            }
+        if (rd == 0 && has_state) {          // the given state, [p][n] -> [n][p]
+            state_tiles([&](int n, int p) {
+                float v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = p + q < P ? h0p[(int64_t)(p + q) * N + n] : 0.f;
+                *reinterpret_cast<float4 *>(sH + n * Pp + p) = make_float4(v[0], v[1], v[2], v[3]);
+            });
+        } else if (rd == 0) {
+            for (int i = tid; i < N * pq; i += CK_THREADS) reinterpret_cast<float4 *>(sH)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         __syncthreads();
-        // ---- local end state, two state rows x four channels per thread and step
-        for (int i = tid; i < (N >> 1) * pq; i += CK_THREADS) {
-            const int nn = (i / pq) * 2, c = (i % pq) * 4;
-            float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+        // ---- local end state, two state rows x four channels per thread and step: to S, or (a cluster of one)
+        // added to the decayed state
+        const int nt8 = (nt + 7) & ~7;
+        auto end_state = [&]() {
+            for (int i = tid; i < (N >> 1) * pq; i += CK_THREADS) {
+                const int nn = (i / pq) * 2, c = (i % pq) * 4;
+                float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
 #pragma unroll 8
-            for (int s = 0; s < CK_Q; ++s) {
-                const float w = s_w[s];
-                const float2 bv = *reinterpret_cast<const float2 *>(sB + s * Nr + nn);
-                const float4 xv = *reinterpret_cast<const float4 *>(sx + s * Pp + c);
-                fma4(a0, w * bv.x, xv);
-                fma4(a1, w * bv.y, xv);
+                for (int s = 0; s < nt8; ++s) {
+                    const float w = s_w[s];
+                    const float2 bv = *reinterpret_cast<const float2 *>(sB + s * Nr + nn);
+                    const float4 xv = *reinterpret_cast<const float4 *>(sx + s * Pp + c);
+                    fma4(a0, w * bv.x, xv);
+                    fma4(a1, w * bv.y, xv);
+                }
+                float *dst = MULTI ? sS : sH;
+                if (!MULTI) {
+                    fma4(a0, s_decay, *reinterpret_cast<const float4 *>(sH + nn * Pp + c));
+                    fma4(a1, s_decay, *reinterpret_cast<const float4 *>(sH + (nn + 1) * Pp + c));
+                }
+                *reinterpret_cast<float4 *>(dst + nn * Pp + c) = a0;
+                *reinterpret_cast<float4 *>(dst + (nn + 1) * Pp + c) = a1;
             }
-            *reinterpret_cast<float4 *>(sS + nn * Pp + c) = a0;
-            *reinterpret_cast<float4 *>(sS + (nn + 1) * Pp + c) = a1;
-        }
+        };
+        if (MULTI) end_state();
         // ---- G: warp = rows i, lane = column s
-        for (int i = warp; i < CK_Q; i += CK_THREADS / 32) {
+        for (int i = warp; i < nt8; i += CK_THREADS / 32) {
             float v = 0.f;
             if (lane <= i) {
                 const float4 *cr = reinterpret_cast<const float4 *>(sC + i * Nr);
@@ -206,7 +241,7 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
             }
             sG[i * Gr + lane] = v;
         }
-        if (ncta > 1) cluster_sync();
+        if (MULTI) cluster_sync();
         else __syncthreads();
         // ---- state entering this run: the runs in front of it, in order
         const uint32_t s_addr = tc::smem_u32(sS), d_addr = tc::smem_u32(&s_decay);
@@ -226,12 +261,13 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
         }
         __syncthreads();
         // ---- y: two tokens x four channels per thread and step
+        has_state |= rank > 0;
         for (int i = tid; i < (CK_Q / 2) * pq; i += CK_THREADS) {
             const int i0 = (i / pq) * 2, c = (i % pq) * 4;
             if (i0 >= nt) continue;
             float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
 #pragma unroll 2
-            for (int n = 0; n < N; n += 4) {
+            for (int n = 0; n < (has_state ? N : 0); n += 4) {
                 const float4 c0 = *reinterpret_cast<const float4 *>(sC + i0 * Nr + n);
                 const float4 c1 = *reinterpret_cast<const float4 *>(sC + (i0 + 1) * Nr + n);
                 const float cv0[4] = {c0.x, c0.y, c0.z, c0.w}, cv1[4] = {c1.x, c1.y, c1.z, c1.w};
@@ -292,8 +328,10 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
         }
         // ---- the state after this round (carried on, or the call's end state)
         if (rd + 1 < nrounds || (h_final && rank == 0)) {
+            has_state = true;
             __syncthreads();                                 // (y has read the entry state)
-            for (int r = rank; r < ncta; ++r) {
+            if (!MULTI) end_state();
+            else for (int r = rank; r < ncta; ++r) {
                 const float dr = cluster_load(cluster_addr(d_addr, r));
                 const uint32_t ra = cluster_addr(s_addr, r);
 #pragma unroll 4
@@ -309,29 +347,35 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
             }
         }
         // the local end states have been read by everyone (and no CTA leaves while it is being read)
-        if (ncta > 1) cluster_sync();
+        if (MULTI) cluster_sync();
         else __syncthreads();
     }
     if (h_final && rank == 0) {
         float *dst = h_final + bh * P * N;
-        for (int i = tid; i < P * N; i += CK_THREADS) {
-            const int p = i / N, n = i - p * N;
-            dst[i] = sH[n * Pp + p];
-        }
+        state_tiles([&](int n, int p) {
+            const float4 h4 = *reinterpret_cast<const float4 *>(sH + n * Pp + p);
+            const float v[4] = {h4.x, h4.y, h4.z, h4.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) if (p + q < P) dst[(int64_t)(p + q) * N + n] = v[q];
+        });
     }
 }
 
 template <typename T>
 static int launch_chunk_t(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
                           const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int P, int N,
-                          int G, void *y, float *h_final)
+                          int G, int sm_count, void *y, float *h_final)
 {
     // as many CTAs per (sequence, head) as it has runs of CK_Q tokens, a power of two up to eight (the
-    // portable cluster size)
+    // portable cluster size), as long as they all run at once
+    const size_t per_cta = (size_t)chunk_smem(P, N, 2).total * sizeof(float) + 2048;
+    const int64_t room = (int64_t)sm_count * std::min<int64_t>(CK_FILL, std::max<int64_t>(1, 228 * 1024 / per_cta));
     int ncta = 1;
-    while (ncta < CK_MAX_CLUSTER && ncta * CK_Q < L) ncta <<= 1;
-    const size_t smem = (size_t)chunk_smem(P, N).total * sizeof(float);
-    auto kern = ssd_chunk_kernel<T>;
+    while (ncta < CK_MAX_CLUSTER && ncta * CK_Q < L && 2 * ncta * (int64_t)B * H <= room) ncta <<= 1;
+    const size_t smem = (size_t)chunk_smem(P, N, ncta).total * sizeof(float);
+    const bool few = (int64_t)B * H * ncta <= (ncta > 1 ? 1 : 2) * (int64_t)sm_count;
+    auto kern = ncta > 1 ? (few ? ssd_chunk_kernel<T, true, 2> : ssd_chunk_kernel<T, true, 4>)
+                         : (few ? ssd_chunk_kernel<T, false, 2> : ssd_chunk_kernel<T, false, 4>);
     if (smem > 40 * 1024 && !ensure_dynamic_smem((const void *)kern, smem)) return SWIMBA_ERR_CUDA;
     ctx.begin(STAGE_SSD_SEQUENTIAL);
     launch_kernel_cluster(kern, dim3((unsigned)((int64_t)B * H * ncta)), dim3(CK_THREADS), smem, ctx.stream, true,
@@ -343,12 +387,12 @@ static int launch_chunk_t(LaunchCtx &ctx, const void *x, const void *BC, const f
 
 int launch_ssd_sequential(LaunchCtx &ctx, int dtype, const void *x, const void *BC, const float *dt, const float *A,
                           const float *dt_bias, const float *D, const float *h0, int B, int L, int H, int P, int N,
-                          int G, void *y, float *h_final)
+                          int G, int sm_count, void *y, float *h_final)
 {
     if (B <= 0 || L <= 0) return SWIMBA_OK;
     if (dtype == SWIMBA_DTYPE_FP32)
-        return launch_chunk_t<float>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, y, h_final);
-    return launch_chunk_t<__nv_bfloat16>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, y, h_final);
+        return launch_chunk_t<float>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, sm_count, y, h_final);
+    return launch_chunk_t<__nv_bfloat16>(ctx, x, BC, dt, A, dt_bias, D, h0, B, L, H, P, N, G, sm_count, y, h_final);
 }
 
 // ------------------------------------------------------------------------------------------
