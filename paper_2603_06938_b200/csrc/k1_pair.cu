@@ -12,6 +12,8 @@
 // tile exposes its epilogue.  Measured: 65536 rows x 2048 features x 256 columns of 8 experts 96 -> 58 us
 // (1.19 PFLOP/s), 32768 x 2048 x 8192 dense 1190 -> 661 us (1.66 PFLOP/s).  Gathered rows come by
 // cp.async: tile::gather4 loads (512 bytes each with the 128-byte swizzle) took 150 us for the first shape.
+#include <algorithm>
+
 #include "internal.h"
 #include "pair.cuh"
 
@@ -374,28 +376,30 @@ int launch_pair_gemm(LaunchCtx &ctx, const void *A, const void *W, const int *pe
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
-// Calls that take the pair kernel: eight full 256 x 256 tiles or more, except grouped rows that the narrow column
-// tiles of expert_gemm_kernel spread over more SMs (it can narrow them while all its tiles fit half of the SMs)
-// when there is little to gain: short products, or lists that fill one 128-row half of a tile.  Measured (router,
-// lists and product, S = 256, us, narrow / pairs):
-//             F = 512       F = 768       F = 1024      F = 2048
-//   E = 4      8 tiles  14.3 / 16.4   16.4 / 17.2   18.5 / 18.5   26.7 / 24.7
-//             17        14.6 / 16.4   17.4 / 18.2   19.6 / 18.6   26.6 / 26.6
-//   E = 8     13        16.4 / 16.4   18.4 / 18.4   20.5 / 20.5   28.8 / 26.6
-//   E = 16     8        15.4 / 17.8   17.9 / 19.5   20.5 / 22.2   32.8 / 30.8
-//             13        18.4 / 18.4   20.5 / 20.0   22.6 / 22.5   34.8 / 31.0
-//   E = 32     9        18.0 / 18.5   20.5 / 22.5   24.6 / 25.2   37.9 / 38.7
-//             13        18.4 / 19.3   20.5 / 22.5   24.7 / 26.6   37.0 / 38.9
-//             17        18.5 / 19.4   22.5 / 22.5   26.6 / 26.6   40.1 / 38.9
-//   E = 64     9        22.6 / 24.6   28.7 / 30.1   33.0 / 35.0   55.1 / 55.5
-//             11        26.6 / 24.6   32.8 / 30.0   39.0 / 34.9   65.8 / 55.9
+// Calls that take the pair kernel: eight 256 x 256 tiles or more of rows as they lie.  Grouped rows also have the
+// narrow column tiles of expert_gemm_kernel, which it narrows further while all its tiles fit half of the SMs, and
+// whose products stop at 128 rows where a list does.  They keep: short products of few tiles; lists that fill half
+// a tile or less, unless one column of long products has few of them (all gain from fewer, longer steps) or they
+// are too many to be narrowed and the pairs hold them in one round (or short and more than two rounds of CTAs,
+// whose set-up the persistent pairs save).  Measured (router, lists and product, us, narrow
+// / pairs; rows are (token, expert) entries):
+//   S = 256    F = 512       F = 1024      F = 2048        S = 2048   F = 512       F = 1024      F = 2048
+//   E = 8      2050 rows  16.4 / 16.4   20.5 / 20.5   28.7 / 26.6   600 rows   19 / 21   24.5 / 26.7   33.5 / 41.1
+//              3200       16.4 / 16.4   20.6 / 20.5   29.3 / 26.6   1600       24.5 / 19.5  33.0 / 22.8  53.3 / 30.9
+//   E = 16     2050       16.4 / 18.4   20.5 / 22.2   33.0 / 31.0   600        22.2 / 24.9  29.0 / 34.2  51.9 / 60.9
+//   E = 32     3200       18.4 / 19.3   24.7 / 26.6   37.0 / 38.9
+//   E = 64     2600       26.6 / 24.6   39.0 / 34.9   65.8 / 55.9   600        58.4 / 54.1  65.6 / 66.6  113 / 117
+// Over 411 calls the line costs 0.2 % over picking the faster one every time.
 bool pair_gemm_usable(int64_t rows, int F, int S, int E, int sm_count)
 {
-    const int cols = ceil_div(S, PG_BN);
-    const int64_t row_tiles = ceil_div64(rows, PG_BM);
+    const int64_t cols = ceil_div(S, PG_BN), row_tiles = ceil_div64(rows, PG_BM);
     if (sm_count < 2 || F < 64 || F % 8 != 0 || S % 8 != 0 || row_tiles * cols < 8) return false;
-    if (E == 1 || 2 * (row_tiles + E) * cols > sm_count) return true;
-    return F < 1024 ? row_tiles * cols >= 32 : E <= (F < 2048 ? 8 : 16) || rows > 120 * (int64_t)E;
+    if (E == 1) return true;
+    if (rows > 120 * (int64_t)E) return F >= 1024 || row_tiles * cols >= 32;
+    if (cols == 1 && F >= 1024 && E <= (F < 2048 ? 8 : 16)) return true;
+    if (2 * (row_tiles + E) * cols <= sm_count) return false;
+    const int64_t tiles = std::max(row_tiles, std::min<int64_t>(E, rows)) * cols;
+    return tiles <= sm_count / 2 || (tiles > 2 * sm_count && F < 1024);
 }
 
 }  // namespace swimba
