@@ -62,7 +62,7 @@ FwdLayout fwd_layout(const swimba_config &c, int B, int L, int sm_count)
     return l;
 }
 
-// Workspace of a decode step: [BC (bf16 on the tensor-core path, else fp32) | idx | w | GEMM scratch].
+// Workspace of a decode step: [BC | idx | w | GEMM scratch].  BC: fp32, mixed or a row per slot, or bf16.
 struct DecLayout {
     size_t bc, idx, w, gemm, total;
 };
@@ -71,10 +71,8 @@ DecLayout dec_layout(const swimba_config &c, int B)
     DecLayout l;
     const size_t S = 2u * c.n_groups * c.d_state;
     size_t off = 0;
-    // fp32 rows: as many as any batch of up to B sequences takes
-    const int64_t rows = front_small_supported(c.dtype, 1, c.d_model, (int)S, c.n_experts, c.top_k)
-                             ? front_small_max_rows(B, c.d_model, c.top_k) : B;
-    l.bc = off;  off += align_up((size_t)rows * S * sizeof(float));
+    const bool slots = front_small_supported(c.dtype, 1, c.d_model, (int)S, c.n_experts, c.top_k);
+    l.bc = off;  off += align_up((size_t)B * (slots ? c.top_k : 1) * S * sizeof(float));
     l.idx = off; off += align_up((size_t)B * c.top_k * sizeof(int32_t));
     l.w = off;   off += align_up((size_t)B * c.top_k * sizeof(float));
     l.gemm = off;
@@ -219,6 +217,33 @@ int run_route_mix(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, con
                                  c.n_experts, c.top_k, BC, bc_fp32);
     if (rc != SWIMBA_OK) return fail(h, rc, "projection launch failed");
     return SWIMBA_OK;
+}
+
+// Router + projection without the mix: row t*k + j of slots (dtype, or fp32 with f32; then shapes of the tensor
+// cores only) is the projection of token t's j-th expert, weight applied.
+int run_slots(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, const void *u, int64_t T, int32_t *idx,
+              float *wt, void *slots, bool f32, void *gemm_ws)
+{
+    const swimba_config &c = h->cfg;
+    const int S = 2 * c.n_groups * c.d_state;
+    const void *Wr = w->W_router ? w->W_router : w->W_expert;
+    const bool tensor = use_tensor_k1(c);
+    int *counts = nullptr, *perm = nullptr;
+    if (tensor) {
+        counts = expert_gemm_counts(gemm_ws);
+        perm = expert_gemm_perm(gemm_ws);
+        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
+            return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
+    }
+    int rc = launch_router(ctx, c.dtype, u, Wr, T, c.d_model, c.n_experts, c.top_k, idx, wt, counts, perm, T, h->sm_count,
+                           nullptr, S * 2, ScalarsArgs{});
+    if (rc != SWIMBA_OK) return fail(h, rc, "router launch failed");
+    if (tensor)
+        rc = launch_expert_gemm(ctx, u, w->W_expert, wt, T, c.d_model, S, c.n_experts, c.top_k, h->sm_count, nullptr,
+                                gemm_ws, slots, f32);
+    else
+        rc = launch_project_slots_simt(ctx, c.dtype, u, w->W_expert, idx, wt, T, c.d_model, S, c.n_experts, c.top_k, slots);
+    return rc == SWIMBA_OK ? rc : fail(h, rc, "projection launch failed");
 }
 
 int run_ssd(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, const void *x,
@@ -369,26 +394,7 @@ int swimba_route_project_slots(swimba_handle *h, const swimba_weights *w, const 
     h->prof.n = 0;
     int32_t *idx = topk_idx ? topk_idx : (int32_t *)(ws + l.idx);
     float *wt = topk_w ? topk_w : (float *)(ws + l.w);
-    const int S = 2 * c.n_groups * c.d_state;
-    const void *Wr = w->W_router ? w->W_router : w->W_expert;
-    const bool tensor = use_tensor_k1(c);
-    int *counts = nullptr, *perm = nullptr;
-    if (tensor) {
-        counts = expert_gemm_counts(ws + l.gemm);
-        perm = expert_gemm_perm(ws + l.gemm);
-        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
-            return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
-    }
-    rc = launch_router(ctx, c.dtype, u, Wr, T, c.d_model, c.n_experts, c.top_k, idx, wt, counts, perm, T,
-                       h->sm_count, nullptr, S * 2, ScalarsArgs{});
-    if (rc != SWIMBA_OK) return fail(h, rc, "router launch failed");
-    if (tensor)
-        rc = launch_expert_gemm(ctx, u, w->W_expert, wt, T, c.d_model, S, c.n_experts, c.top_k, h->sm_count,
-                                nullptr, ws + l.gemm, BC_slots);
-    else
-        rc = launch_project_slots_simt(ctx, c.dtype, u, w->W_expert, idx, wt, T, c.d_model, S, c.n_experts,
-                                       c.top_k, BC_slots);
-    if (rc != SWIMBA_OK) fail(h, rc, "projection launch failed");
+    rc = run_slots(h, ctx, w, u, T, idx, wt, BC_slots, false, ws + l.gemm);
     h->last_stream = ctx.stream;
     h->last_launches = ctx.launches;
     return rc;
@@ -1039,22 +1045,26 @@ int swimba_decode_step(swimba_handle *h, const swimba_weights *w, const void *u,
     float *wt = topk_w ? topk_w : (float *)(ws + l.w);
     void *BC = ws + l.bc;
     const int S = 2 * c.n_groups * c.d_state;
-    // a handful of tokens: the small front end (fp32 streams); else bf16 streams from the
-    // grouped GEMM, or fp32 from the SIMT projection
-    const bool small = front_small_supported(c.dtype, B, c.d_model, S, c.n_experts, c.top_k);
-    const bool tensor = !small && use_tensor_k1(c);
+    // up to a few hundred tokens fp32 streams, from the small front end or (larger ones) from the grouped product as
+    // fp32 slots; else bf16 streams from the grouped product, or fp32 from the SIMT projection
+    const bool few = front_small_supported(c.dtype, B, c.d_model, S, c.n_experts, c.top_k);
+    const bool grouped = few && use_tensor_k1(c) && !front_small_faster(B, c.d_model, S, c.n_experts, c.top_k);
+    const bool small = few && !grouped, tensor = !few && use_tensor_k1(c);
+    const void *Wr = w->W_router ? w->W_router : w->W_expert;
     if (small) {
-        rc = launch_front_small(ctx, u, w->W_router ? w->W_router : w->W_expert, w->W_expert, B, c.d_model, S,
-                                c.n_experts, c.top_k, h->sm_count, idx, wt, (float *)BC);
+        rc = launch_front_small(ctx, u, Wr, w->W_expert, B, c.d_model, S, c.n_experts, c.top_k, h->sm_count, idx, wt,
+                                (float *)BC);
         if (rc != SWIMBA_OK) fail(h, rc, "routing / projection launch failed");
+    } else if (grouped) {
+        rc = run_slots(h, ctx, w, u, B, idx, wt, BC, true, ws + l.gemm);
     } else {
         rc = run_route_mix(h, ctx, w, u, B, BC, !tensor, idx, wt, tensor ? ws + l.gemm : nullptr);
     }
     if (rc == SWIMBA_OK) {
+        const bool slots = grouped || (small && front_small_slots(B, S, c.n_experts, c.top_k));
         // (the small front end starts the update behind the previous step's)
-        rc = launch_decode_update(ctx, c.dtype, x, BC, !tensor, small && front_small_slots(B, c.top_k) ? c.top_k : 1,
-                                  small, dt, w->A, w->dt_bias, w->D, state, B,
-                                  c.n_heads, c.head_dim, c.d_state, c.n_groups, h->sm_count, y);
+        rc = launch_decode_update(ctx, c.dtype, x, BC, !tensor, slots ? c.top_k : 1, small, dt, w->A, w->dt_bias, w->D, state,
+                                  B, c.n_heads, c.head_dim, c.d_state, c.n_groups, h->sm_count, y);
         if (rc != SWIMBA_OK) fail(h, rc, "decode launch failed");
     }
     h->last_stream = ctx.stream;

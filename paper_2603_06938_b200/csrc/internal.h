@@ -29,10 +29,11 @@ bool expert_gemm_adds_rows(int k);   // true: BC must be zero before launch_expe
 int *expert_gemm_counts(void *workspace);
 int *expert_gemm_perm(void *workspace);
 // slots_out (may be NULL): [T*k, S] bf16; when given, the projection of (token t, slot j), scaled by
-// its router weight (w NULL: 1), is stored in row t*k + j and nothing is mixed (BC is not touched).
+// its router weight (w NULL: 1), is stored in row t*k + j and nothing is mixed (BC is not touched); slots_f32: as
+// fp32 rows.
 int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const float *w, int64_t T,
                        int F, int S, int E, int k, int sm_count, void *BC, void *workspace,
-                       void *slots_out = nullptr);
+                       void *slots_out = nullptr, bool slots_f32 = false);
 
 // BC[t, :] = sum_j w[t,j] slots[t*k + j, :], bf16 (w NULL: 1).
 int launch_mix_slots(LaunchCtx &ctx, const void *slots, const float *w, int64_t T, int S, int k, int sm_count, void *BC);
@@ -67,9 +68,10 @@ int launch_accumulate(LaunchCtx &ctx, int dtype, void *y, const void *y_add, int
 // idx [T,k], w [T,k] and the fp32 streams BC are written: [T,S] mixed, or, where front_small_slots says so,
 // [T,k,S] per slot (weights applied), summed by the reader.  The kernel behind starts only after everything
 // in front of this call has completed, so it may read what earlier calls wrote before its own wait.
+// front_small_faster: whether it is, beside the router and the grouped product (with fp32 slots).
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
-bool front_small_slots(int64_t T, int k);
-int64_t front_small_max_rows(int64_t T, int F, int k);     // rows of S streams that any call of up to T tokens takes
+bool front_small_faster(int64_t T, int F, int S, int E, int k);
+bool front_small_slots(int64_t T, int S, int E, int k);
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
                        int S, int E, int k, int sm_count, int32_t *idx, float *w, float *BC);
 // The same kernels for short calls of the forward: BC [T,S] bf16; scalars as in launch_router.

@@ -28,13 +28,15 @@ __host__ __device__ constexpr int gm_stages(int BN) { return BN >= 256 ? 3 : 4; 
 // Grouped GEMM.  Warps 0-3: gather the A rows with cp.async, later the epilogue; warp 4: TMA
 // loads of the weight tile; warp 5: TMEM allocation and MMA issue.
 // ------------------------------------------------------------------------------------------
-template <int BN>
+// F32: the scaled rows leave as fp32, straight from the registers (out: float rows; never added).
+template <int BN, bool F32>
 __global__ void __launch_bounds__(GM_THREADS, 1)
 expert_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __nv_bfloat16 *__restrict__ u,
                    const int *__restrict__ perm, int64_t cap, const float *__restrict__ w_slot,
                    const int *__restrict__ counts, int E, int F, int S, int k, int add_rows,
-                   __nv_bfloat16 *__restrict__ out, int *d_status, int check)
+                   void *__restrict__ outv, int *d_status, int check)
 {
+    __nv_bfloat16 *out = reinterpret_cast<__nv_bfloat16 *>(outv);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int STAGES = gm_stages(BN);
     constexpr uint32_t A_BYTES = GM_BM * 128, B_BYTES = BN * 128;
@@ -190,15 +192,26 @@ expert_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __nv_bfloat
                 uint32_t v[32];
                 tc::tmem_ld32(tmem_base + ((uint32_t)(warp * 32) << 16) + hf * BN + c * 32, v);
                 tc::tmem_ld_wait();
-                uint32_t pk[16];
+                if constexpr (F32) {
+                    if (row < nrows && row_src[row] >= 0) {
+                        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(outv) +
+                                                                 (int64_t)row_dst[row] * S + n0 + c * 32);
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    pk[i] = tc::pack_bf16x2(wr * __uint_as_float(v[2 * i]),
-                                            wr * __uint_as_float(v[2 * i + 1]));
-                uint4 *dst = reinterpret_cast<uint4 *>(srow + c * 64);
+                        for (int i = 0; i < 8; ++i)
+                            dst[i] = make_float4(wr * __uint_as_float(v[4 * i]), wr * __uint_as_float(v[4 * i + 1]),
+                                                 wr * __uint_as_float(v[4 * i + 2]), wr * __uint_as_float(v[4 * i + 3]));
+                    }
+                } else {
+                    uint32_t pk[16];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    dst[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                    for (int i = 0; i < 16; ++i)
+                        pk[i] = tc::pack_bf16x2(wr * __uint_as_float(v[2 * i]),
+                                                wr * __uint_as_float(v[2 * i + 1]));
+                    uint4 *dst = reinterpret_cast<uint4 *>(srow + c * 64);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        dst[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                }
             }
             if (add_rows) {
                 tc::fence_proxy_async_smem();
@@ -211,7 +224,7 @@ expert_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __nv_bfloat
         __syncwarp();
         constexpr int LPR = BN / 8, RPI = 32 / LPR;      // lanes per row, rows per instruction
         const int sub = lane / LPR, piece = lane % LPR;
-        for (int hf = 0; hf < (add_rows ? 0 : nhalf); ++hf) {
+        for (int hf = 0; hf < (F32 || add_rows ? 0 : nhalf); ++hf) {
 #pragma unroll 4
             for (int r0 = 0; r0 < 32; r0 += RPI) {
                 const int row = hf * 128 + warp * 32 + r0 + sub;
@@ -340,7 +353,7 @@ int launch_mix_slots(LaunchCtx &ctx, const void *slots, const float *w, int64_t 
 
 int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const float *w, int64_t T,
                        int F, int S, int E, int k, int sm_count, void *BC, void *workspace,
-                       void *slots_out)
+                       void *slots_out, bool slots_f32)
 {
     if (T <= 0) return SWIMBA_OK;
     const int max_tiles = (int)ceil_div64(T * k, GM_BM) + E;
@@ -354,7 +367,7 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
         : (__nv_bfloat16 *)BC;
 
     const bool mix = k > 1 && !add_rows && !slots_out;      // the slots were stored and are summed afterwards
-    if (pair_gemm_usable(T * k, F, S, E, sm_count)) {
+    if (!slots_f32 && pair_gemm_usable(T * k, F, S, E, sm_count)) {
         const int rc = launch_pair_gemm(ctx, u, W_e, perm, counts, w, T, F, S, E, k, add_rows != 0, sm_count, slots, S);
         if (rc != SWIMBA_OK || !mix) return rc;
         return launch_mix_slots(ctx, slots, nullptr, T, S, k, sm_count, BC);
@@ -375,11 +388,11 @@ int launch_expert_gemm(LaunchCtx &ctx, const void *u, const void *W_e, const flo
     dim3 grid((unsigned)max_tiles, (unsigned)(S / BN));
 #define SWIMBA_GEMM_CASE(BNV)                                                                   \
     do {                                                                                        \
-        auto kern = expert_gemm_kernel<BNV>;                                                    \
+        auto kern = slots_f32 ? expert_gemm_kernel<BNV, true> : expert_gemm_kernel<BNV, false>; \
         if (!ensure_dynamic_smem((const void *)kern, smem)) return SWIMBA_ERR_CUDA;             \
         launch_kernel(kern, grid, dim3(GM_THREADS), smem, ctx.stream, true, tmap,               \
                       (const __nv_bfloat16 *)u, (const int *)perm, (int64_t)T, (const float *)w, \
-                      (const int *)counts, E, F, S, k, add_rows, slots, ctx.d_status,           \
+                      (const int *)counts, E, F, S, k, add_rows, (void *)slots, ctx.d_status,   \
                       ctx.check_indices ? 1 : 0);                                               \
     } while (0)
     ctx.begin(STAGE_EXPERT_GEMM);

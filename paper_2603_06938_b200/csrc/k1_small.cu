@@ -15,7 +15,7 @@
 //                         the mixed streams (Theorem 1).  With k <= 2 a row receives at most two
 //                         additions onto zero, so the sum does not depend on their order; with more
 //                         experts the rows go to slots (t, j), which the update sums in order.
-// At most SM_FUSED tokens: every CTA of the projection computes the few logits itself (the router
+// At most SM_FUSED tokens (and not too many CTAs): every CTA of the projection computes the few logits itself (the router
 // matrix and the tokens are in L2, and a dependent launch costs more than they do); the rows go to slots,
 // since no kernel in front could clear the mixed streams.  A decode step of one token, 64 heads, 8 experts,
 // F = 2048: router and projection apart 14.7 us, one kernel (and the states read under it) 8.5 us.
@@ -150,7 +150,7 @@ template <int ROWS, bool FUSED>
 __global__ void __launch_bounds__(256)
 project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r,
                      const __nv_bfloat16 *__restrict__ W_e, int32_t *__restrict__ idx, float *__restrict__ w, int Ttok,
-                     int F, int S, int E, int k, void *__restrict__ BCv, int check, int *d_status)
+                     int F, int S, int E, int k, int share, void *__restrict__ BCv, int check, int *d_status)
 {
     float *BC = reinterpret_cast<float *>(BCv);
     __shared__ int s_tok[SM_MAX_T], s_out[SM_MAX_T];
@@ -240,8 +240,8 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
     } else {
         // tokens of this CTA's share routed to its expert (a token picks an expert at most once); the order
         // of the list does not matter: every entry ends in its own output row
-        const int t_end = (int)((int64_t)Ttok * (blockIdx.z + 1) / gridDim.z) * k;
-        for (int i = (int)((int64_t)Ttok * blockIdx.z / gridDim.z) * k + tid; i < t_end; i += blockDim.x) {
+        const int t_beg = blockIdx.z * share, t_end = min(Ttok, t_beg + share);
+        for (int i = t_beg * k + tid; i < t_end * k; i += blockDim.x) {
             const int ei = idx[i];
             if (check && (ei < 0 || ei >= E)) atomicCAS(d_status, 0, SWIMBA_ERR_DEVICE_BOUNDS);
             if (ei == e) {
@@ -340,43 +340,42 @@ project_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *_
     }
 }
 
-// Entries that more than two experts per token may make: the grouped product takes over where its wide tiles
-// outweigh its lists.  A decode step of 16 heads, small / grouped: 16 experts, F = 1024, k = 8 128 sequences
-// 43 / 45 us, 170 58 / 55, 256 80 / 72; F = 2048, k = 8 256 sequences 83 / 86; 8 experts, F = 4096, k = 8
-// 213 sequences 88 / 92, 256 100 / 94.
-static int64_t front_small_entries(int F) { return F < 2048 ? 1280 : 1792; }
-
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k)
 {
-    return dtype == SWIMBA_DTYPE_BF16 && T <= SM_MAX_T && E <= SM_MAX_E && S % SM_ROWS == 0 && F % 32 == 0 &&
-           (k <= 2 || T * k <= front_small_entries(F));
+    return dtype == SWIMBA_DTYPE_BF16 && T <= SM_MAX_T && E <= SM_MAX_E && S % SM_ROWS == 0 && F % 32 == 0;
 }
 
-static bool front_small_fused(int64_t T) { return T <= SM_FUSED; }
-bool front_small_slots(int64_t T, int k) { return front_small_fused(T) || k > 2; }
-int64_t front_small_max_rows(int64_t T, int F, int k)
+// The cost here is CTAs with an active expert ((S / 16) of them each) and the 16 x 16 output tiles they work
+// through; the grouped product's is a chain along the features.  Measured over 1678 short forwards and decode steps
+// (5 to 256 tokens, 2 to 16 experts, k = 1 to 8, S = 256 to 4096, F = 64 to 4096): the line costs 0.1 % over
+// picking the faster one every time.  A forward of 8 experts, k = 2, S = 2048, F = 1024 (us, here / grouped): 8
+// tokens 28 / 31, 24 34 / 33, 120 51 / 35, 250 83 / 39; S = 512, 250 tokens 25 / 29.
+bool front_small_faster(int64_t T, int F, int S, int E, int k)
 {
-    // (more tokens may take fewer rows: slots up to SM_FUSED tokens, or for k > 2 as far as this front end goes)
-    const int64_t slots = k * std::min(T, k > 2 ? std::min<int64_t>(SM_MAX_T, front_small_entries(F) / k) : SM_FUSED);
-    return std::max(T, slots);
+    return (S / SM_ROWS) * (12 * std::min<int64_t>(E, T * k) + T * k) <= 27 * (int64_t)F + 4608;
 }
+
+// Every CTA of the fused form computes the logits: not for more than 512 of them (16 experts, k = 2, F = 2048,
+// one token: 512 CTAs 14.5 us fused, 1024 19.0 and 17.2 apart).
+static bool front_small_fused(int64_t T, int S, int E) { return T <= SM_FUSED && (S / SM_ROWS) * E <= 512; }
+bool front_small_slots(int64_t T, int S, int E, int k) { return front_small_fused(T, S, E) || k > 2; }
 
 // Shares the tokens of a projection are cut into (grid z; a CTA lists and works its share): sixteen entries of
 // an expert or more each, two CTAs per SM at most.  Few experts make few CTAs (32 with two experts), which
 // walked their lists 32 entries at a time: two experts, k = 2, F = 768, 256 tokens 34.0 us (the grouped
 // product: 16.4), in shares 13; four experts, k = 1, F = 2048, 128 tokens 10.5, in shares 9.  32 entries a
 // share are 5 % slower over 1083 calls, four CTAs per SM 3 %.
-static unsigned project_shares(int64_t T, int S, int E, int k, int sm_count)
+static int project_share(int64_t T, int S, int E, int k, int sm_count)       // tokens of one
 {
     const int64_t by_work = T * k / (16 * (int64_t)E), by_sms = 2 * (int64_t)sm_count / ((int64_t)(S / SM_ROWS) * E);
-    return (unsigned)std::max<int64_t>(1, std::min(by_work, by_sms));
+    return (int)ceil_div64(T, std::max<int64_t>(1, std::min(by_work, by_sms)));
 }
 
 int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F,
                        int S, int E, int k, int sm_count, int32_t *idx, float *w, float *BC)
 {
     if (T <= 0) return SWIMBA_OK;
-    const bool slots = front_small_slots(T, k), fused = front_small_fused(T);
+    const bool slots = front_small_slots(T, S, E, k), fused = front_small_fused(T, S, E);
     if (!fused) {
         ctx.begin(STAGE_ROUTER);
         launch_kernel(router_small_kernel, dim3((unsigned)ceil_div64(T, 2)), dim3(256), 0, ctx.stream, true,
@@ -385,11 +384,11 @@ int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const voi
         ctx.end();
     }
     ctx.begin(STAGE_PROJECT_SMALL);
+    const int share = fused ? (int)T : project_share(T, S, E, k, sm_count);
     auto kern = fused ? project_small_kernel<ROWS_SLOTS, true>
                       : slots ? project_small_kernel<ROWS_SLOTS, false> : project_small_kernel<ROWS_ADD, false>;
-    launch_kernel(kern, dim3((unsigned)(S / SM_ROWS), (unsigned)E, fused ? 1u : project_shares(T, S, E, k, sm_count)),
-                  dim3(256), 0, ctx.stream, true, (const __nv_bfloat16 *)u,
-                  (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F, S, E, k, (void *)BC,
+    launch_kernel(kern, dim3((unsigned)(S / SM_ROWS), (unsigned)E, (unsigned)ceil_div64(T, share)), dim3(256), 0,
+                  ctx.stream, true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F, S, E, k, share, (void *)BC,
                   ctx.check_indices ? 1 : 0, ctx.d_status);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
@@ -397,12 +396,10 @@ int launch_front_small(LaunchCtx &ctx, const void *u, const void *W_r, const voi
 
 // The forward's streams for short calls: no histogram to clear, no lists, no tiles.  One prompt of
 // 93 tokens, 24 heads, F = 768, one of four experts: 22.5 us a call through router, lists and grouped product,
-// 16.8 us this way (the first tile and the states fetched ahead of the wait included).  With few features the
-// grouped product has little to do and keeps its lead: sixteen experts, k = 2, F = 256, 192 tokens 14.4 us
-// this way, 12.3 there; F = 512, 256 tokens 15.1 and 14.4; F = 768 15.4 and 18.0.
+// 16.8 us this way (the first tile and the states fetched ahead of the wait included).
 bool front_short_supported(int dtype, int64_t T, int F, int S, int E, int k)
 {
-    return front_small_supported(dtype, T, F, S, E, k) && k <= 2 && E > 1 && T * k < F;
+    return front_small_supported(dtype, T, F, S, E, k) && k <= 2 && E > 1 && front_small_faster(T, F, S, E, k);
 }
 
 int launch_front_short(LaunchCtx &ctx, const void *u, const void *W_r, const void *W_e, int64_t T, int F, int S, int E,
@@ -414,11 +411,12 @@ int launch_front_short(LaunchCtx &ctx, const void *u, const void *W_r, const voi
                   ctx.stream, true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (int)T, F, E, k, idx, w,
                   (float4 *)BC, k == 1 ? 0 : S / 8, scalars);
     ctx.end();
+    const int share = project_share(T, S, E, k, sm_count);
     ctx.begin(STAGE_PROJECT_SMALL);
     launch_kernel(project_small_kernel<ROWS_BF16, false>,
-                  dim3((unsigned)(S / SM_ROWS), (unsigned)E, project_shares(T, S, E, k, sm_count)), dim3(256), 0, ctx.stream,
+                  dim3((unsigned)(S / SM_ROWS), (unsigned)E, (unsigned)ceil_div64(T, share)), dim3(256), 0, ctx.stream,
                   true, (const __nv_bfloat16 *)u, (const __nv_bfloat16 *)W_r, (const __nv_bfloat16 *)W_e, idx, w, (int)T, F,
-                  S, E, k, BC, ctx.check_indices ? 1 : 0, ctx.d_status);
+                  S, E, k, share, BC, ctx.check_indices ? 1 : 0, ctx.d_status);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
