@@ -6,6 +6,10 @@
 
 namespace swimba {
 
+// A logit for the choice of experts: NaN (which compares with nothing) and -inf (the mark of a taken expert) rank
+// last, so that a token never picks an expert twice and no expert's list outgrows the number of tokens.
+__device__ __forceinline__ float rankable(float g) { return fmaxf(g, -3.402823466e38f); }
+
 // Router: a block handles chunks of `chunk` consecutive tokens, one warp TPW tokens at a time;
 // the router matrix is staged in shared memory once per block (when it fits) so that every token
 // costs one pass over its own features.
@@ -150,6 +154,8 @@ router_topk_kernel(const T *__restrict__ u, const T *__restrict__ W_r, int64_t T
             }
             // k rounds of "largest remaining logit, lowest index on ties"; weights are NOT
             // renormalised
+#pragma unroll
+            for (int i = 0; i < R; ++i) if (e0 + i < E) gv[i] = rankable(gv[i]);
             for (int j = 0; j < k; ++j) {
                 float bg = gv[0], bp = pv[0];
                 int be = e0;
@@ -341,6 +347,8 @@ router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__re
             }
             // k rounds of "largest remaining logit, lowest index on ties"; weights are NOT
             // renormalised
+#pragma unroll
+            for (int i = 0; i < NT; ++i) if (sub + 8 * i < E) gv[i] = rankable(gv[i]);
             for (int j = 0; j < k; ++j) {
                 float bg = gv[0], bp = pv[0];
                 int be = sub;
@@ -582,6 +590,8 @@ router_stream_kernel(const __grid_constant__ CUtensorMap tmap_u, const __nv_bflo
             }
             // k rounds of "largest remaining logit, lowest index on ties"; weights are NOT
             // renormalised
+#pragma unroll
+            for (int i = 0; i < 2 * NT; ++i) if ((i >> 1) * 8 + 2 * c + (i & 1) < E) gv[i] = rankable(gv[i]);
             for (int j = 0; j < k; ++j) {
                 float bg = gv[0], bp = pv[0];
                 int be = 2 * c;
