@@ -37,9 +37,9 @@
 // every exponent being <= 0 (no overflow, underflow only where the true value underflows), so
 // that it costs two multiplications per entry.
 //
-// Long sequences with few (sequence, head) pairs are cut into segments: a first pass of this
-// kernel computes every segment's local end state (MMA 4 only), segment_scan_kernel (K3) chains
-// them, and a second pass evaluates each segment from its true incoming state.
+// Long sequences with few (sequence, head) pairs are cut into segments: ssd_state_kernel computes every
+// segment's local end state (MMA 4 only), segment_scan_kernel (K3) chains them, and this kernel evaluates each
+// segment from its true incoming state.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -74,8 +74,6 @@ constexpr uint32_t SM_SMALL = SM_HEAD + NHD * SM_HEAD_BYTES;
 constexpr uint32_t TM_G = 0, TM_HEAD = 0, TM_HEAD_COLS = 64, TM_COLS = 512;
 constexpr uint32_t TM_Y = 128, TM_DH = 256, TM_M = 384;
 
-enum { MODE_FULL = 0, MODE_STATE_ONLY = 1 };
-
 struct SeqDesc {            // one sequence of a packed batch
     int tok0, len;          // first token in the packed arrays, tokens
     int tile0, seg0;        // first 128-token tile / first segment of the sequence in the batch-wide lists
@@ -87,17 +85,17 @@ struct SsdParams {
     const float *D;
     const float *h_in;      // initial states: [B,H,P,N] (nseg == 1) or [B,nseg,H,P,N]; may be null
     const float *h_first;   // seg_states >= 2: states entering the first segments, [B,H,P,N]; may be null
-    float *h_out;           // MODE_FULL: h_final [B,H,P,N] (last segment writes) or null
-                            // MODE_STATE_ONLY: local end states [B,nseg,H,P,N]
-    float *seg_decay;       // MODE_STATE_ONLY: [B,nseg,H] product of a_t over the segment
-    int L, Lpad, H, G, nseg, seg_len, mode;
-    int split_tiles;        // > 0 (MODE_FULL, nseg == 1): every (sequence, head pair) is worked by two
-                            // CTAs, see ssd_tiles_kernel
+    float *h_out;           // ssd_tiles_kernel: h_final [B,H,P,N] (last segment writes) or null
+                            // ssd_state_kernel: local end states [B,nseg,H,P,N]
+    float *seg_decay;       // ssd_state_kernel: [B,nseg,H] product of a_t over the segment
+    int L, Lpad, H, G, nseg, seg_len;
+    int split_tiles;        // > 0 (nseg == 1): every (sequence, head pair) is worked by two CTAs, see
+                            // ssd_tiles_kernel
     int *d_status;
     // Packed batch (sequences of different lengths back to back in one [T, ...] array): seqs has one
     // entry per sequence plus a closing one, items lists the (sequence, segment) pairs of this launch
     // (grid.x), the scalar arrays are laid out [H, tiles of the batch], and the per-segment state
-    // arrays are indexed by seqs[b].seg0 + segment.  seg_states: h_in / state-only h_out are those
+    // arrays are indexed by seqs[b].seg0 + segment.  seg_states: h_in / ssd_state_kernel's h_out are those
     // per-segment arrays (else h_in is [sequences, H, P, N]); 2: a sequence's first segment starts from
     // h_first instead; 3: so does a sequence of one segment (in-place states: the first of several reads
     // the scan's copy, since the last one writes over h_first in the same launch).  y: base of the output (ragged last
@@ -211,7 +209,7 @@ __device__ __forceinline__ void scale_units(const uint8_t *s_x, uint8_t *s_xp, c
     }
 }
 
-// The same for the four units of the thread's own row (state-only tiles), with the row's weight
+// The same for the four units of the thread's own row (leading tiles), with the row's weight
 // multiplied by `f` first: w' = w f is split again into two bf16 terms.
 __device__ __forceinline__ void scale_own_row(const uint8_t *s_x, uint8_t *s_xp, uint32_t wp, float f, int i, int hf)
 {
@@ -293,8 +291,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
     const int t_begin = seg * prm.seg_len;
     const int t_end = head_part ? min(L, prm.split_tiles * ST) : min(L, t_begin + prm.seg_len);
     const int ntiles = (t_end - t_begin + ST - 1) / ST;
-    const bool kfull = prm.mode == MODE_FULL;
-    // leading tiles that only carry the state forward (tile j is a full tile iff kfull && j >= n_pre;
+    // leading tiles that only carry the state forward (tile j is a full tile iff j >= n_pre;
     // barriers that only full tiles use count their phases in full tiles, jf = j - n_pre)
     const int n_pre = split ? (head_part ? 0 : min(prm.split_tiles, ntiles)) : 0;
 
@@ -365,7 +362,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         }
         for (int j = 0; j < ntiles; ++j) {
             const int t0 = tok0 + t_begin + j * ST;
-            const bool full = SPLIT ? (kfull && j >= n_pre) : kfull;
+            const bool full = !SPLIT || j >= n_pre;
             tc::mbar_wait(&bars->cb_empty, (j & 1) ^ 1, abort_flag, d_status);
             if (leader) {
                 tc::mbar_arrive_expect_tx(&bars->cb_full, full ? 4 * SLAB : 2 * SLAB);
@@ -388,7 +385,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     }
                 }
                 // scalars of the next tile: the record buffer is single; its last readers are the
-                // mask (full pass) or the w.X scaling (state-only pass) of this tile
+                // mask (full tile) or the w.X scaling (leading tile) of this tile
                 for (int hd = 0; hd < nh; ++hd) {
                     HeadBars *hb = &bars->hd[hd];
                     if (full) tc::mbar_wait(&hb->m_full, (SPLIT ? j - n_pre : j) & 1, abort_flag, d_status);
@@ -446,10 +443,10 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 }
                 __syncwarp();
             };
-            if (hd == 0 && kfull && n_pre == 0 && ntiles > 0) issue_g(0);
+            if (hd == 0 && n_pre == 0 && ntiles > 0) issue_g(0);
             for (int j = 0; j < ntiles; ++j) {
                 const int sx = j & 1;
-                const bool full = SPLIT ? (kfull && j >= n_pre) : kfull;
+                const bool full = !SPLIT || j >= n_pre;
                 const int jf = SPLIT ? j - n_pre : j;
                 if (hd == 0) {
                     tc::mbar_wait(&bars->cb_full, j & 1, abort_flag, d_status);
@@ -478,7 +475,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     tc::tc_fence_after();
                     if (leader) {
 #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)     // (the tiles of a state-only run accumulate)
+                        for (int kk = 0; kk < 8; ++kk)     // (leading tiles accumulate)
                             tc::mma_ss(tmem_u + TM_DH, tc::smem_desc_advance(dBt, kk * 2048),
                                        tc::smem_desc_advance(dXp, kk * 2048), id_hn, (kk > 0) || (!full && j > 0));
                         for (int q = 0; q < nh; ++q) tc::mma_commit(&bars->hd[q].dh_full);
@@ -502,9 +499,9 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 }
                 // MMA 1 of the next tile needs no state: it runs under this tile's state update and
                 // epilogue, and the next tile's mask is built while MMA 3 is still waiting for them
-                if (hd == 0 && kfull && j + 1 < ntiles && j + 1 >= n_pre) issue_g(j + 1);
-                // (state-only pass: the second issuer has no product of its own; it follows the
-                // tile loop at the pace of its head's w.X scaling, whose end frees the X slot)
+                if (hd == 0 && j + 1 < ntiles && j + 1 >= n_pre) issue_g(j + 1);
+                // (leading tiles: the second issuer has no product of its own; it follows the tile loop at
+                // the pace of its head's w.X scaling, whose end frees the X slot)
                 if (!full && hd > 0) tc::mbar_wait(&hb->xp_full, j & 1, abort_flag, d_status);
                 if (leader) tc::mma_commit(&hb->x_free[sx]);
                 __syncwarp();
@@ -522,7 +519,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     __syncwarp();
                 }
             }
-            if (kfull && leader) tc::bulk_wait_read_all();
+            if (leader) tc::bulk_wait_read_all();
         }
     } else if ((uwarp >> 3) < nh) {
         // ------------------------------------------------------------------ compute warps
@@ -547,7 +544,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             // (states of earlier segments come from the scan in front; given ones go past L1)
             const bool wait = !prm.early || (prm.seg_states && !first);
             if (wait) grid_dep_wait();
-            if (h_in && kfull) {
+            if (h_in) {
                 const int64_t base = (prm.seg_states && !first)
                     ? ((((int64_t)seg_base + seg) * H + h) * SP) * SN
                     : (((int64_t)b * H + h) * SP) * SN;
@@ -559,7 +556,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
 #pragma unroll
                 for (int q = 0; q < 16; ++q) Hst[q] = 0;
             }
-            if (kfull && n_pre == 0) {
+            if (n_pre == 0) {
                 // bf16 copy of the state the first tile starts from
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
@@ -570,26 +567,22 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 tc::fence_proxy_async_smem();
                 tc::mbar_arrive(&hb->h_ready);
             }
-            if (kfull) {
-                // blocks of M above the diagonal stay zero for the whole kernel
-                uint32_t zero[8];
+            // blocks of M above the diagonal stay zero for the whole kernel
+            uint32_t zero[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) zero[q] = 0u;
-                for (int c = wq + 1; c < 4; ++c) tc::tmem_st8(tm + TM_M + c * 16 + 8 * hf, zero);
-                tc::tmem_st_wait();
-            }
+            for (int q = 0; q < 8; ++q) zero[q] = 0u;
+            for (int c = wq + 1; c < 4; ++c) tc::tmem_st8(tm + TM_M + c * 16 + 8 * hf, zero);
+            tc::tmem_st_wait();
         }
         grid_dep_wait();         // the step sizes, the streams
-        float seg_l2 = 0.f;      // log2 of the product of a_t over the tiles done so far
         const int64_t rec_row = rec_base + (int64_t)h * rec_hstride;     // tile 0 of this (sequence, head)
         const float *l2p = prm.l2 + rec_row * ST + t_begin;
         float l2_next = ntiles > 0 ? l2p[i] : 0.f;
-        // A run of state-only tiles (a whole segment in the state-only pass, the lead of a split
-        // launch) is one long contraction: with every token weighted by its decay up to the END OF
-        // THE RUN (exponent <= 0), Btilde^T (w . X) accumulates over all tiles of the run in tensor
-        // memory and the state is touched once, at the run's last tile:
+        // The leading tiles of a split launch are one long contraction: with every token weighted by its
+        // decay up to the END OF THE RUN (exponent <= 0), Btilde^T (w . X) accumulates over all tiles of
+        // the run in tensor memory and the state is touched once, at the run's last tile:
         //   H_end = 2^(sum of l_last over the run) H_in + sum_tiles Btilde^T (w' . X).
-        const int run_end = kfull ? n_pre : ntiles;
+        const int run_end = n_pre;
         float run_total = 0.f;   // log2 decay over the whole run
         {
             const TileScalars *rec0 = prm.rec + rec_row + t_begin / ST;
@@ -599,8 +592,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
 
         for (int j = 0; j < ntiles; ++j) {
             const int sx = j & 1;
-            const bool full = SPLIT ? (kfull && j >= n_pre) : kfull;
-            const bool hb_next = SPLIT ? (kfull && j + 1 >= n_pre) : kfull;   // the next tile reads the bf16 state copy
+            const bool full = !SPLIT || j >= n_pre;
+            const bool hb_next = !SPLIT || j + 1 >= n_pre;                    // the next tile reads the bf16 state copy
             const int jf = SPLIT ? j - n_pre : j;
             const uint8_t *s_x = s_head + sx * SLAB;
             // ---- per-token scalars: this row's cumulative log2 decay inside the tile (prefetched);
@@ -615,7 +608,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
 
             // ---- w . X  (rows of the X slab -> rows of the X' slab, this thread's half of the
             // head dim).  Row block wq has wq + 1 blocks of the decay mask to build, all of them on one
-            // scheduler (a warp reads only its quarter of the tensor memory), so in the full pass the 16
+            // scheduler (a warp reads only its quarter of the tensor memory), so in a full tile the 16
             // (row block, 16-byte chunk) units of a lane are dealt 8 / 6 / 2 / 0 to row blocks 0 .. 3; a
             // foreign row's weight is read from shared memory.
             if (full) {
@@ -719,9 +712,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 tc::mbar_arrive(&hb->m_full);
             }
 
-            // ---- state: H = exp(l_last) H + dH  (thread owns state index n = i, 32 channels); inside a
-            // run of state-only tiles only at its last tile, with the decay of the whole run
-            seg_l2 += l2_last;
+            // ---- state: H = exp(l_last) H + dH  (thread owns state index n = i, 32 channels); of the
+            // leading tiles only at the last one, with the decay of the whole run
             if (full || j == run_end - 1) {
             tc::mbar_wait(&hb->dh_full, j & 1, abort_flag, d_status);
             tc::tc_fence_after();
@@ -794,30 +786,19 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             tc::mbar_arrive(&hb->x_free[sx]);
         }
 
-        // ---- final state of the segment
-        if (kfull) {
-            if (prm.h_out && seg == nseg - 1 && !head_part) {
-                float *dst = prm.h_out + (((int64_t)b * H + h) * SP) * SN;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    float2 v = tc::f32x2_get(Hst[q]);
-                    if (prm.add) {
-                        v.x += dst[(int64_t)(p0 + 2 * q) * SN + i];
-                        v.y += dst[(int64_t)(p0 + 2 * q + 1) * SN + i];
-                    }
-                    dst[(int64_t)(p0 + 2 * q) * SN + i] = v.x;
-                    dst[(int64_t)(p0 + 2 * q + 1) * SN + i] = v.y;
-                }
-            }
-        } else {
-            float *dst = prm.h_out + ((((int64_t)seg_base + seg) * H + h) * SP) * SN;
+        // ---- final state
+        if (prm.h_out && seg == nseg - 1 && !head_part) {
+            float *dst = prm.h_out + (((int64_t)b * H + h) * SP) * SN;
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
-                const float2 v = tc::f32x2_get(Hst[q]);
+                float2 v = tc::f32x2_get(Hst[q]);
+                if (prm.add) {
+                    v.x += dst[(int64_t)(p0 + 2 * q) * SN + i];
+                    v.y += dst[(int64_t)(p0 + 2 * q + 1) * SN + i];
+                }
                 dst[(int64_t)(p0 + 2 * q) * SN + i] = v.x;
                 dst[(int64_t)(p0 + 2 * q + 1) * SN + i] = v.y;
             }
-            if (i == 0 && hf == 0) prm.seg_decay[((int64_t)seg_base + seg) * H + h] = tc::ex2_approx(seg_l2);
         }
     }
     tc::tc_fence_before();
@@ -938,7 +919,7 @@ shard_entry_kernel(float *__restrict__ states, const float *__restrict__ seg_dec
 // one long contraction over the segment's tokens accumulated in tensor memory (see the run
 // accumulation in ssd_tiles_kernel).  Nothing but Btilde, x and the tile records is read, so one
 // CTA takes FOUR heads of a group (the Btilde tile is fetched once for all of them: half the
-// shared-operand traffic of a head pair) and the tiles flow through a two-stage ring in which the
+// shared-operand traffic of a head pair) and half tiles flow through a ring of four stages in which the
 // x slabs are scaled IN PLACE: TMA fills a stage, 16 warps (one token row of one head per thread)
 // scale, one thread issues a single 128 x 256 x 128 product per tile, its completion frees the
 // stage.  The state is read from tensor memory once, at the end.
@@ -1360,7 +1341,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
     dim3 grid((unsigned)nseg, (unsigned)(G * pairs_per_group(H, G)), (unsigned)B);
     p.split_tiles = 0;
     if (nseg == 1) {
-        p.h_in = h0; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
+        p.h_in = h0; p.h_out = h_final; p.seg_decay = nullptr;
         p.split_tiles = in_place ? 0 : ssd_split_tiles(B, L, H, G, sm_count);
         if (p.split_tiles > 0) grid = dim3((unsigned)B, (unsigned)(G * pairs_per_group(H, G)), 2u);
         ctx.begin(STAGE_SSD_TILES);
@@ -1372,7 +1353,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
     } else {
         float *states = (float *)seg_ws;
         float *decay = states + (size_t)B * nseg * H * SP * SN;
-        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY;
+        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay;
         {
             // (the last segment's end state is nobody's entry state: the full pass produces it)
             const int rc = launch_state_pass(ctx, x, Bs, L, B, p, (unsigned)(nseg - 1), H, G, (unsigned)B);
@@ -1382,7 +1363,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
             const int rc = launch_segment_scan(ctx, states, decay, h0, B, nseg, H, in_place);
             if (rc != SWIMBA_OK) return rc;
         }
-        p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
+        p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr;
         ctx.begin(STAGE_SSD_TILES);
         launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         ctx.end();
@@ -1639,7 +1620,7 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &pl, const void *x,
         float *decay = (float *)(ws + lay.decay);
         p.items = (const int2 *)(ws + lay.pre);
         const bool in_place = h0 && h0 == h_final;
-        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY; p.seg_states = in_place ? 3 : 2;
+        p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.seg_states = in_place ? 3 : 2;
         const int rc = launch_state_pass(ctx, x, Bs, T, 1, p, (unsigned)pl.pre.size(), H, G, 1u);
         if (rc != SWIMBA_OK) return rc;
         const int PN4 = SP * SN / 4;
@@ -1651,7 +1632,7 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &pl, const void *x,
         p.h_in = states;
     }
     p.items = (const int2 *)(ws + lay.items);
-    p.h_out = h_final; p.seg_decay = nullptr; p.mode = MODE_FULL;
+    p.h_out = h_final; p.seg_decay = nullptr;
     ctx.begin(STAGE_SSD_TILES);
     launch_kernel(ssd_tiles_kernel<false>, dim3((unsigned)pl.items.size() * pairs), dim3(SSD_THREADS), smem,
                   ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
@@ -1739,7 +1720,7 @@ int launch_ssd_shard_summary(LaunchCtx &ctx, const void *x, const void *BC, cons
     SsdParams p = shard_params(ctx, lay, B, L, H, G, workspace);
     float *states = (float *)((char *)workspace + lay.states);
     float *decay = (float *)((char *)workspace + lay.decay);
-    p.h_in = nullptr; p.h_out = states; p.seg_decay = decay; p.mode = MODE_STATE_ONLY;
+    p.h_in = nullptr; p.h_out = states; p.seg_decay = decay;
     {
         const int rc = launch_state_pass(ctx, x, b_stream(BC, G), L, B, p, (unsigned)lay.nseg, H, G, (unsigned)B);
         if (rc != SWIMBA_OK) return rc;
@@ -1770,7 +1751,7 @@ int launch_ssd_shard_finish(LaunchCtx &ctx, const void *x, const void *BC, const
         states, decay, h0, all_state, all_decay, rank, B, lay.nseg, H, PN4);
     ctx.end();
     p.D = D; p.y = y;
-    p.h_in = states; p.h_out = h_end; p.seg_decay = nullptr; p.mode = MODE_FULL;
+    p.h_in = states; p.h_out = h_end; p.seg_decay = nullptr;
     const dim3 grid((unsigned)lay.nseg, (unsigned)(G * pairs_per_group(H, G)), (unsigned)B);
     ctx.begin(STAGE_SSD_TILES);
     launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), ssd_smem_bytes(), ctx.stream, true, tm_b, tm_c,
