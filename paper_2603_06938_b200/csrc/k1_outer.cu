@@ -47,13 +47,6 @@ struct OuterArgs {
     int E, F, S, k, check;
     int *d_status;
 };
-
-__device__ __forceinline__ void reduce_row_f32(float *dst, const void *src, uint32_t bytes)
-{
-    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst),
-                 "r"(tc::smem_u32(src)), "r"(bytes)
-                 : "memory");
-}
 }  // namespace
 
 __global__ void __launch_bounds__(PO_THREADS, 1)
@@ -116,7 +109,7 @@ pair_outer_kernel(const OuterArgs p)
     }
     tc::tc_fence_before();
     __syncthreads();
-    tc::pair_sync();
+    tc::cluster_sync();
     tc::tc_fence_after();
     const uint32_t tmem = sm->tmem_slot;
     const int64_t total = sm->step_end[SWIMBA_MAX_EXPERTS - 1];
@@ -275,7 +268,7 @@ pair_outer_kernel(const OuterArgs p)
                     for (int i = 0; i < 8; ++i) d4[i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
                 }
                 tc::fence_proxy_async_smem();
-                if (row < p.S) reduce_row_f32(dst + c, srow, (uint32_t)min(PO_COLS, ncols - c) * 4);
+                if (row < p.S) tc::bulk_reduce_add_f32(dst + c, srow, (uint32_t)min(PO_COLS, ncols - c) * 4);
                 tc::bulk_commit_group();
             }
             tc::tc_fence_before();
@@ -287,7 +280,7 @@ pair_outer_kernel(const OuterArgs p)
     }
     tc::tc_fence_before();
     __syncthreads();
-    tc::pair_sync();
+    tc::cluster_sync();
     tc::tc_fence_after();
     if (warp == 1) tc::pair_tmem_dealloc(tmem);
 }

@@ -135,7 +135,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
     tc::tc_fence_before();
     __syncthreads();
-    tc::pair_sync();            // barriers and tensor memory of both CTAs are ready
+    tc::cluster_sync();            // barriers and tensor memory of both CTAs are ready
     tc::tc_fence_after();
     const uint32_t tmem = sm->tmem_slot;
     const int ncol = ceil_div(p.S, PG_BN);
@@ -333,7 +333,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
     tc::tc_fence_before();
     __syncthreads();
-    tc::pair_sync();            // nobody reads or signals the other CTA's memory any more
+    tc::cluster_sync();            // nobody reads or signals the other CTA's memory any more
     tc::tc_fence_after();
     if (warp == 1) tc::pair_tmem_dealloc(tmem);
 }

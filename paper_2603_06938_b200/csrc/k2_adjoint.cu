@@ -38,12 +38,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, const void *s
                  "r"(tc::smem_u32(src)), "r"(c0), "r"(c1), "r"(c2)
                  : "memory");
 }
-__device__ __forceinline__ void bulk_reduce_add_f32(void *dst, const void *src, uint32_t bytes)
-{
-    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst),
-                 "r"(tc::smem_u32(src)), "r"(bytes)
-                 : "memory");
-}
 // Eight bf16 values times (w_hi + w_lo), rounded once.
 __device__ __forceinline__ uint4 scale8(const uint4 &v, __nv_bfloat162 w_hi, __nv_bfloat162 w_lo)
 {
@@ -568,7 +562,7 @@ adjoint_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_c
         if (tid < 2 * AT) {
             const int mat = tid >> 7, r = tid & 127;
             if (t0 + r < prm.L)
-                bulk_reduce_add_f32(prm.dBC + ((int64_t)b * prm.L + t0 + r) * (2 * prm.G * AN) + (mat ? g : prm.G + g) * AN,
+                tc::bulk_reduce_add_f32(prm.dBC + ((int64_t)b * prm.L + t0 + r) * (2 * prm.G * AN) + (mat ? g : prm.G + g) * AN,
                                     smem + mat * AT * AC_ROW + r * AC_ROW, AN * 4);
             tc::bulk_commit_group();
             tc::bulk_wait_read_all();

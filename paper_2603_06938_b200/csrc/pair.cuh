@@ -19,14 +19,13 @@ __device__ __forceinline__ uint32_t leader_addr(const void *p)
     asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(p)));
     return r;
 }
-__device__ __forceinline__ void pair_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Arrival at a barrier of the first CTA.  What it announces -- rows in this SM's own shared memory that
-// this SM's tensor core will read, tensor memory of this SM that its tensor core may overwrite -- is
-// ordered by the proxy fence / tcgen05 fence in front; no other SM reads it, so that no cluster-wide
-// release is needed (with one, every step of the product took 2000 cycles).
+// Arrival at a barrier of the first CTA: rows in this SM's shared memory are ready for the pair's products (the
+// products of both SMs read them where they are the second operand), tensor memory of this SM may be overwritten.
+// The form is that of CUTLASS's umma_arrive_2x1SM_sm0, which announces operands written by ordinary stores of
+// either CTA to products on the pair: the writes are made visible to the asynchronous proxy by the proxy fence in
+// front (reads of tensor memory: completed by the tcgen05 fence), and the products read shared memory of both SMs
+// through that proxy.  An arrival with a cluster-wide release and a wait with a cluster-wide acquire in its place:
+// 3 x 1531 tokens of 36 heads, 16 experts, k = 4 89 -> 125 us, the gradients of 4 x 8192 790 -> 868 us.
 __device__ __forceinline__ void remote_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");

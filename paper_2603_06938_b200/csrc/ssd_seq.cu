@@ -48,10 +48,6 @@ __device__ __forceinline__ void ck_store4(__nv_bfloat16 *p, const float (&v)[4])
 {
     *reinterpret_cast<uint2 *>(p) = make_uint2(tc::pack_bf16x2(v[0], v[1]), tc::pack_bf16x2(v[2], v[3]));
 }
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t local, uint32_t rank)
 {
     uint32_t r;
@@ -241,7 +237,7 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
             }
             sG[i * Gr + lane] = v;
         }
-        if (MULTI) cluster_sync();
+        if (MULTI) tc::cluster_sync();
         else __syncthreads();
         // ---- state entering this run: the runs in front of it, in order
         const uint32_t s_addr = tc::smem_u32(sS), d_addr = tc::smem_u32(&s_decay);
@@ -347,7 +343,7 @@ ssd_chunk_kernel(const T *__restrict__ x, const T *__restrict__ BC, const float 
             }
         }
         // the local end states have been read by everyone (and no CTA leaves while it is being read)
-        if (MULTI) cluster_sync();
+        if (MULTI) tc::cluster_sync();
         else __syncthreads();
     }
     if (h_final && rank == 0) {

@@ -153,6 +153,16 @@ __device__ __forceinline__ void bulk_reduce_add_bf16(void *dst_global, const voi
                  "r"(smem_u32(src_smem)), "r"(bytes)
                  : "memory");
 }
+// The same for fp32 elements.
+__device__ __forceinline__ void bulk_reduce_add_f32(void *dst_global, const void *src_smem, uint32_t bytes) {
+    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst_global),
+                 "r"(smem_u32(src_smem)), "r"(bytes)
+                 : "memory");
+}
+// Barrier among all threads of a cluster.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // Waits until the issuing thread's bulk stores have finished READING shared memory.
 __device__ __forceinline__ void bulk_wait_read_all() {
@@ -287,15 +297,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
         "r"(r[30]), "r"(r[31]), "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" ::"r"(r[0]),
-        "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-        "r"(taddr)
-        : "memory");
-}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(r[0]),
@@ -325,25 +326,6 @@ __device__ __forceinline__ float lg2_approx(float v) {
 // Barrier among the first `n` threads of the CTA (n a multiple of 32), hardware barrier `id`.
 __device__ __forceinline__ void named_bar_sync(int id, int n) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
-// Re-deal of the CTA's registers between warpgroups (all four warps of a warpgroup execute the
-// same call): the issuing warps give up what they do not need, the compute warpgroups take it.
-template <int N> __device__ __forceinline__ void reg_alloc() {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
-}
-template <int N> __device__ __forceinline__ void reg_dealloc() {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
-}
-
-// Packed fp32 pairs (one instruction for two lanes of arithmetic): (a, b) <- (a, b) * (x, y) on the
-// raw 32-bit images of two floats.
-__device__ __forceinline__ void mul2(uint32_t &a, uint32_t &b, float x, float y) {
-    asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
-        "mov.b64 ra, {%0, %1};\n\tmov.b64 rb, {%2, %3};\n\t"
-        "mul.rn.f32x2 rc, ra, rb;\n\tmov.b64 {%0, %1}, rc;\n\t}"
-        : "+r"(a), "+r"(b)
-        : "f"(x), "f"(y));
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
