@@ -20,8 +20,9 @@
 // the head dimension) and its own MMA-issuing warp, so that one head's tensor-core and memory
 // latencies are covered by the other warps' CUDA-core work.
 //
-// What bounds it: shared memory (about 4500 of a tile's 5500 cycles carry products, TMA and the CUDA cores'
-// reads and writes at 128 bytes a cycle) and the row-block-3 scheduler, not the tensor cores (30 %).  So G of
+// What bounds it, as far as counters and arithmetic go: shared memory (512 KB a tile of a head pair for products,
+// TMA and the CUDA cores, 4000 of its 5500 cycles at 128 bytes a cycle; the CUDA cores' part is counted at 0.42 of
+// the time, nearly twice its share of that) and the row-block-3 scheduler, not the tensor cores (0.37).  So G of
 // the next tile is issued under this tile's state update (it needs no state) and the mask is built before the
 // product with the carried state is waited for; fp32 work goes two to an instruction; the mask's column
 // weights are read 16 bytes at a time; w.X stays off the warps that have the longest mask rows.  4 x 8192
