@@ -1,4 +1,5 @@
 // Host side of the C ABI: handle, argument validation, workspace layout and kernel sequencing.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -72,7 +73,8 @@ DecLayout dec_layout(const swimba_config &c, int B)
     const size_t S = 2u * c.n_groups * c.d_state;
     size_t off = 0;
     const bool slots = front_small_supported(c.dtype, 1, c.d_model, (int)S, c.n_experts, c.top_k);
-    l.bc = off;  off += align_up((size_t)B * (slots ? c.top_k : 1) * S * sizeof(float));
+    const int rows = slots ? std::max(B, std::min(B, FRONT_SMALL_TOKENS) * c.top_k) : B;   // (grows with B)
+    l.bc = off;  off += align_up((size_t)rows * S * sizeof(float));
     l.idx = off; off += align_up((size_t)B * c.top_k * sizeof(int32_t));
     l.w = off;   off += align_up((size_t)B * c.top_k * sizeof(float));
     l.gemm = off;

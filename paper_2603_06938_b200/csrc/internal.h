@@ -69,6 +69,7 @@ int launch_accumulate(LaunchCtx &ctx, int dtype, void *y, const void *y_add, int
 // [T,k,S] per slot (weights applied), summed by the reader.  The kernel behind starts only after everything
 // in front of this call has completed, so it may read what earlier calls wrote before its own wait.
 // front_small_faster: whether it is, beside the router and the grouped product (with fp32 slots).
+constexpr int FRONT_SMALL_TOKENS = 256;      // per call
 bool front_small_supported(int dtype, int64_t T, int F, int S, int E, int k);
 bool front_small_faster(int64_t T, int F, int S, int E, int k);
 bool front_small_slots(int64_t T, int S, int E, int k);

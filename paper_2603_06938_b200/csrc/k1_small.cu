@@ -27,7 +27,7 @@ namespace swimba {
 
 namespace {
 constexpr int SM_MAX_E = 16;        // experts the small router holds in registers
-constexpr int SM_MAX_T = 256;       // tokens per call
+constexpr int SM_MAX_T = FRONT_SMALL_TOKENS;
 constexpr int SM_ROWS = 16;         // rows of W_e per CTA (the M of m16n8k16)
 constexpr int SM_WARPS = 8;
 constexpr int SM_NT = 4;            // 8-token column tiles worked per pass

@@ -78,3 +78,6 @@ def test_smaller_decode_batches_need_no_more(F, G, E, k, dtype):
     assert sizes == sorted(sizes)
     if E <= 16 and dtype == "bf16":      # the small front end: k fp32 rows per sequence up to B = 4
         assert sizes[3] >= 4 * k * 256 * G * 4
+    # larger batches take no slots of fp32 rows: one row of streams, the lists, 16-bit slots where k > 2
+    S = 256 * G
+    assert sizes[1100] - sizes[256] <= (1100 - 256) * (4 * S + (2 * k * S if k > 2 else 0) + 4 * E + 8 * k) + 4096
