@@ -636,7 +636,9 @@ size_t ssd_adjoint_tiles_workspace_bytes(int B, int L, int H, int G, int sm_coun
 ScalarsArgs ssd_adjoint_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
                                      void *workspace)
 {
-    return ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace);
+    ScalarsArgs sa = ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace);
+    sa.mid = 0;                                   // (this file's kernels take the weights block by block)
+    return sa;
 }
 
 int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, const void *BC, const float *h0, int B,

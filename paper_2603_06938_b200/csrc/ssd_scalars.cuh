@@ -2,12 +2,16 @@
 // transition is shared by all experts: shared-A equation).  Per token t of head h, with
 // Delta_t = softplus(dt_t + dt_bias_h) and l_t = sum_{r <= t, r in t's 128-token tile} Delta_r A_h log2 e,
 // two arrays are produced:
-//   l2[(b*H + h)*Lpad + t] = l_t
+//   l2[(b*H + h)*Lpad + t] = l_t          (forward: the row factor of the decay mask, below)
 //   rec[((b*H + h)*ntile + tile)] = one record per 128-token tile, copied to shared memory as a block:
 //       wp[128]  W(Delta_t 2^(l_last - l_t))      weight of token t in the tile's end state
-//       cb[128]  Delta_t 2^(l_blockend - l_t)     weight of token t at the end of its 32-token block
+//       cb[128]  Delta_t 2^(l_ref - l_t)          weight of token t as a column of the decay mask
 //       ends[4]  l at the end of each 32-token block (ends[3] = l_last)
-// Every exponent is <= 0.  W(w) is w as a two-term bf16 sum packed in one word (high part in the low
+//       aux      (forward only) what follows from the ends, so that no thread of the SSD kernel has to work it out
+// l_ref is l at the end of t's 32-token block; for the forward (`mid`) it is l in the middle of the tile, ends[1],
+// while the tile's halves decay moderately (tile_mid_ref).  Exponents to the block's or the tile's end are <= 0.
+// Row factors: 2^(l_t - l_ref) with the middle as reference; else 2^(l_t - l at the start of t's block), or l_t
+// itself where the block decays by 2^-96 and more (mask_mode).  W(w) is w as a two-term bf16 sum packed in one word (high part in the low
 // half, remainder in the high half): round(w_hi x + round(w_lo x)) is w x rounded once for a bf16 x,
 // up to a term of relative size 2^-17.  Positions past L carry Delta = 0.
 // The work depends on dt only, so it runs either as a kernel of its own or as extra blocks of
@@ -23,8 +27,32 @@ struct TileScalars {            // (the shared-memory image as well)
     uint32_t wp[SCALARS_TILE];
     float cb[SCALARS_TILE];
     float ends[4];
+    struct Aux {
+        float to_ref;       // decay from the tile's start to l_ref (1 unless it is the middle)
+        float from_ref;     // from l_ref to the tile's end (middle only)
+        float total;        // over the tile
+        float blocks;       // 0: l_ref is the middle of the tile, 1: it is not
+    } aux;
 };
 static_assert(sizeof(TileScalars) % 16 == 0, "tile records are moved by 16-byte bulk copies");
+
+// Whether the mask of a tile may be split at its middle, exp(l_t - l_s) = 2^(l_t - ends[1]) 2^(ends[1] - l_s): a
+// column weight and a row factor, both within 2^(+-72), instead of a product per block.  Sums over the tile then
+// stay finite as long as the plain ones are below 2^55; heads that decay faster take the blockwise form.
+__host__ __device__ inline bool tile_mid_ref(float ends1, float ends3)
+{
+    return fabsf(ends1) < 72.f && fabsf(ends3 - ends1) < 72.f;
+}
+
+// What the row factors, and with them the column weights, of rows in block w refer to: the middle of the tile (the
+// column weights as they are); where a head decays too fast for that, the start of the row block (column weights
+// times a factor per block); where even a block decays by 2^-96, nothing (entries are formed one by one).
+enum MaskMode { MASK_MIDDLE, MASK_BLOCKS, MASK_ENTRIES };
+__host__ __device__ inline int mask_mode(const float *ends, int w)
+{
+    if (tile_mid_ref(ends[1], ends[3])) return MASK_MIDDLE;
+    return (w ? ends[w - 1] : 0.f) - ends[w] < 96.f ? MASK_BLOCKS : MASK_ENTRIES;
+}
 
 struct ScalarsArgs {
     const float *dt, *A, *dt_bias;
@@ -35,6 +63,7 @@ struct ScalarsArgs {
     // (first token, valid tokens); tiles start at sequence starts.  dt is then [T, H], the arrays
     // are laid out [H, tiles] and Lpad = 128 * tiles, B = 1.  Null: dense [B, L].
     const int2 *tile_tab = nullptr;
+    int mid = 0;          // 1: the forward's column weights
 };
 
 __host__ __device__ inline int64_t scalars_units(const ScalarsArgs &a)
@@ -98,6 +127,11 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
         const float excl = incl - run;
         const float l_last = __shfl_sync(0xffffffffu, incl, 31);
         const float l_blk = __shfl_sync(0xffffffffu, incl, lane | 7);   // 8 lanes = one 32-token block
+        const float l_mid = __shfl_sync(0xffffffffu, incl, 15);
+        const bool mid = a.mid && tile_mid_ref(l_mid, l_last);
+        const float l_ref = mid ? l_mid : l_blk;
+        const float l_prev = __shfl_sync(0xffffffffu, incl, (lane & 24) - 1);      // (block 0: any lane)
+        const float l_beg = lane < 8 ? 0.f : l_prev;
         float lv[4], cb[4];
         uint32_t wp[4];
 #pragma unroll
@@ -107,9 +141,19 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
             const __nv_bfloat16 w_hi = __float2bfloat16_rn(w);
             wp[i] = (uint32_t)__bfloat16_as_ushort(w_hi) |
                     ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(w - __bfloat162float(w_hi))) << 16);
-            cb[i] = d[i] * exp2f(l_blk - lv[i]);
+            cb[i] = d[i] * exp2f(l_ref - lv[i]);
         }
         TileScalars *rec = a.rec + out[q];
+        if (a.mid) {
+            if (mid || l_beg - l_blk < 96.f) {
+                const float from = mid ? l_mid : l_beg;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) lv[i] = exp2f(lv[i] - from);
+            }
+            if (lane == 31)
+                rec->aux = TileScalars::Aux{mid ? exp2f(l_mid) : 1.f, mid ? exp2f(l_last - l_mid) : 1.f, exp2f(l_last),
+                                            mid ? 0.f : 1.f};
+        }
         reinterpret_cast<float4 *>(a.l2 + out[q] * SCALARS_TILE)[lane] = make_float4(lv[0], lv[1], lv[2], lv[3]);
         reinterpret_cast<uint4 *>(rec->wp)[lane] = make_uint4(wp[0], wp[1], wp[2], wp[3]);
         reinterpret_cast<float4 *>(rec->cb)[lane] = make_float4(cb[0], cb[1], cb[2], cb[3]);
