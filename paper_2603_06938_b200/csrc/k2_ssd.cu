@@ -629,7 +629,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         // token, the share one half of one head's channels.
         const int wq = uwarp & 3, sub = uwarp >> 2;
         const int i = wq * 32 + lane;
-        const int hs = wq >> 1, ps = i & 63;                 // state: head of the pair, channel
+        const int hs = wq >> 1;                              // state: head of the pair
         const int he = sub >> 1, hf = sub & 1;               // epilogue: head of the pair, half of its channels
         const bool has_s = hs < nh, has_e = he < nh;
         const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
@@ -638,6 +638,10 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         // 16-byte chunk c of this thread's part of row i, in the state, x and y slabs alike: base ^ 16 c
         const uint32_t row_off = tc::sw128_offset(i, 4 * hf);
         uint8_t *s_h = smem + SM_H + (sub >> 1) * SLAB;
+        // States to and from global memory: eight rows of 64 bytes at a time (a row per thread touched 32 lines with
+        // every load: 3 us at either end of a CTA), transposed through this warp's part of the bf16 copy's slabs.
+        const int tr_row = lane >> 2, tr_col = 4 * (lane & 3);
+        const uint32_t tr_off = tc::sw128_offset(32 * wq + tr_row, 4 * hf + (lane & 3));
         // of a pair of columns c, c + 1 = 2 (t % 4) of an 8 x 8 diagonal block, the bf16 halves that row t / 4 keeps
         const int below = (lane >> 2) - 2 * (lane & 3);
         const uint32_t keep = below < 0 ? 0u : (below == 0 ? 0xffffu : 0xffffffffu);
@@ -646,7 +650,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(bar);
         };
-        // fp32 master copy of the state: this thread holds H[p = ps][n = 32 sub ..], two to a register pair
+        // fp32 master copy of the state: this thread holds H[p = i % 64][n = 32 sub ..], two to a register pair
         uint64_t Hst[16];
         // its bf16 copy, MMA 3 operand of the next tile, decayed by f
         auto store_h = [&](float f) {
@@ -671,13 +675,24 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             if (h_in && has_s) {
                 const int64_t row = (prm.seg_states && !first) ? ((int64_t)seg_base + seg) * H + head0 + hs
                                                                : (int64_t)b * H + head0 + hs;
-                const float4 *src = reinterpret_cast<const float4 *>(h_in + (row * SP + ps) * SN + 32 * sub);
+                const float *src = h_in + (row * SP + 32 * (wq & 1)) * SN + 32 * sub + tr_row * SN + tr_col;
+                float4 t[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 v = __ldcg(src + q);
-                    Hst[2 * q] = tc::f32x2(v.x, v.y);
-                    Hst[2 * q + 1] = tc::f32x2(v.z, v.w);
+                for (int q = 0; q < 8; ++q) t[q] = __ldcg(reinterpret_cast<const float4 *>(src + 8 * (q & 3) * SN + 16 * (q >> 2)));
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) *reinterpret_cast<float4 *>(s_h + tr_off + q * 1024) = t[4 * half + q];
+                    __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float4 v = *reinterpret_cast<const float4 *>(s_h + (row_off ^ (c << 4)));
+                        Hst[8 * half + 2 * c] = tc::f32x2(v.x, v.y);
+                        Hst[8 * half + 2 * c + 1] = tc::f32x2(v.z, v.w);
+                    }
                 }
+                __syncwarp();
             }
         }
         grid_dep_wait();         // the step sizes, the streams
@@ -800,14 +815,20 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                     // ---- Y = Ctilde Hprev^T scaled in place
                     tc::mbar_wait(&bars->dh_full, dh_ph, abort_flag, d_status);
                     tc::tc_fence_after();
-#pragma unroll 1
-                    for (int c = 0; c < 32; c += 8) {
-                        uint32_t yo[8];
-                        tc::tmem_ld8(tm_y + c, yo);
-                        tc::tmem_ld_wait();
+                    const uint64_t e2 = tc::f32x2(cur.pre, cur.pre);
+                    uint32_t yo[2][16];
+                    tc::tmem_ld16(tm_y, yo[0]);
+                    tc::tmem_ld16(tm_y + 16, yo[1]);
+                    tc::tmem_ld_wait();
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) yo[q] = __float_as_uint(cur.pre * __uint_as_float(yo[q]));
-                        tc::tmem_st8(tm_y + c, yo);
+                    for (int hh = 0; hh < 2; ++hh) {
+#pragma unroll
+                        for (int q = 0; q < 16; q += 2) {
+                            const float2 v = tc::f32x2_get(tc::f32x2_mul(e2, f32x2_bits(yo[hh][q], yo[hh][q + 1])));
+                            yo[hh][q] = __float_as_uint(v.x);
+                            yo[hh][q + 1] = __float_as_uint(v.y);
+                        }
+                        tc::tmem_st16(tm_y + 16 * hh, yo[hh]);
                     }
                 }
                 tc::tmem_st_wait();
@@ -901,16 +922,26 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             nseg = prm.seqs[b + 1].seg0 - prm.seqs[b].seg0;
         }
         if (prm.h_out && seg == nseg - 1 && !head_part && has_s) {
-            float4 *dst = reinterpret_cast<float4 *>(prm.h_out + (((int64_t)b * prm.H + head0 + hs) * SP + ps) * SN + 32 * sub);
+            float *dst = prm.h_out + (((int64_t)b * prm.H + head0 + hs) * SP + 32 * (wq & 1)) * SN + 32 * sub + tr_row * SN + tr_col;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float2 lo = tc::f32x2_get(Hst[2 * q]), hi = tc::f32x2_get(Hst[2 * q + 1]);
-                float4 v = make_float4(lo.x, lo.y, hi.x, hi.y);
-                if (prm.add) {
-                    const float4 w = dst[q];
-                    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+            for (int half = 0; half < 2; ++half) {
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float2 lo = tc::f32x2_get(Hst[8 * half + 2 * c]), hi = tc::f32x2_get(Hst[8 * half + 2 * c + 1]);
+                    *reinterpret_cast<float4 *>(s_h + (row_off ^ (c << 4))) = make_float4(lo.x, lo.y, hi.x, hi.y);
                 }
-                dst[q] = v;
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float4 v = *reinterpret_cast<const float4 *>(s_h + tr_off + q * 1024);
+                    float4 *p = reinterpret_cast<float4 *>(dst + 8 * q * SN + 16 * half);
+                    if (prm.add) {
+                        const float4 w = *p;
+                        v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+                    }
+                    *p = v;
+                }
             }
         }
     }

@@ -8,9 +8,9 @@
 //       cb[128]  Delta_t 2^(l_ref - l_t)          weight of token t as a column of the decay mask
 //       ends[4]  l at the end of each 32-token block (ends[3] = l_last)
 //       aux      (forward only) what follows from the ends, so that no thread of the SSD kernel has to work it out
-// l_ref is l at the end of t's 32-token block; for the forward (`mid`) it is l in the middle of the tile, ends[1],
-// while the tile's halves decay moderately (tile_mid_ref).  Exponents to the block's or the tile's end are <= 0.
-// Row factors: 2^(l_t - l_ref) with the middle as reference; else 2^(l_t - l at the start of t's block), or l_t
+// l_ref is l at the end of t's 32-token block; for the forward (`mid`) the tile's reference while there is one
+// (tile_one_ref).  Exponents to the block's or the tile's end are <= 0.
+// Row factors: 2^(l_t - l_ref) with a reference for the tile; else 2^(l_t - l at the start of t's block), or l_t
 // itself where the block decays by 2^-96 and more (mask_mode).  W(w) is w as a two-term bf16 sum packed in one word (high part in the low
 // half, remainder in the high half): round(w_hi x + round(w_lo x)) is w x rounded once for a bf16 x,
 // up to a term of relative size 2^-17.  Positions past L carry Delta = 0.
@@ -28,29 +28,28 @@ struct TileScalars {            // (the shared-memory image as well)
     float cb[SCALARS_TILE];
     float ends[4];
     struct Aux {
-        float to_ref;       // decay from the tile's start to l_ref (1 unless it is the middle)
-        float from_ref;     // from l_ref to the tile's end (middle only)
+        float to_ref;       // decay from the tile's start to its reference (1 if it has none)
+        float from_ref;     // from there to the tile's end
         float total;        // over the tile
-        float blocks;       // 0: l_ref is the middle of the tile, 1: it is not
+        float blocks;       // 0: the tile has a reference, 1: it has not
     } aux;
 };
 static_assert(sizeof(TileScalars) % 16 == 0, "tile records are moved by 16-byte bulk copies");
 
-// Whether the mask of a tile may be split at its middle, exp(l_t - l_s) = 2^(l_t - ends[1]) 2^(ends[1] - l_s): a
-// column weight and a row factor, both within 2^(+-72), instead of a product per block.  Sums over the tile then
-// stay finite as long as the plain ones are below 2^55; heads that decay faster take the blockwise form.
-__host__ __device__ inline bool tile_mid_ref(float ends1, float ends3)
-{
-    return fabsf(ends1) < 72.f && fabsf(ends3 - ends1) < 72.f;
-}
+// The forward's decay mask in two factors per entry: exp(l_t - l_s) = 2^(l_t - ref) 2^(ref - l_s), a row factor and a
+// column weight, with one reference for the whole tile as long as the tile decays by less than 2^-188: half way, or
+// where the column weights stay below 2^88 (sums over the tile are finite while the plain ones are below
+// 2^39), the row factors below 2^100.  A head that decays faster takes the blockwise form, some 10 % slower.
+__host__ __device__ inline bool tile_one_ref(float l_last) { return fabsf(l_last) < 188.f; }
+__host__ __device__ inline float tile_ref(float l_last) { return l_last > -176.f ? 0.5f * l_last : l_last + 88.f; }
 
-// What the row factors, and with them the column weights, of rows in block w refer to: the middle of the tile (the
-// column weights as they are); where a head decays too fast for that, the start of the row block (column weights
-// times a factor per block); where even a block decays by 2^-96, nothing (entries are formed one by one).
-enum MaskMode { MASK_MIDDLE, MASK_BLOCKS, MASK_ENTRIES };
+// What the row factors, and with them the column weights, of rows in block w refer to: the tile's reference (the
+// column weights as they are); the start of the row block (column weights times a factor per block); where even a
+// block decays by 2^-96, nothing (entries are formed one by one).
+enum MaskMode { MASK_TILE, MASK_BLOCKS, MASK_ENTRIES };
 __host__ __device__ inline int mask_mode(const float *ends, int w)
 {
-    if (tile_mid_ref(ends[1], ends[3])) return MASK_MIDDLE;
+    if (tile_one_ref(ends[3])) return MASK_TILE;
     return (w ? ends[w - 1] : 0.f) - ends[w] < 96.f ? MASK_BLOCKS : MASK_ENTRIES;
 }
 
@@ -63,7 +62,7 @@ struct ScalarsArgs {
     // (first token, valid tokens); tiles start at sequence starts.  dt is then [T, H], the arrays
     // are laid out [H, tiles] and Lpad = 128 * tiles, B = 1.  Null: dense [B, L].
     const int2 *tile_tab = nullptr;
-    int mid = 0;          // 1: the forward's column weights
+    int mid = 0;          // 1: the forward's column weights and row factors
 };
 
 __host__ __device__ inline int64_t scalars_units(const ScalarsArgs &a)
@@ -127,8 +126,8 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
         const float excl = incl - run;
         const float l_last = __shfl_sync(0xffffffffu, incl, 31);
         const float l_blk = __shfl_sync(0xffffffffu, incl, lane | 7);   // 8 lanes = one 32-token block
-        const float l_mid = __shfl_sync(0xffffffffu, incl, 15);
-        const bool mid = a.mid && tile_mid_ref(l_mid, l_last);
+        const bool mid = a.mid && tile_one_ref(l_last);
+        const float l_mid = tile_ref(l_last);
         const float l_ref = mid ? l_mid : l_blk;
         const float l_prev = __shfl_sync(0xffffffffu, incl, (lane & 24) - 1);      // (block 0: any lane)
         const float l_beg = lane < 8 ? 0.f : l_prev;
