@@ -71,6 +71,7 @@ constexpr uint32_t SM_C = B_SLOTS * 2 * SLAB;
 constexpr uint32_t SM_X = SM_C + 2 * SLAB;
 constexpr uint32_t SM_H = SM_X + X_SLOTS * NHD * SLAB;
 constexpr uint32_t SM_SMALL = SM_H + 2 * SLAB;
+constexpr uint32_t H_BYTES = SP * SN * 4;      // one head's fp32 state
 
 // TMEM columns: G, which the masked tiles of both heads overwrite in place; Y; dH; w.X; Ctilde.  (w.X of every
 // second leading tile takes Y's place, which those do not use.)
@@ -120,7 +121,7 @@ enum SsdMode { SSD_DENSE, SSD_SPLIT, SSD_PACKED };
 struct __align__(8) SsdBars {
     uint64_t b_full[B_SLOTS], b_empty[B_SLOTS], c_full, c_empty;
     uint64_t x_full[X_SLOTS], xp_full[2], xp_free[2], y_staged[Y_BARS];
-    uint64_t rec_free, m_full, g_full, yd_full, dh_full;
+    uint64_t rec_free, m_full, g_full, yd_full, dh_full, h_staged;
 };
 
 // What this kernel keeps of a tile's record: the column weights, the block ends, what follows from them, and the row
@@ -399,6 +400,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         }
         tc::mbar_init(&bars->rec_free, NCW);
         tc::mbar_init(&bars->m_full, NCW);
+        tc::mbar_init(&bars->h_staged, NCW);
         tc::mbar_init(&bars->g_full, 1);
         tc::mbar_init(&bars->yd_full, 1);
         tc::mbar_init(&bars->dh_full, 1);
@@ -512,6 +514,17 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             }
         }
         if (ntiles > n_pre) store_y(ntiles - 1);
+        if (prm.h_out && seg == nseg - 1 && !head_part) {    // the final states, staged where Btilde stood
+            tc::mbar_wait(&bars->h_staged, 0, abort_flag, d_status);
+            if (leader) {
+                for (int q = 0; q < nh; ++q) {
+                    float *dst = prm.h_out + ((int64_t)b * H + head0 + q) * SP * SN;
+                    if (prm.add) tc::bulk_reduce_add_f32(dst, smem + SM_B + q * H_BYTES, H_BYTES);
+                    else tc::bulk_store(dst, smem + SM_B + q * H_BYTES, H_BYTES);
+                }
+                tc::bulk_commit_group();
+            }
+        }
         if (leader) tc::bulk_wait_read_all();
     } else if (uwarp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer
@@ -915,14 +928,10 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             }
         }
 
-        // ---- final state
-        if (packed) {
-            const int2 it = prm.items[item];
-            b = it.x; seg = it.y;
-            nseg = prm.seqs[b + 1].seg0 - prm.seqs[b].seg0;
-        }
-        if (prm.h_out && seg == nseg - 1 && !head_part && has_s) {
-            float *dst = prm.h_out + (((int64_t)b * prm.H + head0 + hs) * SP + 32 * (wq & 1)) * SN + 32 * sub + tr_row * SN + tr_col;
+        // ---- final state: as rows of [channel][state index] where Btilde stood (no product reads that any more), from
+        // where they go out as one copy per head
+        if (prm.h_out && seg == nseg - 1 && !head_part) {
+            uint8_t *dst = smem + SM_B + hs * H_BYTES + ((32 * (wq & 1) + tr_row) * SN + 32 * sub + tr_col) * 4;
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
                 __syncwarp();
@@ -933,16 +942,12 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 }
                 __syncwarp();
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float4 v = *reinterpret_cast<const float4 *>(s_h + tr_off + q * 1024);
-                    float4 *p = reinterpret_cast<float4 *>(dst + 8 * q * SN + 16 * half);
-                    if (prm.add) {
-                        const float4 w = *p;
-                        v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-                    }
-                    *p = v;
-                }
+                for (int q = 0; q < 4; ++q)
+                    *reinterpret_cast<float4 *>(dst + (8 * q * SN + 16 * half) * 4) =
+                        *reinterpret_cast<const float4 *>(s_h + tr_off + q * 1024);
             }
+            tc::fence_proxy_async_smem();
+            arrive(&bars->h_staged);
         }
     }
     tc::tc_fence_before();
