@@ -71,7 +71,6 @@ constexpr uint32_t SM_C = B_SLOTS * 2 * SLAB;
 constexpr uint32_t SM_X = SM_C + 2 * SLAB;
 constexpr uint32_t SM_H = SM_X + X_SLOTS * NHD * SLAB;
 constexpr uint32_t SM_SMALL = SM_H + 2 * SLAB;
-constexpr uint32_t H_BYTES = SP * SN * 4;      // one head's fp32 state
 
 // TMEM columns: G, which the masked tiles of both heads overwrite in place; Y; dH; w.X; Ctilde.  (w.X of every
 // second leading tile takes Y's place, which those do not use.)
@@ -121,7 +120,7 @@ enum SsdMode { SSD_DENSE, SSD_SPLIT, SSD_PACKED };
 struct __align__(8) SsdBars {
     uint64_t b_full[B_SLOTS], b_empty[B_SLOTS], c_full, c_empty;
     uint64_t x_full[X_SLOTS], xp_full[2], xp_free[2], y_staged[Y_BARS];
-    uint64_t rec_free, m_full, g_full, yd_full, dh_full, h_staged;
+    uint64_t rec_free, m_full, g_full, yd_full, dh_full;
 };
 
 // What this kernel keeps of a tile's record: the column weights, the block ends, what follows from them, and the row
@@ -400,7 +399,6 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         }
         tc::mbar_init(&bars->rec_free, NCW);
         tc::mbar_init(&bars->m_full, NCW);
-        tc::mbar_init(&bars->h_staged, NCW);
         tc::mbar_init(&bars->g_full, 1);
         tc::mbar_init(&bars->yd_full, 1);
         tc::mbar_init(&bars->dh_full, 1);
@@ -514,17 +512,6 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             }
         }
         if (ntiles > n_pre) store_y(ntiles - 1);
-        if (prm.h_out && seg == nseg - 1 && !head_part) {    // the final states, staged where Btilde stood
-            tc::mbar_wait(&bars->h_staged, 0, abort_flag, d_status);
-            if (leader) {
-                for (int q = 0; q < nh; ++q) {
-                    float *dst = prm.h_out + ((int64_t)b * H + head0 + q) * SP * SN;
-                    if (prm.add) tc::bulk_reduce_add_f32(dst, smem + SM_B + q * H_BYTES, H_BYTES);
-                    else tc::bulk_store(dst, smem + SM_B + q * H_BYTES, H_BYTES);
-                }
-                tc::bulk_commit_group();
-            }
-        }
         if (leader) tc::bulk_wait_read_all();
     } else if (uwarp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer
@@ -637,8 +624,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         }
     } else {
         // ------------------------------------------------------------------ compute warps
-        // Warp (row block wq, share sub).  State and w.X: row i is channel i % 64 of head i / 64, the share 32 state
-        // indices / 32 tokens.  Mask: a block of 32 rows and 32 columns, both heads.  Epilogue: row i is a
+        // Warp (row block wq, share sub).  State and w.X: 32 channels of head wq / 2, the share 32 state indices / 32
+        // tokens.  Mask: a block of 32 rows and 32 columns, both heads.  Epilogue: row i is a
         // token, the share one half of one head's channels.
         const int wq = uwarp & 3, sub = uwarp >> 2;
         const int i = wq * 32 + lane;
@@ -648,13 +635,8 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
         const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
         const uint32_t tm_g = lane_base + TM_G + 32 * sub, tm_y = lane_base + TM_Y + 32 * sub;
         const uint32_t tm_dh = lane_base + TM_DH + 32 * sub;
-        // 16-byte chunk c of this thread's part of row i, in the state, x and y slabs alike: base ^ 16 c
+        // 16-byte chunk c of this thread's part of row i, in the x and y slabs: base ^ 16 c
         const uint32_t row_off = tc::sw128_offset(i, 4 * hf);
-        uint8_t *s_h = smem + SM_H + (sub >> 1) * SLAB;
-        // States to and from global memory: eight rows of 64 bytes at a time (a row per thread touched 32 lines with
-        // every load: 3 us at either end of a CTA), transposed through this warp's part of the bf16 copy's slabs.
-        const int tr_row = lane >> 2, tr_col = 4 * (lane & 3);
-        const uint32_t tr_off = tc::sw128_offset(32 * wq + tr_row, 4 * hf + (lane & 3));
         // of a pair of columns c, c + 1 = 2 (t % 4) of an 8 x 8 diagonal block, the bf16 halves that row t / 4 keeps
         const int below = (lane >> 2) - 2 * (lane & 3);
         const uint32_t keep = below < 0 ? 0u : (below == 0 ? 0xffffu : 0xffffffffu);
@@ -663,20 +645,27 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(bar);
         };
-        // fp32 master copy of the state: this thread holds H[p = i % 64][n = 32 sub ..], two to a register pair
+        // fp32 master copy of the state, rows (channels) 32 wq .. and columns (state indices) 32 sub .. in the fragment
+        // layout: pair 8 m + 4 k + r is row 16 m + 8 k + t / 4, columns 8 r + 2 (t % 4) and the one behind.  (A row per
+        // thread makes every access to the states in global memory touch 32 lines: 3 us at either end of a CTA.)
         uint64_t Hst[16];
         // its bf16 copy, MMA 3 operand of the next tile, decayed by f
+        const uint32_t s_h = tc::smem_u32(smem + SM_H + (sub >> 1) * SLAB) +
+                             tc::sw128_offset(32 * wq + (lane & 7), 4 * hf + (lane >> 3));
         auto store_h = [&](float f) {
             const uint64_t f2 = tc::f32x2(f, f);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int q = 0; q < 4; ++q) {
                 uint32_t o[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) o[q] = tc::f32x2_bf16(tc::f32x2_mul(f2, Hst[4 * c + q]));
-                *reinterpret_cast<uint4 *>(s_h + (row_off ^ (c << 4))) = make_uint4(o[0], o[1], o[2], o[3]);
+                for (int r = 0; r < 4; ++r) o[r] = tc::f32x2_bf16(tc::f32x2_mul(f2, Hst[4 * q + r]));
+                tc::stmatrix_x4(s_h + q * 1024, o[0], o[1], o[2], o[3]);
             }
             tc::fence_proxy_async_smem();
         };
+        // offset of pair 8 m + 4 k + r inside the pair of heads' states, from this thread's first one
+        auto h_off = [&](int e) { return 8 * (e >> 2) * SN + 8 * (e & 3); };
+        const int h_mine = (32 * (wq & 1) + (lane >> 2)) * SN + 32 * sub + 2 * (lane & 3);
         {
             const bool first = seg == 0 && (prm.seg_states == 2 || (prm.seg_states == 3 && nseg == 1));
             const float *h_in = first ? prm.h_first : prm.h_in;
@@ -688,24 +677,12 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             if (h_in && has_s) {
                 const int64_t row = (prm.seg_states && !first) ? ((int64_t)seg_base + seg) * H + head0 + hs
                                                                : (int64_t)b * H + head0 + hs;
-                const float *src = h_in + (row * SP + 32 * (wq & 1)) * SN + 32 * sub + tr_row * SN + tr_col;
-                float4 t[8];
+                const float *src = h_in + row * SP * SN + h_mine;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) t[q] = __ldcg(reinterpret_cast<const float4 *>(src + 8 * (q & 3) * SN + 16 * (q >> 2)));
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    __syncwarp();
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) *reinterpret_cast<float4 *>(s_h + tr_off + q * 1024) = t[4 * half + q];
-                    __syncwarp();
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float4 v = *reinterpret_cast<const float4 *>(s_h + (row_off ^ (c << 4)));
-                        Hst[8 * half + 2 * c] = tc::f32x2(v.x, v.y);
-                        Hst[8 * half + 2 * c + 1] = tc::f32x2(v.z, v.w);
-                    }
+                for (int e = 0; e < 16; ++e) {
+                    const float2 v = __ldcg(reinterpret_cast<const float2 *>(src + h_off(e)));
+                    Hst[e] = tc::f32x2(v.x, v.y);
                 }
-                __syncwarp();
             }
         }
         grid_dep_wait();         // the step sizes, the streams
@@ -861,13 +838,16 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 tc::tc_fence_after();
                 const uint64_t dec2 = tc::f32x2(cur.dec, cur.dec);
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
+                for (int m = 0; m < 2; ++m) {
                     uint32_t dh[16];
-                    tc::tmem_ld16(tm_dh + 16 * hh, dh);
+                    tc::tmem_ld_16x256b_x4(tm_dh + ((uint32_t)(16 * m) << 16), dh);
                     tc::tmem_ld_wait();
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        Hst[8 * hh + q] = tc::f32x2_fma(dec2, Hst[8 * hh + q], f32x2_bits(dh[2 * q], dh[2 * q + 1]));
+                    for (int e = 0; e < 8; ++e) {            // (its registers: columns r first, then rows k)
+                        const int k = e >> 2, r = e & 3;
+                        Hst[8 * m + e] = tc::f32x2_fma(dec2, Hst[8 * m + e],
+                                                       f32x2_bits(dh[4 * r + 2 * k], dh[4 * r + 2 * k + 1]));
+                    }
                 }
                 if (j + 1 < ntiles) store_h(h_next);           // (MMA 3 has read the old copy)
                 tc::tc_fence_before();
@@ -928,26 +908,24 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
             }
         }
 
-        // ---- final state: as rows of [channel][state index] where Btilde stood (no product reads that any more), from
-        // where they go out as one copy per head
-        if (prm.h_out && seg == nseg - 1 && !head_part) {
-            uint8_t *dst = smem + SM_B + hs * H_BYTES + ((32 * (wq & 1) + tr_row) * SN + 32 * sub + tr_col) * 4;
+        // ---- final state
+        if (packed) {
+            const int2 it = prm.items[item];
+            b = it.x; seg = it.y;
+            nseg = prm.seqs[b + 1].seg0 - prm.seqs[b].seg0;
+        }
+        if (prm.h_out && seg == nseg - 1 && !head_part && has_s) {
+            float *dst = prm.h_out + ((int64_t)b * prm.H + head0 + hs) * SP * SN + h_mine;
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                __syncwarp();
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float2 lo = tc::f32x2_get(Hst[8 * half + 2 * c]), hi = tc::f32x2_get(Hst[8 * half + 2 * c + 1]);
-                    *reinterpret_cast<float4 *>(s_h + (row_off ^ (c << 4))) = make_float4(lo.x, lo.y, hi.x, hi.y);
+            for (int e = 0; e < 16; ++e) {
+                float2 v = tc::f32x2_get(Hst[e]);
+                float2 *p = reinterpret_cast<float2 *>(dst + h_off(e));
+                if (prm.add) {
+                    const float2 w = *p;
+                    v.x += w.x; v.y += w.y;
                 }
-                __syncwarp();
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    *reinterpret_cast<float4 *>(dst + (8 * q * SN + 16 * half) * 4) =
-                        *reinterpret_cast<const float4 *>(s_h + tr_off + q * 1024);
+                *p = v;
             }
-            tc::fence_proxy_async_smem();
-            arrive(&bars->h_staged);
         }
     }
     tc::tc_fence_before();

@@ -352,6 +352,14 @@ __device__ __forceinline__ void tmem_st_wait() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// Four 8x8 blocks of 16-bit elements from the fragment layout (thread t: row t / 4, columns 2 (t % 4) and the one
+// behind) to shared memory; thread t gives the address of row t % 8 of block t / 8.
+__device__ __forceinline__ void stmatrix_x4(uint32_t smem_addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(smem_addr), "r"(r0), "r"(r1),
+                 "r"(r2), "r"(r3)
+                 : "memory");
+}
+
 // Byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a 128-byte-swizzled slab whose
 // base is 1024-byte aligned (the layout TMA writes and the descriptors above describe).
 __device__ __forceinline__ uint32_t sw128_offset(int row, int chunk) {
