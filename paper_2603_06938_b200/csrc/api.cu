@@ -668,7 +668,9 @@ int swimba_forward(swimba_handle *h, const swimba_weights *w, const void *u, con
     void *BC = ws + l.bc;
     // The SSD step sizes depend on dt only: their kernel runs beside the router.
     const bool fuse = ssd_tiles_supported(h->cfg.dtype, h->cfg.head_dim, h->cfg.d_state);
-    const ScalarsArgs sa = fuse ? ssd_scalars_args(dt, w->A, w->dt_bias, B, L, h->cfg.n_heads, ws + l.ssd)
+    const ScalarsArgs sa = fuse ? ssd_scalars_args(dt, w->A, w->dt_bias, B, L, h->cfg.n_heads, ws + l.ssd,
+                                                   ssd_long_runs(B, L, h->cfg.n_heads, h->cfg.n_groups, h->cfg.chunk,
+                                                                 h->sm_count))
                                 : ScalarsArgs{};
     rc = run_route_mix(h, ctx, w, u, T, BC, false, idx, wt, ws + l.gemm, fuse ? &sa : nullptr);
     if (rc == SWIMBA_OK) rc = run_ssd(h, ctx, w, x, BC, dt, h0, B, L, y, h_final, ws + l.ssd, fuse, true);

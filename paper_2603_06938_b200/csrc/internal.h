@@ -88,8 +88,11 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count);
 // scalars_done: the step sizes and tile log-decays (ssd_scalars_args over the same workspace) have
 // already been produced earlier in the stream (launch_router with scalars, or launch_ssd_scalars).  early:
 // x and h0 were complete before the first kernel of the same call.
+// runs: what ssd_long_runs says of the call (false for kernels that take the records of the tile kernel).
 ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
-                             void *workspace);
+                             void *workspace, bool runs);
+// Whether the full pass of such a call goes to the kernel for long runs of tiles.
+bool ssd_long_runs(int B, int L, int H, int G, int chunk, int sm_count);
 int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &args);
 size_t ssd_scalars_bytes(int B, int L, int H);       // of the arrays ssd_scalars_args lays out
 // Chains nseg segment states per (sequence, head): states [B,nseg,H,P,N] holds local end states on entry

@@ -636,9 +636,7 @@ size_t ssd_adjoint_tiles_workspace_bytes(int B, int L, int H, int G, int sm_coun
 ScalarsArgs ssd_adjoint_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
                                      void *workspace)
 {
-    ScalarsArgs sa = ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace);
-    sa.mid = 0;                                   // (this file's kernels take the weights block by block)
-    return sa;
+    return ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace, false);
 }
 
 int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, const void *BC, const float *h0, int B,
@@ -673,7 +671,7 @@ int launch_ssd_adjoint_tiles(LaunchCtx &ctx, const void *x, const void *dy, cons
         !ensure_dynamic_smem((const void *)adjoint_tiles_kernel, smem_t))
         return SWIMBA_ERR_CUDA;
     AdjParams p;
-    const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, ws + lay.scal);
+    const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, ws + lay.scal, false);
     p.l2 = sa.l2; p.rec = sa.rec; p.h0 = h0;
     p.seg_states = (float *)(ws + lay.seg_states); p.seg_decay = (float *)(ws + lay.seg_decay);
     p.L = L; p.nt = lay.nt; p.H = H; p.G = G; p.B = B; p.nseg = lay.nseg; p.seg_tiles = lay.seg_tiles;

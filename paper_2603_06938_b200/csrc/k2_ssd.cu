@@ -45,103 +45,45 @@
 #include <cstring>
 #include <vector>
 
-#include "internal.h"
-#include "ssd_scalars.cuh"
-#include "tc05.cuh"
+#include "ssd_tiles.cuh"
 
 namespace swimba {
 
 namespace {
-constexpr int ST = 128;                 // tokens per tile
-constexpr int SP = 64;                  // head dim this kernel is built for
-constexpr int SN = 128;                 // state size this kernel is built for
-constexpr int NHD = 2;                  // heads per CTA
-constexpr int NCW = 16;                 // compute warps
-constexpr int WARP_TMA = NCW, WARP_MMA = NCW + 1;
-constexpr int SSD_THREADS = 32 * (NCW + 2);
-constexpr uint32_t SLAB = 16384;        // 128 rows x 128 bytes
+constexpr int NCW = 8 * NHD;            // compute warps
+// warps 0-7: head 0 compute, 8-15: head 1 compute (warp = 8 head + 4 half + row block),
+// 16: TMA, 17: MMA issuer head 0 (+ MMA 1), 18: MMA issuer head 1
+constexpr int WARP_TMA = NCW, WARP_MMA0 = NCW + 1;
+constexpr int SSD_THREADS = 32 * (NCW + 1 + NHD);
+constexpr int HEAD_THREADS = 256;
 
-// shared memory map (bytes from the 1024-aligned base): Btilde of two tiles, Ctilde of one (two slabs each), x of
-// three tiles, which y replaces in place, and the bf16 states of both heads.  A copy from L2 takes 2000 cycles
-// here, from HBM up to 4000: with one Btilde tile less, or x two tiles deep, they were waited for.
-constexpr int B_SLOTS = 2, X_SLOTS = 3;
-constexpr int Y_BARS = 3;               // (the store of a tile is waited for while two more may be staged)
-constexpr uint32_t SM_B = 0;
-constexpr uint32_t SM_C = B_SLOTS * 2 * SLAB;
-constexpr uint32_t SM_X = SM_C + 2 * SLAB;
-constexpr uint32_t SM_H = SM_X + X_SLOTS * NHD * SLAB;
-constexpr uint32_t SM_SMALL = SM_H + 2 * SLAB;
+// shared memory map (bytes from the 1024-aligned base)
+constexpr uint32_t SM_CB = 0;                        // C0 C1 B0 B1 slabs (single stage)
+constexpr uint32_t SM_HEAD = 4 * SLAB;               // per head: X[2] XP HB YS
+constexpr uint32_t SM_HEAD_BYTES = 5 * SLAB;
+constexpr uint32_t SM_SMALL = SM_HEAD + NHD * SM_HEAD_BYTES;
 
-// TMEM columns: G, which the masked tiles of both heads overwrite in place; Y; dH; w.X; Ctilde.  (w.X of every
-// second leading tile takes Y's place, which those do not use.)
-constexpr uint32_t TM_G = 0, TM_Y = 128, TM_DH = 256, TM_XP = 384, TM_C = 448, TM_COLS = 512;
+// TMEM columns: G, then Y, dH and M (bf16 A operand), each 64 columns per head with the two heads
+// side by side (one MMA of N = 128 can then write both heads' Y or dH)
+constexpr uint32_t TM_G = 0, TM_HEAD = 0, TM_HEAD_COLS = 64, TM_COLS = 512;
+constexpr uint32_t TM_Y = 128, TM_DH = 256, TM_M = 384;
 
-struct SeqDesc {            // one sequence of a packed batch
-    int tok0, len;          // first token in the packed arrays, tokens
-    int tile0, seg0;        // first 128-token tile / first segment of the sequence in the batch-wide lists
+struct __align__(8) HeadBars {
+    uint64_t x_full[2], x_free[2];
+    uint64_t yoff_full, m_full, yd_full, xp_full, dh_full, h_ready, y_free, y_staged;
 };
-
-struct SsdParams {
-    const float *l2;        // [B,H,Lpad] row factors of the decay mask (ssd_scalars.cuh)
-    const TileScalars *rec; // [B,H,Lpad/128] per-tile weights and block ends
-    const float *D;
-    const float *h_in;      // initial states: [B,H,P,N] (nseg == 1) or [B,nseg,H,P,N]; may be null
-    const float *h_first;   // seg_states >= 2: states entering the first segments, [B,H,P,N]; may be null
-    float *h_out;           // ssd_tiles_kernel: h_final [B,H,P,N] (last segment writes) or null
-                            // ssd_state_kernel: local end states [B,nseg,H,P,N]
-    float *seg_decay;       // ssd_state_kernel: [B,nseg,H] product of a_t over the segment
-    int L, Lpad, H, G, nseg, seg_len;
-    int split_tiles;        // > 0 (nseg == 1): every (sequence, head pair) is worked by two CTAs, see
-                            // ssd_tiles_kernel
-    int *d_status;
-    // Packed batch (sequences of different lengths back to back in one [T, ...] array): seqs has one
-    // entry per sequence plus a closing one, items lists the (sequence, segment) pairs of this launch
-    // (grid.x), the scalar arrays are laid out [H, tiles of the batch], and the per-segment state
-    // arrays are indexed by seqs[b].seg0 + segment.  seg_states: h_in / ssd_state_kernel's h_out are those
-    // per-segment arrays (else h_in is [sequences, H, P, N]); 2: a sequence's first segment starts from
-    // h_first instead; 3: so does a sequence of one segment (in-place states: the first of several reads
-    // the scan's copy, since the last one writes over h_first in the same launch).  y: base of the output (ragged last
-    // tiles are stored row by row).  Null seqs: dense [B, L].
-    const SeqDesc *seqs;
-    const int2 *items;
-    int ntile_total, seg_states;
-    void *y;
-    // 1: y and h_out are added to, not overwritten (the slots behind the first of the general form)
-    int add;
-    // 1: x and the initial states are not written by anything in the same call, so that they may be read before
-    // the dependency wait (everything in front of the call has completed when its first kernel runs)
-    int early;
-};
-
-// How a launch divides the work: a CTA per (sequence, head pair, segment); two CTAs per (sequence, head pair), see
-// split_tiles; the items of a packed batch
-enum SsdMode { SSD_DENSE, SSD_SPLIT, SSD_PACKED };
-
 struct __align__(8) SsdBars {
-    uint64_t b_full[B_SLOTS], b_empty[B_SLOTS], c_full, c_empty;
-    uint64_t x_full[X_SLOTS], xp_full[2], xp_free[2], y_staged[Y_BARS];
-    uint64_t rec_free, m_full, g_full, yd_full, dh_full;
-};
-
-// What this kernel keeps of a tile's record: the column weights, the block ends, what follows from them, and the row
-// factors.  Every warp takes what it needs into registers as soon as the record is there, a tile ahead of its
-// use: room for one.
-struct __align__(16) TileRec {
-    float cb[ST], ends[4];
-    TileScalars::Aux aux;
-    float row[ST];
+    uint64_t cb_full, cb_empty, g_full, g_free;
+    HeadBars hd[NHD];
 };
 
 struct __align__(16) SsdSmall {
-    TileRec sc[NHD];         // copied in by the TMA warp
+    TileScalars sc[NHD];     // the current tile's weights and block ends, copied in by the TMA warp
     SsdBars bars;
-    float rest[NCW];         // split launch: per warp, log2 decay over the leading tiles that are left
     uint32_t tmem_slot;
     int abort_flag;
 };
 
-// pairs of heads never straddle a B/C group
-__host__ __device__ inline int pairs_per_group(int H, int G) { return (H / G + NHD - 1) / NHD; }
 }  // namespace
 
 // Stand-alone launch of the step sizes and tile log-decays.
@@ -190,145 +132,69 @@ int launch_wait_selftest(LaunchCtx &ctx, long long limit_cycles, long long *out_
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
+// w . X for units [UB, UE) of one lane's 16 (row block, 16-byte chunk) units of its half of the
+// head dim: x' = w x with the weight given as a two-term bf16 sum (rounded once).  The unit range
+// is known at compile time, so that all loads are issued before the first use.
+template <int UB, int UE>
+__device__ __forceinline__ void scale_units(const uint8_t *s_x, uint8_t *s_xp, const uint32_t *s_wp, int lane, int hf)
+{
+    uint4 xr[UE - UB];
+    uint32_t wp[UE - UB];
+#pragma unroll
+    for (int un = UB; un < UE; ++un) {
+        const int r = (un >> 2) * 32 + lane;
+        wp[un - UB] = s_wp[r];
+        xr[un - UB] = *reinterpret_cast<const uint4 *>(s_x + tc::sw128_offset(r, 4 * hf + (un & 3)));
+    }
+#pragma unroll
+    for (int un = UB; un < UE; ++un) {
+        const int r = (un >> 2) * 32 + lane;
+        const uint32_t hi_u = __byte_perm(wp[un - UB], 0, 0x1010), lo_u = __byte_perm(wp[un - UB], 0, 0x3232);
+        const __nv_bfloat162 w_hi2 = *reinterpret_cast<const __nv_bfloat162 *>(&hi_u);
+        const __nv_bfloat162 w_lo2 = *reinterpret_cast<const __nv_bfloat162 *>(&lo_u);
+        const uint32_t wv[4] = {xr[un - UB].x, xr[un - UB].y, xr[un - UB].z, xr[un - UB].w};
+        uint32_t o[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const __nv_bfloat162 xv = *reinterpret_cast<const __nv_bfloat162 *>(&wv[q]);
+            const __nv_bfloat162 pr = __hfma2(w_hi2, xv, __hmul2(w_lo2, xv));
+            o[q] = *reinterpret_cast<const uint32_t *>(&pr);
+        }
+        *reinterpret_cast<uint4 *>(s_xp + tc::sw128_offset(r, 4 * hf + (un & 3))) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+
+// The same for the four units of the thread's own row (leading tiles), with the row's weight
+// multiplied by `f` first: w' = w f is split again into two bf16 terms.
+__device__ __forceinline__ void scale_own_row(const uint8_t *s_x, uint8_t *s_xp, uint32_t wp, float f, int i, int hf)
+{
+    const float w = (__uint_as_float(wp << 16) + __uint_as_float(wp & 0xffff0000u)) * f;
+    const __nv_bfloat16 w_hi = __float2bfloat16_rn(w);
+    const __nv_bfloat16 w_lo = __float2bfloat16_rn(w - __bfloat162float(w_hi));
+    const __nv_bfloat162 w_hi2 = __halves2bfloat162(w_hi, w_hi), w_lo2 = __halves2bfloat162(w_lo, w_lo);
+    uint4 xr[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) xr[c] = *reinterpret_cast<const uint4 *>(s_x + tc::sw128_offset(i, 4 * hf + c));
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t wv[4] = {xr[c].x, xr[c].y, xr[c].z, xr[c].w};
+        uint32_t o[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const __nv_bfloat162 xv = *reinterpret_cast<const __nv_bfloat162 *>(&wv[q]);
+            const __nv_bfloat162 pr = __hfma2(w_hi2, xv, __hmul2(w_lo2, xv));
+            o[q] = *reinterpret_cast<const uint32_t *>(&pr);
+        }
+        *reinterpret_cast<uint4 *>(s_xp + tc::sw128_offset(i, 4 * hf + c)) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+
 __device__ __forceinline__ uint64_t f32x2_bits(uint32_t a, uint32_t b)
 {
     return tc::f32x2(__uint_as_float(a), __uint_as_float(b));
 }
 
-// Weights of a thread's eight columns (or tokens) of a 32-wide block.
-struct BlockWeights { uint64_t v[4]; };
-__device__ __forceinline__ void load_weights(BlockWeights &w, const float *s_cb, int lane)
-{
-#pragma unroll
-    for (int r = 0; r < 4; ++r) w.v[r] = *reinterpret_cast<const uint64_t *>(s_cb + 8 * r + 2 * (lane & 3));
-}
-
-// w . X of one warp, from the X slab to the A operand of MMA 4 in tensor memory: lanes p0 .. p0+31 (channels of
-// the head), tokens s0 .. s0+31 (16 columns, two to a column).  wx: weights of tokens s0 + 8 c + 2 (t % 4) and
-// the one behind; x' = w x with the weight as a two-term bf16 sum (rounded once).
-__device__ __forceinline__ void scale_to_tmem(const uint8_t *s_x, const BlockWeights &wx, int p0, int s0, int lane,
-                                              uint32_t taddr)
-{
-    uint32_t a[4][4];              // [8 tokens][8 channels], the fragment layout of ldmatrix
-    const uint32_t src = tc::smem_u32(s_x) + tc::sw128_offset(s0 + (lane & 7), (p0 >> 3) + (lane >> 3));
-#pragma unroll
-    for (int c = 0; c < 4; ++c) tc::ldmatrix_x4_trans(src + c * 1024, a[c][0], a[c][1], a[c][2], a[c][3]);
-    const uint64_t minus = tc::f32x2(-1.f, -1.f);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const uint64_t w = wx.v[c];
-        const uint32_t hi_u = tc::f32x2_bf16(w);
-        const uint32_t lo_u = tc::f32x2_bf16(tc::f32x2_fma(f32x2_bits(hi_u << 16, hi_u & 0xffff0000u), minus, w));
-        const __nv_bfloat162 w_hi2 = *reinterpret_cast<const __nv_bfloat162 *>(&hi_u);
-        const __nv_bfloat162 w_lo2 = *reinterpret_cast<const __nv_bfloat162 *>(&lo_u);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const __nv_bfloat162 xv = *reinterpret_cast<const __nv_bfloat162 *>(&a[c][m]);
-            const __nv_bfloat162 pr = __hfma2(w_hi2, xv, __hmul2(w_lo2, xv));
-            a[c][m] = *reinterpret_cast<const uint32_t *>(&pr);
-        }
-    }
-    const uint32_t lo[8] = {a[0][0], a[0][1], a[1][0], a[1][1], a[2][0], a[2][1], a[3][0], a[3][1]};
-    const uint32_t hi[8] = {a[0][2], a[0][3], a[1][2], a[1][3], a[2][2], a[2][3], a[3][2], a[3][3]};
-    tc::tmem_st_16x128b_x4(taddr, lo);
-    tc::tmem_st_16x128b_x4(taddr + (16u << 16), hi);
-}
-
-// Decay mask of a 32 x 32 block in place, M = G cb as bf16 pairs, in the fragment layout: this thread has rows t / 4 + 8 k
-// and columns 8 r + 2 (t % 4) and the one behind, so that it needs 8 weights a head (a row per thread would
-// need all 32, read as broadcasts: a fourth of the kernel's shared-memory wavefronts).  16 columns of G become 8
-// of the first head's M and 8 of the second one's, which is what a K step of MMA 2 takes.  The row factor comes
-// with the epilogue.
-// Entries of rows k = 0, 1 (t / 4 + 8 k) and columns 16 c .. 16 c + 15 for one head: a K step's four registers.  DIAG: the
-// 16 x 16 block on the diagonal; `keep` the bits that a row keeps of the pair in its own 8 x 8 block.
-template <bool DIAG>
-__device__ __forceinline__ void mask_step(uint32_t taddr, const uint32_t (&g)[16], const BlockWeights &w, int c, uint32_t keep)
-{
-    uint32_t o[4];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int e = 4 * (2 * c + r) + 2 * k;
-            o[2 * r + k] = tc::f32x2_bf16(tc::f32x2_mul(f32x2_bits(g[e], g[e + 1]), w.v[2 * c + r]));
-        }
-    if (DIAG) {
-        o[0] &= keep;
-        o[2] = 0u;
-        o[3] &= keep;
-    }
-    tc::tmem_st_16x128b_x2(taddr + 16 * c, o[0], o[1], o[2], o[3]);
-}
-
-template <bool DIAG>
-__device__ __forceinline__ void mask_block(uint32_t taddr, const BlockWeights (&w)[2], uint32_t keep)
-{
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {                    // rows 0 .. 15, 16 .. 31
-        const uint32_t ta = taddr + ((uint32_t)(16 * half) << 16);
-        uint32_t g[16];
-        tc::tmem_ld_16x256b_x4(ta, g);
-        tc::tmem_ld_wait();
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if (!DIAG) {
-                mask_step<false>(ta + 8 * q, g, w[q], 0, 0u);
-                mask_step<false>(ta + 8 * q, g, w[q], 1, 0u);
-            } else if (half == 0) {
-                mask_step<true>(ta + 8 * q, g, w[q], 0, keep);
-                tc::tmem_st_16x128b_x2(ta + 8 * q + 16, 0u, 0u, 0u, 0u);
-            } else {
-                mask_step<false>(ta + 8 * q, g, w[q], 0, 0u);
-                mask_step<true>(ta + 8 * q, g, w[q], 1, keep);
-            }
-        }
-    }
-}
-
-// The same where a 32-token block of a head decays by more than 2^-96 (its diagonal's column weights could overflow):
-// that head's entries carry the row factor, the exponents of a diagonal block are formed entry by entry, all of them
-// <= 0.  Records and row factors (log-decays there) of the tile from global memory: the copy in shared memory
-// belongs to the next tile.
-__device__ __forceinline__ void mask_block_entries(uint32_t taddr, const TileScalars *rec0, const TileScalars *rec1,
-                                                   const float *l2_0, const float *l2_1, int wq, int sub, int lane)
-{
-#pragma unroll 1
-    for (int step = 0; step < 4; ++step) {                    // 16 rows x 16 columns
-        const int half = step >> 1, c = step & 1;
-        const uint32_t ta = taddr + ((uint32_t)(16 * half) << 16) + 16 * c;
-        uint32_t g[8];
-        tc::tmem_ld_16x256b_x2(ta, g);
-        tc::tmem_ld_wait();
-#pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-            const TileScalars *rec = q ? rec1 : rec0;
-            const bool diag = sub == wq;
-            const float Lw = wq ? rec->ends[wq - 1] : 0.f, Lc = rec->ends[sub];      // l before the rows, at the columns' end
-            const int mode = mask_mode(rec->ends, wq);
-            uint32_t o[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {                     // rows k = e % 2, columns 8 (e / 2) ..
-                const int row = 16 * half + (lane >> 2) + 8 * (e & 1), col = 16 * c + 8 * (e >> 1) + 2 * (lane & 3);
-                const float l_i = (q ? l2_1 : l2_0)[32 * wq + row];
-                const float2 cb = *reinterpret_cast<const float2 *>(&rec->cb[32 * sub + col]);
-                float rf = 1.f;
-                if (mode == MASK_BLOCKS) rf = tc::ex2_approx(Lw - Lc);
-                if (mode == MASK_ENTRIES) rf = tc::ex2_approx(l_i - Lw) * tc::ex2_approx(Lw - Lc);
-                float m0 = __uint_as_float(g[2 * e]) * cb.x * rf, m1 = __uint_as_float(g[2 * e + 1]) * cb.y * rf;
-                if (mode == MASK_ENTRIES && diag) {
-                    m0 = __uint_as_float(g[2 * e]) * tc::ex2_approx(l_i - Lc + tc::lg2_approx(cb.x));
-                    m1 = __uint_as_float(g[2 * e + 1]) * tc::ex2_approx(l_i - Lc + tc::lg2_approx(cb.y));
-                }
-                if (diag && col > row) m0 = 0.f;
-                if (diag && col + 1 > row) m1 = 0.f;
-                o[e] = tc::pack_bf16x2(m0, m1);
-            }
-            tc::tmem_st_16x128b_x2(ta + 8 * q, o[0], o[1], o[2], o[3]);
-        }
-    }
-}
-
-template <SsdMode MODE>
+template <bool SPLIT>
 __global__ void __launch_bounds__(SSD_THREADS, 1)
 ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_c,
                  const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_y,
@@ -350,22 +216,22 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
     // sequence but evaluate the first split_tiles tiles for their end state only (about half the
     // cost of a full tile) and produce y from there on; the CTAs of the second plane produce y of
     // those first tiles.  No CTA waits for another.
-    constexpr bool SPLIT = MODE == SSD_SPLIT, packed = MODE == SSD_PACKED;
-    const bool head_part = SPLIT && blockIdx.z == 1;             // y of the leading tiles only
-    int seg = SPLIT ? 0 : blockIdx.x, b = SPLIT ? blockIdx.x : blockIdx.z;
+    constexpr bool split = SPLIT;                                // (prm.split_tiles > 0)
+    const bool head_part = split && blockIdx.z == 1;             // y of the leading tiles only
+    const bool packed = !SPLIT && prm.seqs != nullptr;
+    int seg = split ? 0 : blockIdx.x, b = split ? blockIdx.x : blockIdx.z;
     int L = prm.L, nseg = prm.nseg, tok0 = 0, bco = b;
     const int H = prm.H;
     int seg_base = b * prm.nseg;                     // index of the sequence's first segment
     int64_t rec_base = (int64_t)b * H * (prm.Lpad / ST);   // tile record of head 0, tile 0: + h * rec_hstride
     int rec_hstride = prm.Lpad / ST;
     const int HG = H / prm.G, ppg = pairs_per_group(H, prm.G);
-    int pair = blockIdx.y, item = 0;
+    int pair = blockIdx.y;
     if (packed) {
         // (one grid dimension, the head pair fastest: CTAs start in the order of the items)
         const int npairs = prm.G * ppg;
         pair = blockIdx.x % npairs;
-        item = blockIdx.x / npairs;
-        const int2 it = prm.items[item];
+        const int2 it = prm.items[blockIdx.x / npairs];
         b = it.x; seg = it.y;
         const SeqDesc sd = prm.seqs[b];
         L = sd.len; tok0 = sd.tok0; bco = 0;
@@ -382,30 +248,32 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
     const int ntiles = (t_end - t_begin + ST - 1) / ST;
     // leading tiles that only carry the state forward (tile j is a full tile iff j >= n_pre;
     // barriers that only full tiles use count their phases in full tiles, jf = j - n_pre)
-    const int n_pre = SPLIT ? (head_part ? 0 : min(prm.split_tiles, ntiles)) : 0;
+    const int n_pre = split ? (head_part ? 0 : min(prm.split_tiles, ntiles)) : 0;
 
     if (tid == 0) {
-        for (int s = 0; s < B_SLOTS; ++s) {
-            tc::mbar_init(&bars->b_full[s], 1);
-            tc::mbar_init(&bars->b_empty[s], 1);
-        }
-        tc::mbar_init(&bars->c_full, 1);
-        tc::mbar_init(&bars->c_empty, 1);
-        for (int s = 0; s < X_SLOTS; ++s) tc::mbar_init(&bars->x_full[s], 1);
-        for (int s = 0; s < Y_BARS; ++s) tc::mbar_init(&bars->y_staged[s], NCW);
-        for (int s = 0; s < 2; ++s) {
-            tc::mbar_init(&bars->xp_full[s], NCW);
-            tc::mbar_init(&bars->xp_free[s], 1);
-        }
-        tc::mbar_init(&bars->rec_free, NCW);
-        tc::mbar_init(&bars->m_full, NCW);
+        tc::mbar_init(&bars->cb_full, 1);
+        tc::mbar_init(&bars->cb_empty, 1);
         tc::mbar_init(&bars->g_full, 1);
-        tc::mbar_init(&bars->yd_full, 1);
-        tc::mbar_init(&bars->dh_full, 1);
+        tc::mbar_init(&bars->g_free, HEAD_THREADS * nh);
+        for (int hd = 0; hd < NHD; ++hd) {
+            HeadBars *hb = &bars->hd[hd];
+            for (int s = 0; s < 2; ++s) {
+                tc::mbar_init(&hb->x_full[s], 1);
+                tc::mbar_init(&hb->x_free[s], HEAD_THREADS + 1);
+            }
+            tc::mbar_init(&hb->yoff_full, 1);
+            tc::mbar_init(&hb->m_full, HEAD_THREADS);
+            tc::mbar_init(&hb->yd_full, 1);
+            tc::mbar_init(&hb->xp_full, HEAD_THREADS);
+            tc::mbar_init(&hb->dh_full, 1);
+            tc::mbar_init(&hb->h_ready, HEAD_THREADS);
+            tc::mbar_init(&hb->y_free, HEAD_THREADS);
+            tc::mbar_init(&hb->y_staged, HEAD_THREADS);
+        }
         *abort_flag = 0;
         tc::fence_mbar_init();
     }
-    if (warp == WARP_MMA) {
+    if (warp == WARP_MMA0) {
         tc::tmem_alloc(&sm->tmem_slot, TM_COLS);
         tc::tmem_relinquish();
     }
@@ -424,513 +292,473 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
     // Warp index as a value the compiler knows to be warp-uniform.
     const int uwarp = __shfl_sync(0xffffffffu, warp, 0);
     if (uwarp == WARP_TMA) {
-        // ------------------------------------------------------------------ TMA producer, y stores
+        // ------------------------------------------------------------------ TMA producer
         // (the whole warp runs the loop; one elected lane issues the copies)
         const bool leader = tc::elect_one();
-        auto load_x = [&](int j) {                           // x and, on the same barrier, the tile's record
-            const int s = j % X_SLOTS;
-            tc::mbar_arrive_expect_tx(&bars->x_full[s], nh * (SLAB + (uint32_t)sizeof(TileRec)));
-            for (int hd = 0; hd < nh; ++hd)
-                tc::tma_load_4d(smem + SM_X + (s * NHD + hd) * SLAB, &tmap_x, &bars->x_full[s], 0, head0 + hd,
-                                tok0 + t_begin + j * ST, bco);
+        // record of tile t_begin / ST + j of head head0 + hd
+        auto scal_rec = [&](int hd, int j) {
+            return prm.rec + rec_base + (int64_t)(head0 + hd) * rec_hstride + t_begin / ST + j;
         };
-        auto load_rec = [&](int j) {
-            for (int hd = 0; hd < nh; ++hd) {
-                const int64_t r = rec_base + (int64_t)(head0 + hd) * rec_hstride + t_begin / ST + j;
-                tc::bulk_load(sm->sc[hd].cb, prm.rec[r].cb, (ST + 8) * sizeof(float), &bars->x_full[j % X_SLOTS]);
-                tc::bulk_load(sm->sc[hd].row, prm.l2 + r * ST, ST * sizeof(float), &bars->x_full[j % X_SLOTS]);
-            }
-        };
-        // a stream's tile: Btilde waits for MMA 4 of the tile before the last, Ctilde for the last one's copy
-        auto load_stream = [&](const CUtensorMap *m, int j, uint8_t *dst, uint64_t *full_bar) {
-            tc::mbar_arrive_expect_tx(full_bar, 2 * SLAB);
-            tc::tma_load_3d(dst, m, full_bar, g * SN, tok0 + t_begin + j * ST, bco);
-            tc::tma_load_3d(dst + SLAB, m, full_bar, g * SN + 64, tok0 + t_begin + j * ST, bco);
-        };
-        auto load_b = [&](int j) {
-            const int s = j & 1;
-            tc::mbar_wait(&bars->b_empty[s], ((j >> 1) & 1) ^ 1, abort_flag, d_status);
-            if (leader) load_stream(&tmap_b, j, smem + SM_B + s * 2 * SLAB, &bars->b_full[s]);
-            __syncwarp();
-        };
-        auto load_c = [&](int j) {                           // (full tiles only)
-            const int jf = SPLIT ? j - n_pre : j;
-            tc::mbar_wait(&bars->c_empty, (jf & 1) ^ 1, abort_flag, d_status);
-            if (leader) load_stream(&tmap_c, j, smem + SM_C, &bars->c_full);
-            __syncwarp();
-        };
-        // the y tiles staged over x of tile j (rows past the end of the sequence are clipped by the tensor map; packed
-        // batch: a tile that runs past the end of its sequence is stored row by row by the compute warps, the
-        // rows behind it belong to the next sequence)
-        auto store_y = [&](int j) {
-            const int jf = SPLIT ? j - n_pre : j;
-            tc::mbar_wait(&bars->y_staged[jf % Y_BARS], (jf / Y_BARS) & 1, abort_flag, d_status);
-            if (leader && !(packed && t_begin + (j + 1) * ST > L)) {
-                for (int q = 0; q < nh; ++q) {
-                    const uint8_t *s_y = smem + SM_X + ((j % X_SLOTS) * NHD + q) * SLAB;
-                    if (prm.add) tc::tma_reduce_add_4d(&tmap_y, s_y, 0, head0 + q, tok0 + t_begin + j * ST, bco);
-                    else tc::tma_store_4d(&tmap_y, s_y, 0, head0 + q, tok0 + t_begin + j * ST, bco);
-                }
-                tc::bulk_commit_group();
-            }
-            __syncwarp();
-        };
-        const int ahead = min(X_SLOTS, ntiles);
         if (!prm.early) grid_dep_wait();
-        if (leader)
-            for (int j = 0; j < ahead; ++j) load_x(j);
+        if (leader && ntiles > 0) {
+            for (int hd = 0; hd < nh; ++hd) {               // X of tile 0
+                HeadBars *hb = &bars->hd[hd];
+                tc::mbar_arrive_expect_tx(&hb->x_full[0], SLAB + (uint32_t)sizeof(TileScalars));
+                tc::tma_load_4d(smem + SM_HEAD + hd * SM_HEAD_BYTES, &tmap_x, &hb->x_full[0], 0,
+                                head0 + hd, tok0 + t_begin, bco);
+            }
+        }
         if (prm.early) grid_dep_wait();
-        if (leader)
-            if (ntiles > 0) load_rec(0);
-        __syncwarp();
-        if (ntiles > 0) load_b(0);
-        if (ntiles > 0 && n_pre == 0) load_c(0);
-        if (ntiles > 1) {
-            load_b(1);
-            tc::mbar_wait(&bars->rec_free, 0, abort_flag, d_status);
-            if (leader) load_rec(1);
-            __syncwarp();
-        }
-        for (int j = 0; j < ntiles; ++j) {                   // while tile j is worked
-            if (j + 1 < ntiles && (!SPLIT || j + 1 >= n_pre)) load_c(j + 1);
-            // the tile in front gives back its x slot: a full one once its y has gone out, a leading one once its
-            // w.X is done
-            if (j > 0) {
-                if (!SPLIT || j > n_pre) store_y(j - 1);
-                else tc::mbar_wait(&bars->xp_full[(j - 1) & 1], ((j - 1) >> 1) & 1, abort_flag, d_status);
+        if (leader && ntiles > 0) {
+            for (int hd = 0; hd < nh; ++hd) {               // its scalars
+                HeadBars *hb = &bars->hd[hd];
+                tc::bulk_load(&sm->sc[hd], scal_rec(hd, 0), (uint32_t)sizeof(TileScalars), &hb->x_full[0]);
             }
-            if (j + 2 < ntiles) load_b(j + 2);
-            if (leader && j > 0 && j - 1 + X_SLOTS < ntiles) {
-                tc::bulk_wait_read_all();
-                load_x(j - 1 + X_SLOTS);
-            }
-            __syncwarp();
-            if (j + 2 < ntiles) {                            // (the next tile's record has been taken)
-                tc::mbar_wait(&bars->rec_free, (j + 1) & 1, abort_flag, d_status);
-                if (leader) load_rec(j + 2);
-                __syncwarp();
-            }
-        }
-        if (ntiles > n_pre) store_y(ntiles - 1);
-        if (leader) tc::bulk_wait_read_all();
-    } else if (uwarp == WARP_MMA) {
-        // ------------------------------------------------------------------ MMA issuer
-        // The whole warp runs the loop and the waits; one elected lane issues the MMAs and the
-        // commits.  One warp issues every product: they run in the order of issue, which the
-        // regions of tensor memory that follow one another in the same columns rely on.
-        grid_dep_wait();
-        const bool leader = tc::elect_one();
-        // The products against the shared Ctilde / Btilde tiles (MMA 1, 3, 4) are issued for both heads at once:
-        // the shared operand is read from shared memory once instead of once per head.
-        constexpr uint32_t id_g = tc::idesc_bf16(128, 128, 0, 0);         // C (TMEM) x B (K-major)
-        constexpr uint32_t id_x = tc::idesc_bf16(128, 64, 0, 1);          // M (TMEM) x X (MN-major)
-        constexpr uint32_t id_h = tc::idesc_bf16(128, 128, 0, 1);         // w.X (TMEM) x B (MN-major)
-        const uint32_t id_y = nh == 2 ? tc::idesc_bf16(128, 128, 0, 0) : tc::idesc_bf16(128, 64, 0, 0);   // C (TMEM) x H, K-major
-        const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
-        // descriptors of the first K step; later steps and slots advance the address field
-        const uint64_t dC = tc::smem_desc_sw128(tc::smem_u32(smem + SM_C), 16, 1024);        // K-major
-        const uint64_t dB = tc::smem_desc_sw128(tc::smem_u32(smem + SM_B), 16, 1024);        // K-major
-        const uint64_t dBt = tc::smem_desc_sw128(tc::smem_u32(smem + SM_B), SLAB, 1024);     // MN-major
-        const uint64_t dH = tc::smem_desc_sw128(tc::smem_u32(smem + SM_H), 16, 1024);
-        const uint64_t dX0 = tc::smem_desc_sw128(tc::smem_u32(smem + SM_X), SLAB, 1024);
-        // MMA 1 of tile j: G = Ctilde Btilde^T (K = state index), for both heads, over the masked tile in front of it.
-        // Ctilde is copied to tensor memory first, as soon as MMA 3 of the tile in front has read the last one:
-        // MMA 1 and MMA 3 would each read it from shared memory.
-        auto copy_c = [&](int j) {
-            const int jf = SPLIT ? j - n_pre : j;
-            tc::mbar_wait(&bars->c_full, jf & 1, abort_flag, d_status);
-            tc::tc_fence_after();
-            if (leader) {
-                const uint64_t d = tc::smem_desc_fresh(dC);
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk)
-                    tc::tmem_copy_128x256b(tmem_u + TM_C + kk * 8, tc::smem_desc_advance(d, (kk >> 2) * SLAB + (kk & 3) * 32));
-                tc::mma_commit(&bars->c_empty);
-            }
-            __syncwarp();
-        };
-        auto issue_g = [&](int j) {
-            tc::mbar_wait(&bars->b_full[j & 1], (j >> 1) & 1, abort_flag, d_status);
-            tc::tc_fence_after();
-            if (leader) {
-                const uint64_t d = tc::smem_desc_fresh(tc::smem_desc_advance(dB, (j & 1) * 2 * SLAB));
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk)
-                    tc::mma_ts(tmem_u + TM_G, tmem_u + TM_C + kk * 8,
-                               tc::smem_desc_advance(d, (kk >> 2) * SLAB + (kk & 3) * 32), id_g, kk > 0);
-                tc::mma_commit(&bars->g_full);
-            }
-            __syncwarp();
-        };
-        if (n_pre == 0 && ntiles > 0) {
-            copy_c(0);
-            issue_g(0);
         }
         for (int j = 0; j < ntiles; ++j) {
+            const int t0 = tok0 + t_begin + j * ST;
             const bool full = !SPLIT || j >= n_pre;
-            const int jf = SPLIT ? j - n_pre : j;
-            if (!full) tc::mbar_wait(&bars->b_full[j & 1], (j >> 1) & 1, abort_flag, d_status);
-            // MMA 4: dH[p,n] = sum_s (w_s x_s[p]) Btilde[s,n]   (K = token; A = w.X in TMEM, both heads' channels).  It
-            // and MMA 1 run ahead: under the epilogue of the tile in front.
-            tc::mbar_wait(&bars->xp_full[j & 1], (j >> 1) & 1, abort_flag, d_status);
-            tc::tc_fence_after();
+            tc::mbar_wait(&bars->cb_empty, (j & 1) ^ 1, abort_flag, d_status);
             if (leader) {
-                const uint64_t d = tc::smem_desc_fresh(tc::smem_desc_advance(dBt, (j & 1) * 2 * SLAB));
-                const uint32_t xp = tmem_u + (!full && (j & 1) ? TM_Y : TM_XP);
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk)             // (leading tiles accumulate)
-                    tc::mma_ts(tmem_u + TM_DH, xp + kk * 8, tc::smem_desc_advance(d, kk * 2048),
-                               id_h, (kk > 0) || (!full && j > 0));
-                if (j == n_pre - 1) tc::mma_commit(&bars->dh_full);
-                if (!full) tc::mma_commit(&bars->xp_free[j & 1]);
-                tc::mma_commit(&bars->b_empty[j & 1]);
+                tc::mbar_arrive_expect_tx(&bars->cb_full, full ? 4 * SLAB : 2 * SLAB);
+                if (full) {
+                    tc::tma_load_3d(smem + SM_CB + 0 * SLAB, &tmap_c, &bars->cb_full, g * SN, t0, bco);
+                    tc::tma_load_3d(smem + SM_CB + 1 * SLAB, &tmap_c, &bars->cb_full, g * SN + 64, t0, bco);
+                }
+                tc::tma_load_3d(smem + SM_CB + 2 * SLAB, &tmap_b, &bars->cb_full, g * SN, t0, bco);
+                tc::tma_load_3d(smem + SM_CB + 3 * SLAB, &tmap_b, &bars->cb_full, g * SN + 64, t0, bco);
+            }
+            if (j + 1 < ntiles) {                            // X one tile ahead
+                const int jn = j + 1, sx = jn & 1;
+                for (int hd = 0; hd < nh; ++hd) {
+                    HeadBars *hb = &bars->hd[hd];
+                    tc::mbar_wait(&hb->x_free[sx], ((jn >> 1) & 1) ^ 1, abort_flag, d_status);
+                    if (leader) {
+                        tc::mbar_arrive_expect_tx(&hb->x_full[sx], SLAB + (uint32_t)sizeof(TileScalars));
+                        tc::tma_load_4d(smem + SM_HEAD + hd * SM_HEAD_BYTES + sx * SLAB, &tmap_x,
+                                        &hb->x_full[sx], 0, head0 + hd, t0 + ST, bco);
+                    }
+                }
+                // scalars of the next tile: the record buffer is single; its last readers are the
+                // mask (full tile) or the w.X scaling (leading tile) of this tile
+                for (int hd = 0; hd < nh; ++hd) {
+                    HeadBars *hb = &bars->hd[hd];
+                    if (full) tc::mbar_wait(&hb->m_full, (SPLIT ? j - n_pre : j) & 1, abort_flag, d_status);
+                    else tc::mbar_wait(&hb->xp_full, j & 1, abort_flag, d_status);
+                    if (leader)
+                        tc::bulk_load(&sm->sc[hd], scal_rec(hd, jn), (uint32_t)sizeof(TileScalars), &hb->x_full[sx]);
+                }
             }
             __syncwarp();
-            if (full) {
-                // MMA 3: Y = Ctilde Hprev^T  (K = state index; B = bf16 states, rows = channels; they are stored before
-                // w.X of this tile), once the tile in front has read its Y
-                if (jf > 0) tc::mbar_wait(&bars->y_staged[(jf - 1) % Y_BARS], ((jf - 1) / Y_BARS) & 1, abort_flag, d_status);
+        }
+    } else if (uwarp >= WARP_MMA0) {
+        // ------------------------------------------------------------------ MMA issuers
+        // The whole warp runs the loop and the waits; one elected lane issues the MMAs, the
+        // commits and the y stores.
+        grid_dep_wait();
+        const int hd = uwarp - WARP_MMA0;
+        const bool leader = tc::elect_one();
+        if (hd < nh) {
+            // The products against the shared Ctilde / Btilde tiles (MMA 1, 3, 4) are issued by the
+            // first issuer for both heads at once: with N = 128 the shared operand is read from
+            // shared memory once instead of once per head.  MMA 2 and the y store stay per head.
+            constexpr uint32_t id_g = tc::idesc_bf16(128, 128, 0, 0);     // C (K-major) x B (K-major)
+            constexpr uint32_t id_y = tc::idesc_bf16(128, 64, 0, 1);      // K-major / TMEM A, MN-major B
+            const uint32_t id_yn = nh == 2 ? tc::idesc_bf16(128, 128, 0, 1) : id_y;
+            const uint32_t id_hn = nh == 2 ? tc::idesc_bf16(128, 128, 1, 1) : tc::idesc_bf16(128, 64, 1, 1);
+            HeadBars *hb = &bars->hd[hd];
+            const uint32_t c_addr = tc::smem_u32(smem + SM_CB), b_addr = c_addr + 2 * SLAB;
+            const uint32_t head0_addr = tc::smem_u32(smem + SM_HEAD);
+            const uint32_t head_addr = head0_addr + hd * SM_HEAD_BYTES;
+            const uint8_t *s_y = smem + SM_HEAD + hd * SM_HEAD_BYTES + 4 * SLAB;
+            const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
+            const uint32_t tm = tmem_u + TM_HEAD + hd * TM_HEAD_COLS;
+            // descriptors of the first K step; later steps advance the address field
+            const uint64_t dC = tc::smem_desc_sw128(c_addr, 16, 1024);          // K-major
+            const uint64_t dB = tc::smem_desc_sw128(b_addr, 16, 1024);          // K-major
+            const uint64_t dBt = tc::smem_desc_sw128(b_addr, SLAB, 1024);       // MN-major
+            // MN-major operands over both heads: the second head's 64 columns lie one head region on
+            const uint64_t dH = tc::smem_desc_sw128(head0_addr + 3 * SLAB, SM_HEAD_BYTES, 1024);
+            const uint64_t dXp = tc::smem_desc_sw128(head0_addr + 2 * SLAB, SM_HEAD_BYTES, 1024);
+            const uint64_t dX0 = tc::smem_desc_sw128(head_addr, SLAB, 1024);    // MN-major
+            // MMA 1 of tile jj: G = Ctilde Btilde^T (K = state index), shared by both heads
+            auto issue_g = [&](int jj) {
+                tc::mbar_wait(&bars->cb_full, jj & 1, abort_flag, d_status);
+                const int jjf = SPLIT ? jj - n_pre : jj;
+                if (jjf > 0) tc::mbar_wait(&bars->g_free, (jjf - 1) & 1, abort_flag, d_status);
                 tc::tc_fence_after();
                 if (leader) {
-                    const uint64_t d = tc::smem_desc_fresh(dH);
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        tc::mma_ts(tmem_u + TM_Y, tmem_u + TM_C + kk * 8,
-                                   tc::smem_desc_advance(d, (kk >> 2) * SLAB + (kk & 3) * 32), id_y, kk > 0);
-                    tc::mma_commit(&bars->dh_full);          // (MMA 4 and 3: the state may be advanced, its copy replaced)
+                    for (int kk = 0; kk < 8; ++kk) {
+                        const uint32_t off = (kk >> 2) * SLAB + (kk & 3) * 32;
+                        tc::mma_ss(tmem_u + TM_G, tc::smem_desc_advance(dC, off),
+                                   tc::smem_desc_advance(dB, off), id_g, kk > 0);
+                    }
+                    tc::mma_commit(&bars->g_full);
                 }
                 __syncwarp();
-                if (j + 1 < ntiles) copy_c(j + 1);
-                // MMA 2: Y += M X per head (A = masked tile in TMEM, 16 tokens every 16 columns)
-                tc::mbar_wait(&bars->m_full, jf & 1, abort_flag, d_status);
-                tc::tc_fence_after();
-                if (leader) {
-                    for (int q = 0; q < nh; ++q) {
-                        const uint64_t dX = tc::smem_desc_fresh(tc::smem_desc_advance(dX0, ((j % X_SLOTS) * NHD + q) * SLAB));
+            };
+            if (hd == 0 && n_pre == 0 && ntiles > 0) issue_g(0);
+            for (int j = 0; j < ntiles; ++j) {
+                const int sx = j & 1;
+                const bool full = !SPLIT || j >= n_pre;
+                const int jf = SPLIT ? j - n_pre : j;
+                if (hd == 0) {
+                    tc::mbar_wait(&bars->cb_full, j & 1, abort_flag, d_status);
+                    tc::tc_fence_after();
+                    if (full) {
+                        // MMA 3: Y = Ctilde Hprev^T  (K = state index; B = bf16 states, rows = n)
+                        for (int q = 0; q < nh; ++q) {
+                            tc::mbar_wait(&bars->hd[q].h_ready, jf & 1, abort_flag, d_status);
+                            if (jf > 0) tc::mbar_wait(&bars->hd[q].y_free, (jf - 1) & 1, abort_flag, d_status);
+                        }
+                        tc::tc_fence_after();
+                        if (leader) {
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk) {
+                                const uint32_t off = (kk >> 2) * SLAB + (kk & 3) * 32;
+                                tc::mma_ss(tmem_u + TM_Y, tc::smem_desc_advance(dC, off),
+                                           tc::smem_desc_advance(dH, kk * 2048), id_yn, kk > 0);
+                            }
+                            for (int q = 0; q < nh; ++q) tc::mma_commit(&bars->hd[q].yoff_full);
+                        }
+                        __syncwarp();
+                    }
+                    // MMA 4: dH^T[n,p] = sum_s Btilde[s,n] (w_s x_s[p])   (K = token)
+                    for (int q = 0; q < nh; ++q)
+                        tc::mbar_wait(&bars->hd[q].xp_full, j & 1, abort_flag, d_status);
+                    tc::tc_fence_after();
+                    if (leader) {
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)     // (leading tiles accumulate)
+                            tc::mma_ss(tmem_u + TM_DH, tc::smem_desc_advance(dBt, kk * 2048),
+                                       tc::smem_desc_advance(dXp, kk * 2048), id_hn, (kk > 0) || (!full && j > 0));
+                        for (int q = 0; q < nh; ++q) tc::mma_commit(&bars->hd[q].dh_full);
+                        tc::mma_commit(&bars->cb_empty);     // C and B tiles are no longer needed
+                    }
+                    __syncwarp();
+                }
+                if (full) {
+                    // MMA 2: Y += M X  (A = masked tile in TMEM, 8 columns per 16 tokens of K)
+                    tc::mbar_wait(&hb->m_full, jf & 1, abort_flag, d_status);
+                    tc::tc_fence_after();
+                    const uint64_t dX = tc::smem_desc_advance(dX0, sx * SLAB);
+                    if (leader) {
+                        tc::bulk_wait_read_all();        // previous y tile has left its staging buffer
 #pragma unroll
                         for (int kk = 0; kk < 8; ++kk)
-                            tc::mma_ts(tmem_u + TM_Y + q * 64, tmem_u + TM_G + kk * 16 + q * 8,
-                                       tc::smem_desc_advance(dX, kk * 2048), id_x, 1);
+                            tc::mma_ts(tm + TM_Y, tm + TM_M + kk * 8, tc::smem_desc_advance(dX, kk * 2048),
+                                       id_y, 1);
+                        tc::mma_commit(&hb->yd_full);
                     }
-                    tc::mma_commit(&bars->yd_full);
                 }
+                // MMA 1 of the next tile needs no state: it runs under this tile's state update and
+                // epilogue, and the next tile's mask is built while MMA 3 is still waiting for them
+                if (hd == 0 && j + 1 < ntiles && j + 1 >= n_pre) issue_g(j + 1);
+                // (leading tiles: the second issuer has no product of its own; it follows the tile loop at
+                // the pace of its head's w.X scaling, whose end frees the X slot)
+                if (!full && hd > 0) tc::mbar_wait(&hb->xp_full, j & 1, abort_flag, d_status);
+                if (leader) tc::mma_commit(&hb->x_free[sx]);
                 __syncwarp();
+                if (full) {
+                    // the staged y tile goes out as one TMA store (rows past the end of the
+                    // sequence are clipped by the tensor map)
+                    // (packed batch: a tile that runs past the end of its sequence is stored row by row
+                    // by the compute warps, the rows behind it belong to the next sequence)
+                    tc::mbar_wait(&hb->y_staged, jf & 1, abort_flag, d_status);
+                    if (leader && !(packed && t_begin + (j + 1) * ST > L)) {
+                        if (prm.add) tc::tma_reduce_add_4d(&tmap_y, s_y, 0, head0 + hd, tok0 + t_begin + j * ST, bco);
+                        else tc::tma_store_4d(&tmap_y, s_y, 0, head0 + hd, tok0 + t_begin + j * ST, bco);
+                        tc::bulk_commit_group();
+                    }
+                    __syncwarp();
+                }
             }
-            // MMA 1 of the next tile needs no state
-            if (j + 1 < ntiles && j + 1 >= n_pre) {
-                if (!full) copy_c(j + 1);
-                issue_g(j + 1);
-            }
+            if (leader) tc::bulk_wait_read_all();
         }
-    } else {
+    } else if ((uwarp >> 3) < nh) {
         // ------------------------------------------------------------------ compute warps
-        // Warp (row block wq, share sub).  State and w.X: 32 channels of head wq / 2, the share 32 state indices / 32
-        // tokens.  Mask: a block of 32 rows and 32 columns, both heads.  Epilogue: row i is a
-        // token, the share one half of one head's channels.
-        const int wq = uwarp & 3, sub = uwarp >> 2;
-        const int i = wq * 32 + lane;
-        const int hs = wq >> 1;                              // state: head of the pair
-        const int he = sub >> 1, hf = sub & 1;               // epilogue: head of the pair, half of its channels
-        const bool has_s = hs < nh, has_e = he < nh;
-        const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
-        const uint32_t tm_g = lane_base + TM_G + 32 * sub, tm_y = lane_base + TM_Y + 32 * sub;
-        const uint32_t tm_dh = lane_base + TM_DH + 32 * sub;
-        // 16-byte chunk c of this thread's part of row i, in the x and y slabs: base ^ 16 c
-        const uint32_t row_off = tc::sw128_offset(i, 4 * hf);
-        // of a pair of columns c, c + 1 = 2 (t % 4) of an 8 x 8 diagonal block, the bf16 halves that row t / 4 keeps
-        const int below = (lane >> 2) - 2 * (lane & 3);
-        const uint32_t keep = below < 0 ? 0u : (below == 0 ? 0xffffu : 0xffffffffu);
-        const float Dh = prm.D && has_e ? prm.D[head0 + he] : 0.f;
-        auto arrive = [&](uint64_t *bar) {                   // one arrival per warp, behind all lanes' work
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(bar);
-        };
-        // fp32 master copy of the state, rows (channels) 32 wq .. and columns (state indices) 32 sub .. in the fragment
-        // layout: pair 8 m + 4 k + r is row 16 m + 8 k + t / 4, columns 8 r + 2 (t % 4) and the one behind.  (A row per
-        // thread makes every access to the states in global memory touch 32 lines: 3 us at either end of a CTA.)
+        const int hd = warp >> 3, hf = (warp >> 2) & 1, wq = warp & 3;
+        const int h = head0 + hd;
+        const int i = wq * 32 + lane;                        // token row in the tile == state index n
+        const int p0 = 32 * hf;                              // this thread's half of the head dim
+        HeadBars *hb = &bars->hd[hd];
+        uint8_t *s_head = smem + SM_HEAD + hd * SM_HEAD_BYTES;
+        uint8_t *s_xp = s_head + 2 * SLAB, *s_hb = s_head + 3 * SLAB, *s_y = s_head + 4 * SLAB;
+        const uint32_t *s_wp = sm->sc[hd].wp;
+        const float *s_cb = sm->sc[hd].cb, *s_ends = sm->sc[hd].ends;
+        const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
+        const uint32_t tm = tmem + TM_HEAD + hd * TM_HEAD_COLS + lane_base;
+        const float Dh = prm.D ? prm.D[h] : 0.f;
+        const uint64_t Dh2 = tc::f32x2(Dh, Dh);
+        // fp32 master copy of the state: this thread holds H[n = i][p = p0 .. p0+31], two to a register pair
         uint64_t Hst[16];
-        // its bf16 copy, MMA 3 operand of the next tile, decayed by f
-        const uint32_t s_h = tc::smem_u32(smem + SM_H + (sub >> 1) * SLAB) +
-                             tc::sw128_offset(32 * wq + (lane & 7), 4 * hf + (lane >> 3));
-        auto store_h = [&](float f) {
-            const uint64_t f2 = tc::f32x2(f, f);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t o[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) o[r] = tc::f32x2_bf16(tc::f32x2_mul(f2, Hst[4 * q + r]));
-                tc::stmatrix_x4(s_h + q * 1024, o[0], o[1], o[2], o[3]);
-            }
-            tc::fence_proxy_async_smem();
-        };
-        // offset of pair 8 m + 4 k + r inside the pair of heads' states, from this thread's first one
-        auto h_off = [&](int e) { return 8 * (e >> 2) * SN + 8 * (e & 3); };
-        const int h_mine = (32 * (wq & 1) + (lane >> 2)) * SN + 32 * sub + 2 * (lane & 3);
         {
             const bool first = seg == 0 && (prm.seg_states == 2 || (prm.seg_states == 3 && nseg == 1));
             const float *h_in = first ? prm.h_first : prm.h_in;
             // (states of earlier segments come from the scan in front; given ones go past L1)
             const bool wait = !prm.early || (prm.seg_states && !first);
             if (wait) grid_dep_wait();
+            if (h_in) {
+                const int64_t base = (prm.seg_states && !first)
+                    ? ((((int64_t)seg_base + seg) * H + h) * SP) * SN
+                    : (((int64_t)b * H + h) * SP) * SN;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) Hst[q] = 0;
-            if (h_in && has_s) {
-                const int64_t row = (prm.seg_states && !first) ? ((int64_t)seg_base + seg) * H + head0 + hs
-                                                               : (int64_t)b * H + head0 + hs;
-                const float *src = h_in + row * SP * SN + h_mine;
+                for (int q = 0; q < 16; ++q)
+                    Hst[q] = tc::f32x2(__ldcg(h_in + base + (int64_t)(p0 + 2 * q) * SN + i),
+                                       __ldcg(h_in + base + (int64_t)(p0 + 2 * q + 1) * SN + i));
+            } else {
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const float2 v = __ldcg(reinterpret_cast<const float2 *>(src + h_off(e)));
-                    Hst[e] = tc::f32x2(v.x, v.y);
-                }
+                for (int q = 0; q < 16; ++q) Hst[q] = 0;
             }
+            if (n_pre == 0) {
+                // bf16 copy of the state the first tile starts from
+#pragma unroll
+                for (int ch = 0; ch < 4; ++ch) {
+                    uint4 v = make_uint4(tc::f32x2_bf16(Hst[4 * ch]), tc::f32x2_bf16(Hst[4 * ch + 1]),
+                                         tc::f32x2_bf16(Hst[4 * ch + 2]), tc::f32x2_bf16(Hst[4 * ch + 3]));
+                    *reinterpret_cast<uint4 *>(s_hb + tc::sw128_offset(i, 4 * hf + ch)) = v;
+                }
+                tc::fence_proxy_async_smem();
+                tc::mbar_arrive(&hb->h_ready);
+            }
+            // blocks of M above the diagonal stay zero for the whole kernel
+            uint32_t zero[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) zero[q] = 0u;
+            for (int c = wq + 1; c < 4; ++c) tc::tmem_st8(tm + TM_M + c * 16 + 8 * hf, zero);
+            tc::tmem_st_wait();
         }
         grid_dep_wait();         // the step sizes, the streams
+        const int64_t rec_row = rec_base + (int64_t)h * rec_hstride;     // tile 0 of this (sequence, head)
+        const float *l2p = prm.l2 + rec_row * ST + t_begin;
+        float l2_next = ntiles > 0 ? l2p[i] : 0.f;
         // The leading tiles of a split launch are one long contraction: with every token weighted by its
-        // decay up to the END OF THE RUN (exponent <= 0), (w . X)^T Btilde accumulates over all tiles of
+        // decay up to the END OF THE RUN (exponent <= 0), Btilde^T (w . X) accumulates over all tiles of
         // the run in tensor memory and the state is touched once, at the run's last tile:
-        //   H_end = 2^(sum of l_last over the run) H_in + sum_tiles (w' . X)^T Btilde.
-        if (SPLIT && n_pre > 0 && has_s) {
-            const TileScalars *rec0 = prm.rec + rec_base + (int64_t)(head0 + hs) * rec_hstride + t_begin / ST;
-            float rest = 0.f;
-            for (int jr = 0; jr < n_pre; ++jr) rest += rec0[jr].ends[3];
-            const float dec = tc::ex2_approx(rest);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) Hst[q] = tc::f32x2_mul(Hst[q], tc::f32x2(dec, dec));
-            sm->rest[uwarp] = rest;
-            __syncwarp();
+        //   H_end = 2^(sum of l_last over the run) H_in + sum_tiles Btilde^T (w' . X).
+        const int run_end = n_pre;
+        float run_total = 0.f;   // log2 decay over the whole run
+        {
+            const TileScalars *rec0 = prm.rec + rec_row + t_begin / ST;
+            for (int jr = 0; jr < run_end; ++jr) run_total += rec0[jr].ends[3];
         }
+        float run_done = 0.f;    // ... over the tiles of the run up to and including the current one
 
-        // What a tile's record means for this thread, taken when the record arrives:
-        struct Prep {
-            BlockWeights w[2];     // mask: weights of its columns, both heads
-            BlockWeights wx;       // w.X: weights of its tokens (the same ones)
-            float dec;             // decay of the state over the tile
-            float row;             // epilogue: y = row Y + D x
-            float pre;             // != 1: Y = Ctilde Hprev^T is multiplied by it before M X is added
-            bool entries;          // (MASK_ENTRIES for one of the heads)
-        };
-        const TileRec *const sc0 = &sm->sc[0], *const sc1 = &sm->sc[nh - 1];
-        const TileRec *const scs = hs ? sc1 : sc0, *const sce = he ? sc1 : sc0;
-        auto take_rec = [&](int j, Prep &p) {
-            const bool blocks0 = sc0->aux.blocks != 0.f, blocks1 = sc1->aux.blocks != 0.f;
-            load_weights(p.w[0], sc0->cb + 32 * sub, lane);
-            load_weights(p.w[1], sc1->cb + 32 * sub, lane);
-            p.row = sce->row[i];
-            p.dec = scs->aux.total;
-            // from where the column weights refer to, to the end of the tile (leading tile: of the run)
-            float f = scs->aux.from_ref;
-            if (hs ? blocks1 : blocks0) f = tc::ex2_approx(scs->ends[3] - scs->ends[sub]);
-            if (SPLIT && j < n_pre) {
-                const float rest = sm->rest[uwarp] - scs->ends[3];
-                __syncwarp();
-                sm->rest[uwarp] = rest;
-                f *= tc::ex2_approx(rest);
-                p.dec = 1.f;
-            }
-            const uint64_t f2 = tc::f32x2(f, f);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) p.wx.v[r] = tc::f32x2_mul(f2, hs ? p.w[1].v[r] : p.w[0].v[r]);
-            p.pre = 1.f;
-            p.entries = false;
-            if (blocks0 || blocks1) {
-                const int m0 = mask_mode(sc0->ends, wq), m1 = mask_mode(sc1->ends, wq), me = he ? m1 : m0;
-                const float Lw0 = wq ? sc0->ends[wq - 1] : 0.f, Lw1 = wq ? sc1->ends[wq - 1] : 0.f;
-                const float f0 = m0 == MASK_BLOCKS ? tc::ex2_approx(Lw0 - sc0->ends[sub]) : 1.f;
-                const float f1 = m1 == MASK_BLOCKS ? tc::ex2_approx(Lw1 - sc1->ends[sub]) : 1.f;
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    p.w[0].v[r] = tc::f32x2_mul(p.w[0].v[r], tc::f32x2(f0, f0));
-                    p.w[1].v[r] = tc::f32x2_mul(p.w[1].v[r], tc::f32x2(f1, f1));
-                }
-                if (me == MASK_BLOCKS) p.pre = tc::ex2_approx(he ? Lw1 : Lw0);
-                if (me == MASK_ENTRIES) { p.pre = tc::ex2_approx(p.row); p.row = 1.f; }
-                p.entries = m0 == MASK_ENTRIES || m1 == MASK_ENTRIES;
-            }
-            tc::fence_proxy_async_smem();                    // (the record is refilled by a copy next)
-            arrive(&bars->rec_free);
-        };
-        // w . X of tile j (rows of the X slab -> A operand of MMA 4)
-        auto scale_x = [&](int j, int sx, const BlockWeights &wx) {
-            uint32_t xp = lane_base + 16 * sub + TM_XP;
-            const bool lead = SPLIT && j < n_pre;
-            if (lead) {
-                if (j & 1) xp += TM_Y - TM_XP;
-                // (its columns are free once the product before the previous tile's has read them)
-                if (j > 1) tc::mbar_wait(&bars->xp_free[j & 1], ((j >> 1) & 1) ^ 1, abort_flag, d_status);
-                tc::tc_fence_after();
-            }
-            if (has_s) scale_to_tmem(smem + SM_X + (sx * NHD + hs) * SLAB, wx, 32 * (wq & 1), 32 * sub, lane, xp);
-            if (lead) tc::fence_proxy_async_smem();          // (the x slot is refilled by a copy next)
-            tc::tmem_st_wait();
-            tc::tc_fence_before();
-            arrive(&bars->xp_full[j & 1]);
-        };
-        Prep cur;
-        if (ntiles > 0) {
-            tc::mbar_wait(&bars->x_full[0], 0, abort_flag, d_status);
-            if (n_pre == 0) store_h(scs->aux.to_ref);
-            take_rec(0, cur);
-            scale_x(0, 0, cur.wx);
-        }
-
-        int sx = 0, sx_next = 0;                             // x slots of this tile and of the next one
-        uint32_t x_ph = 0;
-        for (int j = 0; j < ntiles; ++j, sx = sx_next) {
-            sx_next = sx + 1;
-            if (sx_next == X_SLOTS) { sx_next = 0; x_ph ^= 1; }
+        for (int j = 0; j < ntiles; ++j) {
+            const int sx = j & 1;
             const bool full = !SPLIT || j >= n_pre;
+            const bool hb_next = !SPLIT || j + 1 >= n_pre;                    // the next tile reads the bf16 state copy
             const int jf = SPLIT ? j - n_pre : j;
-            const uint32_t dh_ph = (full ? jf + (SPLIT && n_pre > 0 ? 1 : 0) : 0) & 1;
+            const uint8_t *s_x = s_head + sx * SLAB;
+            // ---- per-token scalars: this row's cumulative log2 decay inside the tile (prefetched);
+            // the weights of all rows and the block ends arrive in shared memory
+            const float l2 = l2_next;
+            if (j + 1 < ntiles) l2_next = l2p[(j + 1) * ST + i];
+            tc::mbar_wait(&hb->x_full[sx], (j >> 1) & 1, abort_flag, d_status);
+            const float4 ends = *reinterpret_cast<const float4 *>(s_ends);
+            const float L1 = ends.x, L2 = ends.y, L3 = ends.z, l2_last = ends.w;
+            const float Lw = wq == 0 ? 0.f : (wq == 1 ? L1 : (wq == 2 ? L2 : L3));    // l before my block
+            const float Lend = wq == 0 ? L1 : (wq == 1 ? L2 : (wq == 2 ? L3 : l2_last));  // l at its end
+
+            // ---- w . X  (rows of the X slab -> rows of the X' slab, this thread's half of the
+            // head dim).  Row block wq has wq + 1 blocks of the decay mask to build, all of them on one
+            // scheduler (a warp reads only its quarter of the tensor memory), so in a full tile the 16
+            // (row block, 16-byte chunk) units of a lane are dealt 8 / 6 / 2 / 0 to row blocks 0 .. 3; a
+            // foreign row's weight is read from shared memory.
             if (full) {
-                // ---- decay mask: G (fp32, TMEM) -> M of both heads (bf16, TMEM)
+                if (wq == 0) scale_units<0, 8>(s_x, s_xp, s_wp, lane, hf);
+                else if (wq == 1) scale_units<8, 14>(s_x, s_xp, s_wp, lane, hf);
+                else if (wq == 2) scale_units<14, 16>(s_x, s_xp, s_wp, lane, hf);
+            } else {
+                // a tile of a run: the X' slab is free once the previous tile's product has read it
+                run_done += l2_last;
+                const uint32_t wp = s_wp[i];
+                if (j > 0) tc::mbar_wait(&hb->dh_full, (j - 1) & 1, abort_flag, d_status);
+                scale_own_row(s_x, s_xp, wp, tc::ex2_approx(run_total - run_done), i, hf);
+            }
+            tc::fence_proxy_async_smem();
+            tc::mbar_arrive(&hb->xp_full);
+
+            if (full) {
+                // ---- decay mask: G (fp32, TMEM) -> M (bf16, TMEM); this thread owns row i and
+                // columns 16 hf .. 16 hf + 15 of every 32-column block
                 tc::mbar_wait(&bars->g_full, jf & 1, abort_flag, d_status);
                 tc::tc_fence_after();
-                if (sub > wq) {
-                    uint32_t zero[16];
+                const float r_i = tc::ex2_approx(l2 - Lw);
+                const uint32_t g_addr = tmem + lane_base + TM_G + 16 * hf;
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) zero[q] = 0u;
-                    tc::tmem_st16(tm_g, zero);
-                    tc::tmem_st16(tm_g + 16, zero);
-                } else if (cur.entries) {
-                    const int64_t r = rec_base + (int64_t)head0 * rec_hstride + t_begin / ST + j;
-                    const int64_t r1 = r + (nh == 2 ? rec_hstride : 0);
-                    mask_block_entries(tm_g, prm.rec + r, prm.rec + r1, prm.l2 + r * ST, prm.l2 + r1 * ST, wq, sub, lane);
-                } else if (sub < wq) {
-                    mask_block<false>(tm_g, cur.w, 0u);
-                } else {
-                    mask_block<true>(tm_g, cur.w, keep);
-                }
-                if (cur.pre != 1.f) {
-                    // ---- Y = Ctilde Hprev^T scaled in place
-                    tc::mbar_wait(&bars->dh_full, dh_ph, abort_flag, d_status);
-                    tc::tc_fence_after();
-                    const uint64_t e2 = tc::f32x2(cur.pre, cur.pre);
-                    uint32_t yo[2][16];
-                    tc::tmem_ld16(tm_y, yo[0]);
-                    tc::tmem_ld16(tm_y + 16, yo[1]);
-                    tc::tmem_ld_wait();
+                for (int c = 0; c < 4; ++c) {
+                    if (c <= wq) {
+                        uint32_t cur[16], pk[8];
+                        tc::tmem_ld16(g_addr + c * 32, cur);
+                        ulonglong2 cb4[4];
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
+                        for (int q = 0; q < 4; ++q)
+                            cb4[q] = *reinterpret_cast<const ulonglong2 *>(&s_cb[c * 32 + 16 * hf + 4 * q]);
+                        tc::tmem_ld_wait();
+                        if (c == wq) {
+                            // diagonal block: Delta_j 2^(l_i - l_j) = cb_j 2^(l_i - l_blockend).  The
+                            // second factor is >= 1; when the whole block decays by less than
+                            // 2^-96 it cannot overflow and is applied as a product, else the
+                            // exponent is formed per entry (always <= 0 where j <= i).
+                            const float up = l2 - Lend;
+                            if (Lw - Lend < 96.f) {
+                                const float rf = tc::ex2_approx(up);
+                                const uint64_t rf2 = tc::f32x2(rf, rf);
 #pragma unroll
-                        for (int q = 0; q < 16; q += 2) {
-                            const float2 v = tc::f32x2_get(tc::f32x2_mul(e2, f32x2_bits(yo[hh][q], yo[hh][q + 1])));
-                            yo[hh][q] = __float_as_uint(v.x);
-                            yo[hh][q + 1] = __float_as_uint(v.y);
+                                for (int q = 0; q < 8; ++q) {
+                                    const uint64_t cb = (q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x;
+                                    float2 m = tc::f32x2_get(tc::f32x2_mul(
+                                        tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rf2));
+                                    if (16 * hf + 2 * q > lane) m.x = 0.f;
+                                    if (16 * hf + 2 * q + 1 > lane) m.y = 0.f;
+                                    pk[q] = tc::pack_bf16x2(m.x, m.y);
+                                }
+                            } else {
+#pragma unroll
+                                for (int q = 0; q < 8; ++q) {
+                                    const float2 cb = tc::f32x2_get((q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x);
+                                    float m0 = __uint_as_float(cur[2 * q]) * tc::ex2_approx(up + tc::lg2_approx(cb.x));
+                                    float m1 = __uint_as_float(cur[2 * q + 1]) * tc::ex2_approx(up + tc::lg2_approx(cb.y));
+                                    if (16 * hf + 2 * q > lane) m0 = 0.f;
+                                    if (16 * hf + 2 * q + 1 > lane) m1 = 0.f;
+                                    pk[q] = tc::pack_bf16x2(m0, m1);
+                                }
+                            }
+                        } else {
+                            // l at the end of column block c, relative to the start of my block
+                            const float Lc1 = c == 0 ? L1 : (c == 1 ? L2 : L3);
+                            const float rowf = r_i * tc::ex2_approx(Lw - Lc1);
+                            const uint64_t rowf2 = tc::f32x2(rowf, rowf);
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const uint64_t cb = (q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x;
+                                pk[q] = tc::f32x2_bf16(tc::f32x2_mul(
+                                    tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rowf2));
+                            }
                         }
-                        tc::tmem_st16(tm_y + 16 * hh, yo[hh]);
+                        tc::tmem_st8(tm + TM_M + c * 16 + 8 * hf, pk);
                     }
+                }
+                tc::tc_fence_before();
+                tc::mbar_arrive(&bars->g_free);
+                // ---- Y = exp(l_i) * (Ctilde Hprev^T), in place
+                tc::mbar_wait(&hb->yoff_full, jf & 1, abort_flag, d_status);
+                tc::tc_fence_after();
+                {
+                    const float e_i = tc::ex2_approx(l2);
+                    uint32_t yo[32];
+                    tc::tmem_ld32(tm + TM_Y + p0, yo);
+                    tc::tmem_ld_wait();
+                    const uint64_t e2 = tc::f32x2(e_i, e_i);
+#pragma unroll
+                    for (int q = 0; q < 32; q += 2) {
+                        const float2 v = tc::f32x2_get(tc::f32x2_mul(e2, f32x2_bits(yo[q], yo[q + 1])));
+                        yo[q] = __float_as_uint(v.x);
+                        yo[q + 1] = __float_as_uint(v.y);
+                    }
+                    tc::tmem_st32(tm + TM_Y + p0, yo);
                 }
                 tc::tmem_st_wait();
                 tc::tc_fence_before();
-                arrive(&bars->m_full);
+                // (the scalars record read above is refilled by a bulk copy once m_full completes)
+                tc::fence_proxy_async_smem();
+                tc::mbar_arrive(&hb->m_full);
             }
 
-            // ---- state: H = exp(l_last) H + dH; of the leading tiles only at the last one, with the decay of the
-            // whole run
-            float h_next = 1.f;
-            if (j + 1 < ntiles) {
-                tc::mbar_wait(&bars->x_full[sx_next], x_ph, abort_flag, d_status);
-                h_next = scs->aux.to_ref;
-            }
-            if (full || j == n_pre - 1) {
-                tc::mbar_wait(&bars->dh_full, dh_ph, abort_flag, d_status);
-                tc::tc_fence_after();
-                const uint64_t dec2 = tc::f32x2(cur.dec, cur.dec);
+            // ---- state: H = exp(l_last) H + dH  (thread owns state index n = i, 32 channels); of the
+            // leading tiles only at the last one, with the decay of the whole run
+            if (full || j == run_end - 1) {
+            tc::mbar_wait(&hb->dh_full, j & 1, abort_flag, d_status);
+            tc::tc_fence_after();
+            const float dec = tc::ex2_approx(full ? l2_last : run_total);
+            const uint64_t dec2 = tc::f32x2(dec, dec);
+            uint32_t dhv[2][16];
+            tc::tmem_ld16(tm + TM_DH + p0, dhv[0]);
+            tc::tmem_ld16(tm + TM_DH + p0 + 16, dhv[1]);
+            tc::tmem_ld_wait();
 #pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    uint32_t dh[16];
-                    tc::tmem_ld_16x256b_x4(tm_dh + ((uint32_t)(16 * m) << 16), dh);
-                    tc::tmem_ld_wait();
+            for (int hh = 0; hh < 2; ++hh) {
+                const uint32_t (&dh)[16] = dhv[hh];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {            // (its registers: columns r first, then rows k)
-                        const int k = e >> 2, r = e & 3;
-                        Hst[8 * m + e] = tc::f32x2_fma(dec2, Hst[8 * m + e],
-                                                       f32x2_bits(dh[4 * r + 2 * k], dh[4 * r + 2 * k + 1]));
+                for (int q = 0; q < 8; ++q)
+                    Hst[8 * hh + q] = tc::f32x2_fma(dec2, Hst[8 * hh + q], f32x2_bits(dh[2 * q], dh[2 * q + 1]));
+                if (hb_next) {
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2) {
+                        const int ch = 2 * hh + c2;
+                        uint4 v = make_uint4(tc::f32x2_bf16(Hst[4 * ch]), tc::f32x2_bf16(Hst[4 * ch + 1]),
+                                             tc::f32x2_bf16(Hst[4 * ch + 2]), tc::f32x2_bf16(Hst[4 * ch + 3]));
+                        *reinterpret_cast<uint4 *>(s_hb + tc::sw128_offset(i, 4 * hf + ch)) = v;
                     }
                 }
-                if (j + 1 < ntiles) store_h(h_next);           // (MMA 3 has read the old copy)
-                tc::tc_fence_before();
             }
-            // ---- w . X of the next tile while MMA 2 runs
-            const float row = cur.row;
-            if (j + 1 < ntiles) {
-                take_rec(j + 1, cur);
-                scale_x(j + 1, sx_next, cur.wx);
+            if (hb_next) {
+                tc::fence_proxy_async_smem();
+                tc::tc_fence_before();
+                tc::mbar_arrive(&hb->h_ready);
+            }
             }
             if (full) {
-                // ---- epilogue: y_i = row Y_i + D x_i, staged for the TMA store where x_i stood
-                uint8_t *s_y = smem + SM_X + (sx * NHD + he) * SLAB;
-                tc::mbar_wait(&bars->yd_full, jf & 1, abort_flag, d_status);
+                // ---- epilogue: y_i = Y_i + D x_i, staged in shared memory for the TMA store
+                tc::mbar_wait(&hb->yd_full, jf & 1, abort_flag, d_status);
                 tc::tc_fence_after();
-                if (has_e) {
-                    const uint64_t D2 = tc::f32x2(Dh, Dh), r2 = tc::f32x2(row, row);
+                uint32_t ydv[2][16];
+                tc::tmem_ld16(tm + TM_Y + p0, ydv[0]);
+                tc::tmem_ld16(tm + TM_Y + p0 + 16, ydv[1]);
+                tc::tmem_ld_wait();
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t yd[16];
-                        tc::tmem_ld16(tm_y + 16 * hh, yd);
-                        uint4 xr[2];
+                for (int hh = 0; hh < 2; ++hh) {
+                    const uint32_t (&yd)[16] = ydv[hh];
 #pragma unroll
-                        for (int c = 0; c < 2; ++c)
-                            xr[c] = *reinterpret_cast<const uint4 *>(s_y + (row_off ^ ((2 * hh + c) << 4)));
-                        tc::tmem_ld_wait();
+                    for (int c2 = 0; c2 < 2; ++c2) {
+                        const uint32_t off = tc::sw128_offset(i, 4 * hf + 2 * hh + c2);
+                        const uint4 xr = *reinterpret_cast<const uint4 *>(s_x + off);
+                        const uint32_t xw[4] = {xr.x, xr.y, xr.z, xr.w};
+                        uint32_t o[4];
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
-                            const uint32_t xw[4] = {xr[c].x, xr[c].y, xr[c].z, xr[c].w};
-                            uint32_t o[4];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int e = 8 * c + 2 * q;
-                                o[q] = tc::f32x2_bf16(tc::f32x2_fma(
-                                    D2, f32x2_bits(xw[q] << 16, xw[q] & 0xffff0000u),
-                                    tc::f32x2_mul(r2, f32x2_bits(yd[e], yd[e + 1]))));
-                            }
-                            *reinterpret_cast<uint4 *>(s_y + (row_off ^ ((2 * hh + c) << 4))) = make_uint4(o[0], o[1], o[2], o[3]);
+                        for (int q = 0; q < 4; ++q) {
+                            const int e0 = c2 * 8 + 2 * q;
+                            o[q] = tc::f32x2_bf16(tc::f32x2_fma(Dh2, f32x2_bits(xw[q] << 16, xw[q] & 0xffff0000u),
+                                                                f32x2_bits(yd[e0], yd[e0 + 1])));
                         }
-                    }
-                    if (packed && j == ntiles - 1) {
-                        const int2 it = prm.items[item];
-                        const SeqDesc sd = prm.seqs[it.x];
-                        const int t = it.y * prm.seg_len + j * ST;               // the tile's first token
-                        if (t + ST > sd.len && t + i < sd.len) {
+                        *reinterpret_cast<uint4 *>(s_y + off) = make_uint4(o[0], o[1], o[2], o[3]);
+                        if (packed && t_begin + (j + 1) * ST > L && t_begin + j * ST + i < L) {
                             __nv_bfloat16 *yrow = reinterpret_cast<__nv_bfloat16 *>(prm.y) +
-                                ((int64_t)(sd.tok0 + t + i) * prm.H + head0 + he) * SP + 32 * hf;
-#pragma unroll 1
-                            for (int c = 0; c < 4; ++c)
-                                *reinterpret_cast<uint4 *>(yrow + 8 * c) =
-                                    *reinterpret_cast<const uint4 *>(s_y + (row_off ^ (c << 4)));
+                                ((int64_t)(tok0 + t_begin + j * ST + i) * H + h) * SP;
+                            *reinterpret_cast<uint4 *>(yrow + p0 + 16 * hh + 8 * c2) = make_uint4(o[0], o[1], o[2], o[3]);
                         }
                     }
                 }
                 tc::tc_fence_before();
+                tc::mbar_arrive(&hb->y_free);
                 tc::fence_proxy_async_smem();
-                arrive(&bars->y_staged[jf % Y_BARS]);
+                tc::mbar_arrive(&hb->y_staged);
+            } else {
+                tc::tc_fence_before();
             }
+            tc::mbar_arrive(&hb->x_free[sx]);
         }
 
         // ---- final state
-        if (packed) {
-            const int2 it = prm.items[item];
-            b = it.x; seg = it.y;
-            nseg = prm.seqs[b + 1].seg0 - prm.seqs[b].seg0;
-        }
-        if (prm.h_out && seg == nseg - 1 && !head_part && has_s) {
-            float *dst = prm.h_out + ((int64_t)b * prm.H + head0 + hs) * SP * SN + h_mine;
+        if (prm.h_out && seg == nseg - 1 && !head_part) {
+            float *dst = prm.h_out + (((int64_t)b * H + h) * SP) * SN;
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                float2 v = tc::f32x2_get(Hst[e]);
-                float2 *p = reinterpret_cast<float2 *>(dst + h_off(e));
+            for (int q = 0; q < 16; ++q) {
+                float2 v = tc::f32x2_get(Hst[q]);
                 if (prm.add) {
-                    const float2 w = *p;
-                    v.x += w.x; v.y += w.y;
+                    v.x += dst[(int64_t)(p0 + 2 * q) * SN + i];
+                    v.y += dst[(int64_t)(p0 + 2 * q + 1) * SN + i];
                 }
-                *p = v;
+                dst[(int64_t)(p0 + 2 * q) * SN + i] = v.x;
+                dst[(int64_t)(p0 + 2 * q + 1) * SN + i] = v.y;
             }
         }
     }
     tc::tc_fence_before();
     __syncthreads();
-    if (warp == WARP_MMA) tc::tmem_dealloc(tmem, TM_COLS);
+    if (warp == WARP_MMA0) tc::tmem_dealloc(tmem, TM_COLS);
 }
 
 // K3: chain the segments.  states[b,s,h,:,:] holds segment s's local end state (computed from a
@@ -1358,15 +1186,23 @@ size_t ssd_workspace_bytes(int B, int L, int H, int G, int chunk, int sm_count)
 }
 
 ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bias, int B, int L, int H,
-                             void *workspace)
+                             void *workspace, bool runs)
 {
     ScalarsArgs a;
     a.dt = dt; a.A = A; a.dt_bias = dt_bias; a.l2 = (float *)workspace;
     a.rec = (TileScalars *)((char *)workspace +
                             ((size_t)B * H * (ceil_div(L, ST) * ST) * sizeof(float) + 255) / 256 * 256);
     a.L = L; a.Lpad = ceil_div(L, ST) * ST; a.H = H; a.B = B;
-    a.mid = 1;
+    a.one_ref = runs ? 1 : 0;
     return a;
+}
+
+// Tiles a CTA has to walk for the run kernel to be the faster one: see launch_ssd_run.
+constexpr int RUN_TILES = 8;
+
+bool ssd_long_runs(int B, int L, int H, int G, int chunk, int sm_count)
+{
+    return ceil_div(std::min(ssd_segment_len(B, L, H, G, chunk, sm_count), L), ST) >= RUN_TILES;
 }
 
 // Split of a one-segment launch (see ssd_tiles_kernel): 0 when one CTA per (sequence, head pair)
@@ -1439,21 +1275,23 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
         if (!encode_tmap_bf16_cached(ctx.tmaps, &tm_y, y, 4, dims, str, box)) return SWIMBA_ERR_CUDA;
     }
     const size_t smem = ssd_smem_bytes();
-    if (!ensure_dynamic_smem((const void *)ssd_tiles_kernel<SSD_DENSE>, smem) ||
-        !ensure_dynamic_smem((const void *)ssd_tiles_kernel<SSD_SPLIT>, smem))
+    if (!ensure_dynamic_smem((const void *)ssd_tiles_kernel<false>, smem) ||
+        !ensure_dynamic_smem((const void *)ssd_tiles_kernel<true>, smem))
         return SWIMBA_ERR_CUDA;
 
     const int seg_len = ssd_segment_len(B, L, H, G, chunk, sm_count);
     const int nseg = ceil_div(L, seg_len);
     const int Lpad = ceil_div(L, ST) * ST;
     char *seg_ws = (char *)workspace + ssd_scalars_bytes(B, L, H);
+    const bool runs = ssd_long_runs(B, L, H, G, chunk, sm_count);
+    if (runs && !ensure_ssd_run()) return SWIMBA_ERR_CUDA;
     if (!scalars_done) {
-        const int rc = launch_ssd_scalars(ctx, ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace));
+        const int rc = launch_ssd_scalars(ctx, ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace, runs));
         if (rc != SWIMBA_OK) return rc;
     }
     SsdParams p;
     {
-        const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, workspace);
+        const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, workspace, runs);
         p.l2 = sa.l2;
         p.rec = sa.rec;
     }
@@ -1473,10 +1311,12 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
         p.split_tiles = in_place ? 0 : ssd_split_tiles(B, L, H, G, sm_count);
         if (p.split_tiles > 0) grid = dim3((unsigned)B, (unsigned)(G * pairs_per_group(H, G)), 2u);
         ctx.begin(STAGE_SSD_TILES);
-        if (p.split_tiles > 0)
-            launch_kernel(ssd_tiles_kernel<SSD_SPLIT>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
+        if (runs)
+            launch_ssd_run(ctx, grid, tm_b, tm_c, tm_x, tm_y, p);
+        else if (p.split_tiles > 0)
+            launch_kernel(ssd_tiles_kernel<true>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         else
-            launch_kernel(ssd_tiles_kernel<SSD_DENSE>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
+            launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         ctx.end();
     } else {
         float *states = (float *)seg_ws;
@@ -1493,7 +1333,10 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
         }
         p.h_in = states; p.h_out = h_final; p.seg_decay = nullptr;
         ctx.begin(STAGE_SSD_TILES);
-        launch_kernel(ssd_tiles_kernel<SSD_DENSE>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
+        if (runs)
+            launch_ssd_run(ctx, grid, tm_b, tm_c, tm_x, tm_y, p);
+        else
+            launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), smem, ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
         ctx.end();
     }
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
@@ -1544,7 +1387,7 @@ int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_s
     if (B <= 0 || L <= 0) return SWIMBA_OK;
     const int64_t T = (int64_t)B * L;
     const int GN = G * SN;
-    const ScalarsArgs sa = ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace);
+    const ScalarsArgs sa = ssd_scalars_args(dt, A, dt_bias, B, L, H, workspace, ssd_long_runs(B, L, H, G, chunk, sm_count));
     const int64_t extra = scalars_blocks(sa, 256);
     int64_t blocks = ceil_div64(T * (GN / 8), 256);
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
@@ -1700,7 +1543,6 @@ ScalarsArgs ssd_packed_scalars_args(const PackedPlan &pl, const float *dt, const
     sa.rec = (TileScalars *)(ws + lay.rec);
     sa.L = (int)T; sa.Lpad = pl.total_tiles * ST; sa.H = H; sa.B = 1;
     sa.tile_tab = (const int2 *)(ws + lay.tiles);
-    sa.mid = 1;
     return sa;
 }
 
@@ -1729,7 +1571,7 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &pl, const void *x,
         if (!encode_tmap_bf16_cached(ctx.tmaps, &tm_y, y, 4, dims, str, box)) return SWIMBA_ERR_CUDA;
     }
     const size_t smem = ssd_smem_bytes();
-    if (!ensure_dynamic_smem((const void *)ssd_tiles_kernel<SSD_PACKED>, smem)) return SWIMBA_ERR_CUDA;
+    if (!ensure_dynamic_smem((const void *)ssd_tiles_kernel<false>, smem)) return SWIMBA_ERR_CUDA;
 
     SsdParams p;
     p.l2 = (const float *)(ws + lay.l2); p.rec = (const TileScalars *)(ws + lay.rec); p.D = D;
@@ -1763,7 +1605,7 @@ int launch_ssd_tiles_packed(LaunchCtx &ctx, const PackedPlan &pl, const void *x,
     p.items = (const int2 *)(ws + lay.items);
     p.h_out = h_final; p.seg_decay = nullptr;
     ctx.begin(STAGE_SSD_TILES);
-    launch_kernel(ssd_tiles_kernel<SSD_PACKED>, dim3((unsigned)pl.items.size() * pairs), dim3(SSD_THREADS), smem,
+    launch_kernel(ssd_tiles_kernel<false>, dim3((unsigned)pl.items.size() * pairs), dim3(SSD_THREADS), smem,
                   ctx.stream, true, tm_b, tm_c, tm_x, tm_y, p);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
@@ -1804,13 +1646,13 @@ bool shard_maps(LaunchCtx &ctx, const void *x, const void *BC, const void *y, in
     const uint32_t box[4] = {SP, 1, ST, 1};
     if (!encode_tmap_bf16_cached(ctx.tmaps, tm_x, x, 4, dims, str, box)) return false;
     if (!encode_tmap_bf16_cached(ctx.tmaps, tm_y, y, 4, dims, str, box)) return false;
-    return ensure_dynamic_smem((const void *)ssd_tiles_kernel<SSD_DENSE>, ssd_smem_bytes());
+    return ensure_dynamic_smem((const void *)ssd_tiles_kernel<false>, ssd_smem_bytes());
 }
 
 SsdParams shard_params(LaunchCtx &ctx, const ShardLayout &lay, int B, int L, int H, int G, void *workspace)
 {
     SsdParams p;
-    const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, (char *)workspace + lay.scal);
+    const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, (char *)workspace + lay.scal, false);
     p.l2 = sa.l2; p.rec = sa.rec;
     p.D = nullptr;
     p.L = L; p.Lpad = ceil_div(L, ST) * ST; p.H = H; p.G = G; p.nseg = lay.nseg; p.seg_len = lay.seg_len;
@@ -1833,7 +1675,7 @@ ScalarsArgs ssd_shard_scalars_args(const float *dt, const float *A, const float 
                                    int G, int chunk, int sm_count, void *workspace)
 {
     const ShardLayout lay = shard_layout(B, L, H, G, chunk, sm_count);
-    return ssd_scalars_args(dt, A, dt_bias, B, L, H, (char *)workspace + lay.scal);
+    return ssd_scalars_args(dt, A, dt_bias, B, L, H, (char *)workspace + lay.scal, ssd_long_runs(B, L, H, G, chunk, sm_count));
 }
 
 int launch_ssd_shard_summary(LaunchCtx &ctx, const void *x, const void *BC, const float *dt, const float *A,
@@ -1843,7 +1685,8 @@ int launch_ssd_shard_summary(LaunchCtx &ctx, const void *x, const void *BC, cons
     if (B <= 0 || L <= 0) return SWIMBA_OK;
     const ShardLayout lay = shard_layout(B, L, H, G, chunk, sm_count);
     if (!scalars_done) {
-        const int rc = launch_ssd_scalars(ctx, ssd_scalars_args(dt, A, dt_bias, B, L, H, (char *)workspace + lay.scal));
+        const int rc = launch_ssd_scalars(ctx, ssd_scalars_args(dt, A, dt_bias, B, L, H, (char *)workspace + lay.scal,
+                                                             ssd_long_runs(B, L, H, G, chunk, sm_count)));
         if (rc != SWIMBA_OK) return rc;
     }
     SsdParams p = shard_params(ctx, lay, B, L, H, G, workspace);
@@ -1882,9 +1725,14 @@ int launch_ssd_shard_finish(LaunchCtx &ctx, const void *x, const void *BC, const
     p.D = D; p.y = y;
     p.h_in = states; p.h_out = h_end; p.seg_decay = nullptr;
     const dim3 grid((unsigned)lay.nseg, (unsigned)(G * pairs_per_group(H, G)), (unsigned)B);
+    const bool runs = ssd_long_runs(B, L, H, G, chunk, sm_count);
+    if (runs && !ensure_ssd_run()) return SWIMBA_ERR_CUDA;
     ctx.begin(STAGE_SSD_TILES);
-    launch_kernel(ssd_tiles_kernel<SSD_DENSE>, grid, dim3(SSD_THREADS), ssd_smem_bytes(), ctx.stream, true, tm_b, tm_c,
-                  tm_x, tm_y, p);
+    if (runs)
+        launch_ssd_run(ctx, grid, tm_b, tm_c, tm_x, tm_y, p);
+    else
+        launch_kernel(ssd_tiles_kernel<false>, grid, dim3(SSD_THREADS), ssd_smem_bytes(), ctx.stream, true, tm_b, tm_c,
+                      tm_x, tm_y, p);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }

@@ -2,13 +2,13 @@
 // transition is shared by all experts: shared-A equation).  Per token t of head h, with
 // Delta_t = softplus(dt_t + dt_bias_h) and l_t = sum_{r <= t, r in t's 128-token tile} Delta_r A_h log2 e,
 // two arrays are produced:
-//   l2[(b*H + h)*Lpad + t] = l_t          (forward: the row factor of the decay mask, below)
+//   l2[(b*H + h)*Lpad + t] = l_t          (one_ref: the row factor of the decay mask, below)
 //   rec[((b*H + h)*ntile + tile)] = one record per 128-token tile, copied to shared memory as a block:
 //       wp[128]  W(Delta_t 2^(l_last - l_t))      weight of token t in the tile's end state
 //       cb[128]  Delta_t 2^(l_ref - l_t)          weight of token t as a column of the decay mask
 //       ends[4]  l at the end of each 32-token block (ends[3] = l_last)
-//       aux      (forward only) what follows from the ends, so that no thread of the SSD kernel has to work it out
-// l_ref is l at the end of t's 32-token block; for the forward (`mid`) the tile's reference while there is one
+//       aux      (one_ref only) what follows from the ends, so that no thread of the SSD kernel has to work it out
+// l_ref is l at the end of t's 32-token block; with one_ref the tile's reference while there is one
 // (tile_one_ref).  Exponents to the block's or the tile's end are <= 0.
 // Row factors: 2^(l_t - l_ref) with a reference for the tile; else 2^(l_t - l at the start of t's block), or l_t
 // itself where the block decays by 2^-96 and more (mask_mode).  W(w) is w as a two-term bf16 sum packed in one word (high part in the low
@@ -62,7 +62,7 @@ struct ScalarsArgs {
     // (first token, valid tokens); tiles start at sequence starts.  dt is then [T, H], the arrays
     // are laid out [H, tiles] and Lpad = 128 * tiles, B = 1.  Null: dense [B, L].
     const int2 *tile_tab = nullptr;
-    int mid = 0;          // 1: the forward's column weights and row factors
+    int one_ref = 0;      // 1: column weights and row factors for the run kernel (k2_run.cu)
 };
 
 __host__ __device__ inline int64_t scalars_units(const ScalarsArgs &a)
@@ -126,7 +126,7 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
         const float excl = incl - run;
         const float l_last = __shfl_sync(0xffffffffu, incl, 31);
         const float l_blk = __shfl_sync(0xffffffffu, incl, lane | 7);   // 8 lanes = one 32-token block
-        const bool mid = a.mid && tile_one_ref(l_last);
+        const bool mid = a.one_ref && tile_one_ref(l_last);
         const float l_mid = tile_ref(l_last);
         const float l_ref = mid ? l_mid : l_blk;
         const float l_prev = __shfl_sync(0xffffffffu, incl, (lane & 24) - 1);      // (block 0: any lane)
@@ -143,7 +143,7 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
             cb[i] = d[i] * exp2f(l_ref - lv[i]);
         }
         TileScalars *rec = a.rec + out[q];
-        if (a.mid) {
+        if (a.one_ref) {
             if (mid || l_beg - l_blk < 96.f) {
                 const float from = mid ? l_mid : l_beg;
 #pragma unroll
