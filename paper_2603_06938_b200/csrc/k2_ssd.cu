@@ -1120,8 +1120,9 @@ bool ssd_tiles_supported(int dtype, int P, int N)
 static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 
 // Segment length (tokens, multiple of 128); L itself if one segment per sequence is best.  Costs in units of
-// a full tile of a head pair (3.3 us), from a sweep of lengths 400..32768 at 12..128 (sequence, head) pairs:
-// a segment's full pass takes its tiles plus 1.2, the state-only pass 0.35 a tile plus 1.2 (four heads per
+// a full tile of a head pair in the tile kernel (3.3 us), from a sweep of lengths 400..32768 at 12..128 (sequence, head)
+// pairs: a segment's full pass takes its tiles plus 1.2, or from RUN_TILES tiles on 0.8 of its tiles plus 1.6; the
+// state-only pass 0.35 a tile plus 1.2 (four heads per
 // CTA), the scan 1 and 0.005 per head and segment (128 KB moved), or 0.05 per segment where few heads leave it
 // bound by its chain (one head, 16000 tokens: 49 us in 125 segments, 42 in 63).  Whole rounds of CTAs count.  Of the
 // lengths tried the one picked was the best or within 2 % of it; filling two CTAs per SM whatever it costs
@@ -1131,6 +1132,14 @@ static size_t ssd_smem_bytes() { return SM_SMALL + sizeof(SsdSmall); }
 // ssd_segment_states can reserve for every shorter call without knowing its pick.
 constexpr int SEG_ROUNDS = 4, SEG_TILES = 12;
 
+// Tiles a CTA has to walk for the run kernel (k2_run.cu) to be the faster one.  Whole calls, run kernel against tile
+// kernel: 6 sequences of 48 heads and 2 tiles with states 31.0 / 30.4 us, 4 tiles 37.3 / 37.5, 6 tiles 43.1 / 45.4,
+// 8 tiles 49.8 / 53.3, 16 tiles 77.6 / 85.7; 16 sequences of 40 heads and 6 tiles (5 rounds of CTAs) 85 / 96.
+constexpr int RUN_TILES = 6;
+
+// Time of a CTA that walks n tiles, in tiles of the tile kernel.
+static float walk_cost(int n) { return n >= RUN_TILES ? 0.8f * n + 1.6f : (float)n + 1.2f; }
+
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
 {
     const int64_t ctas = (int64_t)B * G * pairs_per_group(H, G);
@@ -1139,12 +1148,12 @@ int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count)
     if (2 * ctas > sm_count || tiles <= 2) return tiles * ST;
     const int q_tiles = chunk >= ST ? chunk / ST : 1;                 // segments are whole chunks
     const int64_t most = std::max<int64_t>(SEG_ROUNDS * (int64_t)sm_count / ctas, tiles / SEG_TILES);
-    float best_cost = (float)tiles + 1.2f;
+    float best_cost = walk_cost(tiles);
     int best = tiles;
     for (int st = q_tiles; st < tiles; st += q_tiles) {
         const int64_t nseg = ceil_div(tiles, st);
         if (nseg > most) continue;
-        const float cost = (float)ceil_div64(ctas * nseg, sm_count) * ((float)st + 1.2f) +
+        const float cost = (float)ceil_div64(ctas * nseg, sm_count) * walk_cost(st) +
                            (float)ceil_div64(quads * (nseg - 1), sm_count) * (0.35f * st + 1.2f) + 1.f +
                            (float)(nseg - 1) * std::max(0.005f * B * H, 0.05f);
         if (cost < best_cost) { best_cost = cost; best = st; }
@@ -1197,9 +1206,6 @@ ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bi
     return a;
 }
 
-// Tiles a CTA has to walk for the run kernel to be the faster one: see launch_ssd_run.
-constexpr int RUN_TILES = 8;
-
 bool ssd_long_runs(int B, int L, int H, int G, int chunk, int sm_count)
 {
     return ceil_div(std::min(ssd_segment_len(B, L, H, G, chunk, sm_count), L), ST) >= RUN_TILES;
@@ -1211,21 +1217,24 @@ bool ssd_long_runs(int B, int L, int H, int G, int chunk, int sm_count)
 // state-only tiles at about 0.47 of a full one; the CTAs that produce y of the leading tiles run
 // on the SMs left over, in ceil(ctas / spare) rounds of a tiles and 1.2 for starting and draining one.
 // a minimises the later of the two.  4 sequences of 64 heads and 64 tiles: 219 us at a = 7, 228 us at the
-// a = 8 that a rule without the 1.2 picks, 234 us unsplit.
+// a = 8 that a rule without the 1.2 picks, 234 us unsplit.  In the run kernel, in its tiles: 0.5 of a full one and 1.65
+// (a CTA of 4 tiles takes 23800 cycles, of 8 tiles 40600; the same sequences 292 us a call at a = 7, 293 at 5 and 6).
 static int ssd_split_tiles(int B, int L, int H, int G, int sm_count)
 {
     const int64_t ctas = (int64_t)B * G * pairs_per_group(H, G);
     const int n = ceil_div(L, ST);
     if (2 * ctas <= sm_count || ctas >= sm_count || n < 4) return 0;
     const int64_t spare = sm_count - ctas, rounds = ceil_div64(ctas, spare);
-    float best = (float)n + 1.2f;
+    const bool run = n >= RUN_TILES;
+    const float ends = run ? 1.65f : 1.2f, saved = run ? 0.5f : 0.53f;
+    float best = (float)n + ends;
     int best_a = 0;
     for (int a = 1; a < n; ++a) {
-        const float whole = (float)n + 1.2f - 0.53f * a, lead = (float)rounds * ((float)a + 1.2f);
+        const float whole = (float)n + ends - saved * a, lead = (float)rounds * ((float)a + ends);
         const float m = whole > lead ? whole : lead;
         if (m < best) { best = m; best_a = a; }
     }
-    return best < 0.97f * ((float)n + 1.2f) ? best_a : 0;
+    return best < 0.97f * ((float)n + ends) ? best_a : 0;
 }
 
 int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &sa)
