@@ -44,7 +44,7 @@ struct __align__(8) RunBars {
 // use: room for one.
 struct __align__(16) TileRec {
     float cb[ST], ends[4];
-    TileScalars::Aux aux;
+    TileAux aux;
     float row[ST];
 };
 
@@ -290,7 +290,8 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
         auto load_rec = [&](int j) {
             for (int hd = 0; hd < nh; ++hd) {
                 const int64_t r = rec_base + (int64_t)(head0 + hd) * rec_hstride + t_begin / ST + j;
-                tc::bulk_load(sm->sc[hd].cb, prm.rec[r].cb, (ST + 8) * sizeof(float), &bars->x_full[j % X_SLOTS]);
+                tc::bulk_load(sm->sc[hd].cb, prm.rec[r].cb, (ST + 4) * sizeof(float), &bars->x_full[j % X_SLOTS]);
+                tc::bulk_load(&sm->sc[hd].aux, prm.aux + r, (uint32_t)sizeof(TileAux), &bars->x_full[j % X_SLOTS]);
                 tc::bulk_load(sm->sc[hd].row, prm.l2 + r * ST, ST * sizeof(float), &bars->x_full[j % X_SLOTS]);
             }
         };

@@ -1179,14 +1179,19 @@ static size_t ssd_states_bytes(int64_t n, int H)
     return (size_t)n * H * SP * SN * sizeof(float) + ((size_t)n * H * sizeof(float) + 255) / 256 * 256;
 }
 
-// Workspace: [log-decays B*H*Lpad float] [per-tile records B*H*(Lpad/128)] [segment states]
+// Workspace: [log-decays B*H*Lpad float] [per-tile records B*H*(Lpad/128)] [aux of them] [segment states]
 // [segment decays].
+static size_t aux_bytes(int B, int L, int H)
+{
+    return ((size_t)B * H * ceil_div(L, ST) * sizeof(TileAux) + 255) / 256 * 256;
+}
+
 size_t ssd_scalars_bytes(int B, int L, int H)
 {
     const size_t Lpad = (size_t)ceil_div(L, ST) * ST;
     const size_t l2_bytes = ((size_t)B * H * Lpad * sizeof(float) + 255) / 256 * 256;
     const size_t rec_bytes = ((size_t)B * H * (Lpad / ST) * sizeof(TileScalars) + 255) / 256 * 256;
-    return l2_bytes + rec_bytes;
+    return l2_bytes + rec_bytes + aux_bytes(B, L, H);
 }
 
 size_t ssd_workspace_bytes(int B, int L, int H, int G, int chunk, int sm_count)
@@ -1202,7 +1207,7 @@ ScalarsArgs ssd_scalars_args(const float *dt, const float *A, const float *dt_bi
     a.rec = (TileScalars *)((char *)workspace +
                             ((size_t)B * H * (ceil_div(L, ST) * ST) * sizeof(float) + 255) / 256 * 256);
     a.L = L; a.Lpad = ceil_div(L, ST) * ST; a.H = H; a.B = B;
-    a.one_ref = runs ? 1 : 0;
+    if (runs) a.aux = (TileAux *)((char *)workspace + ssd_scalars_bytes(B, L, H) - aux_bytes(B, L, H));
     return a;
 }
 
@@ -1303,6 +1308,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
         const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, workspace, runs);
         p.l2 = sa.l2;
         p.rec = sa.rec;
+        p.aux = sa.aux;
     }
     p.D = D;
     p.L = L; p.Lpad = Lpad; p.H = H; p.G = G; p.nseg = nseg; p.seg_len = seg_len;
@@ -1661,8 +1667,8 @@ bool shard_maps(LaunchCtx &ctx, const void *x, const void *BC, const void *y, in
 SsdParams shard_params(LaunchCtx &ctx, const ShardLayout &lay, int B, int L, int H, int G, void *workspace)
 {
     SsdParams p;
-    const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, (char *)workspace + lay.scal, false);
-    p.l2 = sa.l2; p.rec = sa.rec;
+    const ScalarsArgs sa = ssd_scalars_args(nullptr, nullptr, nullptr, B, L, H, (char *)workspace + lay.scal, true);
+    p.l2 = sa.l2; p.rec = sa.rec; p.aux = sa.aux;
     p.D = nullptr;
     p.L = L; p.Lpad = ceil_div(L, ST) * ST; p.H = H; p.G = G; p.nseg = lay.nseg; p.seg_len = lay.seg_len;
     p.split_tiles = 0;

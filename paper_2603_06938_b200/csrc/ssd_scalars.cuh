@@ -2,13 +2,12 @@
 // transition is shared by all experts: shared-A equation).  Per token t of head h, with
 // Delta_t = softplus(dt_t + dt_bias_h) and l_t = sum_{r <= t, r in t's 128-token tile} Delta_r A_h log2 e,
 // two arrays are produced:
-//   l2[(b*H + h)*Lpad + t] = l_t          (one_ref: the row factor of the decay mask, below)
+//   l2[(b*H + h)*Lpad + t] = l_t          (for the run kernel: the row factor of its decay mask, below)
 //   rec[((b*H + h)*ntile + tile)] = one record per 128-token tile, copied to shared memory as a block:
 //       wp[128]  W(Delta_t 2^(l_last - l_t))      weight of token t in the tile's end state
 //       cb[128]  Delta_t 2^(l_ref - l_t)          weight of token t as a column of the decay mask
 //       ends[4]  l at the end of each 32-token block (ends[3] = l_last)
-//       aux      (one_ref only) what follows from the ends, so that no thread of the SSD kernel has to work it out
-// l_ref is l at the end of t's 32-token block; with one_ref the tile's reference while there is one
+// l_ref is l at the end of t's 32-token block; for the run kernel (ScalarsArgs::aux) the tile's reference while there is one
 // (tile_one_ref).  Exponents to the block's or the tile's end are <= 0.
 // Row factors: 2^(l_t - l_ref) with a reference for the tile; else 2^(l_t - l at the start of t's block), or l_t
 // itself where the block decays by 2^-96 and more (mask_mode).  W(w) is w as a two-term bf16 sum packed in one word (high part in the low
@@ -27,14 +26,15 @@ struct TileScalars {            // (the shared-memory image as well)
     uint32_t wp[SCALARS_TILE];
     float cb[SCALARS_TILE];
     float ends[4];
-    struct Aux {
-        float to_ref;       // decay from the tile's start to its reference (1 if it has none)
-        float from_ref;     // from there to the tile's end
-        float total;        // over the tile
-        float blocks;       // 0: the tile has a reference, 1: it has not
-    } aux;
+};
+struct TileAux {        // what follows from a tile's block ends, so that no thread of the run kernel has to work it out
+    float to_ref;       // decay from the tile's start to its reference (1 if it has none)
+    float from_ref;     // from there to the tile's end
+    float total;        // over the tile
+    float blocks;       // 0: the tile has a reference, 1: it has not
 };
 static_assert(sizeof(TileScalars) % 16 == 0, "tile records are moved by 16-byte bulk copies");
+
 
 // The forward's decay mask in two factors per entry: exp(l_t - l_s) = 2^(l_t - ref) 2^(ref - l_s), a row factor and a
 // column weight, with one reference for the whole tile as long as the tile decays by less than 2^-188: half way, or
@@ -62,7 +62,7 @@ struct ScalarsArgs {
     // (first token, valid tokens); tiles start at sequence starts.  dt is then [T, H], the arrays
     // are laid out [H, tiles] and Lpad = 128 * tiles, B = 1.  Null: dense [B, L].
     const int2 *tile_tab = nullptr;
-    int one_ref = 0;      // 1: column weights and row factors for the run kernel (k2_run.cu)
+    TileAux *aux = nullptr;          // given: column weights, row factors and this for the run kernel (k2_run.cu)
 };
 
 __host__ __device__ inline int64_t scalars_units(const ScalarsArgs &a)
@@ -75,7 +75,8 @@ __host__ __device__ inline int64_t scalars_units(const ScalarsArgs &a)
 // synchronisation: lane l owns tokens 4l .. 4l+3 of a tile; the loads of all NU units are issued
 // before the first use.  The tile's running log-decay is summed token by token inside a lane and
 // by a shuffle scan across lanes.
-template <int NU>
+// ONE_REF: ScalarsArgs::aux is given.
+template <int NU, bool ONE_REF>
 __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t unit0, int lane)
 {
     const int ntile = a.Lpad / SCALARS_TILE;
@@ -126,11 +127,16 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
         const float excl = incl - run;
         const float l_last = __shfl_sync(0xffffffffu, incl, 31);
         const float l_blk = __shfl_sync(0xffffffffu, incl, lane | 7);   // 8 lanes = one 32-token block
-        const bool mid = a.one_ref && tile_one_ref(l_last);
-        const float l_mid = tile_ref(l_last);
-        const float l_ref = mid ? l_mid : l_blk;
-        const float l_prev = __shfl_sync(0xffffffffu, incl, (lane & 24) - 1);      // (block 0: any lane)
-        const float l_beg = lane < 8 ? 0.f : l_prev;
+        float l_ref = l_blk, l_row = 0.f;                    // what column weights and row factors refer to
+        bool has_ref = false, rows = false;
+        if (ONE_REF) {
+            const float l_prev = __shfl_sync(0xffffffffu, incl, (lane & 24) - 1);      // (block 0: any lane)
+            const float l_beg = lane < 8 ? 0.f : l_prev;
+            has_ref = tile_one_ref(l_last);
+            if (has_ref) l_ref = tile_ref(l_last);
+            l_row = has_ref ? l_ref : l_beg;
+            rows = has_ref || l_beg - l_blk < 96.f;
+        }
         float lv[4], cb[4];
         uint32_t wp[4];
 #pragma unroll
@@ -143,15 +149,14 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
             cb[i] = d[i] * exp2f(l_ref - lv[i]);
         }
         TileScalars *rec = a.rec + out[q];
-        if (a.one_ref) {
-            if (mid || l_beg - l_blk < 96.f) {
-                const float from = mid ? l_mid : l_beg;
+        if (ONE_REF) {
+            if (rows) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) lv[i] = exp2f(lv[i] - from);
+                for (int i = 0; i < 4; ++i) lv[i] = exp2f(lv[i] - l_row);
             }
             if (lane == 31)
-                rec->aux = TileScalars::Aux{mid ? exp2f(l_mid) : 1.f, mid ? exp2f(l_last - l_mid) : 1.f, exp2f(l_last),
-                                            mid ? 0.f : 1.f};
+                a.aux[out[q]] = TileAux{has_ref ? exp2f(l_ref) : 1.f, has_ref ? exp2f(l_last - l_ref) : 1.f, exp2f(l_last),
+                                        has_ref ? 0.f : 1.f};
         }
         reinterpret_cast<float4 *>(a.l2 + out[q] * SCALARS_TILE)[lane] = make_float4(lv[0], lv[1], lv[2], lv[3]);
         reinterpret_cast<uint4 *>(rec->wp)[lane] = make_uint4(wp[0], wp[1], wp[2], wp[3]);
@@ -164,7 +169,8 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
 __device__ __forceinline__ void ssd_scalars_block(const ScalarsArgs &a, int64_t block)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    ssd_scalars_warp<2>(a, (block * nwarp + warp) * 2, lane);
+    if (a.aux) ssd_scalars_warp<2, true>(a, (block * nwarp + warp) * 2, lane);
+    else ssd_scalars_warp<2, false>(a, (block * nwarp + warp) * 2, lane);
 }
 
 // Blocks of `threads` threads that cover all units.

@@ -20,6 +20,7 @@ struct SeqDesc {            // one sequence of a packed batch
 struct SsdParams {
     const float *l2;        // [B,H,Lpad] log2-decay accumulated inside the 128-token tile
     const TileScalars *rec; // [B,H,Lpad/128] per-tile weights and block ends
+    const TileAux *aux;     // run kernel: [B,H,Lpad/128]
     const float *D;
     const float *h_in;      // initial states: [B,H,P,N] (nseg == 1) or [B,nseg,H,P,N]; may be null
     const float *h_first;   // seg_states >= 2: states entering the first segments, [B,H,P,N]; may be null
