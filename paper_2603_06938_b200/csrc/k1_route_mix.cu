@@ -223,7 +223,7 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&d)[4], uint32_t a0, uin
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <int NT>
+template <int NT, bool ONE_REF>
 __global__ void __launch_bounds__(256, NT <= 2 ? 4 : 2)
 router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r,
                   int64_t Ttok, int F, int E, int k, int32_t *__restrict__ idx, float *__restrict__ w,
@@ -235,7 +235,7 @@ router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__re
     if ((int)blockIdx.x < scalar_blocks) {
         // leading blocks: SSD step sizes and tile log-decays of the same call (they depend on dt
         // only); being short, they also stagger the start of the router blocks behind them
-        ssd_scalars_block(scalars, blockIdx.x);
+        ssd_scalars_block<ONE_REF>(scalars, blockIdx.x);
         return;
     }
     const int rblock = (int)blockIdx.x - scalar_blocks;       // index among the router blocks
@@ -740,7 +740,7 @@ static int launch_router_mma(LaunchCtx &ctx, const __nv_bfloat16 *u, const __nv_
     ctx.begin(STAGE_ROUTER);
 #define SWIMBA_ROUTER_MMA_CASE(NTV)                                                             \
     do {                                                                                        \
-        auto kern = router_mma_kernel<NTV>;                                                     \
+        auto kern = scalars.aux ? router_mma_kernel<NTV, true> : router_mma_kernel<NTV, false>; \
         if (smem > 32 * 1024 &&  /* static shared memory counts toward the 48 KB default */     \
             !ensure_dynamic_smem((const void *)kern,             \
                                  smem))                                     \

@@ -59,7 +59,7 @@ router_small_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__
     grid_dep_launch();
     if ((int)blockIdx.x >= (Ttok + 1) / 2) {
         // SSD step sizes and tile log-decays of the same call (they depend on dt only)
-        ssd_scalars_block(scalars, blockIdx.x - (Ttok + 1) / 2);
+        ssd_scalars_block<false>(scalars, blockIdx.x - (Ttok + 1) / 2);
         return;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

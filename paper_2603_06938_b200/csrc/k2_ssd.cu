@@ -87,6 +87,7 @@ struct __align__(16) SsdSmall {
 }  // namespace
 
 // Stand-alone launch of the step sizes and tile log-decays.
+template <bool ONE_REF>
 __global__ void __launch_bounds__(256)
 ssd_scalars_kernel(const ScalarsArgs args)
 {
@@ -94,7 +95,7 @@ ssd_scalars_kernel(const ScalarsArgs args)
     // kernel behind this one (the streaming router, which writes without waiting) be let in.
     grid_dep_wait();
     grid_dep_launch();
-    ssd_scalars_block(args, blockIdx.x);
+    ssd_scalars_block<ONE_REF>(args, blockIdx.x);
 }
 
 // Self-test of the bounded wait every tensor-core kernel here relies on: one warp waits, with the
@@ -1246,7 +1247,7 @@ int launch_ssd_scalars(LaunchCtx &ctx, const ScalarsArgs &sa)
 {
     if (scalars_units(sa) <= 0) return SWIMBA_OK;
     ctx.begin(STAGE_SSD_SCALARS);
-    launch_kernel(ssd_scalars_kernel, dim3((unsigned)scalars_blocks(sa, 256)), dim3(256), 0, ctx.stream,
+    launch_kernel(sa.aux ? ssd_scalars_kernel<true> : ssd_scalars_kernel<false>, dim3((unsigned)scalars_blocks(sa, 256)), dim3(256), 0, ctx.stream,
                   true, sa);
     ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
@@ -1361,6 +1362,7 @@ int launch_ssd_tiles_streams(LaunchCtx &ctx, const void *x, const SsdStream &Bs,
 //   Cmix[t, :] = sum_j slots[t*k + j, GN:2GN]      (the slots carry their router weights)
 // and the same for every slot's evaluation, whose injection stream is read straight from the slots.  The
 // leading blocks compute the step sizes, which are shared by the slots too.
+template <bool ONE_REF>
 __global__ void __launch_bounds__(256)
 slot_readout_kernel(const __nv_bfloat16 *__restrict__ slots, int64_t T, int GN, int k,
                     __nv_bfloat16 *__restrict__ Cmix, int scalar_blocks, const ScalarsArgs scalars)
@@ -1368,7 +1370,7 @@ slot_readout_kernel(const __nv_bfloat16 *__restrict__ slots, int64_t T, int GN, 
     grid_dep_wait();
     grid_dep_launch();
     if ((int)blockIdx.x < scalar_blocks) {
-        ssd_scalars_block(scalars, blockIdx.x);
+        ssd_scalars_block<ONE_REF>(scalars, blockIdx.x);
         return;
     }
     const int vpr = GN >> 3;
@@ -1407,7 +1409,7 @@ int launch_ssd_slots_tiles(LaunchCtx &ctx, const void *x_slots, const void *BC_s
     int64_t blocks = ceil_div64(T * (GN / 8), 256);
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
     ctx.begin(STAGE_SLOT_STREAMS);
-    launch_kernel(slot_readout_kernel, dim3((unsigned)(extra + blocks)), dim3(256), 0, ctx.stream, true,
+    launch_kernel(sa.aux ? slot_readout_kernel<true> : slot_readout_kernel<false>, dim3((unsigned)(extra + blocks)), dim3(256), 0, ctx.stream, true,
                   (const __nv_bfloat16 *)BC_slots, T, GN, k, (__nv_bfloat16 *)cmix, (int)extra, sa);
     ctx.end();
     for (int j = 0; j < k; ++j) {
