@@ -201,7 +201,7 @@ int run_route_mix(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, con
     if (tensor) {
         counts = expert_gemm_counts(gemm_ws);
         perm = expert_gemm_perm(gemm_ws);
-        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
+        if (launch_zero(ctx, ZeroRegions{{counts}, {sizeof(int) * SWIMBA_MAX_EXPERTS}}, h->sm_count) != SWIMBA_OK)
             return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
     const bool zero_bc = tensor && expert_gemm_adds_rows(c.top_k);
@@ -234,7 +234,7 @@ int run_slots(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, const v
     if (tensor) {
         counts = expert_gemm_counts(gemm_ws);
         perm = expert_gemm_perm(gemm_ws);
-        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
+        if (launch_zero(ctx, ZeroRegions{{counts}, {sizeof(int) * SWIMBA_MAX_EXPERTS}}, h->sm_count) != SWIMBA_OK)
             return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
     int rc = launch_router(ctx, c.dtype, u, Wr, T, c.d_model, c.n_experts, c.top_k, idx, wt, counts, perm, T, h->sm_count,
@@ -498,7 +498,7 @@ int dense_linear(swimba_handle *h, LaunchCtx &ctx, const void *in, const void *W
     if (tensor) {
         counts = expert_gemm_counts(gws);
         perm = expert_gemm_perm(gws);
-        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
+        if (launch_zero(ctx, ZeroRegions{{counts}, {sizeof(int) * SWIMBA_MAX_EXPERTS}}, h->sm_count) != SWIMBA_OK)
             return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
     // one expert: the router only writes idx = 0, w = 1 and the identity list (W stands in for the
@@ -959,13 +959,17 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
     LaunchCtx ctx{(cudaStream_t)cuda_stream, h->d_status, 0, &h->prof, (c.flags & SWIMBA_FLAG_CHECK_INDICES) != 0, &h->tmaps};
     h->prof.n = 0;
     const size_t S = 2u * c.n_groups * c.d_state;
-    // the gradients of an empty batch are zero
-    if (cudaMemsetAsync(dW_expert, 0, (size_t)c.n_experts * S * c.d_model * sizeof(float), ctx.stream) != cudaSuccess ||
-        (dW_router &&
-         cudaMemsetAsync(dW_router, 0, (size_t)c.n_experts * c.d_model * sizeof(float), ctx.stream) != cudaSuccess))
-        return fail(h, SWIMBA_ERR_CUDA, "clearing the gradients failed");
+    // features come in eights: both sizes are multiples of 16
+    const size_t dwe_bytes = (size_t)c.n_experts * S * c.d_model * sizeof(float);
+    const size_t dwr_bytes = (size_t)c.n_experts * c.d_model * sizeof(float);
     h->last_stream = ctx.stream;
-    if (T == 0) { h->last_launches = 0; return SWIMBA_OK; }
+    if (T == 0) {                                                  // the gradients of an empty batch are zero
+        if (cudaMemsetAsync(dW_expert, 0, dwe_bytes, ctx.stream) != cudaSuccess ||
+            (dW_router && cudaMemsetAsync(dW_router, 0, dwr_bytes, ctx.stream) != cudaSuccess))
+            return fail(h, SWIMBA_ERR_CUDA, "clearing the gradients failed");
+        h->last_launches = 0;
+        return SWIMBA_OK;
+    }
     if (!u || !x || !dy || !workspace) return fail(h, SWIMBA_ERR_NULL_ARG, "u, x, dy or workspace is NULL");
     const BwdLayout l = bwd_layout(c, B, L, h->sm_count);
     if (workspace_bytes < l.total) return fail(h, SWIMBA_ERR_WORKSPACE_TOO_SMALL, "workspace too small");
@@ -975,8 +979,6 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
     void *BC = ws + l.f.bc;
     void *slots = ws + l.slots;
     float *dBC = (float *)(ws + l.dbc), *pi = (float *)(ws + l.pi);
-    if (cudaMemsetAsync(dBC, 0, (size_t)T * S * sizeof(float), ctx.stream) != cudaSuccess)
-        return fail(h, SWIMBA_ERR_CUDA, "clearing dBC failed");
     // forward quantities again: routing (with the softmax over all experts), the unscaled projection of every
     // kept slot, and the mixed streams as its weighted sum
     const bool tiles = ssd_tiles_supported(c.dtype, c.head_dim, c.d_state), tensor = use_tensor_k1(c);
@@ -987,9 +989,11 @@ int swimba_backward_weights(swimba_handle *h, const swimba_weights *w, const voi
     if (tensor) {
         counts = expert_gemm_counts(ws + l.f.gemm);
         perm = expert_gemm_perm(ws + l.f.gemm);
-        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
-            return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
+    if (launch_zero(ctx, ZeroRegions{{dBC, dW_expert, dW_router, counts},
+                                     {(size_t)T * S * sizeof(float), dwe_bytes, dW_router ? dwr_bytes : 0,
+                                      counts ? sizeof(int) * SWIMBA_MAX_EXPERTS : 0}}, h->sm_count) != SWIMBA_OK)
+        return fail(h, SWIMBA_ERR_CUDA, "clearing the gradients failed");
     rc = launch_router(ctx, c.dtype, u, Wr, T, c.d_model, c.n_experts, c.top_k, idx, wt, counts, perm, T, h->sm_count,
                        nullptr, 0, sa, pi);
     if (rc != SWIMBA_OK) return fail(h, rc, "router launch failed");

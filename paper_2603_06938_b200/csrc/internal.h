@@ -85,6 +85,12 @@ bool ssd_tiles_supported(int dtype, int P, int N);
 size_t ssd_workspace_bytes(int B, int L, int H, int G, int chunk, int sm_count);
 // Tokens per segment the tile path cuts a sequence into (a multiple of 128; >= L: one segment).
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count);
+// Clears up to four regions (16-byte aligned, sizes multiples of 16; null: none) as the first kernel of a call.  The kernel
+// behind it may be launched programmatically and waits with grid_dep_wait: a memset in its place cost 1.5 us more,
+// the gap between it and the first kernel.
+struct ZeroRegions { void *p[4]; size_t bytes[4]; };
+int launch_zero(LaunchCtx &ctx, const ZeroRegions &z, int sm_count);
+
 // scalars_done: the step sizes and tile log-decays (ssd_scalars_args over the same workspace) have
 // already been produced earlier in the stream (launch_router with scalars, or launch_ssd_scalars).  early:
 // x and h0 were complete before the first kernel of the same call.

@@ -1,5 +1,7 @@
 // K1 (SIMT part): router logits + softmax + top-k, and the plain projection/mix used by the
 // fp32 path and by decode.  (Router softmax equation and top-k rule; Theorem 1, mixed streams.)
+#include <algorithm>
+
 #include "internal.h"
 #include "tc05.cuh"
 #include <type_traits>
@@ -223,6 +225,16 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&d)[4], uint32_t a0, uin
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+__global__ void __launch_bounds__(256)
+zero_kernel(const ZeroRegions z)
+{
+    grid_dep_launch();
+    const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        for (size_t i = first; i < z.bytes[r] / 16; i += step) reinterpret_cast<uint4 *>(z.p[r])[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 template <int NT, bool ONE_REF>
 __global__ void __launch_bounds__(256, NT <= 2 ? 4 : 2)
 router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__restrict__ W_r,
@@ -238,6 +250,7 @@ router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__re
         ssd_scalars_block<ONE_REF>(scalars, blockIdx.x);
         return;
     }
+    grid_dep_wait();        // the cleared histogram (launch_zero; no kernel of an earlier call can still run)
     const int rblock = (int)blockIdx.x - scalar_blocks;       // index among the router blocks
     constexpr int EPAD = 8 * NT;
     extern __shared__ __align__(16) unsigned char router_smem[];
@@ -745,7 +758,7 @@ static int launch_router_mma(LaunchCtx &ctx, const __nv_bfloat16 *u, const __nv_
             !ensure_dynamic_smem((const void *)kern,             \
                                  smem))                                     \
             return SWIMBA_ERR_CUDA;                                                             \
-        launch_kernel(kern, dim3((unsigned)(extra + blocks)), dim3(256), smem, ctx.stream, false, \
+        launch_kernel(kern, dim3((unsigned)(extra + blocks)), dim3(256), smem, ctx.stream, counts != nullptr, \
                       u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, stage_w, chunk,         \
                       (uint4 *)zero_out, zero_bytes_per_token / 16, (int)blocks, (int)extra,    \
                       scalars, pi_out);                                                                 \
@@ -821,6 +834,16 @@ static int launch_router_t(LaunchCtx &ctx, const T *u, const T *W_r, int64_t Tto
     else SWIMBA_ROUTER_CASE(64, 1);
 #undef SWIMBA_ROUTER_CASE
     ctx.end();
+    return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
+}
+
+int launch_zero(LaunchCtx &ctx, const ZeroRegions &z, int sm_count)
+{
+    size_t most = 0;
+    for (size_t b : z.bytes) most = std::max(most, b);
+    const size_t blocks = std::min<size_t>((most / 16 + 255) / 256, (size_t)sm_count * 8);
+    launch_kernel(zero_kernel, dim3((unsigned)std::max<size_t>(blocks, 1)), dim3(256), 0, ctx.stream, false, z);
+    ctx.launches++;
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 
