@@ -201,7 +201,7 @@ int run_route_mix(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, con
     if (tensor) {
         counts = expert_gemm_counts(gemm_ws);
         perm = expert_gemm_perm(gemm_ws);
-        if (launch_zero(ctx, ZeroRegions{{counts}, {sizeof(int) * SWIMBA_MAX_EXPERTS}}, h->sm_count) != SWIMBA_OK)
+        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
             return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
     const bool zero_bc = tensor && expert_gemm_adds_rows(c.top_k);
@@ -234,7 +234,7 @@ int run_slots(swimba_handle *h, LaunchCtx &ctx, const swimba_weights *w, const v
     if (tensor) {
         counts = expert_gemm_counts(gemm_ws);
         perm = expert_gemm_perm(gemm_ws);
-        if (launch_zero(ctx, ZeroRegions{{counts}, {sizeof(int) * SWIMBA_MAX_EXPERTS}}, h->sm_count) != SWIMBA_OK)
+        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
             return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
     int rc = launch_router(ctx, c.dtype, u, Wr, T, c.d_model, c.n_experts, c.top_k, idx, wt, counts, perm, T, h->sm_count,
@@ -498,7 +498,7 @@ int dense_linear(swimba_handle *h, LaunchCtx &ctx, const void *in, const void *W
     if (tensor) {
         counts = expert_gemm_counts(gws);
         perm = expert_gemm_perm(gws);
-        if (launch_zero(ctx, ZeroRegions{{counts}, {sizeof(int) * SWIMBA_MAX_EXPERTS}}, h->sm_count) != SWIMBA_OK)
+        if (cudaMemsetAsync(counts, 0, sizeof(int) * SWIMBA_MAX_EXPERTS, ctx.stream) != cudaSuccess)
             return fail(h, SWIMBA_ERR_CUDA, "clearing the expert histogram failed");
     }
     // one expert: the router only writes idx = 0, w = 1 and the identity list (W stands in for the

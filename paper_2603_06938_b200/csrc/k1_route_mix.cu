@@ -225,6 +225,8 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&d)[4], uint32_t a0, uin
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// Stores only: bound by HBM writes (and by its launch at small calls).  An ordinary launch, so that nothing of an earlier
+// call is left when the kernel behind it starts.
 __global__ void __launch_bounds__(256)
 zero_kernel(const ZeroRegions z)
 {
@@ -250,7 +252,7 @@ router_mma_kernel(const __nv_bfloat16 *__restrict__ u, const __nv_bfloat16 *__re
         ssd_scalars_block<ONE_REF>(scalars, blockIdx.x);
         return;
     }
-    grid_dep_wait();        // the cleared histogram (launch_zero; no kernel of an earlier call can still run)
+    grid_dep_wait();        // the cleared histogram of a gradient call (launch_zero)
     const int rblock = (int)blockIdx.x - scalar_blocks;       // index among the router blocks
     constexpr int EPAD = 8 * NT;
     extern __shared__ __align__(16) unsigned char router_smem[];
@@ -758,7 +760,7 @@ static int launch_router_mma(LaunchCtx &ctx, const __nv_bfloat16 *u, const __nv_
             !ensure_dynamic_smem((const void *)kern,             \
                                  smem))                                     \
             return SWIMBA_ERR_CUDA;                                                             \
-        launch_kernel(kern, dim3((unsigned)(extra + blocks)), dim3(256), smem, ctx.stream, counts != nullptr, \
+        launch_kernel(kern, dim3((unsigned)(extra + blocks)), dim3(256), smem, ctx.stream, pi_out != nullptr, \
                       u, W_r, Ttok, F, E, k, idx, w, counts, perm, cap, stage_w, chunk,         \
                       (uint4 *)zero_out, zero_bytes_per_token / 16, (int)blocks, (int)extra,    \
                       scalars, pi_out);                                                                 \
