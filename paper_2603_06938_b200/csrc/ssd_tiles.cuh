@@ -1,4 +1,4 @@
-// What the two kernels over 128-token tiles share (k2_ssd.cu, k2_run.cu): sizes and parameters.
+// What the two kernels over 128-token tiles share (k2_ssd.cu, which picks by RUN_TILES, and k2_run.cu): sizes and parameters.
 #pragma once
 #include "internal.h"
 #include "ssd_scalars.cuh"
