@@ -653,7 +653,9 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
                 } else {
                     mask_block<true>(tm_g, cur.w, keep);
                 }
-                if (cur.pre != 1.f) {
+                // (one answer for the warp, tensor memory being accessed by whole warps: with MASK_ENTRIES the factor is each
+                // row's own, and 1 for rows that nothing has decayed in front of)
+                if (__any_sync(0xffffffffu, cur.pre != 1.f)) {
                     // ---- Y = Ctilde Hprev^T scaled in place
                     tc::mbar_wait(&bars->dh_full, dh_ph, abort_flag, d_status);
                     tc::tc_fence_after();

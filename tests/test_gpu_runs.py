@@ -4,6 +4,7 @@ counts, two groups, leading tiles, segments, given states; heads that decay too 
 import math
 
 import pytest
+import torch
 
 from paper_2603_06938_b200 import synth
 
@@ -24,5 +25,20 @@ def test_long_runs_match_oracle(B, L, H, G, fast):
             inp["A"][head] = -16.0
             inp["dt_bias"][head] = math.log(math.expm1(step))
         inp["dt"] *= 0.1
+    got = hp.gpu_forward(cfg, inp)
+    hp.compare_forward(cfg, inp, got, *hp.tolerances(cfg))
+
+
+def test_vanishing_steps_in_front_of_fast_tokens():
+    """Eight tokens of step size 0 lead every 32-token block of two heads, the others decay by 2^-99 in all: of one
+    warp's rows some have decayed by nothing, some by more than 2^-96."""
+    B, L, H = 25, 769, 6
+    cfg = synth.LayerConfig("runs", "bf16", B, L, 32, H, 64, 128, 1, 4, 2, 128, h0_std=0.2)
+    inp = synth.make_inputs(cfg, seed=70)
+    for head in (0, H - 1):
+        inp["A"][head] = -16.0
+        inp["dt_bias"][head] = math.log(math.expm1(0.179))
+        inp["dt"][..., head] = 0.0
+        inp["dt"][:, torch.arange(L) % 32 < 8, head] = -200.0
     got = hp.gpu_forward(cfg, inp)
     hp.compare_forward(cfg, inp, got, *hp.tolerances(cfg))
