@@ -490,10 +490,10 @@ adjoint_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_c
                 const uint32_t sa = lane_base + TC_S + (n & 1) * 128 + cq * 32;
                 const float *cb = sc->cb + cq * 32;
                 const float up = l_i - l_end;          // row factor 2^up: <= 1 below the diagonal blocks
-                // a diagonal block's row factor is >= 1: it is applied as a product while the block's decay
-                // stays above 2^-96, else the exponent is formed per entry (where it is <= 0)
+                // a diagonal block's row factor is >= 1 and below 2^96: it is applied as a product.  Columns of a block
+                // that decays by more come without a factor: their exponents are formed per entry (where <= 0)
                 const float l_beg = cq == 0 ? 0.f : sc->ends[cq - 1];
-                const bool prod = cq < wq || l_beg - l_end < 96.f;
+                const bool prod = !block_fast(l_beg, l_end);
                 const float rf = tc::ex2_approx(prod ? up : 0.f);
                 const uint64_t rf2 = tc::f32x2(rf, rf);
                 uint32_t v[32];
@@ -516,8 +516,9 @@ adjoint_tiles_kernel(const __grid_constant__ CUtensorMap tmap_bc, const __grid_c
 #pragma unroll
                     for (int e = 0; e < 32; e += 2) {
                         // (behind the diagonal the exponent is positive: the entry there is zero, its factor must be finite)
-                        const float f0 = e <= lane ? tc::ex2_approx(up + tc::lg2_approx(cb[e])) : 0.f;
-                        const float f1 = e + 1 <= lane ? tc::ex2_approx(up + tc::lg2_approx(cb[e + 1])) : 0.f;
+                        const float *lc = l2s + cq * 32;
+                        const float f0 = cq < wq || e <= lane ? cb[e] * tc::ex2_approx(l_i - lc[e]) : 0.f;
+                        const float f1 = cq < wq || e + 1 <= lane ? cb[e + 1] * tc::ex2_approx(l_i - lc[e + 1]) : 0.f;
                         acc[e / 2] = tc::f32x2_fma(tc::f32x2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
                                                    tc::f32x2(f0, f1), acc[e / 2]);
                     }

@@ -71,6 +71,16 @@ __device__ __forceinline__ void load_weights(BlockWeights &w, const float *s_cb,
     for (int r = 0; r < 4; ++r) w.v[r] = *reinterpret_cast<const uint64_t *>(s_cb + 8 * r + 2 * (lane & 3));
 }
 
+// Their decay to the end of the block, where the record has Delta alone and l in place of row factors (block_fast).
+__device__ __forceinline__ void decay_weights(BlockWeights &w, const TileRec *rec, int block, int lane)
+{
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float2 l = *reinterpret_cast<const float2 *>(&rec->row[32 * block + 8 * r + 2 * (lane & 3)]);
+        w.v[r] = tc::f32x2_mul(w.v[r], tc::f32x2(tc::ex2_approx(rec->ends[block] - l.x), tc::ex2_approx(rec->ends[block] - l.y)));
+    }
+}
+
 // w . X of one warp, from the X slab to the A operand of MMA 4 in tensor memory: lanes p0 .. p0+31 (channels of
 // the head), tokens s0 .. s0+31 (16 columns, two to a column).  wx: weights of tokens s0 + 8 c + 2 (t % 4) and
 // the one behind; x' = w x with the weight as a two-term bf16 sum (rounded once).
@@ -153,10 +163,10 @@ __device__ __forceinline__ void mask_block(uint32_t taddr, const BlockWeights (&
     }
 }
 
-// The same where a 32-token block of a head decays by more than 2^-96 (its diagonal's column weights could overflow):
-// that head's entries carry the row factor, the exponents of a diagonal block are formed entry by entry, all of them
-// <= 0.  Records and row factors (log-decays there) of the tile from global memory: the copy in shared memory
-// belongs to the next tile.
+// The same where a 32-token block of a head decays by 2^-96 and more (block_fast): that head's entries carry the row
+// factor, and where the columns lie in such a block, exponents are formed entry by entry, all of them <= 0.
+// Records and row factors (log-decays there) of the tile from global memory: the copy in shared memory belongs
+// to the next tile.
 __device__ __forceinline__ void mask_block_entries(uint32_t taddr, const TileScalars *rec0, const TileScalars *rec1,
                                                    const float *l2_0, const float *l2_1, int wq, int sub, int lane)
 {
@@ -173,20 +183,26 @@ __device__ __forceinline__ void mask_block_entries(uint32_t taddr, const TileSca
             const bool diag = sub == wq;
             const float Lw = wq ? rec->ends[wq - 1] : 0.f, Lc = rec->ends[sub];      // l before the rows, at the columns' end
             const int mode = mask_mode(rec->ends, wq);
+            const bool fast_cols = mask_mode(rec->ends, sub) == MASK_ENTRIES;
+            const float *l2 = q ? l2_1 : l2_0;
             uint32_t o[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {                     // rows k = e % 2, columns 8 (e / 2) ..
                 const int row = 16 * half + (lane >> 2) + 8 * (e & 1), col = 16 * c + 8 * (e >> 1) + 2 * (lane & 3);
-                const float l_i = (q ? l2_1 : l2_0)[32 * wq + row];
-                const float2 cb = *reinterpret_cast<const float2 *>(&rec->cb[32 * sub + col]);
+                const float l_i = l2[32 * wq + row];
+                float2 cb = *reinterpret_cast<const float2 *>(&rec->cb[32 * sub + col]);
                 float rf = 1.f;
-                if (mode == MASK_BLOCKS) rf = tc::ex2_approx(Lw - Lc);
-                if (mode == MASK_ENTRIES) rf = tc::ex2_approx(l_i - Lw) * tc::ex2_approx(Lw - Lc);
-                float m0 = __uint_as_float(g[2 * e]) * cb.x * rf, m1 = __uint_as_float(g[2 * e + 1]) * cb.y * rf;
-                if (mode == MASK_ENTRIES && diag) {
-                    m0 = __uint_as_float(g[2 * e]) * tc::ex2_approx(l_i - Lc + tc::lg2_approx(cb.x));
-                    m1 = __uint_as_float(g[2 * e + 1]) * tc::ex2_approx(l_i - Lc + tc::lg2_approx(cb.y));
+                if (fast_cols) {                              // (cb: Delta of the columns)
+                    const float2 l_s = *reinterpret_cast<const float2 *>(&l2[32 * sub + col]);
+                    const float to = mode == MASK_ENTRIES ? l_i : Lw;
+                    cb.x *= tc::ex2_approx(to - l_s.x);
+                    cb.y *= tc::ex2_approx(to - l_s.y);
+                } else if (mode == MASK_BLOCKS) {
+                    rf = tc::ex2_approx(Lw - Lc);
+                } else if (mode == MASK_ENTRIES) {
+                    rf = tc::ex2_approx(l_i - Lw) * tc::ex2_approx(Lw - Lc);
                 }
+                float m0 = __uint_as_float(g[2 * e]) * cb.x * rf, m1 = __uint_as_float(g[2 * e + 1]) * cb.y * rf;
                 if (diag && col > row) m0 = 0.f;
                 if (diag && col + 1 > row) m1 = 0.f;
                 o[e] = tc::pack_bf16x2(m0, m1);
@@ -568,6 +584,10 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
             const bool blocks0 = sc0->aux.blocks != 0.f, blocks1 = sc1->aux.blocks != 0.f;
             load_weights(p.w[0], sc0->cb + 32 * sub, lane);
             load_weights(p.w[1], sc1->cb + 32 * sub, lane);
+            if (blocks0 || blocks1) {                        // weights of a fast block's columns come without their decay
+                if (mask_mode(sc0->ends, sub) == MASK_ENTRIES) decay_weights(p.w[0], sc0, sub, lane);
+                if (mask_mode(sc1->ends, sub) == MASK_ENTRIES) decay_weights(p.w[1], sc1, sub, lane);
+            }
             p.row = sce->row[i];
             p.dec = scs->aux.total;
             // from where the column weights refer to, to the end of the tile (leading tile: of the run)

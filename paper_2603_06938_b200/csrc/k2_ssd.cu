@@ -36,7 +36,8 @@
 // columns in block b < w) factors as
 //   exp(l_i - L_w) * exp(L_w - L_{b+1}) * exp(L_{b+1} - l_s),     L_w = l at the end of block w-1,
 // every exponent being <= 0 (no overflow, underflow only where the true value underflows), so
-// that it costs two multiplications per entry.
+// that it costs two multiplications per entry.  Columns of a block that decays by 2^-96 and more are evaluated entry by
+// entry in every row block (their weights come without a factor: ssd_scalars.cuh, block_fast).
 //
 // Long sequences with few (sequence, head) pairs are cut into segments: ssd_state_kernel computes every
 // segment's local end state (MMA 4 only), segment_scan_kernel (K3) chains them, and this kernel evaluates each
@@ -193,6 +194,34 @@ __device__ __forceinline__ void scale_own_row(const uint8_t *s_x, uint8_t *s_xp,
 __device__ __forceinline__ uint64_t f32x2_bits(uint32_t a, uint32_t b)
 {
     return tc::f32x2(__uint_as_float(a), __uint_as_float(b));
+}
+
+// A row of the decay mask (this thread's 16 columns of every block up to its own) where one of those blocks decays by
+// 2^-96 and more (block_fast): its weights are the columns' Delta, and the exponents l_i - l_j are formed entry by entry.
+__device__ __forceinline__ void mask_row_entries(uint32_t g_addr, uint32_t m_addr, const float *s_cb, const float *s_ends,
+                                                 const float *l2_tile, float l_i, int wq, int hf, int lane)
+{
+#pragma unroll 1
+    for (int c = 0; c <= wq; ++c) {
+        const float Lc1 = s_ends[c];
+        const bool fast = block_fast(c ? s_ends[c - 1] : 0.f, Lc1);
+        uint32_t cur[16], pk[8];
+        tc::tmem_ld16(g_addr + c * 32, cur);
+        tc::tmem_ld_wait();
+        const int col0 = c * 32 + 16 * hf;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float2 cb = *reinterpret_cast<const float2 *>(&s_cb[col0 + 2 * q]);
+            float2 to = make_float2(Lc1, Lc1);                // what cb refers to
+            if (fast) to = *reinterpret_cast<const float2 *>(&l2_tile[col0 + 2 * q]);
+            float m0 = __uint_as_float(cur[2 * q]) * (cb.x * tc::ex2_approx(l_i - to.x));
+            float m1 = __uint_as_float(cur[2 * q + 1]) * (cb.y * tc::ex2_approx(l_i - to.y));
+            if (c == wq && 16 * hf + 2 * q > lane) m0 = 0.f;
+            if (c == wq && 16 * hf + 2 * q + 1 > lane) m1 = 0.f;
+            pk[q] = tc::pack_bf16x2(m0, m1);
+        }
+        tc::tmem_st8(m_addr + c * 16, pk);
+    }
 }
 
 template <bool SPLIT>
@@ -588,6 +617,11 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                 tc::tc_fence_after();
                 const float r_i = tc::ex2_approx(l2 - Lw);
                 const uint32_t g_addr = tmem + lane_base + TM_G + 16 * hf;
+                const bool any_fast = block_fast(0.f, L1) || (wq > 0 && block_fast(L1, L2)) ||
+                                      (wq > 1 && block_fast(L2, L3)) || (wq > 2 && block_fast(L3, l2_last));
+                if (any_fast) {
+                    mask_row_entries(g_addr, tm + TM_M + 8 * hf, s_cb, s_ends, prm.l2 + (rec_row + t_begin / ST + j) * ST, l2, wq, hf, lane);
+                } else {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     if (c <= wq) {
@@ -600,32 +634,17 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                         tc::tmem_ld_wait();
                         if (c == wq) {
                             // diagonal block: Delta_j 2^(l_i - l_j) = cb_j 2^(l_i - l_blockend).  The
-                            // second factor is >= 1; when the whole block decays by less than
-                            // 2^-96 it cannot overflow and is applied as a product, else the
-                            // exponent is formed per entry (always <= 0 where j <= i).
-                            const float up = l2 - Lend;
-                            if (Lw - Lend < 96.f) {
-                                const float rf = tc::ex2_approx(up);
-                                const uint64_t rf2 = tc::f32x2(rf, rf);
+                            // second factor is >= 1, and below 2^96
+                            const float rf = tc::ex2_approx(l2 - Lend);
+                            const uint64_t rf2 = tc::f32x2(rf, rf);
 #pragma unroll
-                                for (int q = 0; q < 8; ++q) {
-                                    const uint64_t cb = (q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x;
-                                    float2 m = tc::f32x2_get(tc::f32x2_mul(
-                                        tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rf2));
-                                    if (16 * hf + 2 * q > lane) m.x = 0.f;
-                                    if (16 * hf + 2 * q + 1 > lane) m.y = 0.f;
-                                    pk[q] = tc::pack_bf16x2(m.x, m.y);
-                                }
-                            } else {
-#pragma unroll
-                                for (int q = 0; q < 8; ++q) {
-                                    const float2 cb = tc::f32x2_get((q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x);
-                                    float m0 = __uint_as_float(cur[2 * q]) * tc::ex2_approx(up + tc::lg2_approx(cb.x));
-                                    float m1 = __uint_as_float(cur[2 * q + 1]) * tc::ex2_approx(up + tc::lg2_approx(cb.y));
-                                    if (16 * hf + 2 * q > lane) m0 = 0.f;
-                                    if (16 * hf + 2 * q + 1 > lane) m1 = 0.f;
-                                    pk[q] = tc::pack_bf16x2(m0, m1);
-                                }
+                            for (int q = 0; q < 8; ++q) {
+                                const uint64_t cb = (q & 1) ? cb4[q >> 1].y : cb4[q >> 1].x;
+                                float2 m = tc::f32x2_get(tc::f32x2_mul(
+                                    tc::f32x2_mul(f32x2_bits(cur[2 * q], cur[2 * q + 1]), cb), rf2));
+                                if (16 * hf + 2 * q > lane) m.x = 0.f;
+                                if (16 * hf + 2 * q + 1 > lane) m.y = 0.f;
+                                pk[q] = tc::pack_bf16x2(m.x, m.y);
                             }
                         } else {
                             // l at the end of column block c, relative to the start of my block
@@ -641,6 +660,7 @@ ssd_tiles_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_consta
                         }
                         tc::tmem_st8(tm + TM_M + c * 16 + 8 * hf, pk);
                     }
+                }
                 }
                 tc::tc_fence_before();
                 tc::mbar_arrive(&bars->g_free);

@@ -5,7 +5,8 @@
 //   l2[(b*H + h)*Lpad + t] = l_t          (for the run kernel: the row factor of its decay mask, below)
 //   rec[((b*H + h)*ntile + tile)] = one record per 128-token tile, copied to shared memory as a block:
 //       wp[128]  W(Delta_t 2^(l_last - l_t))      weight of token t in the tile's end state
-//       cb[128]  Delta_t 2^(l_ref - l_t)          weight of token t as a column of the decay mask
+//       cb[128]  Delta_t 2^(l_ref - l_t)          weight of token t as a column of the decay mask; in a block that
+//                                                 decays by 2^-96 and more (block_fast) Delta_t itself
 //       ends[4]  l at the end of each 32-token block (ends[3] = l_last)
 // l_ref is l at the end of t's 32-token block; for the run kernel (ScalarsArgs::aux) the tile's reference while there is one
 // (tile_one_ref).  Exponents to the block's or the tile's end are <= 0.
@@ -43,6 +44,11 @@ static_assert(sizeof(TileScalars) % 16 == 0, "tile records are moved by 16-byte 
 __host__ __device__ inline bool tile_one_ref(float l_last) { return fabsf(l_last) < 188.f; }
 __host__ __device__ inline float tile_ref(float l_last) { return l_last > -176.f ? 0.5f * l_last : l_last + 88.f; }
 
+// A 32-token block whose decay factors cannot be taken apart: Delta_t 2^(l_blockend - l_t) of its first tokens leaves
+// fp32's range (from 2^-126 on, less for a small Delta_t), and the mask's diagonal needs Delta_t back.  Its column
+// weights are Delta_t, and whoever reads them forms 2^(l - l_t) from the l array (exponents <= 0).
+__host__ __device__ inline bool block_fast(float l_beg, float l_end) { return !(l_beg - l_end < 96.f); }
+
 // What the row factors, and with them the column weights, of rows in block w refer to: the tile's reference (the
 // column weights as they are); the start of the row block (column weights times a factor per block); where even a
 // block decays by 2^-96, nothing (entries are formed one by one).
@@ -50,7 +56,7 @@ enum MaskMode { MASK_TILE, MASK_BLOCKS, MASK_ENTRIES };
 __host__ __device__ inline int mask_mode(const float *ends, int w)
 {
     if (tile_one_ref(ends[3])) return MASK_TILE;
-    return (w ? ends[w - 1] : 0.f) - ends[w] < 96.f ? MASK_BLOCKS : MASK_ENTRIES;
+    return block_fast(w ? ends[w - 1] : 0.f, ends[w]) ? MASK_ENTRIES : MASK_BLOCKS;
 }
 
 struct ScalarsArgs {
@@ -127,16 +133,16 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
         const float excl = incl - run;
         const float l_last = __shfl_sync(0xffffffffu, incl, 31);
         const float l_blk = __shfl_sync(0xffffffffu, incl, lane | 7);   // 8 lanes = one 32-token block
+        const float l_prev = __shfl_sync(0xffffffffu, incl, (lane & 24) - 1);          // (block 0: any lane)
+        const float l_beg = lane < 8 ? 0.f : l_prev;
         float l_ref = l_blk, l_row = 0.f;                    // what column weights and row factors refer to
-        bool has_ref = false, rows = false;
+        bool has_ref = false;
         if (ONE_REF) {
-            const float l_prev = __shfl_sync(0xffffffffu, incl, (lane & 24) - 1);      // (block 0: any lane)
-            const float l_beg = lane < 8 ? 0.f : l_prev;
             has_ref = tile_one_ref(l_last);
             if (has_ref) l_ref = tile_ref(l_last);
             l_row = has_ref ? l_ref : l_beg;
-            rows = has_ref || l_beg - l_blk < 96.f;
         }
+        const bool fast = !has_ref && block_fast(l_beg, l_blk);
         float lv[4], cb[4];
         uint32_t wp[4];
 #pragma unroll
@@ -146,11 +152,11 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
             const __nv_bfloat16 w_hi = __float2bfloat16_rn(w);
             wp[i] = (uint32_t)__bfloat16_as_ushort(w_hi) |
                     ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(w - __bfloat162float(w_hi))) << 16);
-            cb[i] = d[i] * exp2f(l_ref - lv[i]);
+            cb[i] = fast ? d[i] : d[i] * exp2f(l_ref - lv[i]);
         }
         TileScalars *rec = a.rec + out[q];
         if (ONE_REF) {
-            if (rows) {
+            if (!fast) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) lv[i] = exp2f(lv[i] - l_row);
             }

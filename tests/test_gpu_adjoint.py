@@ -19,8 +19,7 @@ def test_weight_gradients_at_the_edges_of_the_adjoint(B, L, H, G, strong):
     cfg = tb.cfg_of(B=B, L=L, H=H, G=G, h0_std=0.3)
     inp = synth.make_inputs(cfg, seed=600 + L)
     if strong:        # the last head halves 16 * 0.149 * 32 / ln 2 = 110 times per 32 tokens (+- a few): past the
-        # 96 where factors are applied one by one, short of the 126 at which the tile records' fp32 weights
-        # (in the forward as well) reach zero
+        # 96 where exponents are formed entry by entry
         inp["A"] = -torch.linspace(4.0, 16.0, H)
         inp["dt_bias"] = torch.full((H,), float(np.log(np.expm1(0.149))))
         inp["dt"] = 0.1 * inp["dt"]
