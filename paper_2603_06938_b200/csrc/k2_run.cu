@@ -51,7 +51,9 @@ struct __align__(16) TileRec {
 struct __align__(16) RunSmall {
     TileRec sc[NHD];         // copied in by the TMA warp
     RunBars bars;
-    float rest[NCW];         // split launch: per warp, log2 decay over the leading tiles that are left
+    // split launch: per warp, log2 decay over all leading tiles, and over those worked so far: summed in the same order, so
+    // that the difference is 0 at the last one (a remainder counted down keeps every subtraction's rounding)
+    float run_total[NCW], run_done[NCW];
     uint32_t tmem_slot;
     int abort_flag;
 };
@@ -560,12 +562,13 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
         //   H_end = 2^(sum of l_last over the run) H_in + sum_tiles (w' . X)^T Btilde.
         if (SPLIT && n_pre > 0 && has_s) {
             const TileScalars *rec0 = prm.rec + rec_base + (int64_t)(head0 + hs) * rec_hstride + t_begin / ST;
-            float rest = 0.f;
-            for (int jr = 0; jr < n_pre; ++jr) rest += rec0[jr].ends[3];
-            const float dec = tc::ex2_approx(rest);
+            float total = 0.f;
+            for (int jr = 0; jr < n_pre; ++jr) total += rec0[jr].ends[3];
+            const float dec = tc::ex2_approx(total);
 #pragma unroll
             for (int q = 0; q < 16; ++q) Hst[q] = tc::f32x2_mul(Hst[q], tc::f32x2(dec, dec));
-            sm->rest[uwarp] = rest;
+            sm->run_total[uwarp] = total;
+            sm->run_done[uwarp] = 0.f;
             __syncwarp();
         }
 
@@ -594,10 +597,10 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
             float f = scs->aux.from_ref;
             if (hs ? blocks1 : blocks0) f = tc::ex2_approx(scs->ends[3] - scs->ends[sub]);
             if (SPLIT && j < n_pre) {
-                const float rest = sm->rest[uwarp] - scs->ends[3];
+                const float done = sm->run_done[uwarp] + scs->ends[3];
                 __syncwarp();
-                sm->rest[uwarp] = rest;
-                f *= tc::ex2_approx(rest);
+                sm->run_done[uwarp] = done;
+                f *= tc::ex2_approx(sm->run_total[uwarp] - done);
                 p.dec = 1.f;
             }
             const uint64_t f2 = tc::f32x2(f, f);
