@@ -363,12 +363,10 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
         }
         for (int j = 0; j < ntiles; ++j) {                   // while tile j is worked
             if (j + 1 < ntiles && (!SPLIT || j + 1 >= n_pre)) load_c(j + 1);
-            // the tile in front gives back its x slot: a full one once its y has gone out, a leading one once its
-            // w.X is done
-            if (j > 0) {
-                if (!SPLIT || j > n_pre) store_y(j - 1);
-                else tc::mbar_wait(&bars->xp_full[(j - 1) & 1], ((j - 1) >> 1) & 1, abort_flag, d_status);
-            }
+            // the tile in front gives back its x slot: a full one once its y has gone out; a leading one's w.X was
+            // done when the record of tile j was taken, which has been waited for.  (Not on xp_full: two tiles share
+            // a barrier there, and tile j + 1, whose record is out, could have completed its phase too.)
+            if (j > 0 && (!SPLIT || j > n_pre)) store_y(j - 1);
             if (j + 2 < ntiles) load_b(j + 2);
             if (leader && j > 0 && j - 1 + X_SLOTS < ntiles) {
                 tc::bulk_wait_read_all();
