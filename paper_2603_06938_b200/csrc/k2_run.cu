@@ -384,8 +384,10 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
     } else if (uwarp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer
         // The whole warp runs the loop and the waits; one elected lane issues the MMAs and the
-        // commits.  One warp issues every product: they run in the order of issue, which the
-        // regions of tensor memory that follow one another in the same columns rely on.
+        // commits.  The order of issue is relied upon where PTX promises it: products into one accumulator in one
+        // shape, a product behind a copy.  Everything else that follows in the same columns waits for a commit:
+        // MMA 2 (another shape than MMA 3) and the copy of the next Ctilde for MMA 3, MMA 1 for MMA 2, whose masked tile
+        // it overwrites.
         grid_dep_wait();
         const bool leader = tc::elect_one();
         // The products against the shared Ctilde / Btilde tiles (MMA 1, 3, 4) are issued for both heads at once:
@@ -468,6 +470,7 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
                     tc::mma_commit(&bars->dh_full);          // (MMA 4 and 3: the state may be advanced, its copy replaced)
                 }
                 __syncwarp();
+                tc::mbar_wait(&bars->dh_full, (jf + (SPLIT && n_pre > 0 ? 1 : 0)) & 1, abort_flag, d_status);
                 if (j + 1 < ntiles) copy_c(j + 1);
                 // MMA 2: Y += M X per head (A = masked tile in TMEM, 16 tokens every 16 columns)
                 tc::mbar_wait(&bars->m_full, jf & 1, abort_flag, d_status);
@@ -483,6 +486,7 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
                     tc::mma_commit(&bars->yd_full);
                 }
                 __syncwarp();
+                if (j + 1 < ntiles) tc::mbar_wait(&bars->yd_full, jf & 1, abort_flag, d_status);
             }
             // MMA 1 of the next tile needs no state
             if (j + 1 < ntiles && j + 1 >= n_pre) {

@@ -1,6 +1,6 @@
 """The waits of the SSD run kernel (csrc/k2_run.cu), restated: copy warp, product warp and two compute warps as
 programs over mbarriers, run in random order with every copy and product completing as late or as early as it
-likes.  A wait names the phase it means; the hardware compares one parity bit, so a barrier that has gone
+likes (products and tensor-memory copies in the order of issue where PTX promises that).  A wait names the phase it means; the hardware compares one parity bit, so a barrier that has gone
 more than one phase past it would be waited for until the limit.  Everything in flight holds the memory it reads
 and writes: nobody may touch that before a wait has seen it complete.
 
@@ -91,11 +91,14 @@ def product_warp(nt, n_pre):
                 yield "wait", ("y_staged", (jf - 1) % Y_BARS), (jf - 1) // Y_BARS
             yield "tc", "mma", ("Y", 128), ("C", ("h",)), ("Y",)
             yield "commit", ("dh_full",)
+            yield "wait", ("dh_full",), jf + (n_pre > 0)
             if j + 1 < nt:
                 yield from copy_c(j + 1)
             yield "wait", ("m_full",), jf
             yield "tc", "mma", ("Y", 64), ("G", ("x", j % X_SLOTS)), ("Y",)
             yield "commit", ("yd_full",)
+            if j + 1 < nt:
+                yield "wait", ("yd_full",), jf
         if j + 1 < nt and j + 1 >= n_pre:
             if not full:
                 yield from copy_c(j + 1)
@@ -150,6 +153,11 @@ def clash(a_reads, a_writes, b_reads, b_writes):
     return bool(set(a_writes) & (set(b_reads) | set(b_writes)) or set(a_reads) & set(b_writes))
 
 
+def in_order(before, op):
+    """Whether two tensor-core operations of one thread are promised to run in the order of issue."""
+    return op[1] == "mma" and (before[1] == "cp" or before[2] == op[2])
+
+
 def simulate(nt, n_pre, rng):
     agents = [copy_warp(nt, n_pre), product_warp(nt, n_pre)]
     agents += [compute_warp(nt, n_pre, scale) for scale in (rng.random() < 0.3,) for _ in range(WARPS)]
@@ -186,7 +194,7 @@ def simulate(nt, n_pre, rng):
             free(op, op[2], op[3])
             copies.append(op)
         elif op[0] == "tc":
-            free(op, op[3], op[4], lambda before: True)
+            free(op, op[3], op[4], lambda before: in_order(before, op))
             queue.append(op)
         elif op[0] == "commit":
             queue.append(op)
