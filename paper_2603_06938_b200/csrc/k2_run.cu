@@ -589,28 +589,31 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
             const bool blocks0 = sc0->aux.blocks != 0.f, blocks1 = sc1->aux.blocks != 0.f;
             load_weights(p.w[0], sc0->cb + 32 * sub, lane);
             load_weights(p.w[1], sc1->cb + 32 * sub, lane);
-            if (blocks0 || blocks1) {                        // weights of a fast block's columns come without their decay
-                if (mask_mode(sc0->ends, sub) == MASK_ENTRIES) decay_weights(p.w[0], sc0, sub, lane);
-                if (mask_mode(sc1->ends, sub) == MASK_ENTRIES) decay_weights(p.w[1], sc1, sub, lane);
-            }
             p.row = sce->row[i];
             p.dec = scs->aux.total;
-            // from where the column weights refer to, to the end of the tile (leading tile: of the run)
-            float f = scs->aux.from_ref;
-            if (hs ? blocks1 : blocks0) f = tc::ex2_approx(scs->ends[3] - scs->ends[sub]);
+            p.pre = 1.f;
+            p.entries = false;
+            float lead = 1.f;                                // leading tiles: from the end of the tile to the end of the run
             if (SPLIT && j < n_pre) {
                 const float done = sm->run_done[uwarp] + scs->ends[3];
                 __syncwarp();
                 sm->run_done[uwarp] = done;
-                f *= tc::ex2_approx(sm->run_total[uwarp] - done);
+                lead = tc::ex2_approx(sm->run_total[uwarp] - done);
                 p.dec = 1.f;
             }
-            const uint64_t f2 = tc::f32x2(f, f);
+            // w.X: from where the column weights refer to, to the end of the tile
+            auto take_wx = [&](float f) {
+                const uint64_t f2 = tc::f32x2(f, f);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) p.wx.v[r] = tc::f32x2_mul(f2, hs ? p.w[1].v[r] : p.w[0].v[r]);
-            p.pre = 1.f;
-            p.entries = false;
-            if (blocks0 || blocks1) {
+                for (int r = 0; r < 4; ++r) p.wx.v[r] = tc::f32x2_mul(f2, hs ? p.w[1].v[r] : p.w[0].v[r]);
+            };
+            if (!(blocks0 || blocks1)) {
+                take_wx(scs->aux.from_ref * lead);
+            } else {
+                // weights of a fast block's columns come without their decay
+                if (mask_mode(sc0->ends, sub) == MASK_ENTRIES) decay_weights(p.w[0], sc0, sub, lane);
+                if (mask_mode(sc1->ends, sub) == MASK_ENTRIES) decay_weights(p.w[1], sc1, sub, lane);
+                take_wx(((hs ? blocks1 : blocks0) ? tc::ex2_approx(scs->ends[3] - scs->ends[sub]) : scs->aux.from_ref) * lead);
                 const int m0 = mask_mode(sc0->ends, wq), m1 = mask_mode(sc1->ends, wq), me = he ? m1 : m0;
                 const float Lw0 = wq ? sc0->ends[wq - 1] : 0.f, Lw1 = wq ? sc1->ends[wq - 1] : 0.f;
                 const float f0 = m0 == MASK_BLOCKS ? tc::ex2_approx(Lw0 - sc0->ends[sub]) : 1.f;
