@@ -36,16 +36,17 @@ struct TileAux {        // what follows from a tile's block ends, so that no thr
 };
 static_assert(sizeof(TileScalars) % 16 == 0, "tile records are moved by 16-byte bulk copies");
 
-
 // The forward's decay mask in two factors per entry: exp(l_t - l_s) = 2^(l_t - ref) 2^(ref - l_s), a row factor and a
-// column weight, with one reference for the whole tile as long as the tile decays by less than 2^-188: half way, or
-// where the column weights stay below 2^88 (sums over the tile are finite while the plain ones are below
-// 2^39), the row factors below 2^100.  A head that decays faster takes the blockwise form, some 10 % slower.
-__host__ __device__ inline bool tile_one_ref(float l_last) { return fabsf(l_last) < 188.f; }
-__host__ __device__ inline float tile_ref(float l_last) { return l_last > -176.f ? 0.5f * l_last : l_last + 88.f; }
+// column weight, with one reference for the whole tile, half way, as long as the tile decays by less than 2^-176, and
+// from block to block beyond that (some 10 % slower).  What the factors take of the exponents is lost to magnitudes: entries
+// C.B Delta and states keep bf16's bits from 2^-38 on (factors down to 2^-88), readouts are finite up to 2^31 (up to
+// 2^88, and 2^96 inside a block).  A bound of 2^-128 here and 2^-64 there would leave 2^-62 and 2^56: calls with a head that
+// decays by 2^-64 to 2^-96 a block then took up to 1.2 times as long (4 x 8192 tokens, 64 heads: 320 -> 392 us).
+__host__ __device__ inline bool tile_one_ref(float l_last) { return fabsf(l_last) < 176.f; }
+__host__ __device__ inline float tile_ref(float l_last) { return 0.5f * l_last; }
 
-// A 32-token block whose decay factors cannot be taken apart: Delta_t 2^(l_blockend - l_t) of its first tokens leaves
-// fp32's range (from 2^-126 on, less for a small Delta_t), and the mask's diagonal needs Delta_t back.  Its column
+// A 32-token block whose decay factors are not taken apart: Delta_t 2^(l_blockend - l_t) of its first tokens may leave
+// fp32's range (at 2^-126, before that for a small Delta_t), and the mask's diagonal needs Delta_t back.  Its column
 // weights are Delta_t, and whoever reads them forms 2^(l - l_t) from the l array (exponents <= 0).
 __host__ __device__ inline bool block_fast(float l_beg, float l_end) { return !(l_beg - l_end < 96.f); }
 

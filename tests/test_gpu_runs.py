@@ -1,6 +1,6 @@
 """The SSD kernel for long runs of tiles at its edges: six tiles (the fewest it takes) and one more token, odd head
 counts, two groups, leading tiles, segments, given states; heads that decay too fast for one reference per tile
-(more than 2^-188 over its 128 tokens), and for products of factors at all (2^-96 over 32)."""
+(2^-176 and more over its 128 tokens), and for products of factors at all (2^-96 over 32)."""
 import math
 
 import numpy as np
@@ -84,3 +84,29 @@ def test_leading_tiles_hand_over_the_state_of_fast_heads():
             got, ref = (a[b, :, i].reshape(L // 128, 128, 64)[1:, :48].reshape(L // 128 - 1, -1)
                         for a in (y.cpu()[:, :, heads].double().numpy(), y_ref))
             assert np.abs((got * ref).sum(1) / (ref * ref).sum(1) - 1.0).max() <= 8e-3
+
+
+@pytest.mark.parametrize("bc_scale,x_scale", [(2.0 ** 10, 2.0 ** 4), (2.0 ** -17, 1.0)])
+def test_range_of_magnitudes(bc_scale, x_scale):
+    """Readouts of some 2^25, and entries C.B Delta of some 2^-35: heads whose factors are the furthest apart, at 2^-100 to
+    2^-372 a tile (2^-93 a block), on the kernel for six tiles and more."""
+    B, L, H = 38, 900, 8
+    cfg = synth.LayerConfig("runs", "bf16", B, L, 32, H, 64, 128, 1, 4, 2, 128)
+    inp = synth.make_inputs(cfg, seed=78)
+    inp["D"] = None
+    inp["A"][:] = -16.0
+    step = torch.tensor([100.0, 140.0, 172.0, 180.0, 187.0, 190.0, 300.0, 372.0]) * (math.log(2.0) / (16 * 128))
+    inp["dt_bias"] = torch.log(torch.expm1(step))
+    inp["dt"] *= 0.01
+    inp["x"] *= x_scale
+    bc = (bc_scale * torch.randn(B, L, cfg.S, generator=torch.Generator().manual_seed(79))).to(torch.bfloat16)
+    h = hp.create_handle(cfg)
+    w, keep = hp.device_weights(inp)
+    assert sb.swimba_ssd_segments(h, B, L) == 1
+    y, hf = torch.empty(B, L, H, 64, dtype=torch.bfloat16, device="cuda"), torch.empty(B, H, 64, 128, device="cuda")
+    ws = torch.empty(sb.swimba_workspace_bytes(h, B, L), dtype=torch.uint8, device="cuda")
+    sb.swimba_ssd(h, w, hp.dev(inp["x"]), hp.dev(bc), hp.dev(inp["dt"]), None, B, L, y, hf, ws)
+    assert sb.swimba_status(h) == 0
+    sb.swimba_destroy(h)
+    y_ref, h_ref = oracle.ssm_recurrence(*(synth.f64(t) for t in (inp["x"], bc, inp["dt"], inp["A"], inp["dt_bias"])))
+    hp.check_outputs(cfg, inp, y.cpu(), hf.cpu(), dict(y=y_ref, h_final=h_ref), *hp.tolerances(cfg))
