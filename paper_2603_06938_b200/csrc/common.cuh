@@ -17,7 +17,7 @@ enum Stage {
     STAGE_MIX_SLOTS = 5, STAGE_PROJECT_SIMT = 6, STAGE_SSD_SEQUENTIAL = 7, STAGE_DECODE_UPDATE = 8,
     STAGE_SSD_TILES = 9, STAGE_SEGMENT_SCAN = 10, STAGE_SSD_SCALARS = 11, STAGE_SLOT_STREAMS = 12,
     STAGE_SLOT_SUM = 13, STAGE_PROJECT_SMALL = 14, STAGE_CONV = 15, STAGE_GATED_NORM = 16,
-    STAGE_DT_COLUMNS = 17, STAGE_SSD_ADJOINT = 18, STAGE_DPI_DG = 20,
+    STAGE_DT_COLUMNS = 17, STAGE_SSD_ADJOINT = 18, STAGE_CLEAR = 19, STAGE_DPI_DG = 20,
     STAGE_DW_ROUTER = 21, STAGE_DW_EXPERT = 22, STAGE_ADJOINT_STATES = 23, STAGE_SSD_STATE = 24,
 };
 

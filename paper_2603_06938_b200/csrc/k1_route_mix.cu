@@ -844,8 +844,9 @@ int launch_zero(LaunchCtx &ctx, const ZeroRegions &z, int sm_count)
     size_t most = 0;
     for (size_t b : z.bytes) most = std::max(most, b);
     const size_t blocks = std::min<size_t>((most / 16 + 255) / 256, (size_t)sm_count * 8);
+    ctx.begin(STAGE_CLEAR);
     launch_kernel(zero_kernel, dim3((unsigned)std::max<size_t>(blocks, 1)), dim3(256), 0, ctx.stream, false, z);
-    ctx.launches++;
+    ctx.end();
     return cudaGetLastError() == cudaSuccess ? SWIMBA_OK : SWIMBA_ERR_CUDA;
 }
 

@@ -131,3 +131,18 @@ def test_weight_gradients_without_step_sizes_or_initial_state():
                                   k=cfg.k, G=cfg.G, h0=None, forced_idx=idx.numpy())
     assert rel_per_expert(dWe, ref["dW_e"]) <= 2e-2
     assert np.abs(dWr.double().numpy() - ref["dW_r"]).max() <= 2e-2 * np.abs(ref["dW_r"]).max()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_profile_names_every_kernel_of_a_gradient_call(dtype):
+    cfg = cfg_of(dtype)
+    inp = synth.make_inputs(cfg, seed=7)
+    h = hp.create_handle(cfg)
+    w, keep = hp.device_weights(inp)
+    u, x, dt = hp.dev(inp["u"]), hp.dev(inp["x"]), hp.dev(inp["dt"])
+    dWr, dWe = torch.empty(cfg.E, cfg.F, device="cuda"), torch.empty(cfg.E, cfg.S, cfg.F, device="cuda")
+    ws = torch.empty(sb.swimba_backward_workspace_bytes(h, cfg.B, cfg.L), dtype=torch.uint8, device="cuda")
+    sb.swimba_profile(h, True)
+    sb.swimba_backward_weights(h, w, u, x, dt, None, torch.ones_like(x), cfg.B, cfg.L, dWr, dWe, None, ws)
+    assert len(sb.swimba_profile_read(h)) == sb.swimba_last_launch_count(h)
+    sb.swimba_destroy(h)
