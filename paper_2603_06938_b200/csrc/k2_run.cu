@@ -165,51 +165,59 @@ __device__ __forceinline__ void mask_block(uint32_t taddr, const BlockWeights (&
     }
 }
 
-// The same where a 32-token block of a head decays by 2^-96 and more (block_fast): that head's entries carry the row
-// factor, and where the columns lie in such a block, exponents are formed entry by entry, all of them <= 0.
-// Records and row factors (log-decays there) of the tile from global memory: the copy in shared memory belongs
-// to the next tile.
-__device__ __forceinline__ void mask_block_entries(uint32_t taddr, const TileScalars *rec0, const TileScalars *rec1,
-                                                   const float *l2_0, const float *l2_1, int wq, int sub, int lane)
+// The same where this row block of a head decays by 2^-96 and more (block_fast; heads in `fast`, one bit each): that head's
+// entries carry the row factor 2^lr, which lane t has for row t.  On the diagonal the weights are Delta and exponents
+// are formed entry by entry, those kept all <= 0; rows and columns are the same tokens there.  4 x 8192 tokens of
+// 64 heads, one of them like that: 235 us (200 without, 218 in the tile kernel); with l and Delta read from global memory where
+// they are used 440.
+__device__ __forceinline__ void mask_block_entries(uint32_t taddr, const BlockWeights (&w)[2], const float (&lr)[2], int fast,
+                                                   bool diag, uint32_t keep, int lane)
 {
-#pragma unroll 1
-    for (int step = 0; step < 4; ++step) {                    // 16 rows x 16 columns
-        const int half = step >> 1, c = step & 1;
-        const uint32_t ta = taddr + ((uint32_t)(16 * half) << 16) + 16 * c;
-        uint32_t g[8];
-        tc::tmem_ld_16x256b_x2(ta, g);
-        tc::tmem_ld_wait();
-#pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-            const TileScalars *rec = q ? rec1 : rec0;
-            const bool diag = sub == wq;
-            const float Lw = wq ? rec->ends[wq - 1] : 0.f, Lc = rec->ends[sub];      // l before the rows, at the columns' end
-            const int mode = mask_mode(rec->ends, wq);
-            const bool fast_cols = mask_mode(rec->ends, sub) == MASK_ENTRIES;
-            const float *l2 = q ? l2_1 : l2_0;
-            uint32_t o[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {                     // rows k = e % 2, columns 8 (e / 2) ..
-                const int row = 16 * half + (lane >> 2) + 8 * (e & 1), col = 16 * c + 8 * (e >> 1) + 2 * (lane & 3);
-                const float l_i = l2[32 * wq + row];
-                float2 cb = *reinterpret_cast<const float2 *>(&rec->cb[32 * sub + col]);
-                float rf = 1.f;
-                if (fast_cols) {                              // (cb: Delta of the columns)
-                    const float2 l_s = *reinterpret_cast<const float2 *>(&l2[32 * sub + col]);
-                    const float to = mode == MASK_ENTRIES ? l_i : Lw;
-                    cb.x *= tc::ex2_approx(to - l_s.x);
-                    cb.y *= tc::ex2_approx(to - l_s.y);
-                } else if (mode == MASK_BLOCKS) {
-                    rf = tc::ex2_approx(Lw - Lc);
-                } else if (mode == MASK_ENTRIES) {
-                    rf = tc::ex2_approx(l_i - Lw) * tc::ex2_approx(Lw - Lc);
-                }
-                float m0 = __uint_as_float(g[2 * e]) * cb.x * rf, m1 = __uint_as_float(g[2 * e + 1]) * cb.y * rf;
-                if (diag && col > row) m0 = 0.f;
-                if (diag && col + 1 > row) m1 = 0.f;
-                o[e] = tc::pack_bf16x2(m0, m1);
+    for (int half = 0; half < 2; ++half) {
+        const uint32_t ta = taddr + ((uint32_t)(16 * half) << 16);
+        uint32_t g[16];
+        tc::tmem_ld_16x256b_x4(ta, g);
+        tc::tmem_ld_wait();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const bool entries = diag && (fast >> q & 1);
+            const float l = fast >> q & 1 ? lr[q] : 0.f;
+            float row[2];                                    // l of rows k, their factor where the weights have one
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                row[k] = __shfl_sync(0xffffffffu, l, 16 * half + 8 * k + (lane >> 2));
+                if (!entries) row[k] = tc::ex2_approx(row[k]);
             }
-            tc::tmem_st_16x128b_x2(ta + 8 * q, o[0], o[1], o[2], o[3]);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (diag && c > half) {                      // (above the diagonal)
+                    tc::tmem_st_16x128b_x2(ta + 8 * q + 16 * c, 0u, 0u, 0u, 0u);
+                    continue;
+                }
+                uint32_t o[4];
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    float col[2] = {0.f, 0.f};
+                    if (entries) {
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) col[e] = __shfl_sync(0xffffffffu, l, 16 * c + 8 * r + 2 * (lane & 3) + e);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const uint64_t f = entries ? tc::f32x2(tc::ex2_approx(row[k] - col[0]), tc::ex2_approx(row[k] - col[1]))
+                                                   : tc::f32x2(row[k], row[k]);
+                        const int e = 4 * (2 * c + r) + 2 * k;
+                        o[2 * r + k] = tc::f32x2_bf16(tc::f32x2_mul(f32x2_bits(g[e], g[e + 1]), tc::f32x2_mul(w[q].v[2 * c + r], f)));
+                    }
+                }
+                if (diag && c == half) {                     // the 16 x 16 block on the diagonal
+                    o[0] &= keep;
+                    o[2] = 0u;
+                    o[3] &= keep;
+                }
+                tc::tmem_st_16x128b_x2(ta + 8 * q + 16 * c, o[0], o[1], o[2], o[3]);
+            }
         }
     }
 }
@@ -581,7 +589,8 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
             float dec;             // decay of the state over the tile
             float row;             // epilogue: y = row Y + D x
             float pre;             // != 1: Y = Ctilde Hprev^T is multiplied by it before M X is added
-            bool entries;          // (MASK_ENTRIES for one of the heads)
+            int fast;              // heads with MASK_ENTRIES for these rows, one bit each; of them, if any:
+            float lr[2];           // l of row 32 wq + lane, relative to the block's start (garbage for the others)
         };
         const TileRec *const sc0 = &sm->sc[0], *const sc1 = &sm->sc[nh - 1];
         const TileRec *const scs = hs ? sc1 : sc0, *const sce = he ? sc1 : sc0;
@@ -592,7 +601,7 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
             p.row = sce->row[i];
             p.dec = scs->aux.total;
             p.pre = 1.f;
-            p.entries = false;
+            p.fast = 0;
             float lead = 1.f;                                // leading tiles: from the end of the tile to the end of the run
             if (SPLIT && j < n_pre) {
                 const float done = sm->run_done[uwarp] + scs->ends[3];
@@ -602,30 +611,36 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
                 p.dec = 1.f;
             }
             // w.X: from where the column weights refer to, to the end of the tile
-            auto take_wx = [&](float f) {
+            auto take_wx = [&](float f, const BlockWeights &w0, const BlockWeights &w1) {
                 const uint64_t f2 = tc::f32x2(f, f);
 #pragma unroll
-                for (int r = 0; r < 4; ++r) p.wx.v[r] = tc::f32x2_mul(f2, hs ? p.w[1].v[r] : p.w[0].v[r]);
+                for (int r = 0; r < 4; ++r) p.wx.v[r] = tc::f32x2_mul(f2, hs ? w1.v[r] : w0.v[r]);
             };
             if (!(blocks0 || blocks1)) {
-                take_wx(scs->aux.from_ref * lead);
+                take_wx(scs->aux.from_ref * lead, p.w[0], p.w[1]);
             } else {
-                // weights of a fast block's columns come without their decay
-                if (mask_mode(sc0->ends, sub) == MASK_ENTRIES) decay_weights(p.w[0], sc0, sub, lane);
-                if (mask_mode(sc1->ends, sub) == MASK_ENTRIES) decay_weights(p.w[1], sc1, sub, lane);
-                take_wx(((hs ? blocks1 : blocks0) ? tc::ex2_approx(scs->ends[3] - scs->ends[sub]) : scs->aux.from_ref) * lead);
                 const int m0 = mask_mode(sc0->ends, wq), m1 = mask_mode(sc1->ends, wq), me = he ? m1 : m0;
                 const float Lw0 = wq ? sc0->ends[wq - 1] : 0.f, Lw1 = wq ? sc1->ends[wq - 1] : 0.f;
-                const float f0 = m0 == MASK_BLOCKS ? tc::ex2_approx(Lw0 - sc0->ends[sub]) : 1.f;
-                const float f1 = m1 == MASK_BLOCKS ? tc::ex2_approx(Lw1 - sc1->ends[sub]) : 1.f;
+                // (weights of a fast block's columns come without their decay: w.X needs it, its own rows do not)
+                BlockWeights w0 = p.w[0], w1 = p.w[1];
+                if (mask_mode(sc0->ends, sub) == MASK_ENTRIES) decay_weights(w0, sc0, sub, lane);
+                if (mask_mode(sc1->ends, sub) == MASK_ENTRIES) decay_weights(w1, sc1, sub, lane);
+                take_wx(((hs ? blocks1 : blocks0) ? tc::ex2_approx(scs->ends[3] - scs->ends[sub]) : scs->aux.from_ref) * lead,
+                        w0, w1);
+                const float f0 = m0 == MASK_TILE ? 1.f : tc::ex2_approx(Lw0 - sc0->ends[sub]);
+                const float f1 = m1 == MASK_TILE ? 1.f : tc::ex2_approx(Lw1 - sc1->ends[sub]);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    p.w[0].v[r] = tc::f32x2_mul(p.w[0].v[r], tc::f32x2(f0, f0));
-                    p.w[1].v[r] = tc::f32x2_mul(p.w[1].v[r], tc::f32x2(f1, f1));
+                    if (!(sub == wq && m0 == MASK_ENTRIES)) p.w[0].v[r] = tc::f32x2_mul(w0.v[r], tc::f32x2(f0, f0));
+                    if (!(sub == wq && m1 == MASK_ENTRIES)) p.w[1].v[r] = tc::f32x2_mul(w1.v[r], tc::f32x2(f1, f1));
                 }
                 if (me == MASK_BLOCKS) p.pre = tc::ex2_approx(he ? Lw1 : Lw0);
                 if (me == MASK_ENTRIES) { p.pre = tc::ex2_approx(p.row); p.row = 1.f; }
-                p.entries = m0 == MASK_ENTRIES || m1 == MASK_ENTRIES;
+                if (m0 == MASK_ENTRIES || m1 == MASK_ENTRIES) {
+                    p.fast = (m0 == MASK_ENTRIES ? 1 : 0) | (m1 == MASK_ENTRIES ? 2 : 0);
+                    p.lr[0] = sc0->row[i] - Lw0;
+                    p.lr[1] = sc1->row[i] - Lw1;
+                }
             }
             tc::fence_proxy_async_smem();                    // (the record is refilled by a copy next)
             arrive(&bars->rec_free);
@@ -672,10 +687,8 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
                     for (int q = 0; q < 16; ++q) zero[q] = 0u;
                     tc::tmem_st16(tm_g, zero);
                     tc::tmem_st16(tm_g + 16, zero);
-                } else if (cur.entries) {
-                    const int64_t r = rec_base + (int64_t)head0 * rec_hstride + t_begin / ST + j;
-                    const int64_t r1 = r + (nh == 2 ? rec_hstride : 0);
-                    mask_block_entries(tm_g, prm.rec + r, prm.rec + r1, prm.l2 + r * ST, prm.l2 + r1 * ST, wq, sub, lane);
+                } else if (cur.fast) {
+                    mask_block_entries(tm_g, cur.w, cur.lr, cur.fast, sub == wq, keep, lane);
                 } else if (sub < wq) {
                     mask_block<false>(tm_g, cur.w, 0u);
                 } else {
