@@ -87,8 +87,7 @@ size_t ssd_workspace_bytes(int B, int L, int H, int G, int chunk, int sm_count);
 int ssd_segment_len(int B, int L, int H, int G, int chunk, int sm_count);
 // Clears up to four regions (16-byte aligned, sizes multiples of 16; null: none) as the first kernel of a gradient call;
 // the kernel behind it may be launched programmatically and waits with grid_dep_wait.  Four memsets in its place cost
-// 8 us more at 4 x 8192 tokens (795 -> 787), and 122 -> 115, 183 -> 171 and 180 -> 171 us at smaller calls: mostly the gaps between
-// them.  A forward clears its histogram alone and keeps the memset: with this kernel and the router launched behind it
+// 8 us more at 4 x 8192 tokens (795 -> 787): mostly the gaps between them.  A forward clears its histogram alone and keeps the memset: with this kernel and the router launched behind it
 // programmatically calls went anywhere between 0.973 and 1.034 of their rate.
 struct ZeroRegions { void *p[4]; size_t bytes[4]; };
 int launch_zero(LaunchCtx &ctx, const ZeroRegions &z, int sm_count);

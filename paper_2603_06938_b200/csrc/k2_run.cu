@@ -1,14 +1,16 @@
 // The chunked SSD evaluation of k2_ssd.cu for CTAs that walk many tiles in a row (same division of the work, same
-// products; names of the products and of the factors as there).  What the tile loop there waits for is shared
-// memory's data pipe: 4000 to 5500 of a tile's 5500 cycles.  So here
+// products; names of the products and of the factors as there).  What the tile loop there waits for is, as far as counters
+// and bytes tell, shared memory's data pipe: of a tile's 5500 cycles 4300 are counted as wavefronts of the CUDA cores and of
+// the tensor cores' operands, TMA's 128 KB are another 1000.  So here
 //   - w.X goes from the x slab to the tensor memory by ldmatrix and is MMA 4's A operand (no scaled copy in shared
 //     memory), Ctilde is copied to tensor memory once and is the A operand of MMA 1 and MMA 3;
 //   - G is read once for both heads, masked in place and in the fragment layout (8 weights a head and thread);
 //   - exp(l_i - l_s) = 2^(l_i - ref) 2^(ref - l_s) with one reference a tile (ssd_scalars.cuh): one product an entry, no
 //     scaling of Ctilde Hprev^T (the bf16 state copy decays to the reference), the row factor in the epilogue;
 //   - w.X of the next tile is made while MMA 2 runs, y replaces x in place, x is three tiles ahead.
-// A tile takes 4350 cycles (4500 of them counted as wavefronts of that pipe: it is the bound again), a CTA 2000 to 3500
-// more to start and to drain, so that runs of fewer than RUN_TILES tiles stay with the other kernel.
+// A tile takes 4350 cycles: 3300 counted as wavefronts (2050 of the CUDA cores, 1240 operands), 1000 for TMA by its bytes, so that
+// the pipe is the bound again.  A CTA takes 2000 to 3500 more to start and to drain: runs of fewer than RUN_TILES tiles stay
+// with the other kernel.
 #include "ssd_tiles.cuh"
 
 namespace swimba {

@@ -26,7 +26,7 @@
 // the next tile is issued under this tile's state update (it needs no state) and the mask is built before the
 // product with the carried state is waited for; fp32 work goes two to an instruction; the mask's column
 // weights are read 16 bytes at a time; w.X stays off the warps that have the longest mask rows.  4 x 8192
-// tokens of 64 heads: 228 us a call before these and with 8 leading tiles, 215 with 7, 205 with the mask
+// tokens of 64 heads (while such calls came here; they go to k2_run.cu now): 228 us a call before these and with 8 leading tiles, 215 with 7, 205 with the mask
 // first, 200 with packed pairs and the new shares of w.X, 193 with the wide reads and one barrier for x and
 // the scalars.  Measured and not taken: the streams loaded as soon as they are free (217: G then displaces
 // the products that are waited for), tensor-memory loads one block ahead (232), 112 registers (no change).
