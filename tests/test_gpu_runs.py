@@ -1,5 +1,6 @@
 """The SSD kernel for long runs of tiles at its edges: six tiles (the fewest it takes) and one more token, odd head
-counts, two groups, leading tiles, segments, given states; heads that decay too fast for one reference per tile
+counts, two groups, leading tiles, given states (and segments of two tiles, which the other kernel works: longer ones are in
+test_gpu_run_forms.py); heads that decay too fast for one reference per tile
 (2^-176 and more over its 128 tokens), and for products of factors at all (2^-96 over 32)."""
 import math
 
