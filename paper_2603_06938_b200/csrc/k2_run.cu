@@ -597,7 +597,7 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
         const TileRec *const sc0 = &sm->sc[0], *const sc1 = &sm->sc[nh - 1];
         const TileRec *const scs = hs ? sc1 : sc0, *const sce = he ? sc1 : sc0;
         auto take_rec = [&](int j, Prep &p) {
-            const bool blocks0 = sc0->aux.blocks != 0.f, blocks1 = sc1->aux.blocks != 0.f;
+            const float blocks0 = sc0->aux.blocks, blocks1 = sc1->aux.blocks;
             load_weights(p.w[0], sc0->cb + 32 * sub, lane);
             load_weights(p.w[1], sc1->cb + 32 * sub, lane);
             p.row = sce->row[i];
@@ -618,16 +618,23 @@ ssd_run_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant
 #pragma unroll
                 for (int r = 0; r < 4; ++r) p.wx.v[r] = tc::f32x2_mul(f2, hs ? w1.v[r] : w0.v[r]);
             };
-            if (!(blocks0 || blocks1)) {
+            if (blocks0 == 0.f && blocks1 == 0.f) {
                 take_wx(scs->aux.from_ref * lead, p.w[0], p.w[1]);
             } else {
-                const int m0 = mask_mode(sc0->ends, wq), m1 = mask_mode(sc1->ends, wq), me = he ? m1 : m0;
+                int m0 = blocks0 == 0.f ? MASK_TILE : MASK_BLOCKS, m1 = blocks1 == 0.f ? MASK_TILE : MASK_BLOCKS;
                 const float Lw0 = wq ? sc0->ends[wq - 1] : 0.f, Lw1 = wq ? sc1->ends[wq - 1] : 0.f;
                 // (weights of a fast block's columns come without their decay: w.X needs it, its own rows do not)
                 BlockWeights w0 = p.w[0], w1 = p.w[1];
-                if (mask_mode(sc0->ends, sub) == MASK_ENTRIES) decay_weights(w0, sc0, sub, lane);
-                if (mask_mode(sc1->ends, sub) == MASK_ENTRIES) decay_weights(w1, sc1, sub, lane);
-                take_wx(((hs ? blocks1 : blocks0) ? tc::ex2_approx(scs->ends[3] - scs->ends[sub]) : scs->aux.from_ref) * lead,
+                if (blocks0 == 2.f) {
+                    m0 = mask_mode(sc0->ends, wq);
+                    if (mask_mode(sc0->ends, sub) == MASK_ENTRIES) decay_weights(w0, sc0, sub, lane);
+                }
+                if (blocks1 == 2.f) {
+                    m1 = mask_mode(sc1->ends, wq);
+                    if (mask_mode(sc1->ends, sub) == MASK_ENTRIES) decay_weights(w1, sc1, sub, lane);
+                }
+                const int me = he ? m1 : m0;
+                take_wx(((hs ? blocks1 : blocks0) != 0.f ? tc::ex2_approx(scs->ends[3] - scs->ends[sub]) : scs->aux.from_ref) * lead,
                         w0, w1);
                 const float f0 = m0 == MASK_TILE ? 1.f : tc::ex2_approx(Lw0 - sc0->ends[sub]);
                 const float f1 = m1 == MASK_TILE ? 1.f : tc::ex2_approx(Lw1 - sc1->ends[sub]);

@@ -32,13 +32,13 @@ struct TileAux {        // what follows from a tile's block ends, so that no thr
     float to_ref;       // decay from the tile's start to its reference (1 if it has none)
     float from_ref;     // from there to the tile's end
     float total;        // over the tile
-    float blocks;       // 0: the tile has a reference, 1: it has not
+    float blocks;       // 0: the tile has a reference, 1: it has not, 2: some of its blocks are fast as well (block_fast)
 };
 static_assert(sizeof(TileScalars) % 16 == 0, "tile records are moved by 16-byte bulk copies");
 
 // The forward's decay mask in two factors per entry: exp(l_t - l_s) = 2^(l_t - ref) 2^(ref - l_s), a row factor and a
 // column weight, with one reference for the whole tile, half way, as long as the tile decays by less than 2^-176, and
-// from block to block beyond that (some 10 % slower).  What the factors take of the exponents is lost to magnitudes: entries
+// from block to block beyond that (5 to 20 % slower).  What the factors take of the exponents is lost to magnitudes: entries
 // C.B Delta and states keep bf16's bits from 2^-38 on (factors down to 2^-88), readouts are finite up to 2^31 (up to
 // 2^88, and 2^96 inside a block).  A bound of 2^-128 would leave 2^-62 at the lower end and costs 1 % of whole calls (8 x
 // 2048, 4 x 8192, 65536 and 3 x 1531 tokens), where heads lie between.
@@ -161,9 +161,10 @@ __device__ __forceinline__ void ssd_scalars_warp(const ScalarsArgs &a, int64_t u
 #pragma unroll
                 for (int i = 0; i < 4; ++i) lv[i] = exp2f(lv[i] - l_row);
             }
+            const bool any_fast = __any_sync(0xffffffffu, fast);
             if (lane == 31)
                 a.aux[out[q]] = TileAux{has_ref ? exp2f(l_ref) : 1.f, has_ref ? exp2f(l_last - l_ref) : 1.f, exp2f(l_last),
-                                        has_ref ? 0.f : 1.f};
+                                        has_ref ? 0.f : (any_fast ? 2.f : 1.f)};
         }
         reinterpret_cast<float4 *>(a.l2 + out[q] * SCALARS_TILE)[lane] = make_float4(lv[0], lv[1], lv[2], lv[3]);
         reinterpret_cast<uint4 *>(rec->wp)[lane] = make_uint4(wp[0], wp[1], wp[2], wp[3]);
